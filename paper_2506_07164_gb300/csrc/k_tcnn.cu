@@ -9,7 +9,7 @@
 // bf16 (rounded from fp32 master copies that Adam updates); every product is
 // accumulated in fp32.  One block per tile; activations stay in shared
 // memory.  Training uses a plain forward that saves activations to global
-// memory for the backward pass; inference uses a register-blocked forward.
+// memory for the backward pass; inference runs on the tensor cores.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -59,37 +59,18 @@ namespace tn {
 
 __device__ __forceinline__ float relu(float x) { return x > 0.f ? x : 0.f; }
 
-// Source of one 64 x 64 input patch: either a dense tile array, or a
-// proposal tile of a pyramid level read in place.
+// Source of the 64 x 64 input patches: a dense tile array, or the proposal
+// tiles of pyramid levels read in place.  Proposal tile t is quarter t & 3 of
+// detect tile t / 4 of the plan's item table ((image, (y0 << 16) | x0): the
+// 128 x 32 tiles of all images in order), so no search over the images.
 struct PatchSrc {
     const uint8_t* tiles;   // dense: n x 4096 bytes, or nullptr
     const ofk::Img* imgs;   // in place: image descriptors
-    const int32_t* list;    // image index per job
-    const int32_t* prefix;  // first tile of each job
-    int n_list;
+    const uint2* items;     // in place: the detect tiles
 };
 
-__device__ void load_patch(const PatchSrc& S, int t, float* in, int border) {
-    if (S.tiles) {
-        const uint8_t* p = S.tiles + (size_t)t * S0 * S0;
-        for (int i = threadIdx.x; i < S0 * S0; i += blockDim.x) in[i] = ((float)p[i] - 128.f) * (1.f / 64.f);
-        return;
-    }
-    int lo = 0, hi = S.n_list - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(S.prefix + mid) <= t) lo = mid; else hi = mid - 1;
-    }
-    const ofk::Img& I = S.imgs[__ldg(S.list + lo)];
-    const int k = t - __ldg(S.prefix + lo);
-    const int ptx = I.tiles_x * 4;
-    const int x0 = I.tile_x0 + 32 * (k % ptx) - 16, y0 = border + 32 * (k / ptx) - 16;
-    for (int i = threadIdx.x; i < S0 * S0; i += blockDim.x) {
-        const int x = x0 + (i & 63), y = y0 + (i >> 6);
-        // Pixels outside the image are 0 in the uint8 patch, i.e. -2 after normalisation.
-        const float v = (x >= 0 && x < I.w && y >= 0 && y < I.h) ? (float)I.img[(size_t)y * I.pitch + x] : 0.f;
-        in[i] = (v - 128.f) * (1.f / 64.f);
-    }
+__device__ void load_patch(const uint8_t* __restrict__ p, float* in) {
+    for (int i = threadIdx.x; i < S0 * S0; i += blockDim.x) in[i] = ((float)p[i] - 128.f) * (1.f / 64.f);
 }
 
 // out[o][y][x] = relu(b[o] + sum_c sum_k w[o][c][k] in[c][2y+ky-1][2x+kx-1])
@@ -121,8 +102,8 @@ __device__ void conv_s2(const float* __restrict__ in, int C, int Sin, const floa
 // Forward pass of tiles [0, n); logits to `logits` (may be null); when `save`
 // is set, activations to save[t * SAVE ...].
 __global__ void __launch_bounds__(THREADS)
-k_forward(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float* __restrict__ logits,
-          float* __restrict__ save, int border) {
+k_forward(const uint8_t* __restrict__ tiles, int n, const __nv_bfloat16* __restrict__ wq, float* __restrict__ logits,
+          float* __restrict__ save) {
     extern __shared__ float sm[];
     float* in = sm;
     float* a1 = in + S0 * S0;
@@ -133,7 +114,7 @@ k_forward(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float* __re
     for (int i = threadIdx.x; i < NP; i += blockDim.x) w[i] = __bfloat162float(wq[i]);
     __syncthreads();
     for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        load_patch(src, t, in, border);
+        load_patch(tiles + (size_t)t * S0 * S0, in);
         __syncthreads();
         conv_s2(in, 1, S0, w + W1, w + B1, C1, a1);
         __syncthreads();
@@ -170,151 +151,362 @@ k_forward(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float* __re
     }
 }
 
-// Inference forward, register-blocked.  Activations live in zero-padded
-// planes (no bounds tests); weights are transposed to [c][k][o] so one
-// 16-byte broadcast load serves four output channels; a thread accumulates
-// all channels of one output pixel (layers 1, 2) or four channels (layer 3).
-// Same function as k_forward; products are summed over (c, ky, kx) in the
-// same order.
-constexpr int P0 = S0 + 2, P1 = S1 + 2, P2 = S2 + 2;
-constexpr int FAST_SMEM = (P0 * P0 + C1 * P1 * P1 + C2 * P2 * P2 + A3 + NP + 32) * 4;
+// A 64 x 64 patch is 256 16-byte chunks (4 per row).  Chunk q of tile t; pixels
+// outside the image are 0.  Level images and their pitches are multiples of
+// 16 bytes, and a patch starts at a multiple of 16, so a chunk is one aligned
+// load (whole inside the row's pitch); bytes past the row's w are cleared.
+struct Patch {
+    const uint8_t* p;       // dense: the tile; in place: the level image
+    int x0, y0, w, h, pitch;  // in place; pitch 0: dense
+};
 
-__global__ void __launch_bounds__(THREADS)
-k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float* __restrict__ logits, int border) {
-    extern __shared__ __align__(16) float sm[];
-    float* in = sm;                    // P0 x P0
-    float* a1 = in + P0 * P0;          // C1 x P1 x P1
-    float* a2 = a1 + C1 * P1 * P1;     // C2 x P2 x P2
-    float* a3 = a2 + C2 * P2 * P2;     // C3 x 8 x 8
-    float* w = a3 + A3;                // transposed weights + biases + head
-    float* red = w + NP;
-    const int tid = threadIdx.x;
-    // Zero everything once: padding cells are never written afterwards.
-    for (int i = tid; i < (int)(FAST_SMEM / 4); i += blockDim.x) sm[i] = 0.f;
-    __syncthreads();
-    // w1t[k][o], w2t[c][k][o], w3t[c][k][o] at the same offsets as W1, W2, W3.
-    for (int i = tid; i < NP; i += blockDim.x) {
-        float v = __bfloat162float(wq[i]);
-        int dst = i;
-        if (i < B1) {  // W1[o][0][k]
-            const int o = i / 9, k = i % 9;
-            dst = W1 + k * C1 + o;
-        } else if (i >= W2 && i < B2) {
-            const int j = i - W2, o = j / (C1 * 9), c = (j / 9) % C1, k = j % 9;
-            dst = W2 + (c * 9 + k) * C2 + o;
-        } else if (i >= W3 && i < B3) {
-            const int j = i - W3, o = j / (C2 * 9), c = (j / 9) % C2, k = j % 9;
-            dst = W3 + (c * 9 + k) * C3 + o;
-        }
-        w[dst] = v;
+__device__ __forceinline__ Patch find_patch(const PatchSrc& S, int t) {
+    Patch P;
+    if (S.tiles) {
+        P.p = S.tiles + (size_t)t * S0 * S0;
+        P.x0 = P.y0 = P.w = P.h = P.pitch = 0;
+        return P;
     }
-    __syncthreads();
-    for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        // Input patch into the interior of the padded plane.
-        if (src.tiles) {
-            const uint8_t* p = src.tiles + (size_t)t * S0 * S0;
-            for (int i = tid; i < S0 * S0; i += blockDim.x)
-                in[((i >> 6) + 1) * P0 + (i & 63) + 1] = ((float)p[i] - 128.f) * (1.f / 64.f);
-        } else {
-            int lo = 0, hi = src.n_list - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (__ldg(src.prefix + mid) <= t) lo = mid; else hi = mid - 1;
+    const uint2 e = __ldg(S.items + (t >> 2));
+    const ofk::Img& I = S.imgs[e.x];
+    P.p = I.img;
+    P.x0 = (int)(e.y & 0xFFFFu) + 32 * (t & 3) - 16;
+    P.y0 = (int)(e.y >> 16) - 16;
+    P.w = I.w;
+    P.h = I.h;
+    P.pitch = I.pitch;
+    return P;
+}
+
+__device__ __forceinline__ uint4 load_chunk(const Patch& P, int q) {
+    if (P.pitch == 0) {
+        const uint8_t* p = P.p + 16 * q;
+        if ((reinterpret_cast<uintptr_t>(P.p) & 15) == 0) return __ldg(reinterpret_cast<const uint4*>(p));
+        uint32_t v[4] = {0u, 0u, 0u, 0u};  // a caller's unaligned tile array
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i >> 2] |= (uint32_t)__ldg(p + i) << (8 * (i & 3));
+        return make_uint4(v[0], v[1], v[2], v[3]);
+    }
+    const int x = P.x0 + 16 * (q & 3), y = P.y0 + (q >> 2);
+    if (x < 0 || x >= P.w || y < 0 || y >= P.h) return make_uint4(0u, 0u, 0u, 0u);
+    uint4 v = __ldg(reinterpret_cast<const uint4*>(P.p + (size_t)y * P.pitch + x));
+    const int n = P.w - x;  // valid bytes
+    if (n < 16) {
+        uint32_t* m = &v.x;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) m[i] &= n >= 4 * i + 4 ? 0xFFFFFFFFu : n <= 4 * i ? 0u : (1u << (8 * (n - 4 * i))) - 1u;
+    }
+    return v;
+}
+
+// ---------------------------------------------------------------------------
+// Inference on the tensor cores, without losing precision.
+//
+// An fp32 activation is the exact sum of three bf16 numbers (its leading 8
+// significant bits, the next 8, the last 8: truncations), the weights are bf16
+// already, so every product of a layer is an exact bf16 product and the layer
+// is a matrix product with three times the depth.  The tensor cores' fp32
+// accumulation truncates, though: a long chain of the leading parts would bias
+// the logits (5e-7 of their norm).  So the leading parts' products of one
+// 16-deep step are summed from zero and added to the running sum with an fp32
+// addition; only the lower parts, 2^-8 and 2^-16 of the size, stay in a chain.
+// Against 64 bits the logits are 3e-8 off (norms, committed network), the fp32
+// FMA chain of the training forward 8.4e-8.
+//
+// The layers are far too narrow (8 or 16 channels) for tcgen05's 128-row
+// tiles to be filled by channels, and a sum from zero per step would cost a
+// TMEM read per step, so warp-level m16n8k16 products with pixels as rows and
+// channels as columns carry the work; all weight fragments stay in registers.
+// Activations are stored channels-last, 8 channels = 16 bytes per pixel, one
+// plane per part (and per channel half), columns split by parity, so that
+// each tap of 8 neighbouring output pixels is 128 contiguous bytes: one 8 x 8
+// matrix of ldmatrix, no im2col copy and no bank conflict.  The input (exact
+// in bf16) keeps rows of pixels: an output's three taps of a row and a zero
+// weight are two aligned words.
+//
+// A block of 8 warps takes one tile at a time, two blocks per SM; a layer's
+// planes have buffers of their own, so a tile needs two barriers, and the next
+// tile's pixels are staged while layer 2 runs.  Bound by shared memory (65 % of
+// its wavefront rate; tensor pipe 36 %, issue 50 %).  16,384 patches: 755 us as
+// fp32 FMAs over shared-memory operands, 397 us register-blocked with packed
+// fp32 FMAs (the smem reads of the weights then bound it), 240 us here.
+constexpr int FWD_THREADS = 256, FWD_BLOCKS = 2;
+constexpr int TI_ROW = 48, TI_X = 4;                       // input rows: words per row (pixel pairs), word of pixel 0
+constexpr int TI_BYTES = 65 * TI_ROW * 4;                  // row 0: zeros
+constexpr int T1_ROW = 33, T1_O = 17;                      // layer-1 rows: 17 even padded columns, then 16 odd ones
+constexpr int T1_PLANE = 33 * T1_ROW * 16;                 // one part: 33 rows (row 0: zeros), 8 channels
+constexpr int T2_ROW = 21, T2_O = 13;                      // layer-2 rows: 9 even columns, (gap), 8 odd ones
+constexpr int T2_PLANE = 17 * T2_ROW * 16;                 // one part and channel half: 17 rows
+constexpr int FWD_RED = 2 * 4 * C3;                        // per tile parity and row pair: channel sums
+constexpr int FWD_SMEM = TI_BYTES + 3 * T1_PLANE + 6 * T2_PLANE + FWD_RED * 4;
+static_assert(TI_BYTES % 16 == 0 && T1_PLANE % 16 == 0 && T2_PLANE % 16 == 0, "16-byte rows for ldmatrix");
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm2(uint32_t (&r)[2], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"(a)
+                 : "memory");
+}
+// d = a b + c, a 16 x 16 (pixels x depth), b 16 x 8 (depth x channels).
+__device__ __forceinline__ void mma16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2], const float (&c)[4]) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%10, %11, %12, %13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+__device__ __forceinline__ void mma8(float (&d)[4], const uint32_t (&a)[2], uint32_t b, const float (&c)[4]) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%7, %8, %9, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(b), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
+}
+
+// The three bf16 parts of two non-negative activations (channels 2t, 2t + 1),
+// packed: truncations, so that finite values never round up to infinity; an
+// infinity is its own leading part.
+__device__ __forceinline__ void split3(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+    auto rest = [](float v) {
+        const float r = v - __uint_as_float(__float_as_uint(v) & 0xFFFF0000u);
+        return r;
+    };
+    const bool xi = x > 3.402823466e38f, yi = y > 3.402823466e38f;
+    const float rx = xi ? 0.f : rest(x), ry = yi ? 0.f : rest(y);
+    const float sx = rest(rx), sy = rest(ry);
+    h = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
+    m = __byte_perm(__float_as_uint(rx), __float_as_uint(ry), 0x7632);
+    l = __byte_perm(__float_as_uint(sx), __float_as_uint(sy), 0x7632);
+}
+
+// Two consecutive input channels (or taps) of a weight matrix as one fragment word.
+__device__ __forceinline__ uint32_t pack_w(const __nv_bfloat16* __restrict__ w, int i0, int i1) {
+    const uint32_t lo = i0 >= 0 ? __bfloat16_as_ushort(w[i0]) : 0u, hi = i1 >= 0 ? __bfloat16_as_ushort(w[i1]) : 0u;
+    return lo | (hi << 16);
+}
+
+// Chunk q (16 pixels) of the patch as bf16 (v - 128) / 64, exact, into the input plane.
+__device__ __forceinline__ void stage_bf16(uint32_t* __restrict__ in, int q, const uint4& v) {
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    uint32_t o[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t wd = u[i >> 1];
+        const float a = fmaf(__uint_as_float(__byte_perm(wd, 0x4B000000u, (i & 1) ? 0x7552 : 0x7550)), 1.f / 64.f, -131074.f);
+        const float b = fmaf(__uint_as_float(__byte_perm(wd, 0x4B000000u, (i & 1) ? 0x7553 : 0x7551)), 1.f / 64.f, -131074.f);
+        o[i] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+    }
+    uint4* d = reinterpret_cast<uint4*>(in + ((q >> 2) + 1) * TI_ROW + TI_X + 8 * (q & 3));
+    d[0] = make_uint4(o[0], o[1], o[2], o[3]);
+    d[1] = make_uint4(o[4], o[5], o[6], o[7]);
+}
+
+__global__ void __launch_bounds__(FWD_THREADS, FWD_BLOCKS)
+k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float* __restrict__ logits) {
+    extern __shared__ __align__(128) uint8_t fsm[];
+    uint32_t* const in = reinterpret_cast<uint32_t*>(fsm);
+    uint8_t* const p1 = fsm + TI_BYTES;
+    uint8_t* const p2 = p1 + 3 * T1_PLANE;
+    float* const red = reinterpret_cast<float*>(p2 + 6 * T2_PLANE);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t4 = lane & 3;
+    // Zero the planes once: the pad words are never written afterwards.
+    for (int i = tid; i < (TI_BYTES + 3 * T1_PLANE + 6 * T2_PLANE) / 16; i += FWD_THREADS)
+        reinterpret_cast<uint4*>(fsm)[i] = make_uint4(0u, 0u, 0u, 0u);
+
+    // Weight fragments.  Layer 1: depth 4 ky + j, j = 0 a zero weight (the pixel
+    // two to the left), j = kx + 1; layer 2: two taps of 8 channels per step, the
+    // ninth alone; layer 3 (this warp's channel half): a tap of 16 channels per step.
+    uint32_t b1[2], b2[2][4][2], b2e[2], b3[9][2];
+    {
+        auto w1 = [&](int k) {  // depth k of layer 1, channel g; -1: zero weight
+            return k < 12 && (k & 3) ? W1 + g * 9 + (k >> 2) * 3 + (k & 3) - 1 : -1;
+        };
+        b1[0] = pack_w(wq, w1(2 * t4), w1(2 * t4 + 1));
+        b1[1] = pack_w(wq, w1(2 * t4 + 8), w1(2 * t4 + 9));
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int r = W2 + (8 * j + g) * C1 * 9 + 2 * t4 * 9;  // output channel 8 j + g, input channel 2 t
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                b2[j][s][0] = pack_w(wq, r + 2 * s, r + 9 + 2 * s);
+                b2[j][s][1] = pack_w(wq, r + 2 * s + 1, r + 9 + 2 * s + 1);
             }
-            const ofk::Img& I = src.imgs[__ldg(src.list + lo)];
-            const int k = t - __ldg(src.prefix + lo);
-            const int ptx = I.tiles_x * 4;
-            const int x0 = I.tile_x0 + 32 * (k % ptx) - 16, y0 = border + 32 * (k / ptx) - 16;
-            for (int i = tid; i < S0 * S0; i += blockDim.x) {
-                const int x = x0 + (i & 63), y = y0 + (i >> 6);
-                const float v = (x >= 0 && x < I.w && y >= 0 && y < I.h) ? (float)I.img[(size_t)y * I.pitch + x] : 0.f;
-                in[((i >> 6) + 1) * P0 + (i & 63) + 1] = (v - 128.f) * (1.f / 64.f);
+            b2e[j] = pack_w(wq, r + 8, r + 9 + 8);
+        }
+        const int r = W3 + (8 * (warp & 1) + g) * C2 * 9 + 2 * t4 * 9;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            b3[k][0] = pack_w(wq, r + k, r + 9 + k);
+            b3[k][1] = pack_w(wq, r + 8 * 9 + k, r + 9 * 9 + k);
+        }
+    }
+    auto bias = [&](int i) { return __bfloat162float(wq[i]); };
+    const float bb1[2] = {bias(B1 + 2 * t4), bias(B1 + 2 * t4 + 1)};
+    const float bb2[4] = {bias(B2 + 2 * t4), bias(B2 + 2 * t4 + 1), bias(B2 + 8 + 2 * t4), bias(B2 + 9 + 2 * t4)};
+    const float bb3[2] = {bias(B3 + 8 * (warp & 1) + 2 * t4), bias(B3 + 8 * (warp & 1) + 2 * t4 + 1)};
+    const float wf = bias(WF + (lane & 15)), bf = bias(BF);
+    const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+
+    // ldmatrix row addresses of this lane (relative to the plane and the output row).
+    auto col1 = [](int kx) { return kx == 1 ? T1_O : kx >> 1; };  // E[x], O[x], E[x + 1]
+    uint32_t off2[4], off2e;
+    {
+        const int x = (lane & 7) + 8 * ((lane >> 3) & 1);
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const int tap = 2 * s + (lane >> 4);
+            off2[s] = (uint32_t)(((tap / 3) * T1_ROW + col1(tap % 3) + x) * 16);
+        }
+        off2e = (uint32_t)((2 * T1_ROW + 1 + x) * 16);
+    }
+    const uint32_t s1 = smem_addr(p1), s2 = smem_addr(p2);
+    // Layer 3: output row 2 (warp / 2) + (bit 3 of the lane), column lane & 7, channel half = bit 4.
+    const uint32_t a3base =
+        s2 + (uint32_t)((lane >> 4) * T2_PLANE + (2 * (2 * (warp >> 1) + ((lane >> 3) & 1)) * T2_ROW + (lane & 7)) * 16);
+
+    auto finish = [&](int t, int par) {  // warp 0: the head of a finished tile
+        const float* r = red + par * 4 * C3 + (lane & 15);
+        float z = ((r[0] + r[C3]) + (r[2 * C3] + r[3 * C3])) * (1.f / 64.f) * wf;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+        if (lane == 0) logits[t] = z + bf;
+    };
+
+    int t = blockIdx.x, last = -1;
+    __syncthreads();
+    if (t < n) stage_bf16(in, tid, load_chunk(find_patch(src, t), tid));
+    __syncthreads();
+    for (int par = 0; t < n; par ^= 1) {
+        const int tn = t + gridDim.x;
+        uint4 pix = make_uint4(0u, 0u, 0u, 0u);
+        if (tn < n) pix = load_chunk(find_patch(src, tn), tid);
+        // Layer 1: 64 products of 16 pixels (a row's half: even columns 2 g + 16 h, odd ones).
+#pragma unroll 2
+        for (int i = warp; i < 64; i += 8) {
+            const int y = i >> 1, h = i & 1;
+            const uint32_t* r = in + (2 * y + (t4 >> 1)) * TI_ROW + TI_X - 1 + 2 * g + 16 * h + (t4 & 1);
+            const uint32_t* r2 = in + (2 * y + 2) * TI_ROW + TI_X - 1 + 2 * g + 16 * h + t4;
+            uint32_t a[4] = {r[0], r[1], 0u, 0u};
+            if (t4 < 2) {
+                a[2] = r2[0];
+                a[3] = r2[1];
+            }
+            float d[4];
+            mma16(d, a, b1, zero);
+            uint32_t hh, mm, ll;
+            uint8_t* o = p1 + ((y + 1) * T1_ROW + g + 8 * h) * 16 + 4 * t4;
+            split3(relu(d[0] + bb1[0]), relu(d[1] + bb1[1]), hh, mm, ll);
+            *reinterpret_cast<uint32_t*>(o + T1_O * 16) = hh;  // even columns: odd padded columns
+            *reinterpret_cast<uint32_t*>(o + T1_O * 16 + T1_PLANE) = mm;
+            *reinterpret_cast<uint32_t*>(o + T1_O * 16 + 2 * T1_PLANE) = ll;
+            split3(relu(d[2] + bb1[0]), relu(d[3] + bb1[1]), hh, mm, ll);
+            *reinterpret_cast<uint32_t*>(o + 16) = hh;
+            *reinterpret_cast<uint32_t*>(o + 16 + T1_PLANE) = mm;
+            *reinterpret_cast<uint32_t*>(o + 16 + 2 * T1_PLANE) = ll;
+        }
+        __syncthreads();
+        if (warp == 0 && last >= 0) finish(last, par ^ 1);
+        if (tn < n) stage_bf16(in, tid, pix);
+        // Layer 2: two output rows per warp, 16 pixels x 16 channels each.
+#pragma unroll 1
+        for (int y = warp; y < S2; y += 8) {
+            const uint32_t row = s1 + (uint32_t)(2 * y * T1_ROW * 16);
+            float acc[2][4] = {}, low[2][4] = {};
+#pragma unroll
+            for (int s = 0; s < 5; ++s) {
+                uint32_t ah[4], am[4], al[4];
+                if (s < 4) {
+                    ldsm4(ah, row + off2[s]);
+                    ldsm4(am, row + off2[s] + T1_PLANE);
+                    ldsm4(al, row + off2[s] + 2 * T1_PLANE);
+                } else {
+                    uint32_t q[2];
+                    ldsm2(q, row + off2e);
+                    ah[0] = q[0], ah[1] = q[1];
+                    ldsm2(q, row + off2e + T1_PLANE);
+                    am[0] = q[0], am[1] = q[1];
+                    ldsm2(q, row + off2e + 2 * T1_PLANE);
+                    al[0] = q[0], al[1] = q[1];
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    float d[4];
+                    if (s < 4) {
+                        mma16(d, ah, b2[j][s], zero);
+                        mma16(low[j], al, b2[j][s], low[j]);
+                        mma16(low[j], am, b2[j][s], low[j]);
+                    } else {
+                        const uint32_t h2[2] = {ah[0], ah[1]}, m2[2] = {am[0], am[1]}, l2[2] = {al[0], al[1]};
+                        mma8(d, h2, b2e[j], zero);
+                        mma8(low[j], l2, b2e[j], low[j]);
+                        mma8(low[j], m2, b2e[j], low[j]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[j][i] += d[i];
+                }
+            }
+            // Pixels g and g + 8: padded columns g + 1 (odd for even g) and g + 9.
+            uint8_t* o = p2 + ((y + 1) * T2_ROW + ((g & 1) ? (g + 1) >> 1 : T2_O + (g >> 1))) * 16 + 4 * t4;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    uint32_t hh, mm, ll;
+                    split3(relu(acc[j][2 * i] + low[j][2 * i] + bb2[2 * j]),
+                           relu(acc[j][2 * i + 1] + low[j][2 * i + 1] + bb2[2 * j + 1]), hh, mm, ll);
+                    uint8_t* d = o + 64 * i + j * T2_PLANE;
+                    *reinterpret_cast<uint32_t*>(d) = hh;
+                    *reinterpret_cast<uint32_t*>(d + 2 * T2_PLANE) = mm;
+                    *reinterpret_cast<uint32_t*>(d + 4 * T2_PLANE) = ll;
+                }
             }
         }
         __syncthreads();
-        // Layer 1: 32 x 32 pixels, 4 per thread, 8 channels each.
-        for (int px = tid; px < S1 * S1; px += blockDim.x) {
-            const int y = px >> 5, x = px & 31;
-            float acc[C1];
-#pragma unroll
-            for (int o = 0; o < C1; ++o) acc[o] = w[B1 + o];
+        // Layer 3: two output rows of 8 pixels, 8 channels per warp; their sums for the mean.
+        {
+            float acc[4] = {}, lm[4] = {}, lw[4] = {};
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
-                const float v = in[(2 * y + k / 3) * P0 + 2 * x + k % 3];
-                const float4 wa = *reinterpret_cast<const float4*>(w + W1 + k * C1);
-                const float4 wb = *reinterpret_cast<const float4*>(w + W1 + k * C1 + 4);
-                acc[0] = fmaf(wa.x, v, acc[0]); acc[1] = fmaf(wa.y, v, acc[1]);
-                acc[2] = fmaf(wa.z, v, acc[2]); acc[3] = fmaf(wa.w, v, acc[3]);
-                acc[4] = fmaf(wb.x, v, acc[4]); acc[5] = fmaf(wb.y, v, acc[5]);
-                acc[6] = fmaf(wb.z, v, acc[6]); acc[7] = fmaf(wb.w, v, acc[7]);
+                const uint32_t a0 = a3base + (uint32_t)(((k / 3) * T2_ROW + (k % 3 == 1 ? T2_O : (k % 3) >> 1)) * 16);
+                uint32_t ah[4], am[4], al[4];
+                ldsm4(ah, a0);
+                ldsm4(am, a0 + 2 * T2_PLANE);
+                ldsm4(al, a0 + 4 * T2_PLANE);
+                float d[4];
+                mma16(d, ah, b3[k], zero);
+                mma16(lm, am, b3[k], lm);
+                mma16(lw, al, b3[k], lw);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i] += d[i];
             }
+            float v0 = relu(acc[0] + (lm[0] + lw[0]) + bb3[0]) + relu(acc[2] + (lm[2] + lw[2]) + bb3[0]);
+            float v1 = relu(acc[1] + (lm[1] + lw[1]) + bb3[1]) + relu(acc[3] + (lm[3] + lw[3]) + bb3[1]);
 #pragma unroll
-            for (int o = 0; o < C1; ++o) a1[o * P1 * P1 + (y + 1) * P1 + x + 1] = relu(acc[o]);
-        }
-        __syncthreads();
-        // Layer 2: 16 x 16 pixels, one per thread, 16 channels each.
-        {
-            const int y = tid >> 4, x = tid & 15;
-            float acc[C2];
-#pragma unroll
-            for (int o = 0; o < C2; ++o) acc[o] = w[B2 + o];
-            for (int c = 0; c < C1; ++c) {
-                const float* ic = a1 + c * P1 * P1;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float v = ic[(2 * y + k / 3) * P1 + 2 * x + k % 3];
-                    const float* wk = w + W2 + (c * 9 + k) * C2;
-#pragma unroll
-                    for (int o4 = 0; o4 < C2; o4 += 4) {
-                        const float4 ww = *reinterpret_cast<const float4*>(wk + o4);
-                        acc[o4] = fmaf(ww.x, v, acc[o4]);
-                        acc[o4 + 1] = fmaf(ww.y, v, acc[o4 + 1]);
-                        acc[o4 + 2] = fmaf(ww.z, v, acc[o4 + 2]);
-                        acc[o4 + 3] = fmaf(ww.w, v, acc[o4 + 3]);
-                    }
-                }
+            for (int o = 4; o < 32; o <<= 1) {
+                v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o);
+                v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, o);
             }
-#pragma unroll
-            for (int o = 0; o < C2; ++o) a2[o * P2 * P2 + (y + 1) * P2 + x + 1] = relu(acc[o]);
-        }
-        __syncthreads();
-        // Layer 3: 8 x 8 pixels x 4 channel groups.
-        {
-            const int pxl = tid & 63, g = tid >> 6;
-            const int y = pxl >> 3, x = pxl & 7;
-            float acc[4];
-#pragma unroll
-            for (int o = 0; o < 4; ++o) acc[o] = w[B3 + 4 * g + o];
-            for (int c = 0; c < C2; ++c) {
-                const float* ic = a2 + c * P2 * P2;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const float v = ic[(2 * y + k / 3) * P2 + 2 * x + k % 3];
-                    const float4 ww = *reinterpret_cast<const float4*>(w + W3 + (c * 9 + k) * C3 + 4 * g);
-                    acc[0] = fmaf(ww.x, v, acc[0]); acc[1] = fmaf(ww.y, v, acc[1]);
-                    acc[2] = fmaf(ww.z, v, acc[2]); acc[3] = fmaf(ww.w, v, acc[3]);
-                }
-            }
-#pragma unroll
-            for (int o = 0; o < 4; ++o) a3[(4 * g + o) * 64 + pxl] = relu(acc[o]);
-        }
-        __syncthreads();
-        {
-            const int warp = tid >> 5, lane = tid & 31;
-            for (int c = warp; c < C3; c += 8) {
-                float sgap = a3[c * 64 + lane] + a3[c * 64 + 32 + lane];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) sgap += __shfl_xor_sync(0xFFFFFFFFu, sgap, o);
-                if (lane == 0) red[c] = sgap * (1.f / 64.f);
+            if (g == 0) {
+                float* r = red + (par * 4 + (warp >> 1)) * C3 + 8 * (warp & 1) + 2 * t4;
+                r[0] = v0;
+                r[1] = v1;
             }
         }
-        __syncthreads();
-        if (tid == 0) {
-            float z = w[BF];
-            for (int c = 0; c < C3; ++c) z = fmaf(w[WF + c], red[c], z);
-            logits[t] = z;
-        }
-        __syncthreads();
+        last = t;
+        t = tn;
+    }
+    __syncthreads();
+    if (warp == 0 && last >= 0) {
+        // Parity of the last tile: tiles alternate from 0.
+        const int k = (last - (int)blockIdx.x) / (int)gridDim.x;
+        finish(last, k & 1);
     }
 }
 
@@ -493,6 +685,14 @@ int grid_for(int n) {
     return n < 2 * sms ? n : 2 * sms;
 }
 
+// Blocks of the inference kernel: every SM's three, at most one per tile.
+int fwd_grid(int n) {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return n < FWD_BLOCKS * sms ? n : FWD_BLOCKS * sms;
+}
+
 constexpr int SMEM_BWD = (S0 * S0 + A1 + A2 + A3 + 2 * NP) * 4;
 
 // Proposal mask of one listed image per block (see of_detect_learned).
@@ -581,13 +781,12 @@ int launch_extract(const Img* imgs, int img, int border, uint8_t* dst, int n, vo
     return cudaGetLastError() == cudaSuccess ? OF_OK : tn::fail(OF_ERR_CUDA, "extract launch failed");
 }
 
-// Forward over the proposal tiles of a batch (in place from the pyramid).
-int tcnn_forward_tiles(of_tcnn* N, const Img* imgs, const int32_t* list, const int32_t* prefix, int n_list,
-                       int n_tiles, int border, float* logits, void* stream) {
+// Forward over the proposal tiles of a batch (in place from the pyramid); items: the batch's 128 x 32 detect tiles.
+int tcnn_forward_tiles(of_tcnn* N, const Img* imgs, const uint2* items, int n_tiles, float* logits, void* stream) {
     if (n_tiles <= 0) return OF_OK;
-    tn::PatchSrc src{nullptr, imgs, list, prefix, n_list};
-    tn::k_forward_fast<<<tn::grid_for(n_tiles), tn::THREADS, tn::FAST_SMEM, (cudaStream_t)stream>>>(
-        src, n_tiles, N->w, logits, border);
+    tn::PatchSrc src{nullptr, imgs, items};
+    tn::k_forward_fast<<<tn::fwd_grid(n_tiles), tn::FWD_THREADS, tn::FWD_SMEM, (cudaStream_t)stream>>>(
+        src, n_tiles, N->w, logits);
     return cudaGetLastError() == cudaSuccess ? OF_OK : tn::fail(OF_ERR_CUDA, "tile-net forward launch failed");
 }
 }  // namespace ofk
@@ -599,7 +798,7 @@ of_tcnn* of_tcnn_create(uint64_t seed) {
     if (!attr) {
         cudaFuncSetAttribute(tn::k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::SMEM_FWD);
         cudaFuncSetAttribute(tn::k_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::SMEM_BWD);
-        cudaFuncSetAttribute(tn::k_forward_fast, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::FAST_SMEM);
+        cudaFuncSetAttribute(tn::k_forward_fast, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::FWD_SMEM);
         attr = true;
     }
     of_tcnn* N = new of_tcnn();
@@ -679,9 +878,8 @@ int of_tcnn_get_params(of_tcnn* N, int which, float* host) {
 int of_tcnn_forward(of_tcnn* N, const uint8_t* tiles, int n, float* logits, void* stream) {
     if (!N || !tiles || !logits || n < 0) return tn::fail(OF_ERR_ARG, "bad arguments");
     if (n == 0) return OF_OK;
-    tn::PatchSrc src{tiles, nullptr, nullptr, nullptr, 0};
-    tn::k_forward_fast<<<tn::grid_for(n), tn::THREADS, tn::FAST_SMEM, (cudaStream_t)stream>>>(src, n, N->w, logits,
-                                                                                          0);
+    tn::PatchSrc src{tiles, nullptr, nullptr};
+    tn::k_forward_fast<<<tn::fwd_grid(n), tn::FWD_THREADS, tn::FWD_SMEM, (cudaStream_t)stream>>>(src, n, N->w, logits);
     return cudaGetLastError() == cudaSuccess ? OF_OK : tn::fail(OF_ERR_CUDA, "tile-net forward launch failed");
 }
 
@@ -693,8 +891,7 @@ int of_tcnn_loss_grad(of_tcnn* N, const uint8_t* tiles, const float* labels, int
     cudaStream_t st = (cudaStream_t)stream;
     cudaMemsetAsync(N->grad, 0, sizeof(float) * tn::NP, st);
     cudaMemsetAsync(N->loss, 0, sizeof(float), st);
-    tn::PatchSrc src{tiles, nullptr, nullptr, nullptr, 0};
-    tn::k_forward<<<tn::grid_for(n), tn::THREADS, tn::SMEM_FWD, st>>>(src, n, N->w, nullptr, N->save, 0);
+    tn::k_forward<<<tn::grid_for(n), tn::THREADS, tn::SMEM_FWD, st>>>(tiles, n, N->w, nullptr, N->save);
     tn::k_bce<<<(n + 255) / 256, 256, 0, st>>>(N->save, labels, n, pos_weight, N->dz, N->loss);
     tn::k_backward<<<tn::grid_for(n), tn::THREADS, tn::SMEM_BWD, st>>>(tiles, n, N->w, N->save, N->dz, N->grad);
     if (cudaGetLastError() != cudaSuccess) return tn::fail(OF_ERR_CUDA, "tile-net training launch failed");

@@ -33,8 +33,7 @@ int launch_propose(const Img* imgs, const int32_t* list, const int32_t* prefix, 
                    uint8_t* pos, uint8_t* mask, float threshold, float min_conf, int dilate, int32_t* stats,
                    void* stream);
 int launch_extract(const Img* imgs, int img, int border, uint8_t* dst, int n, void* stream);
-int tcnn_forward_tiles(of_tcnn* N, const Img* imgs, const int32_t* list, const int32_t* prefix, int n_list,
-                       int n_tiles, int border, float* logits, void* stream);
+int tcnn_forward_tiles(of_tcnn* N, const Img* imgs, const uint2* items, int n_tiles, float* logits, void* stream);
 }
 
 using namespace ofk;
@@ -1579,7 +1578,7 @@ int of_detect_learned(of_handle* H, const of_frame* frames, int n_frames, int le
     OF_CK(cudaMemsetAsync(d_stats, 0, 4 * sizeof(int32_t), st));
     if (n_features == 0) OF_CK(cudaMemsetAsync(out_counts, 0, sizeof(int32_t) * n_frames, st));
     OF_CK(cudaGraphLaunch(P->stage_exec[0], st));  // pyramid
-    rc = tcnn_forward_tiles(net, P->d_img(), P->d_dl(), d_pp, n_list, n_tiles, P->s.border, d_logit, st);
+    rc = tcnn_forward_tiles(net, P->d_img(), P->d_idt() + P->groups[1][0].dti_off, n_tiles, d_logit, st);
     if (rc == OF_OK)
         rc = launch_propose(P->d_img(), P->d_dl(), d_pp, n_list, d_logit, P->lbuf + P->off_pos,
                             P->lbuf + P->off_mask, threshold, min_confidence, dilate, d_stats, st);
