@@ -81,7 +81,7 @@ typedef struct of_tuning {
     int32_t nms_blocks_per_sm;    /* persistent NMS + Harris grid = SMs x this */
     int32_t fast_order;           /* tile walk: 0 round-robin, 1 contiguous chunks */
     int32_t nms_order;
-    int32_t resize_tma;           /* 1: persistent TMA resize on the levels whose source box fits */
+    int32_t resize_tma;           /* 1: fused pyramid, several levels per launch, where its source boxes fit */
     int32_t stream_groups;        /* k > 1: the frames run as k groups on k forked graph branches (1..8) */
     int32_t fast_cell_tiles;      /* FAST form.  1: FAST on whole-cell tiles applies the cell threshold
                                      itself (cells of 8..30 pixels); 2: the same on 120 x 120 cell-aligned
@@ -185,7 +185,7 @@ int64_t of_inspect(of_handle* h, int what, int frame, int level, void* dst, int6
 
 /* Autotuner (batched path): for this batch shape, time each candidate
  * launch configuration -- pyramid kernel (staged tiles of 32 or 64 rows, or
- * the persistent TMA kernel), persistent grid size and tile order of the FAST
+ * the fused kernel), persistent grid size and tile order of the FAST
  * and NMS kernels, the FAST tile height (32..256 rows) and NMS tile height
  * (32..128 rows), the FAST form (0..4, see of_tuning), and whether the frames
  * run as one group or as 2..8 groups

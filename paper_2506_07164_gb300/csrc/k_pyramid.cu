@@ -1,7 +1,8 @@
 // Pyramid resize: level l is a bilinear resize of level l-1 (the pyramid of
 // an ORB front end, Sec. 1; level sizes "decrease exponentially", Sec. 6.1).
 //
-// One launch resizes level l of every frame in the batch.  Each block owns a
+// Staged kernel (scales the fused kernel below does not take, or by choice):
+// one launch resizes level l of every frame in the batch.  Each block owns a
 // 128 x TH output tile (TH = 32 or 64, chosen by the autotuner): it stages the tile's source window in shared memory
 // with aligned 16-byte loads (direct loads when the window is larger than the
 // buffer, i.e. scales above ~2), then each thread writes 4 consecutive output
@@ -146,10 +147,21 @@ void launch_resize(const Resize* jobs, const int32_t* tile_prefix, int n_jobs, i
 }
 
 // ---------------------------------------------------------------------------
-// Persistent TMA resize, separable and exact.
+// Fused pyramid: a run of levels in one launch, no level waits for another.
 //
-// The bilinear value above factors into a horizontal and a vertical step,
-// both exact in unsigned 32-bit arithmetic when every weight is doubled:
+// Every level is resized from the one before it, so level by level the pyramid
+// is a chain of dependent launches (7 for 8 levels: 38 us for one 1080p frame,
+// nearly all of it latency), each reading back what the last one wrote.  Here a
+// block owns a rectangle of every level of the run -- equal shares of the
+// image -- and computes it from its piece of the source level alone: it loads
+// that piece once (one TMA box), then resizes it level by level in shared
+// memory, each level over its own rectangle plus the few pixels its rectangles
+// of the later levels need (7 levels at scale 1.2: 1.3 times the pixels for a
+// 128 x 128 source piece), and writes what it owns to global memory.  Pixels
+// near the seams are computed by two blocks, identically.
+//
+// The bilinear value factors into a horizontal and a vertical step, both exact
+// in unsigned 32-bit arithmetic when every weight is doubled:
 //   h(r, x) = (4096 - 2ax) S[r][x0] + 2ax S[r][x0 + 1]           (< 2^20)
 //   v       = (4096 - 2ay) h(y0, x) + 2ay h(y0 + 1, x) + 2^23    (< 2^32)
 //   out     = v >> 24 = ((sum of the original products) + 2^21) >> 22.
@@ -157,172 +169,135 @@ void launch_resize(const Resize* jobs, const int32_t* tile_prefix, int n_jobs, i
 // one __byte_perm picks the byte pairs of two outputs into the low and high
 // halves of a word; out is byte 3 of v, so four outputs pack with three byte
 // permutes.  Where a source index is clamped (x0 = w - 1, y0 = h - 1) the
-// tables give that sample's partner weight 0, so the zero fill of the TMA
-// box past the image edge never contributes.
-//
-// Each block walks 128 x 64 output tiles (all frames of one level) and
-// fetches the next tile's source window by TMA into the other buffer while
-// it filters the current one.  Warp w owns output rows 8w .. 8w + 7; each
-// lane owns 4 consecutive output columns and keeps the horizontal values of
-// the two source rows under the current output row in registers, computing
-// each source row once as the warp moves down.
+// tables give that sample's partner weight 0, so what lies past the edge never
+// contributes.  The plan's tables (pyramid_axis) hold, per tile column and row,
+// every level's ranges, byte selectors, weights and source rows, relative to
+// the tile.  A thread owns 4 columns of a strip of rows and keeps the
+// horizontal values of the two source rows under the current output row in
+// registers as it moves down.  Measured (stage time): one 1080p frame 38 -> 16
+// us, one 4K frame 51 -> 28, 64 frames of four sizes 166 -> 122, 128 1080p
+// frames 459 -> 340; batches are bound by instruction issue (72 %).
 
-struct RsTile {
-    int32_t job, x0, y0, sx0, sy0;
-};
-
-// Horizontal pass of one staged source row for a lane's 4 columns.
-__device__ __forceinline__ void hrow(const uint8_t* __restrict__ row, int wa, int wb, const uint32_t (&sel)[4],
+// Horizontal pass of one source row for a thread's 4 columns.
+__device__ __forceinline__ void hrow(const uint32_t* __restrict__ row, uint32_t wa, uint32_t wb, uint32_t sel,
                                      const uint32_t (&wgt)[4], uint32_t (&h)[4]) {
-    const uint32_t* rp = reinterpret_cast<const uint32_t*>(row);
-    const uint32_t a0 = rp[wa], a1 = rp[wa + 1], b0 = rp[wb], b1 = rp[wb + 1];
-    // sel[0]: the byte pairs of outputs 0 and 1 in one word (low half, high half); sel[2]: outputs 2 and 3.
-    const uint32_t p01 = __byte_perm(a0, a1, sel[0]), p23 = __byte_perm(b0, b1, sel[2]);
+    const uint32_t a0 = row[wa], a1 = row[wa + 1], b0 = row[wb], b1 = row[wb + 1];
+    const uint32_t p01 = __byte_perm(a0, a1, sel), p23 = __byte_perm(b0, b1, sel >> 16);
     h[0] = __dp2a_lo(wgt[0], p01, 0u);
     h[1] = __dp2a_hi(wgt[1], p01, 0u);
     h[2] = __dp2a_lo(wgt[2], p23, 0u);
     h[3] = __dp2a_hi(wgt[3], p23, 0u);
 }
 
-__global__ void __launch_bounds__(RT_THREADS)
-k_resize_tma(const Resize* __restrict__ jobs, const uint2* __restrict__ items, int n_tiles,
-             const CUtensorMap* __restrict__ maps, const Call* __restrict__ call, int buf_bytes) {
-    extern __shared__ __align__(128) uint8_t rdyn[];
-    __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ RsTile tinfo[2];
-    // Two buffers of buf_bytes (a multiple of 128) from a 128-byte boundary;
-    // the launch reserves 128 bytes of slack for the rounding.
-    uint8_t* rbuf = rdyn + ((128u - (smem_u32(rdyn) & 127u)) & 127u);
+__global__ void __launch_bounds__(PY_THREADS, 4)
+k_pyramid(const PyrJob* __restrict__ jobs, const uint2* __restrict__ items, const CUtensorMap* __restrict__ maps,
+          const Call* __restrict__ call, int s_bytes, int t_bytes, int x_words) {
+    // The piece of the source level (and of levels 2, 4, ...), of levels 1, 3, ..., then the tables.
+    extern __shared__ __align__(128) uint8_t pdyn[];
+    __shared__ __align__(8) uint64_t mbar;
+    uint8_t* const S = pdyn + ((128u - (smem_u32(pdyn) & 127u)) & 127u);
+    uint8_t* const T = S + s_bytes;
+    int32_t* const xs = reinterpret_cast<int32_t*>(T + t_bytes);
+    int32_t* const ys = xs + x_words;
     const int tid = threadIdx.x;
+    const uint2 it = __ldg(items + blockIdx.x);  // (job, (tile row << 16) | tile column)
+    const PyrJob& J = jobs[it.x];
+    const int32_t* const xg = J.xblk + (size_t)(it.y & 0xFFFFu) * J.xstride;
+    const int32_t* const yg = J.yblk + (size_t)(it.y >> 16) * J.ystride;
     if (tid == 0) {
-        mbar_init(&mbar[0], 1);
-        mbar_init(&mbar[1], 1);
+        mbar_init(&mbar, 1);
         fence_barrier_init();
+        tensormap_acquire(maps + it.x);
+        mbar_arrive_expect_tx(&mbar, (uint32_t)(J.box_w * J.box_h));
+        tma_load_2d(S, maps + it.x, __ldg(xg), __ldg(yg), &mbar);
     }
+    for (int i = tid; i < J.xstride / 4; i += PY_THREADS)
+        reinterpret_cast<int4*>(xs)[i] = __ldg(reinterpret_cast<const int4*>(xg) + i);
+    for (int i = tid; i < J.ystride / 4; i += PY_THREADS)
+        reinterpret_cast<int4*>(ys)[i] = __ldg(reinterpret_cast<const int4*>(yg) + i);
+    const int nl = J.nl;
     __syncthreads();
-    auto issue = [&](int t, int b) {
-        // Tile t from the plan's item table: (job, (Y0 << 16) | X0).
-        const uint2 e = __ldg(items + t);
-        const int j = (int)e.x;
-        const Resize& J = jobs[j];
-        const int X0 = (int)(e.y & 0xFFFFu), Y0 = (int)(e.y >> 16);
-        const int sx0 = (__ldg(J.xtab + X0) >> 12) & ~15;
-        const int sy0 = __ldg(J.ytab + Y0) >> 12;
-        tinfo[b] = RsTile{j, X0, Y0, sx0, sy0};
-        tensormap_acquire(maps + j);
-        mbar_arrive_expect_tx(&mbar[b], (uint32_t)(J.box_w * J.box_h));
-        tma_load_2d(rbuf + b * buf_bytes, maps + j, sx0, sy0, &mbar[b]);
-    };
-    const int g = gridDim.x;
-    if (tid == 0 && (int)blockIdx.x < n_tiles) issue(blockIdx.x, 0);
-
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int it = 0;; ++it) {
-        const int t = blockIdx.x + it * g;
-        if (t >= n_tiles) break;
-        const int tn = t + g;
-        const int b = it & 1;
-        if (tid == 0 && tn < n_tiles) {
-            fence_proxy_async_smem();
-            issue(tn, b ^ 1);
+    const bool ok = mbar_wait(&mbar, 0);
+    if (__syncthreads_or(!ok)) {
+        if (tid == 0) {
+            atomicOr(call->status, OF_DEV_TIMEOUT);
+            mbar_wait(&mbar, 0, OF_WAIT_LIMIT_NS / 8);  // let the copy land before the shared memory goes away
         }
-        const bool ok = mbar_wait(&mbar[b], (it >> 1) & 1);
-        if (__syncthreads_or(!ok)) {
-            if (tid == 0) {
-                atomicOr(call->status, OF_DEV_TIMEOUT);
-                mbar_wait(&mbar[b], (it >> 1) & 1, OF_WAIT_LIMIT_NS / 8);
-                if (tn < n_tiles) mbar_wait(&mbar[b ^ 1], ((it + 1) >> 1) & 1, OF_WAIT_LIMIT_NS / 8);
-            }
-            return;
-        }
-        const RsTile ti = tinfo[b];
-        const Resize& J = jobs[ti.job];
-        const uint8_t* s = rbuf + b * buf_bytes;
-        const int bw = J.box_w;
-        const int nx = min(RS_TILE_W, J.dw - ti.x0), ny = min(RT_TILE_H, J.dh - ti.y0);
-        const int lx = 4 * lane;
-        if (lx < nx) {
-            const int n = min(4, nx - lx);
-            int xo[4];
-            uint32_t wgt[4], sel[4];
+        return;
+    }
+    const int32_t* xe = xs + 4 * (nl + 1);
+    const int32_t* ye = ys + 4 * (nl + 1);
+    int spw = J.box_w / 4;  // words per row of the level being read
+    for (int l = 1; l <= nl; ++l) {
+        const int4 hx = reinterpret_cast<const int4*>(xs)[l], hy = reinterpret_cast<const int4*>(ys)[l];
+        const uint32_t* const src = reinterpret_cast<const uint32_t*>((l & 1) ? S : T);
+        uint32_t* const dst = reinterpret_cast<uint32_t*>((l & 1) ? T : S);
+        const int ncg = hx.y & 255, nr = hy.y & 0xFFFF, dpw = hy.y >> 16;
+        const uint32_t m = (uint32_t)hx.y >> 8;
+        // Strips of rp rows: as many as the threads give (strip = tid / ncg).
+        const int strips = (int)(m >> 8), strip = (int)(((uint32_t)tid * m) >> 16), cg = tid - strip * ncg;
+        if (ncg > 0 && strip < strips) {
+            const int rp = (int)(((float)(nr + strips - 1) + 0.5f) * __frcp_rn((float)strips));  // ceil(nr / strips)
+            int r = strip * rp;
+            const int re = min(r + rp, nr);
+            const int4 ea = *reinterpret_cast<const int4*>(xe + 8 * cg);
+            const int2 eb = *reinterpret_cast<const int2*>(xe + 8 * cg + 4);
+            const uint32_t wa = (uint32_t)ea.x & 0xFFFFu, wb = (uint32_t)ea.x >> 16, sel = (uint32_t)ea.y;
+            const uint32_t wgt[4] = {(uint32_t)ea.z, (uint32_t)ea.w, (uint32_t)eb.x, (uint32_t)eb.y};
+            const int x = hx.x + 4 * cg;
+            // Owned rows of the strip: none when the columns are another tile's.
+            const bool mine = x >= hx.z && x < hx.w;
+            const int o0 = mine ? hy.z - hy.x : nr, o1 = hy.w - hy.x;
+            const int pitch = J.dpitch[l - 1];
+            // Word stores: x and the pitch are multiples of 4; a level's rows are padded to 16 bytes.
+            uint8_t* g = J.dst[l - 1] + (ptrdiff_t)(hy.x + r) * pitch + x;
+            uint32_t* d = dst + r * dpw + cg;
+            const bool keep = l < nl;
+            uint32_t ha[4], hb[4] = {0u, 0u, 0u, 0u};
+            int next = -1;  // word offset of the row below the last one read
+#pragma unroll 2
+            for (; r < re; ++r, g += pitch, d += dpw) {
+                const uint32_t e = (uint32_t)ye[r];
+                const int off = (int)(e >> 16);
+                const uint32_t a2 = e & 0xFFFFu;
+                // Consecutive output rows mostly read consecutive source rows: the
+                // upper one is then the last lower one.  Only the other lanes branch.
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int e = __ldg(J.xtab + ti.x0 + lx + min(i, n - 1));
-                xo[i] = (e >> 12) - ti.sx0;  // byte offset of x0 in the staged row
-                const uint32_t a2 = 2u * (uint32_t)(e & 4095);
-                wgt[i] = (4096u - a2) | (a2 << 16);
-            }
-            // Columns 0-1 read the word pair at wa, columns 2-3 the pair at wb;
-            // consecutive x0 differ by at most 3, so each byte pair lies in its 8 bytes.
-            const int wa = xo[0] >> 2, wb = xo[2] >> 2;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t o = (uint32_t)(xo[i] - 4 * (i < 2 ? wa : wb));
-                sel[i] = o | ((o + 1u) << 4);
-            }
-            sel[0] |= sel[1] << 8;  // outputs 0 and 1 share one permute
-            sel[2] |= sel[3] << 8;
-            // The job's fields, read once (the stores below could alias them).
-            const int dpitch = J.dpitch;
-            const int32_t* ytab = J.ytab + ti.y0;
-            uint8_t* d = J.dst + (size_t)ti.y0 * dpitch + ti.x0 + lx;
-            uint32_t ha[4], hb[4];
-            int cur = -4;
-            const int ly_end = min(8 * warp + 8, ny);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {  // unrolled: the row-table loads are issued together
-                const int ly = 8 * warp + k;
-                if (ly >= ly_end) break;
-                const int e = __ldg(ytab + ly);
-                const int r0 = (e >> 12) - ti.sy0;
-                const uint32_t a2 = 2u * (uint32_t)(e & 4095);
-                if (r0 == cur + 1) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) ha[i] = hb[i];
-                    hrow(s + (r0 + 1) * bw, wa, wb, sel, wgt, hb);
-                } else if (r0 != cur) {
-                    hrow(s + r0 * bw, wa, wb, sel, wgt, ha);
-                    hrow(s + (r0 + 1) * bw, wa, wb, sel, wgt, hb);
-                }
-                cur = r0;
+                for (int i = 0; i < 4; ++i) ha[i] = hb[i];
+                if (off != next) hrow(src + off, wa, wb, sel, wgt, ha);
+                next = off + spw;
+                hrow(src + next, wa, wb, sel, wgt, hb);
                 uint32_t v[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) v[i] = (4096u - a2) * ha[i] + a2 * hb[i] + (1u << 23);
                 const uint32_t packed =
                     __byte_perm(__byte_perm(v[0], v[1], 0x0073), __byte_perm(v[2], v[3], 0x0073), 0x5410);
-                uint8_t* dr = d + (size_t)ly * dpitch;
-                if (n == 4) {
-                    *reinterpret_cast<uint32_t*>(dr) = packed;  // x0 + lx is a multiple of 4, dpitch of 16
-                } else {
-                    for (int i = 0; i < n; ++i) dr[i] = (uint8_t)(packed >> (8 * i));
-                }
+                if (keep) *d = packed;
+                if (r >= o0 && r < o1) *reinterpret_cast<uint32_t*>(g) = packed;
             }
         }
-        __syncthreads();  // buffer b is free for the tile after next
+        xe += 8 * ncg;
+        ye += nr;
+        spw = dpw;
+        __syncthreads();
     }
 }
 
-void launch_resize_tma(const Resize* jobs, const uint2* items, int n_tiles, const CUtensorMap* maps,
-                       const Call* call, int buf_bytes, int grid, void* stream) {
-    if (n_tiles <= 0) return;
-    grid = grid < n_tiles ? grid : n_tiles;
-    k_resize_tma<<<grid, RT_THREADS, 2 * buf_bytes + 128, (cudaStream_t)stream>>>(jobs, items, n_tiles, maps, call,
-                                                                                   buf_bytes);
+int pyramid_smem(int s_bytes, int t_bytes, int x_words, int y_words) {
+    return s_bytes + t_bytes + 4 * (x_words + y_words) + 128;
 }
 
-// The kernel's dynamic shared-memory limit is raised once to the largest
-// size any plan may use (two buffers of RT_MAX_BUF), so graphs captured for
+void launch_pyramid(const PyrJob* jobs, const uint2* items, int n_tiles, const CUtensorMap* maps, const Call* call,
+                    int s_bytes, int t_bytes, int x_words, int y_words, void* stream) {
+    if (n_tiles <= 0) return;
+    k_pyramid<<<n_tiles, PY_THREADS, pyramid_smem(s_bytes, t_bytes, x_words, y_words), (cudaStream_t)stream>>>(
+        jobs, items, maps, call, s_bytes, t_bytes, x_words);
+}
+
+// Raised once to the largest size any plan may use, so graphs captured for
 // different plans never depend on which plan set it last.
-int resize_tma_blocks_per_sm(int buf_bytes) {
-    if (buf_bytes <= 0 || buf_bytes > RT_MAX_BUF) return 0;
-    if (cudaFuncSetAttribute(k_resize_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * RT_MAX_BUF + 128) !=
-        cudaSuccess)
-        return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_resize_tma, RT_THREADS, 2 * buf_bytes + 128) !=
-        cudaSuccess)
-        return 0;
-    return n;
+bool pyramid_raise_smem() {
+    return cudaFuncSetAttribute(k_pyramid, cudaFuncAttributeMaxDynamicSharedMemorySize, PY_MAX_SMEM) == cudaSuccess;
 }
 
 }  // namespace ofk

@@ -228,28 +228,35 @@ struct Plan {
         int slot_begin = 0, slot_end = 0;
         std::vector<int> rs_job, rs_n;              // per level: first resize job, jobs
         std::vector<int> rsp_off[2], rs_tiles[2];   // per level and resize tile height
-        std::vector<int> rsi_off;                   // per level: offset of its 64-row tiles in items_rs
+        std::vector<int> py_off, py_n;              // per fused run: its tiles in items_py
     };
     std::vector<Group> groups[kMaxGroups + 1];
     std::vector<int32_t> gp_det, gp_rs, gp_fast, gp_rows, gp_nms64, gp_ftall[2], gp_fal, gp_cstrip;
     // Work-item tables of the per-warp kernels, per group: (image, (y0 << 16) | x0).
     std::vector<uint2> items_cs, items_dt;
     std::vector<uint16_t> slot_img;  // image of every output slot (orientation kernel)
-    std::vector<uint2> items_rs;  // TMA resize tiles per group and level: (job in the level's launch, (Y0 << 16) | X0)
+    // Fused pyramid: the levels 1 .. L-1 as runs of levels, one launch each.
+    struct Run {
+        int job_begin = 0, s_bytes = 0, t_bytes = 0, x_words = 0, y_words = 0;
+    };
+    std::vector<Run> runs;           // empty: the staged kernel resizes level by level
+    std::vector<PyrJob> h_pj;        // jobs of all runs (one per frame and run)
+    std::vector<int> pj_frame, pj_level;  // frame and source level of each job
+    std::vector<std::pair<int, int>> pj_tiles;  // tile columns and rows of each job
+    std::vector<int32_t> pblk;       // the jobs' axis tables
+    std::vector<uint2> items_py;     // (job in its run, (tile row << 16) | tile column) per group and run
     bool cell_tiles = false;     // the cell size allows the cell-tile FAST kernel
     bool apply_flags = false;    // the threshold pass can set the cell flags (else the general FAST kernel does)
     bool strip_ok = false;       // the cell size allows the cell-row strip kernel (cells of 8..33 pixels)
     bool aligned_ok = false;     // ... and the cell-aligned general FAST kernel (cells of 15 or 30 pixels)
-    std::vector<int> rt_buf;        // TMA resize buffer bytes of level l (0: staged kernel only)
-    std::vector<int> rt_bps;        // TMA resize resident blocks per SM of level l
     int det_tiles = 0, max_quota = 0, total_slots = 0, n_img = 0;
     Call h_call{};
     uint8_t* dbuf = nullptr;
     size_t off_call = 0, off_img = 0, off_rs = 0, off_dl = 0, off_tab = 0, off_ftab = 0;
     size_t off_gdp = 0, off_grs = 0, off_gfp = 0, off_grp = 0, off_gnp = 0, off_gft[2] = {0, 0}, off_gfal = 0,
-           off_gcs = 0, off_ics = 0, off_idt = 0, off_irs = 0, off_sli = 0;
+           off_gcs = 0, off_ics = 0, off_idt = 0, off_ipy = 0, off_sli = 0, off_pj = 0, off_pblk = 0;
     size_t off_maps = 0;
-    std::vector<CUtensorMap> h_maps;  // [image maps | score maps] (n_img each) | resize source maps
+    std::vector<CUtensorMap> h_maps;  // [image maps | score maps] (n_img each) | source maps of the pyramid jobs
     of_tuning tun{};  // launch configuration (defaults, or the autotuner's choice)
     bool tuned = false;
     // Learned path: proposal tiles per listed image, device buffers
@@ -282,7 +289,8 @@ struct Plan {
     const int32_t* d_gcs() const { return reinterpret_cast<const int32_t*>(dbuf + off_gcs); }
     const uint2* d_ics() const { return reinterpret_cast<const uint2*>(dbuf + off_ics); }
     const uint2* d_idt() const { return reinterpret_cast<const uint2*>(dbuf + off_idt); }
-    const uint2* d_irs() const { return reinterpret_cast<const uint2*>(dbuf + off_irs); }
+    const uint2* d_ipy() const { return reinterpret_cast<const uint2*>(dbuf + off_ipy); }
+    const PyrJob* d_pj() const { return reinterpret_cast<const PyrJob*>(dbuf + off_pj); }
     const uint16_t* d_sli() const { return reinterpret_cast<const uint16_t*>(dbuf + off_sli); }
     const int32_t* d_gnp() const { return reinterpret_cast<const int32_t*>(dbuf + off_gnp); }
     const int32_t* d_gft(int i) const { return reinterpret_cast<const int32_t*>(dbuf + off_gft[i]); }
@@ -379,19 +387,21 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
     const int nl = s.levels;
     switch (stage) {
         case 0:
+            if (P->tun.resize_tma && !P->runs.empty()) {
+                for (size_t c = 0; c < P->runs.size(); ++c) {
+                    const Plan::Run& R = P->runs[c];
+                    launch_pyramid(P->d_pj() + R.job_begin, P->d_ipy() + G.py_off[c], G.py_n[c],
+                                   P->d_maps() + 2 * P->n_img + R.job_begin, P->d_call(), R.s_bytes, R.t_bytes,
+                                   R.x_words, R.y_words, st);
+                }
+                break;
+            }
             for (int l = 1; l < nl; ++l) {
                 const int nj = G.rs_n[l];
                 if (nj <= 0) continue;
-                if (P->tun.resize_tma && P->rt_buf[l] > 0) {
-                    static_assert(RS_TILE_HS[1] == RT_TILE_H, "TMA resize uses the 64-row tile prefix");
-                    launch_resize_tma(P->d_rs() + G.rs_job[l], P->d_irs() + G.rsi_off[l], G.rs_tiles[1][l],
-                                      P->d_maps() + 2 * P->n_img + G.rs_job[l], P->d_call(), P->rt_buf[l],
-                                      H->n_sms * P->rt_bps[l], st);
-                } else {
-                    const int v = P->tun.resize_tile_h == RS_TILE_HS[0] ? 0 : 1;
-                    launch_resize(P->d_rs() + G.rs_job[l], P->d_grs() + G.rsp_off[v][l], nj, G.rs_tiles[v][l],
-                                  RS_TILE_HS[v], st);
-                }
+                const int v = P->tun.resize_tile_h == RS_TILE_HS[0] ? 0 : 1;
+                launch_resize(P->d_rs() + G.rs_job[l], P->d_grs() + G.rsp_off[v][l], nj, G.rs_tiles[v][l],
+                              RS_TILE_HS[v], st);
             }
             break;
         case 1:
@@ -542,6 +552,132 @@ cudaError_t instantiate_graphs(of_handle* H, Plan* P) {
     return e;
 }
 
+// Source map of a pyramid job: its frame's source level, boxes of the job's tiles.
+int encode_pyr_map(Plan* P, int j) {
+    const Img& I = P->h_img[P->pj_frame[j] * P->s.levels + P->pj_level[j]];
+    const PyrJob& J = P->h_pj[j];
+    return encode_u8(&P->h_maps[2 * P->n_img + j], I.img, I.w, I.h, I.pitch, J.box_w, J.box_h);
+}
+
+// Tile of the source level (pixels a side) and bound on a run's computed over
+// owned pixels, by the pixels of the batch.  Small batches are bound by the
+// latency of one block's levels: one run, tiles small enough to give every SM a
+// block (one VGA frame: tiles of 64 / 96 / 128: 12.5 / 13.6 / 15.6 us; one
+// 1080p frame: 18 / 16 / 16; four: 39 / 30 / 27).  Large ones are bound by
+// instructions, so by the seams: larger tiles and shorter runs, each of which
+// reads its source level back once (32 1080p frames: 128 px, one run 128 us,
+// 160 px 119, 160 px and seams within 6 % -- levels 1-2, 3-4, 5-7 -- 105; 8
+// frames: 44, 42, 46).
+struct PyrShape {
+    int tile;
+    double max_seam;
+};
+PyrShape pyr_shape(const std::vector<FrameKey>& frames) {
+    int64_t px = 0;
+    for (const auto& f : frames) px += (int64_t)f.w * f.h;
+    if (px >= 24000000) return {160, 1.06};
+    return {px < 800000 ? 64 : px < 3000000 ? 96 : 128, 1.9};
+}
+
+// Split the levels 1 .. L-1 of every frame into runs that k_pyramid computes in
+// one launch each: a run takes as many levels as keep the seams within the
+// shape's bound.  Frames of one size share their tables.  No runs (the staged
+// kernel) when some level's source steps or pieces do not fit (scales above 3).
+void plan_pyramid(Plan* P) {
+    const int nl = P->s.levels, nf = (int)P->frames.size();
+    struct Piece {
+        int level, nl, ntx, nty, xoff, yoff;
+        ofh::PyrAxis x, y;
+    };
+    std::map<std::pair<int, int>, std::vector<Piece>> made;  // per frame size: its runs
+    const PyrShape shape = pyr_shape(P->frames);
+    size_t n_runs = 0;
+    bool ok = nl > 1 && pyramid_raise_smem();
+    for (int f = 0; f < nf && ok; ++f) {
+        const std::pair<int, int> key(P->frames[f].w, P->frames[f].h);
+        if (made.count(key)) continue;
+        std::vector<Piece>& v = made[key];
+        std::vector<int32_t> ws, hs;
+        for (int l = 0; l < nl && P->h_img[f * nl + l].w > 0; ++l) {
+            ws.push_back(P->h_img[f * nl + l].w);
+            hs.push_back(P->h_img[f * nl + l].h);
+        }
+        for (int a = 0; a + 1 < (int)ws.size() && ok;) {
+            bool found = false;
+            for (int t = shape.tile; t >= 32 && !found; t = t > 128 ? 128 : t / 2)
+                for (int n = std::min((int)ws.size() - 1 - a, PY_MAX_LEVELS); n >= 1 && !found; --n) {
+                    Piece p;
+                    p.level = a;
+                    p.nl = n;
+                    p.ntx = (ws[a] + t - 1) / t;
+                    p.nty = (hs[a] + t - 1) / t;
+                    p.x = ofh::pyramid_axis(ws.data() + a, n, p.ntx, 256);
+                    std::vector<int32_t> row_words(n + 1);
+                    for (int l = 0; l <= n; ++l) row_words[l] = std::max(p.x.extent[l], 16) / 4;
+                    p.y = ofh::pyramid_axis(hs.data() + a, n, p.nty, 256, row_words.data());
+                    if (!p.x.ok || !p.y.ok) continue;
+                    const double seam = (double)p.x.computed * p.y.computed / ((double)p.x.owned * p.y.owned);
+                    if (n > 1 && seam > shape.max_seam) continue;
+                    p.xoff = (int)P->pblk.size();
+                    P->pblk.insert(P->pblk.end(), p.x.blk.begin(), p.x.blk.end());
+                    p.yoff = (int)P->pblk.size();
+                    P->pblk.insert(P->pblk.end(), p.y.blk.begin(), p.y.blk.end());
+                    v.push_back(p);
+                    a += n;
+                    found = true;
+                }
+            ok = found;
+        }
+        n_runs = std::max(n_runs, v.size());
+    }
+    for (size_t c = 0; c < n_runs && ok; ++c) {
+        Plan::Run R;
+        R.job_begin = (int)P->h_pj.size();
+        for (int f = 0; f < nf; ++f) {
+            const std::vector<Piece>& v = made[std::make_pair(P->frames[f].w, P->frames[f].h)];
+            if (c >= v.size()) continue;
+            const Piece& p = v[c];
+            PyrJob J;
+            std::memset(&J, 0, sizeof(J));
+            J.xblk = reinterpret_cast<const int32_t*>((intptr_t)p.xoff);  // word offsets until the block has an address
+            J.yblk = reinterpret_cast<const int32_t*>((intptr_t)p.yoff);
+            J.xstride = p.x.stride;
+            J.ystride = p.y.stride;
+            J.nl = p.nl;
+            J.box_w = std::max(p.x.extent[0], 16);
+            J.box_h = std::max(p.y.extent[0], 1);
+            // The source piece and the even levels share S, the odd levels T; a row and 16
+            // bytes past the end are read where a clamped source's weight is 0.
+            int s = (J.box_h + 1) * J.box_w + 16, t = 0;
+            for (int l = 1; l <= p.nl; ++l) {
+                const Img& D = P->h_img[f * nl + p.level + l];
+                J.dst[l - 1] = const_cast<uint8_t*>(D.img);
+                J.dpitch[l - 1] = D.pitch;
+                const int n = (p.y.extent[l] + 1) * std::max(p.x.extent[l], 16) + 16;
+                (l & 1 ? t : s) = std::max(l & 1 ? t : s, n);
+            }
+            R.s_bytes = std::max(R.s_bytes, (s + 127) & ~127);
+            R.t_bytes = std::max(R.t_bytes, (t + 127) & ~127);
+            R.x_words = std::max(R.x_words, J.xstride);
+            R.y_words = std::max(R.y_words, J.ystride);
+            P->h_pj.push_back(J);
+            P->pj_frame.push_back(f);
+            P->pj_level.push_back(p.level);
+            P->pj_tiles.emplace_back(p.ntx, p.nty);
+        }
+        ok = pyramid_smem(R.s_bytes, R.t_bytes, R.x_words, R.y_words) <= PY_MAX_SMEM;
+        P->runs.push_back(R);
+    }
+    if (!ok) {
+        P->runs.clear();
+        P->h_pj.clear();
+        P->pj_frame.clear();
+        P->pj_level.clear();
+        P->pj_tiles.clear();
+        P->pblk.clear();
+    }
+}
+
 int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings& s,
                Plan** out) {
     Plan* P = new Plan();
@@ -669,44 +805,7 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
         }
     }
     P->rs_begin[nl] = (int)P->h_rs.size();
-    // Source boxes of the persistent TMA resize; a level uses it when every
-    // job's box fits (<= 256 x 256) and consecutive x0 differ by at most 3.
-    P->rt_buf.assign(nl + 1, 0);
-    P->rt_bps.assign(nl + 1, 0);
-    for (int l = 1; l < nl; ++l) {
-        bool ok = P->rs_begin[l + 1] > P->rs_begin[l];
-        int buf = 0;
-        for (int i = P->rs_begin[l]; i < P->rs_begin[l + 1]; ++i) {
-            Resize& R = P->h_rs[i];
-            const int32_t* xt = P->tables.data() + tab_idx[i].first;
-            const int32_t* yt = P->tables.data() + tab_idx[i].second;
-            int bw = 0, bh = 0, step = 0;
-            for (int X0 = 0; X0 < R.dw; X0 += RS_TILE_W) {
-                const int last = std::min(X0 + RS_TILE_W, R.dw) - 1;
-                bw = std::max(bw, (xt[last] >> 12) + 2 - ((xt[X0] >> 12) & ~15));
-            }
-            for (int Y0 = 0; Y0 < R.dh; Y0 += RT_TILE_H) {
-                const int last = std::min(Y0 + RT_TILE_H, R.dh) - 1;
-                bh = std::max(bh, (yt[last] >> 12) + 2 - (yt[Y0] >> 12));
-            }
-            for (int d = 1; d < R.dw; ++d) step = std::max(step, (xt[d] >> 12) - (xt[d - 1] >> 12));
-            bw = (bw + 15) & ~15;
-            if (bw <= 256 && bh <= 256 && step <= 3) {
-                R.box_w = bw;
-                R.box_h = bh;
-                buf = std::max(buf, (bw * bh + 16 + 127) & ~127);  // +16: a lane's word pair may end past the box
-            } else {
-                ok = false;
-            }
-        }
-        if (ok && buf <= RT_MAX_BUF) {
-            const int bps = resize_tma_blocks_per_sm(buf);
-            if (bps > 0) {
-                P->rt_buf[l] = buf;
-                P->rt_bps[l] = bps;
-            }
-        }
-    }
+    plan_pyramid(P);
     for (int i = 0; i < P->n_img; ++i) {
         const Img& I = P->h_img[i];
         if (I.tiles_x > 0) {
@@ -777,7 +876,6 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
             G.slot_end = f1 < nf ? P->h_img[f1 * nl].slot0 : P->total_slots;
             G.rs_job.assign(nl + 1, 0);
             G.rs_n.assign(nl + 1, 0);
-            G.rsi_off.assign(nl + 1, 0);
             for (int v = 0; v < 2; ++v) {
                 G.rsp_off[v].assign(nl + 1, 0);
                 G.rs_tiles[v].assign(nl + 1, 0);
@@ -789,12 +887,6 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                 while (e < P->rs_begin[l + 1] && P->rs_frame[e] < f1) ++e;
                 G.rs_job[l] = b;
                 G.rs_n[l] = e - b;
-                G.rsi_off[l] = (int)P->items_rs.size();
-                for (int i = b; i < e; ++i)  // tile t = ty * tiles_x + tx of job i - b, as the prefixes count
-                    for (int ty = 0; ty < (P->h_rs[i].dh + RT_TILE_H - 1) / RT_TILE_H; ++ty)
-                        for (int tx = 0; tx < P->h_rs[i].tiles_x; ++tx)
-                            P->items_rs.push_back(make_uint2(
-                                (uint32_t)(i - b), ((uint32_t)(ty * RT_TILE_H) << 16) | (uint32_t)(tx * RS_TILE_W)));
                 for (int v = 0; v < 2; ++v) {
                     G.rsp_off[v][l] = (int)P->gp_rs.size();
                     int tiles = 0;
@@ -804,6 +896,18 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                     }
                     G.rs_tiles[v][l] = tiles;
                 }
+            }
+            for (size_t c = 0; c < P->runs.size(); ++c) {
+                const int j0r = P->runs[c].job_begin;
+                const int j1r = c + 1 < P->runs.size() ? P->runs[c + 1].job_begin : (int)P->h_pj.size();
+                G.py_off.push_back((int)P->items_py.size());
+                for (int j = j0r; j < j1r; ++j) {
+                    if (P->pj_frame[j] < f0 || P->pj_frame[j] >= f1) continue;
+                    for (int ty = 0; ty < P->pj_tiles[j].second; ++ty)
+                        for (int tx = 0; tx < P->pj_tiles[j].first; ++tx)
+                            P->items_py.push_back(make_uint2((uint32_t)(j - j0r), ((uint32_t)ty << 16) | (uint32_t)tx));
+                }
+                G.py_n.push_back((int)P->items_py.size() - G.py_off.back());
             }
             P->groups[k].push_back(G);
         }
@@ -851,8 +955,8 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     P->tun.nms_order = 0;
 
     // Tensor maps: image boxes for FAST and NMS, score boxes for NMS, then
-    // the source box of each resize job (TMA resize).
-    P->h_maps.assign(2 * P->n_img + P->h_rs.size(), CUtensorMap{});
+    // the source box of each pyramid job.
+    P->h_maps.assign(2 * P->n_img + P->h_pj.size(), CUtensorMap{});
     for (int i = 0; i < P->n_img; ++i) {
         const Img& I = P->h_img[i];
         int rc = encode_u8(&P->h_maps[i], I.img, I.w, I.h, I.pitch, SROW, IMG_BOX_ROWS);
@@ -863,10 +967,8 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
             return rc;
         }
     }
-    for (size_t i = 0; i < P->h_rs.size(); ++i) {
-        const Resize& R = P->h_rs[i];
-        if (R.box_w == 0) continue;
-        const int rc = encode_u8(&P->h_maps[2 * P->n_img + i], R.src, R.sw, R.sh, R.spitch, R.box_w, R.box_h);
+    for (size_t j = 0; j < P->h_pj.size(); ++j) {
+        const int rc = encode_pyr_map(P, (int)j);
         if (rc != OF_OK) {
             free_plan(P);
             return rc;
@@ -914,8 +1016,12 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_cs.size(), 1), 16);
     P->off_idt = off;
     off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_dt.size(), 1), 16);
-    P->off_irs = off;
-    off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_rs.size(), 1), 16);
+    P->off_ipy = off;
+    off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_py.size(), 1), 16);
+    P->off_pj = off;
+    off = align_up(off + sizeof(PyrJob) * std::max<size_t>(P->h_pj.size(), 1), 16);
+    P->off_pblk = off;
+    off = align_up(off + sizeof(int32_t) * std::max<size_t>(P->pblk.size(), 1), 16);
     // Output slot -> image (slots of image i: [slot0, slot0 + layout quota)).
     P->slot_img.assign(std::max(P->total_slots, 1), 0);
     for (int i = 0; i < P->n_img; ++i) {
@@ -939,6 +1045,12 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
         P->h_rs[i].xtab = d_tab + tab_idx[i].first;
         P->h_rs[i].ytab = d_tab + tab_idx[i].second;
     }
+    // The jobs' table offsets become addresses.
+    const int32_t* d_pblk = reinterpret_cast<const int32_t*>(P->dbuf + P->off_pblk);
+    for (PyrJob& J : P->h_pj) {
+        J.xblk = d_pblk + reinterpret_cast<intptr_t>(J.xblk);
+        J.yblk = d_pblk + reinterpret_cast<intptr_t>(J.yblk);
+    }
     std::vector<uint8_t> blob(off, 0);
     auto put = [&](size_t at, const void* src, size_t n) {
         if (n) std::memcpy(blob.data() + at, src, n);
@@ -960,7 +1072,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     put(P->off_gcs, P->gp_cstrip.data(), sizeof(int32_t) * P->gp_cstrip.size());
     put(P->off_ics, P->items_cs.data(), sizeof(uint2) * P->items_cs.size());
     put(P->off_idt, P->items_dt.data(), sizeof(uint2) * P->items_dt.size());
-    put(P->off_irs, P->items_rs.data(), sizeof(uint2) * P->items_rs.size());
+    put(P->off_ipy, P->items_py.data(), sizeof(uint2) * P->items_py.size());
+    put(P->off_pj, P->h_pj.data(), sizeof(PyrJob) * P->h_pj.size());
+    put(P->off_pblk, P->pblk.data(), sizeof(int32_t) * P->pblk.size());
     put(P->off_sli, P->slot_img.data(), sizeof(uint16_t) * P->slot_img.size());
     e = cudaMemcpy(P->dbuf, blob.data(), off, cudaMemcpyHostToDevice);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
@@ -1060,12 +1174,12 @@ int bind_plan(of_handle* H, Plan* P, const of_frame* frames, of_keypoint* out, i
             Resize& R = P->h_rs[i];
             for (int f = 0; f < nf; ++f)
                 if (R.dst == P->h_img[f * nl + 1].img) R.src = P->h_img[f * nl].img;
-            if (R.box_w > 0) {
-                const int rc = encode_u8(&P->h_maps[2 * P->n_img + i], R.src, R.sw, R.sh, R.spitch, R.box_w,
-                                         R.box_h);
-                if (rc != OF_OK) return rc;
-            }
         }
+    }
+    for (size_t j = 0; j < P->h_pj.size(); ++j) {
+        if (P->pj_level[j] != 0 || P->frames[P->pj_frame[j]].copy) continue;
+        const int rc = encode_pyr_map(P, (int)j);
+        if (rc != OF_OK) return rc;
     }
     P->h_call.out = out;
     P->h_call.counts = counts;
@@ -1156,7 +1270,7 @@ int prepare_batch(of_handle* H, const of_frame* frames, int n_frames, int levels
 // Time the candidate launch configurations of a bound plan on its own data
 // and keep the fastest per stage:
 //   pyramid  staged kernel with 128 x 32 or 128 x 64 output tiles, or the
-//            persistent TMA kernel;
+//            fused kernel (runs of levels);
 //   FAST     general kernel on 32-, 64-, 128- or 256-row tiles (the tall
 //            ones when the threshold pass sets the flags) or the cell-tile
 //            kernel; 1 .. max resident blocks per SM; round-robin or
@@ -1188,8 +1302,8 @@ int autotune_plan(of_handle* H, Plan* P, int reps) {
     int rc = OF_OK;
     enqueue_stages(H, P, 0, kStages, st);  // every buffer populated once
     // Pyramid (idempotent).
-    // Candidates: the staged kernel with 32- or 64-row tiles, then the
-    // persistent TMA kernel (on the levels it covers; staged 64 elsewhere).
+    // Candidates: the staged kernel with 32- or 64-row tiles, then the fused
+    // kernel (where it covers the levels; else staged 64 again).
     float best = 1e30f;
     int best_h = P->tun.resize_tile_h, best_tma = P->tun.resize_tma;
     for (int c = 0; c < 3 && rc == OF_OK; ++c) {

@@ -94,16 +94,23 @@ struct Resize {
     int32_t sw, sh, spitch;
     int32_t dw, dh, dpitch;
     int32_t tiles_x, tiles_y;
-    // Source box of the persistent TMA kernel (box_w a multiple of 16, both
-    // <= 256): the largest source window of one RS_TILE_W x RT_TILE_H output
-    // tile.  0 when the job is not eligible (scale too large).
-    int32_t box_w, box_h;
 };
 
-// Persistent TMA resize: 128 x 64 output tiles, 8 warps of 8 output rows.
-constexpr int RT_TILE_H = 64;
-constexpr int RT_THREADS = 256;
-constexpr int RT_MAX_BUF = 100 * 1024;  // largest source buffer (two per block)
+// One frame of a fused run of pyramid levels (k_pyramid): nl levels from one
+// source level.  Tables per tile column and row as pyramid_axis writes them.
+constexpr int PY_MAX_LEVELS = 15;
+struct PyrJob {
+    const int32_t* xblk;
+    const int32_t* yblk;
+    int32_t xstride, ystride;  // words per tile, multiples of 4
+    int32_t nl;
+    int32_t box_w, box_h;      // the tiles' piece of the source level (box_w a multiple of 16)
+    int32_t pad;
+    uint8_t* dst[PY_MAX_LEVELS];
+    int32_t dpitch[PY_MAX_LEVELS];
+};
+constexpr int PY_THREADS = 256;
+constexpr int PY_MAX_SMEM = 160 * 1024;
 
 // Per-call constants.
 struct Call {
@@ -134,9 +141,11 @@ __host__ __device__ __forceinline__ int tile_of(int order, int block, int grid, 
 namespace ofk {
 void launch_resize(const Resize* jobs, const int32_t* tile_prefix, int n_jobs, int n_tiles,
                    int tile_h, void* stream);
-void launch_resize_tma(const Resize* jobs, const uint2* items, int n_tiles, const CUtensorMap* maps,
-                       const Call* call, int buf_bytes, int grid, void* stream);
-int resize_tma_blocks_per_sm(int buf_bytes);  // also raises the kernel's shared-memory limit
+// Fused pyramid levels: one block per (frame, tile); items (job, (tile row << 16) | tile column).
+void launch_pyramid(const PyrJob* jobs, const uint2* items, int n_tiles, const CUtensorMap* maps, const Call* call,
+                    int s_bytes, int t_bytes, int x_words, int y_words, void* stream);
+int pyramid_smem(int s_bytes, int t_bytes, int x_words, int y_words);
+bool pyramid_raise_smem();
 // General FAST on 128 x tile_h tiles (32, 64, 128 or 256 rows); flags: also
 // set the cell flags (else the threshold pass sets them).
 void launch_fast(const Img* imgs, const int32_t* img_list, const int32_t* tile_prefix,

@@ -7,6 +7,8 @@
 
 #include "of_plan.h"
 
+#include <algorithm>
+
 namespace ofh {
 
 // Level l has scale s_l = scale^l, a float64 running product starting at 1;
@@ -81,6 +83,116 @@ bool k_fraction(float k, int64_t* num, int64_t* den) {
     *num = n;
     *den = d;
     return true;
+}
+
+// A level's column groups n (at most 64) and ceil(2^16 / n), which divides thread numbers by n: n | m << 8.
+static int32_t pack_groups(int n) { return n > 0 ? n | ((65536 + n - 1) / n << 8) : 0; }
+
+PyrAxis pyramid_axis(const int32_t* sizes, int nl, int nt, int max_extent, const int32_t* row_words) {
+    const bool columns = row_words == nullptr;
+    PyrAxis A;
+    A.nt = nt;
+    A.nl = nl;
+    A.ok = true;
+    std::vector<std::vector<int32_t>> tab(nl + 1);
+    for (int l = 1; l <= nl; ++l) {
+        tab[l].resize(sizes[l]);
+        resize_table(sizes[l - 1], sizes[l], tab[l].data());
+        if (columns)
+            for (int d = 1; d < sizes[l]; ++d)
+                if ((tab[l][d] >> 12) - (tab[l][d - 1] >> 12) > 3) A.ok = false;
+    }
+    // Tile boundaries: equal shares of every level, columns at multiples of 4.
+    auto bound = [&](int l, int i) {
+        if (i >= nt) return sizes[l];
+        const int b = (int)((int64_t)sizes[l] * i / nt);
+        return columns ? b & ~3 : b;
+    };
+    struct Range {
+        int c0 = 0, c1 = 0, o0 = 0, o1 = 0;
+    };
+    std::vector<std::vector<Range>> tiles(nt, std::vector<Range>(nl + 1));
+    A.extent.assign(nl + 1, 0);
+    int words = 0;
+    for (int i = 0; i < nt; ++i) {
+        int n = 4 * (nl + 1);
+        for (int l = nl; l >= 0; --l) {
+            Range& R = tiles[i][l];
+            int n0 = 0, n1 = 0;  // needed: the owned range and the sources of the next level's computed range
+            if (l > 0) {
+                R.o0 = n0 = bound(l, i);
+                R.o1 = n1 = std::max(bound(l, i + 1), R.o0);
+            }
+            if (l < nl && tiles[i][l + 1].c1 > tiles[i][l + 1].c0) {
+                const Range& N = tiles[i][l + 1];
+                const int d1 = std::min(N.c1, (int)sizes[l + 1]) - 1;
+                const int s0 = tab[l + 1][N.c0] >> 12, s1 = std::min((tab[l + 1][d1] >> 12) + 1, sizes[l] - 1) + 1;
+                if (n1 > n0) {
+                    n0 = std::min(n0, s0);
+                    n1 = std::max(n1, s1);
+                } else {
+                    n0 = s0;
+                    n1 = s1;
+                }
+            }
+            if (n1 > n0) {
+                const int q = !columns ? 1 : l > 0 ? 4 : 16;
+                R.c0 = n0 / q * q;
+                R.c1 = (n1 + q - 1) / q * q;
+            }
+            A.extent[l] = std::max(A.extent[l], R.c1 - R.c0);
+            if (l > 0) {
+                n += columns ? (R.c1 - R.c0) / 4 * 8 : R.c1 - R.c0;
+                A.computed += R.c1 - R.c0;
+                A.owned += R.o1 - R.o0;
+            }
+        }
+        words = std::max(words, n);
+    }
+    if (A.extent[0] > max_extent) A.ok = false;
+    A.stride = (words + 3) / 4 * 4;
+    A.blk.assign((size_t)A.stride * nt, 0);
+    if (!A.ok) return A;
+    for (int i = 0; i < nt; ++i) {
+        int32_t* b = A.blk.data() + (size_t)A.stride * i;
+        int32_t* e = b + 4 * (nl + 1);
+        for (int l = 0; l <= nl; ++l) {
+            const Range& R = tiles[i][l];
+            b[4 * l] = R.c0;
+            b[4 * l + 1] = !columns ? (R.c1 - R.c0) | row_words[l] << 16 : l > 0 ? pack_groups((R.c1 - R.c0) / 4) : R.c1 - R.c0;
+            b[4 * l + 2] = R.o0;
+            b[4 * l + 3] = R.o1;
+            if (l == 0) continue;
+            const int s0 = tiles[i][l - 1].c0;
+            if (!columns) {
+                for (int d = R.c0; d < R.c1; ++d) {
+                    const int t = tab[l][d];
+                    *e++ = (int32_t)((uint32_t)(((t >> 12) - s0) * row_words[l - 1]) << 16) | 2 * (t & 4095);
+                }
+                continue;
+            }
+            for (int d = R.c0; d < R.c1; d += 4) {
+                int xo[4];
+                uint32_t wgt[4], sel[4];
+                for (int k = 0; k < 4; ++k) {
+                    const int t = tab[l][std::min(d + k, sizes[l] - 1)];
+                    const uint32_t a2 = 2u * (uint32_t)(t & 4095);
+                    xo[k] = (t >> 12) - s0;
+                    wgt[k] = (4096u - a2) | (a2 << 16);
+                }
+                const int wa = xo[0] >> 2, wb = xo[2] >> 2;
+                for (int k = 0; k < 4; ++k) {
+                    const uint32_t o = (uint32_t)(xo[k] - 4 * (k < 2 ? wa : wb));
+                    sel[k] = o | ((o + 1u) << 4);
+                }
+                e[0] = wa | (wb << 16);
+                e[1] = (int32_t)(sel[0] | (sel[1] << 8) | (sel[2] << 16) | (sel[3] << 24));
+                for (int k = 0; k < 4; ++k) e[2 + k] = (int32_t)wgt[k];
+                e += 8;
+            }
+        }
+    }
+    return A;
 }
 
 float response_scale(int64_t den) {
