@@ -88,12 +88,12 @@ typedef struct of_tuning {
                                      tiles with the general kernel's layout (cells of 15 or 30 pixels);
                                      0: general FAST (fast_tile_h rows), then a threshold pass; 3: general
                                      FAST on 128 x 32 tiles with per-warp pipelines, then the pass; 4: the
-                                     same on strips one cell row high, which also set the cell flags, then
-                                     the pass applies them (cells of 8..33 pixels).  With nms_tile_h 32 the
-                                     NMS kernel applies the cell flags itself: the pass then only sets
-                                     flags where FAST does not */
+                                     same on strips one cell row high (a part of one in small batches), which
+                                     also set the cell flags (cells of 8..33 pixels).  After form 4, and with
+                                     nms_tile_h 32, the NMS kernel applies the cell flags itself: the pass
+                                     then only sets flags where FAST does not */
     int32_t nms_tile_h;           /* NMS + Harris tile height: 32 (per-warp kernel on the 128 x 32 detect
-                                     tiles), 64 or 128 rows (block kernels) */
+                                     tiles, 8 or 16 rows in small batches), 64 or 128 rows (block kernels) */
     int32_t fast_tile_h;          /* general FAST tile height: 32, 64, 128 or 256 rows */
     int32_t candidates_tried;     /* configurations timed */
     float resize_ms, fast_ms, nms_ms;  /* best measured time of each tuned stage (all levels);

@@ -59,8 +59,8 @@ class OfTuning(C.Structure):
     stream_groups (1..8): frame groups on forked graph branches; fast_cell_tiles:
     0 general FAST + threshold pass, 1 cell-tile kernel, 2 cell-aligned general kernel,
     3 general FAST with per-warp pipelines + threshold pass, 4 the same on cell-row strips
-    that also set the cell flags + the pass applying them (with nms_tile_h 32 the per-warp
-    NMS kernel applies the flags itself and the pass only sets flags FAST leaves unset);
+    that also set the cell flags (after form 4, and with nms_tile_h 32, the NMS kernel
+    applies the flags itself and the pass only sets flags FAST leaves unset);
     fast_tile_h (32/64/128/256) and nms_tile_h (32/64/128): tile heights.  The last
     four fields report the autotuner's search (candidates, best stage times in ms)."""
 

@@ -40,6 +40,7 @@
 #include <cuda_runtime.h>
 
 #include "of_internal.h"
+#include "of_launch.cuh"
 #include "of_tile.cuh"
 #include "of_tma.cuh"
 
@@ -599,6 +600,12 @@ int fast_warp_blocks_per_sm() {
 // Work items come from the plan's item table (image, x0, y0): lane 0 reads
 // one entry per item instead of searching the image list, which was a chain
 // of dependent loads the rest of the warp waited on (FAST 2.06 -> 1.99 ms).
+// In small batches an item is a part of a cell row (`sub` rows; its flags OR
+// into the same cells): 1480 strips of a 1080p frame are fewer than the 2432
+// resident warps.  Items go to blocks first, then to their warps, so that few
+// items spread over all SMs (8 1080p frames: 151 -> 141 us, a stereo pair of
+// 720p frames 32 -> 28).  Launched beside the pyramid's end, the strips of
+// level 0, the caller's frame, do not wait for it.
 // An image's last tile column often holds few region columns (18..52 on
 // three of the eight 1080p levels): with at most 64 (32) of them the lanes
 // form 2 (4) row groups over the first 64 (32) columns, so fewer lanes idle.
@@ -606,7 +613,7 @@ int fast_warp_blocks_per_sm() {
 __global__ void __launch_bounds__(DET_THREADS, 2)
 k_fast_cstrip(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_tiles,
               const CUtensorMap* __restrict__ maps, const Call* __restrict__ call, int t_hi, int t_lo, int border,
-              int cell, uint32_t cell_magic, int order) {
+              int cell, int sub, uint32_t cell_magic, int order) {
     // cell_magic = 2^32 / cell rounded up: n / cell == umulhi(n, cell_magic) for 0 <= n < 2^16.
     extern __shared__ __align__(128) uint8_t fw_dyn[];
     uint8_t* const base = fw_dyn + ((128u - (smem_u32(fw_dyn) & 127u)) & 127u);
@@ -614,18 +621,26 @@ k_fast_cstrip(const Img* __restrict__ imgs, const uint2* __restrict__ items, int
     __shared__ TileInfo tinfo[FW_WARPS][2];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint8_t* const wbuf = base + w * 2 * FAST_BUF;
+    pdl_trigger();
     if (lane == 0) {
         mbar_init(&mbar[w][0], 1);
         mbar_init(&mbar[w][1], 1);
         fence_barrier_init();
     }
     __syncwarp();
-    const int nw = gridDim.x * FW_WARPS, gw = blockIdx.x * FW_WARPS + w;
+    const int nw = gridDim.x * FW_WARPS, gw = w * gridDim.x + blockIdx.x;
+    // Level 0 is the caller's frame (or its copy, made before the chain): its
+    // strips need not wait for the pyramid's kernel.
+    bool waited = false;  // lane 0
     auto issue = [&](int t, int b) {  // lane 0
         const TileInfo ti = item_info(items, t);
         const int ii = ti.img;
         tinfo[w][b] = ti;
         tensormap_acquire(maps + ii);
+        if (!waited && imgs[ii].level != 0) {
+            pdl_wait();
+            waited = true;
+        }
         mbar_arrive_expect_tx(&mbar[w][b], FAST_BOX);
         tma_load_2d(wbuf + b * FAST_BUF, maps + ii, ti.x0 - HALO_X, ti.y0 - 4, &mbar[w][b]);
     };
@@ -658,7 +673,8 @@ k_fast_cstrip(const Img* __restrict__ imgs, const uint2* __restrict__ items, int
         const uint8_t* const s = wbuf + b * FAST_BUF;
         const int X0 = ti.x0, y0 = ti.y0;
         const int rx0 = border, rx1 = I.w - border;
-        const int nrows = min(cell, I.h - border - y0);
+        const int cy = (int)__umulhi((uint32_t)(y0 - border), cell_magic);
+        const int nrows = min(min(sub, cell - (y0 - border - cy * cell)), I.h - border - y0);
         // A tile column with at most 64 (32) columns of the detect region left:
         // the lanes split into 2 (4) row groups that each score columns
         // X0 .. X0+63 (X0+31) over hq = nrows / groups rows (rounded up).  The
@@ -725,20 +741,21 @@ k_fast_cstrip(const Img* __restrict__ imgs, const uint2* __restrict__ items, int
                                   ((strong & ~mask_a) ? 2u << (ca - cx0) : 0u);
             const uint32_t flags = __reduce_or_sync(0xFFFFFFFFu, bits);
             if ((flags >> lane) & 1u)
-                atomicOr(&I.cell[(size_t)__umulhi((uint32_t)(y0 - border), cell_magic) * I.ncx + cx0 + lane], 1u);
+                atomicOr(&I.cell[(size_t)cy * I.ncx + cx0 + lane], 1u);
         }
         __syncwarp();  // every lane is done with buffer b before lane 0 refills it
     }
+    pdl_wait();
 }
 
 void launch_fast_cstrip(const Img* imgs, const uint2* items, int n_strips, const CUtensorMap* maps, const Call* call,
-                        int t_hi, int t_lo, int border, int cell, int grid, int order, void* stream) {
+                        int t_hi, int t_lo, int border, int cell, int sub, int grid, int order, void* stream,
+                        bool pdl) {
     if (n_strips <= 0) return;
-    const int warps = (n_strips + FW_WARPS - 1) / FW_WARPS;
-    grid = grid < warps ? grid : warps;
+    grid = grid < n_strips ? grid : n_strips;
     const uint32_t magic = 0xFFFFFFFFu / (uint32_t)cell + 1u;
-    k_fast_cstrip<<<grid, DET_THREADS, FW_DYN, (cudaStream_t)stream>>>(imgs, items, n_strips, maps, call, t_hi, t_lo,
-                                                                       border, cell, magic, order);
+    launch_chain(k_fast_cstrip, grid, DET_THREADS, FW_DYN, (cudaStream_t)stream, pdl, 1, imgs, items, n_strips, maps, call,
+                 t_hi, t_lo, border, cell, sub, magic, order);
 }
 
 int fast_cstrip_blocks_per_sm() {
@@ -790,6 +807,8 @@ k_fast_cells(const Img* __restrict__ imgs, const int32_t* __restrict__ list, con
     const int tw = cpt * cell, th = cr * cell;
     const int srow0 = wcr * cell + CT_RPT * wr;  // the warp's first staged row (staged row 0 = tile row -3)
     const int loads = ((cr - 1) * cell + CT_RPT * nw + 6 + IMG_BOX_ROWS - 1) / IMG_BOX_ROWS;  // 1 or 2
+    pdl_trigger();
+    pdl_wait();
     if (tid == 0) {
         mbar_init(&mbar[0], 1);
         mbar_init(&mbar[1], 1);
@@ -964,12 +983,12 @@ k_fast_cells(const Img* __restrict__ imgs, const int32_t* __restrict__ list, con
 
 void launch_fast_cells(const Img* imgs, const int32_t* img_list, const int32_t* tile_prefix, int n_list,
                        int n_tiles, const CUtensorMap* maps, const Call* call, int t_hi, int t_lo, int border,
-                       int cell, int grid, int order, void* stream) {
+                       int cell, int grid, int order, void* stream, bool pdl) {
     if (n_tiles <= 0) return;
     grid = grid < n_tiles ? grid : n_tiles;
     const int threads = 32 * ct_warps(cell) * ct_cell_rows(cell), cpt = CT_MAX_W / cell;
-    k_fast_cells<<<grid, threads, 0, (cudaStream_t)stream>>>(imgs, img_list, tile_prefix, n_list, n_tiles, maps,
-                                                              call, t_hi, t_lo, border, cell, cpt, order);
+    launch_chain(k_fast_cells, grid, threads, 0, (cudaStream_t)stream, pdl, 1, imgs, img_list, tile_prefix, n_list,
+                 n_tiles, maps, call, t_hi, t_lo, border, cell, cpt, order);
 }
 
 int fast_cells_blocks_per_sm(int cell) {

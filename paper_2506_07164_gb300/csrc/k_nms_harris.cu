@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "of_internal.h"
+#include "of_launch.cuh"
 #include "of_tile.cuh"
 #include "of_tma.cuh"
 
@@ -270,6 +271,7 @@ k_nms_harris(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
     __shared__ int nq;
 
     const int tid = threadIdx.x;
+    pdl_trigger();
     if (tid == 0) {
         mbar_init(&mbar[0], 1);
         mbar_init(&mbar[1], 1);
@@ -285,6 +287,7 @@ k_nms_harris(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
         tinfo[b] = NmsTile{ii, x0, y0};
         tensormap_acquire(score_maps + ii);
         tensormap_acquire(img_maps + ii);
+        pdl_wait();  // FAST's scores (and the pyramid's levels)
         mbar_arrive_expect_tx(&mbar[b], G::S_LOADS * S_BOX + G::I_LOADS * I_BOX);
 #pragma unroll
         for (int k = 0; k < G::S_LOADS; ++k)
@@ -298,6 +301,7 @@ k_nms_harris(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
     const int g = gridDim.x;
     if (tid == 0 && tile_of(order, blockIdx.x, g, n_tiles, 0) < n_tiles) issue(tile_of(order, blockIdx.x, g, n_tiles, 0), 0);
 
+    pdl_wait();
     const int lane = tid & 31, ty = tid >> 5;
     const int64_t knum = call->knum, kden = call->kden;
     for (int it = 0;; ++it) {
@@ -418,6 +422,8 @@ k_nms_harris(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
 // keys of the queued survivors (rounds of 32, one survivor per lane; a 32-row
 // tile holds ~90 at t = 20, so lanes are ~90 % busy) and refill the image
 // buffer.  No block barrier: a warp never waits for another warp.
+// Small batches take tiles of 8 or 16 of the 32 rows (`rows`; the boxes stay),
+// so that more warps share a frame; tiles go to blocks first, then to warps.
 //
 // APPLY: the maps hold s(p) - (t_lo - 1) where s(p) >= t_lo (FAST's output)
 // and the cell flags are set.  Each staged score word becomes S(p) in
@@ -483,7 +489,8 @@ template <bool APPLY, bool SMALL_T>
 __global__ void __launch_bounds__(DET_THREADS, 2)
 k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_tiles,
            const CUtensorMap* __restrict__ img_maps, const CUtensorMap* __restrict__ score_maps,
-           const Call* __restrict__ call, int t_hi, int t_lo, int border, int cell, uint32_t cell_magic, int order) {
+           const Call* __restrict__ call, int t_hi, int t_lo, int border, int cell, int rows, uint32_t cell_magic,
+           int order) {
     extern __shared__ __align__(128) uint8_t nw_raw[];
     uint8_t* const dyn = nw_raw + ((128u - (smem_u32(nw_raw) & 127u)) & 127u);
     __shared__ __align__(8) uint64_t mbar[NW_WARPS][2];  // [0] score box, [1] image box
@@ -491,13 +498,14 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
     uint8_t* const sS = dyn + w * NW_BYTES;
     uint8_t* const sI = sS + NW_SBUF;
     uint16_t* const queue = reinterpret_cast<uint16_t*>(sI + I_BOX);
+    pdl_trigger();
     if (lane == 0) {
         mbar_init(&mbar[w][0], 1);
         mbar_init(&mbar[w][1], 1);
         fence_barrier_init();
     }
     __syncwarp();
-    const int nw = gridDim.x * NW_WARPS, gw = blockIdx.x * NW_WARPS + w;
+    const int nw = gridDim.x * NW_WARPS, gw = w * gridDim.x + blockIdx.x;
     auto locate = [&](int t) {  // the plan's item table: (image, (y0 << 16) | x0)
         const uint2 e = __ldg(items + t);
         return NmsTile{(int)e.x, (int)(e.y & 0xFFFFu), (int)(e.y >> 16)};
@@ -517,9 +525,14 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
     if (t < n_tiles) {
         cur = locate(t);
         if (lane == 0) {
-            issue_s(cur);
-            issue_i(cur);
+            tensormap_acquire(score_maps + cur.img);
+            tensormap_acquire(img_maps + cur.img);
         }
+    }
+    pdl_wait();  // FAST's scores and flags (and the pyramid's levels)
+    if (t < n_tiles && lane == 0) {
+        issue_s(cur);
+        issue_i(cur);
     }
     const int64_t knum = call->knum, kden = call->kden;
     const uint32_t th = (uint32_t)(t_hi - t_lo + 1);  // t_hi in the maps' offset scores
@@ -551,7 +564,7 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
             const int rx0 = border, rx1 = I.w - border, ry0 = border, ry1 = I.h - border;
             const int xc = X0 + 4 * lane;
             const int xh = lane == 0 ? X0 - 4 : X0 + TILE_W;  // the halo word (used by lanes 0 and 31)
-            const int nrows = min(TILE_H, ry1 - Y0);
+            const int nrows = min(rows, ry1 - Y0);
             const uint8_t* const srow = sS + HALO_X + 4 * lane;
             const int hoff = xh - xc;
             // Zero the staged bytes outside the detect region, and outside the
@@ -710,28 +723,27 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
 template <bool APPLY, bool SMALL_T>
 static void launch_nms_warp_t(const Img* imgs, const uint2* items, int n_tiles, const CUtensorMap* img_maps,
                               const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo, int border,
-                              int cell, int grid, int order, void* stream) {
+                              int cell, int rows, int grid, int order, void* stream, bool pdl) {
     const uint32_t magic = 0xFFFFFFFFu / (uint32_t)cell + 1u;
-    k_nms_warp<APPLY, SMALL_T><<<grid, DET_THREADS, NW_DYN, (cudaStream_t)stream>>>(
-        imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell, magic, order);
+    launch_chain(k_nms_warp<APPLY, SMALL_T>, grid, DET_THREADS, NW_DYN, (cudaStream_t)stream, pdl, 1, imgs, items, n_tiles,
+                 img_maps, score_maps, call, t_hi, t_lo, border, cell, rows, magic, order);
 }
 
 void launch_nms_warp(const Img* imgs, const uint2* items, int n_tiles, const CUtensorMap* img_maps,
                      const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo, int border, int cell,
-                     int grid, int order, void* stream, bool apply) {
+                     int rows, int grid, int order, void* stream, bool apply, bool pdl) {
     if (n_tiles <= 0) return;
-    const int warps = (n_tiles + NW_WARPS - 1) / NW_WARPS;
-    grid = grid < warps ? grid : warps;
+    grid = grid < n_tiles ? grid : n_tiles;
     apply = apply && t_hi != t_lo;
     if (!apply)
-        launch_nms_warp_t<false, true>(imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell,
-                                       grid, order, stream);
+        launch_nms_warp_t<false, true>(imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell, rows,
+                                       grid, order, stream, pdl);
     else if (t_hi - t_lo + 1 <= 128)
-        launch_nms_warp_t<true, true>(imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell,
-                                      grid, order, stream);
+        launch_nms_warp_t<true, true>(imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell, rows,
+                                      grid, order, stream, pdl);
     else
-        launch_nms_warp_t<true, false>(imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell,
-                                       grid, order, stream);
+        launch_nms_warp_t<true, false>(imgs, items, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell, rows,
+                                       grid, order, stream, pdl);
 }
 
 // Resident blocks per SM of the per-warp NMS kernel (also raises its dynamic shared-memory limit).
@@ -751,22 +763,21 @@ int nms_warp_blocks_per_sm() {
 template <bool FINAL, int TH>
 void launch_nms_t(const Img* imgs, const int32_t* img_list, const int32_t* tile_prefix, int n_list, int n_tiles,
                   const CUtensorMap* img_maps, const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo,
-                  int border, int cell, int grid, int order, void* stream) {
+                  int border, int cell, int grid, int order, void* stream, bool pdl) {
     const uint32_t magic = 0xFFFFFFFFu / (uint32_t)cell + 1u;
-    k_nms_harris<FINAL, TH><<<grid, DET_THREADS, NmsGeom<TH>::DYN_BYTES, (cudaStream_t)stream>>>(
-        imgs, img_list, tile_prefix, n_list, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell, magic,
-        order);
+    launch_chain(k_nms_harris<FINAL, TH>, grid, DET_THREADS, NmsGeom<TH>::DYN_BYTES, (cudaStream_t)stream, pdl, 1, imgs,
+                 img_list, tile_prefix, n_list, n_tiles, img_maps, score_maps, call, t_hi, t_lo, border, cell, magic, order);
 }
 
 void launch_nms_harris(const Img* imgs, const int32_t* img_list, const int32_t* tile_prefix,
                        int n_list, int n_tiles, const CUtensorMap* img_maps, const CUtensorMap* score_maps,
                        const Call* call, int t_hi, int t_lo, int border, int cell, int grid, int order,
-                       void* stream, bool final_scores, int tile_h) {
+                       void* stream, bool final_scores, int tile_h, bool pdl) {
     if (n_tiles <= 0) return;
     grid = grid < n_tiles ? grid : n_tiles;
 #define OF_NMS_LAUNCH(FI, TH)                                                                                  \
     launch_nms_t<FI, TH>(imgs, img_list, tile_prefix, n_list, n_tiles, img_maps, score_maps, call, t_hi, t_lo, \
-                         border, cell, grid, order, stream)
+                         border, cell, grid, order, stream, pdl)
     if (final_scores) {
         if (tile_h == 64) OF_NMS_LAUNCH(true, 64);
         else if (tile_h == 128) OF_NMS_LAUNCH(true, 128);

@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "of_internal.h"
+#include "of_launch.cuh"
 
 namespace ofk {
 
@@ -22,7 +23,11 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
          const Call* __restrict__ call, const uint16_t* __restrict__ slot_img) {
     const int slot = slot_begin + blockIdx.x * ORIENT_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
-    if (slot >= slot_end) return;
+    pdl_trigger();
+    if (slot >= slot_end) {
+        pdl_wait();
+        return;
+    }
     // The slot's image: from the plan's slot table, else a search over slot0.
     int lo = img_begin, hi = img_begin + n_img - 1;
     if (slot_img) {
@@ -37,9 +42,16 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
     const int rank = slot - I.slot0;
     const int levels = call->levels;
     const Img* F = imgs + I.frame * levels;
+    // Descriptor fields, read before the wait.
+    const uint8_t* img = I.img;
+    const int pitch = I.pitch, quota = I.quota, level = I.level;
+    const int32_t* const ctr = I.ctr;
+    const uint32_t* const kyx = I.kyx;
+    const bool first = slot == I.frame * call->n_features;
+    pdl_wait();  // the kept keypoints
 
     // The frame's first slot publishes its keypoint count.
-    if (slot == I.frame * call->n_features) {
+    if (first) {
         if (lane == 0) {
             int total = 0;
             for (int l = 0; l < levels; ++l) total += F[l].ctr[1];
@@ -47,14 +59,12 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
             call->counts[I.frame] = *call->status ? OF_ERR_TIMEOUT : total;
         }
     }
-    if (rank >= I.quota || rank >= I.ctr[1]) return;
+    if (rank >= quota) return;
+    const uint32_t yx = kyx[rank];  // issued beside the count; unused beyond it
+    if (rank >= ctr[1]) return;
     int base = 0;
-    for (int l = 0; l < I.level; ++l) base += F[l].ctr[1];
-
-    const uint32_t yx = I.kyx[rank];
+    for (int l = 0; l < level; ++l) base += F[l].ctr[1];
     const int x = (int)(yx & 0xFFFFu), y = (int)(yx >> 16);
-    const uint8_t* img = I.img;
-    const int pitch = I.pitch;
 
     // Harris sums over the 7 x 7 window.
     int a = 0, b = 0, c = 0;
@@ -139,15 +149,15 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
 }
 
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,
-                         void* stream, const uint16_t* slot_img) {
+                         void* stream, const uint16_t* slot_img, bool pdl) {
     if (slot_end <= slot_begin || n_img <= 0) return;
     const int blocks = (slot_end - slot_begin + ORIENT_WARPS - 1) / ORIENT_WARPS;
-    k_orient<<<blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream>>>(imgs, img_begin, n_img, slot_begin, slot_end,
-                                                                       call, slot_img);
+    launch_chain(k_orient, blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream, pdl, 1, imgs, img_begin, n_img, slot_begin,
+                 slot_end, call, slot_img);
 }
 
 void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream) {
-    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, stream, nullptr);
+    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, stream, nullptr, false);
 }
 
 // ---------------------------------------------------------------- inspect

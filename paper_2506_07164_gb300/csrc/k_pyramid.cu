@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include "of_internal.h"
+#include "of_launch.cuh"
 #include "of_tma.cuh"
 
 namespace ofk {
@@ -200,6 +201,7 @@ k_pyramid(const PyrJob* __restrict__ jobs, const uint2* __restrict__ items, cons
     int32_t* const xs = reinterpret_cast<int32_t*>(T + t_bytes);
     int32_t* const ys = xs + x_words;
     const int tid = threadIdx.x;
+    pdl_trigger();
     const uint2 it = __ldg(items + blockIdx.x);  // (job, (tile row << 16) | tile column)
     const PyrJob& J = jobs[it.x];
     const int32_t* const xg = J.xblk + (size_t)(it.y & 0xFFFFu) * J.xstride;
@@ -208,6 +210,7 @@ k_pyramid(const PyrJob* __restrict__ jobs, const uint2* __restrict__ items, cons
         mbar_init(&mbar, 1);
         fence_barrier_init();
         tensormap_acquire(maps + it.x);
+        pdl_wait();  // a later run reads the levels of the run before it
         mbar_arrive_expect_tx(&mbar, (uint32_t)(J.box_w * J.box_h));
         tma_load_2d(S, maps + it.x, __ldg(xg), __ldg(yg), &mbar);
     }
@@ -217,6 +220,7 @@ k_pyramid(const PyrJob* __restrict__ jobs, const uint2* __restrict__ items, cons
         reinterpret_cast<int4*>(ys)[i] = __ldg(reinterpret_cast<const int4*>(yg) + i);
     const int nl = J.nl;
     __syncthreads();
+    pdl_wait();
     const bool ok = mbar_wait(&mbar, 0);
     if (__syncthreads_or(!ok)) {
         if (tid == 0) {
@@ -288,10 +292,10 @@ int pyramid_smem(int s_bytes, int t_bytes, int x_words, int y_words) {
 }
 
 void launch_pyramid(const PyrJob* jobs, const uint2* items, int n_tiles, const CUtensorMap* maps, const Call* call,
-                    int s_bytes, int t_bytes, int x_words, int y_words, void* stream) {
+                    int s_bytes, int t_bytes, int x_words, int y_words, void* stream, bool pdl) {
     if (n_tiles <= 0) return;
-    k_pyramid<<<n_tiles, PY_THREADS, pyramid_smem(s_bytes, t_bytes, x_words, y_words), (cudaStream_t)stream>>>(
-        jobs, items, maps, call, s_bytes, t_bytes, x_words);
+    launch_chain(k_pyramid, n_tiles, PY_THREADS, pyramid_smem(s_bytes, t_bytes, x_words, y_words),
+                 (cudaStream_t)stream, pdl, 1, jobs, items, maps, call, s_bytes, t_bytes, x_words);
 }
 
 // Raised once to the largest size any plan may use, so graphs captured for

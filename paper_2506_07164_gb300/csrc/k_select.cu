@@ -33,6 +33,7 @@
 #include <mutex>
 
 #include "of_internal.h"
+#include "of_launch.cuh"
 
 namespace ofk {
 
@@ -181,9 +182,13 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
 
     const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;  // block's place in its image's cluster
     const Img& I = imgs[blockIdx.x / C];
-    const int n = min(I.ctr[0], I.cand_cap);
-    const int q = I.quota;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int q = I.quota;
+    const int32_t* const ctr = I.ctr;
+    pdl_trigger();
+    for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) hist[i] = 0u;
+    pdl_wait();  // the candidates
+    const int n = min(ctr[0], I.cand_cap);
     if (q <= 0 || n <= 0) {  // the same for all blocks of the cluster
         if (tid == 0 && rank == 0) I.ctr[1] = 0;
         return;
@@ -208,7 +213,6 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         st.n_take = m;
         s_cnt = 0;
     }
-    for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) hist[i] = 0u;
     __syncthreads();
 
     // This block's candidate pairs: first, step (in pairs of keys).
@@ -467,20 +471,9 @@ int select_smem_bytes(int max_quota) {
 }
 
 template <int C>
-static void launch_select_t(const Img* imgs, int n_img, const Call* call, int mq, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_img * C);
-    cfg.blockDim = dim3(SELECT_THREADS);
-    cfg.dynamicSmemBytes = select_smem_bytes(mq);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = C > 1 ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, k_select<C>, imgs, call, select_sort_cap(mq));
+static void launch_select_t(const Img* imgs, int n_img, const Call* call, int mq, cudaStream_t st, bool pdl) {
+    launch_chain(k_select<C>, n_img * C, SELECT_THREADS, select_smem_bytes(mq), st, pdl, C, imgs, call,
+                 select_sort_cap(mq));
 }
 
 // Blocks per image, by the images of the launch.  A cluster shortens the scan
@@ -490,14 +483,14 @@ static void launch_select_t(const Img* imgs, int n_img, const Call* call, int mq
 // to 304.  Measured stage times (1080p, 8 levels; 1 / 2 / 4 / 8 blocks): 8
 // images 41 / 33 / 27 / 22 us, 32 images 43 / 35 / 26 / 28, 128 images 49 / 39
 // / 35 / 41, 304 images 64 / 57 / 64 / 84, 1024 images 97 / 119 / 149 / 218.
-void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream) {
+void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream, bool pdl) {
     if (n_img <= 0) return;
     const int mq = max_quota > 0 ? max_quota : 1;
     const cudaStream_t st = (cudaStream_t)stream;
-    if (n_img <= 16) launch_select_t<8>(imgs, n_img, call, mq, st);
-    else if (n_img <= 128) launch_select_t<4>(imgs, n_img, call, mq, st);
-    else if (n_img <= 304) launch_select_t<2>(imgs, n_img, call, mq, st);
-    else launch_select_t<1>(imgs, n_img, call, mq, st);
+    if (n_img <= 16) launch_select_t<8>(imgs, n_img, call, mq, st, pdl);
+    else if (n_img <= 128) launch_select_t<4>(imgs, n_img, call, mq, st, pdl);
+    else if (n_img <= 304) launch_select_t<2>(imgs, n_img, call, mq, st, pdl);
+    else launch_select_t<1>(imgs, n_img, call, mq, st, pdl);
 }
 
 // The limit is a per-device attribute of the kernel shared by every handle,

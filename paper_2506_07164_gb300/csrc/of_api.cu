@@ -219,8 +219,9 @@ struct Plan {
         int img_begin = 0, n_img = 0;
         int dl_begin = 0, n_list = 0, det_tiles = 0, dp_off = 0;
         int fast_tiles = 0, fp_off = 0;             // cell-tile FAST: tiles and prefix offset in gp_fast
-        int cs_strips = 0, cs_off = 0;              // cell-strip FAST: strips and prefix offset in gp_cstrip
+        int cs_strips = 0;                          // cell-strip FAST: strips
         int csi_off = 0, dti_off = 0;               // item tables: cell strips, 128 x 32 detect tiles
+        int nm_tiles = 0, nmi_off = 0;              // 128 x nms_rows tiles of the per-warp NMS kernel and their table
         int nms64_tiles = 0, np_off = 0;            // NMS with 64-row tiles: tiles and prefix offset in gp_nms64
         int ftall_tiles[2] = {0, 0}, ftall_off[2] = {0, 0};  // FAST on FT_HS[i]-row tiles: tiles, offset in gp_ftall[i]
         int fal_tiles = 0, fal_off = 0;             // cell-aligned FAST: tiles and prefix offset in gp_fal
@@ -231,9 +232,12 @@ struct Plan {
         std::vector<int> py_off, py_n;              // per fused run: its tiles in items_py
     };
     std::vector<Group> groups[kMaxGroups + 1];
-    std::vector<int32_t> gp_det, gp_rs, gp_fast, gp_rows, gp_nms64, gp_ftall[2], gp_fal, gp_cstrip;
+    std::vector<int32_t> gp_det, gp_rs, gp_fast, gp_rows, gp_nms64, gp_ftall[2], gp_fal;
     // Work-item tables of the per-warp kernels, per group: (image, (y0 << 16) | x0).
-    std::vector<uint2> items_cs, items_dt;
+    std::vector<uint2> items_cs, items_dt, items_nm;
+    int strip_rows = 0;  // rows of a FAST strip (a cell row or part of one)
+    int nms_rows = 0;    // rows of a per-warp NMS tile (32: the detect tiles)
+    bool pdl = false;    // chain the kernels by programmatic launches
     std::vector<uint16_t> slot_img;  // image of every output slot (orientation kernel)
     // Fused pyramid: the levels 1 .. L-1 as runs of levels, one launch each.
     struct Run {
@@ -254,7 +258,7 @@ struct Plan {
     uint8_t* dbuf = nullptr;
     size_t off_call = 0, off_img = 0, off_rs = 0, off_dl = 0, off_tab = 0, off_ftab = 0;
     size_t off_gdp = 0, off_grs = 0, off_gfp = 0, off_grp = 0, off_gnp = 0, off_gft[2] = {0, 0}, off_gfal = 0,
-           off_gcs = 0, off_ics = 0, off_idt = 0, off_ipy = 0, off_sli = 0, off_pj = 0, off_pblk = 0;
+           off_ics = 0, off_idt = 0, off_inm = 0, off_ipy = 0, off_sli = 0, off_pj = 0, off_pblk = 0;
     size_t off_maps = 0;
     std::vector<CUtensorMap> h_maps;  // [image maps | score maps] (n_img each) | source maps of the pyramid jobs
     of_tuning tun{};  // launch configuration (defaults, or the autotuner's choice)
@@ -286,8 +290,8 @@ struct Plan {
     const int32_t* d_grs() const { return reinterpret_cast<const int32_t*>(dbuf + off_grs); }
     const int32_t* d_gfp() const { return reinterpret_cast<const int32_t*>(dbuf + off_gfp); }
     const int32_t* d_grp() const { return reinterpret_cast<const int32_t*>(dbuf + off_grp); }
-    const int32_t* d_gcs() const { return reinterpret_cast<const int32_t*>(dbuf + off_gcs); }
     const uint2* d_ics() const { return reinterpret_cast<const uint2*>(dbuf + off_ics); }
+    const uint2* d_inm() const { return reinterpret_cast<const uint2*>(dbuf + off_inm); }
     const uint2* d_idt() const { return reinterpret_cast<const uint2*>(dbuf + off_idt); }
     const uint2* d_ipy() const { return reinterpret_cast<const uint2*>(dbuf + off_ipy); }
     const PyrJob* d_pj() const { return reinterpret_cast<const PyrJob*>(dbuf + off_pj); }
@@ -310,12 +314,10 @@ bool cell_form(const Plan* P) {
 bool strip_form(const Plan* P) { return P->strip_ok && P->tun.fast_cell_tiles == 4; }
 bool warp_form(const Plan* P) { return P->tun.fast_cell_tiles == 3 && P->apply_flags; }
 bool fast_sets_flags(const Plan* P) { return strip_form(P) || (!cell_form(P) && !P->apply_flags); }
-// The per-warp NMS kernel (32-row tiles) applies the flags to its staged
-// score words itself; the pass then only sets flags where FAST did not (for
-// images with proposal tiles at least: FAST skips their flags).
-bool nms_applies(const Plan* P) {
-    return P->tun.nms_tile_h == 32 && !cell_form(P) && P->s.t_hi != P->s.t_lo;
-}
+// The per-warp NMS kernel (nms_tile_h 32), and the block kernels after the
+// cell-row strips, apply flags and proposal tiles to their staged scores
+// themselves; the pass then only sets flags where FAST did not.
+bool nms_applies(const Plan* P) { return !cell_form(P) && (P->tun.nms_tile_h == 32 || strip_form(P)); }
 
 int plan_fast_bps(const Plan* P) {
     if (P->aligned_ok && P->tun.fast_cell_tiles == 2) return fast_aligned_blocks_per_sm();
@@ -378,11 +380,15 @@ struct DeviceGuard {
 };
 
 // Enqueue stage `stage` of one frame group of a plan on `st` (stage 0 here is
-// the resize chain only; the clearing memset is enqueued once per call):
+// the resize chain only; the clearing memset is enqueued once per call).  pdl:
+// a kernel of this chain is the last thing on `st`, so the next one may start
+// beside its end (false after the memset or an event, and for plans without
+// pdl); kept up to date here.
 //   0 resize levels 1..L-1 (pyramid)   1 FAST score + cell flags
 //   2 (threshold pass,) NMS + Harris keys
 //   3 top-N per level                  4 orientation + output records
-void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage, cudaStream_t st) {
+void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage, cudaStream_t st,
+                         bool& pdl) {
     const Settings& s = P->s;
     const int nl = s.levels;
     switch (stage) {
@@ -392,7 +398,8 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
                     const Plan::Run& R = P->runs[c];
                     launch_pyramid(P->d_pj() + R.job_begin, P->d_ipy() + G.py_off[c], G.py_n[c],
                                    P->d_maps() + 2 * P->n_img + R.job_begin, P->d_call(), R.s_bytes, R.t_bytes,
-                                   R.x_words, R.y_words, st);
+                                   R.x_words, R.y_words, st, pdl);
+                    pdl = P->pdl && (pdl || G.py_n[c] > 0);
                 }
                 break;
             }
@@ -402,6 +409,7 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
                 const int v = P->tun.resize_tile_h == RS_TILE_HS[0] ? 0 : 1;
                 launch_resize(P->d_rs() + G.rs_job[l], P->d_grs() + G.rsp_off[v][l], nj, G.rs_tiles[v][l],
                               RS_TILE_HS[v], st);
+                pdl = P->pdl;
             }
             break;
         case 1:
@@ -413,11 +421,12 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
                                     H->n_sms * P->tun.fast_blocks_per_sm, P->tun.fast_order, st);
             else if (strip_form(P))
                 launch_fast_cstrip(P->d_img(), P->d_ics() + G.csi_off, G.cs_strips, P->d_maps(), P->d_call(), s.t_hi,
-                                   s.t_lo, s.border, s.cell, H->n_sms * P->tun.fast_blocks_per_sm, P->tun.fast_order, st);
+                                   s.t_lo, s.border, s.cell, P->strip_rows, H->n_sms * P->tun.fast_blocks_per_sm,
+                                   P->tun.fast_order, st, pdl);
             else if (cell_form(P))
                 launch_fast_cells(P->d_img(), P->d_dl() + G.dl_begin, P->d_gfp() + G.fp_off, G.n_list, G.fast_tiles,
                                   P->d_maps(), P->d_call(), s.t_hi, s.t_lo, s.border, s.cell,
-                                  H->n_sms * P->tun.fast_blocks_per_sm, P->tun.fast_order, st);
+                                  H->n_sms * P->tun.fast_blocks_per_sm, P->tun.fast_order, st, pdl);
             else if (warp_form(P))
                 launch_fast_warp(P->d_img(), P->d_dl() + G.dl_begin, P->d_gdp() + G.dp_off, G.n_list, G.det_tiles,
                                  P->d_maps(), P->d_call(), s.t_lo, s.border, H->n_sms * P->tun.fast_blocks_per_sm,
@@ -437,40 +446,44 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
                 launch_fast(P->d_img(), P->d_dl() + G.dl_begin, P->d_gdp() + G.dp_off, G.n_list, G.det_tiles,
                             P->d_maps(), P->d_call(), s.t_hi, s.t_lo, s.border, s.cell,
                             H->n_sms * P->tun.fast_blocks_per_sm, P->tun.fast_order, st, fast_sets_flags(P), 32);
+            pdl = P->pdl && (pdl || G.n_list > 0);
             break;
         case 2: {
             if (!cell_form(P)) {
-                const int flags = strip_form(P) ? 2 : fast_sets_flags(P) ? 0 : 1;
-                const bool apply = !nms_applies(P);
-                // Flags of images with proposal tiles only (flags 2, no apply): the
+                // Flags of images with proposal tiles only (cell-row strips): the
                 // learned path launches that pass itself (learned_flag_pass).
+                const int flags = strip_form(P) || fast_sets_flags(P) || s.t_hi == s.t_lo ? 0 : 1;
+                const bool apply = !nms_applies(P);
                 if (apply || flags == 1)
                     launch_cell_apply(P->d_img(), P->d_dl() + G.dl_begin, P->d_grp() + G.rp_off, G.n_list,
                                       G.n_bands, s.t_hi, s.t_lo, s.border, s.cell, H->n_sms * 8, st, flags, apply);
             }
-            const bool fin = true;
+            const bool fin = !nms_applies(P);
             if (P->tun.nms_tile_h == 32)
-                launch_nms_warp(P->d_img(), P->d_idt() + G.dti_off, G.det_tiles, P->d_maps(), P->d_maps() + P->n_img,
-                                P->d_call(), s.t_hi, s.t_lo, s.border, s.cell, H->n_sms * P->tun.nms_blocks_per_sm,
-                                P->tun.nms_order, st, nms_applies(P));
+                launch_nms_warp(P->d_img(), P->nms_rows == TILE_H ? P->d_idt() + G.dti_off : P->d_inm() + G.nmi_off,
+                                P->nms_rows == TILE_H ? G.det_tiles : G.nm_tiles, P->d_maps(), P->d_maps() + P->n_img,
+                                P->d_call(), s.t_hi, s.t_lo, s.border, s.cell, P->nms_rows,
+                                H->n_sms * P->tun.nms_blocks_per_sm, P->tun.nms_order, st, s.t_hi != s.t_lo && !cell_form(P),
+                                pdl);
             else if (P->tun.nms_tile_h == 64)
                 launch_nms_harris(P->d_img(), P->d_dl() + G.dl_begin, P->d_gnp() + G.np_off, G.n_list,
                                   G.nms64_tiles, P->d_maps(), P->d_maps() + P->n_img, P->d_call(), s.t_hi, s.t_lo,
                                   s.border, s.cell, H->n_sms * P->tun.nms_blocks_per_sm, P->tun.nms_order, st, fin,
-                                  64);
+                                  64, pdl);
             else  // 128 rows: the tiling of the 128-row FAST tiles
                 launch_nms_harris(P->d_img(), P->d_dl() + G.dl_begin, P->d_gft(0) + G.ftall_off[0], G.n_list,
                                   G.ftall_tiles[0], P->d_maps(), P->d_maps() + P->n_img, P->d_call(), s.t_hi,
                                   s.t_lo, s.border, s.cell, H->n_sms * P->tun.nms_blocks_per_sm, P->tun.nms_order, st,
-                                  fin, FT_HS[0]);
+                                  fin, FT_HS[0], pdl);
             break;
         }
         case 3:
-            launch_select(P->d_img() + G.img_begin, G.n_img, P->d_call(), P->max_quota, st);
+            launch_select(P->d_img() + G.img_begin, G.n_img, P->d_call(), P->max_quota, st, pdl);
+            pdl = P->pdl;
             break;
         case 4:
             launch_orient_range(P->d_img(), G.img_begin, G.n_img, G.slot_begin, G.slot_end, P->d_call(), st,
-                                P->n_img <= 65536 ? P->d_sli() : nullptr);
+                                P->n_img <= 65536 ? P->d_sli() : nullptr, pdl);
             break;
     }
 }
@@ -482,10 +495,9 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
 //   3 top-N per level              4 orientation + output records
 // Learned path, between FAST and NMS: the cell flags of the images with
 // proposal tiles, which the cell-row strip kernel leaves to the threshold
-// pass, when the stage-2 graphs run no pass (the per-warp NMS kernel applies
-// the thresholds itself).
+// pass (the stage-2 graphs run none after it).
 void learned_flag_pass(of_handle* H, Plan* P, cudaStream_t st) {
-    if (cell_form(P) || !strip_form(P) || !nms_applies(P)) return;
+    if (!strip_form(P) || P->s.t_hi == P->s.t_lo) return;
     const Plan::Group& G = P->groups[1][0];
     const Settings& s = P->s;
     launch_cell_apply(P->d_img(), P->d_dl() + G.dl_begin, P->d_grp() + G.rp_off, G.n_list, G.n_bands, s.t_hi, s.t_lo,
@@ -493,9 +505,13 @@ void learned_flag_pass(of_handle* H, Plan* P, cudaStream_t st) {
 }
 
 void enqueue_stages(of_handle* H, Plan* P, int first, int last, cudaStream_t st) {
+    bool pdl = false;
     for (int stage = first; stage < last; ++stage) {
-        if (stage == 0) cudaMemsetAsync(H->arena, 0, P->lay.zero_end, st);
-        enqueue_group_stage(H, P, P->groups[1][0], stage, st);
+        if (stage == 0) {
+            cudaMemsetAsync(H->arena, 0, P->lay.zero_end, st);
+            pdl = false;
+        }
+        enqueue_group_stage(H, P, P->groups[1][0], stage, st, pdl);
     }
 }
 
@@ -508,8 +524,9 @@ void enqueue_forked(of_handle* H, Plan* P, int k, cudaStream_t cs) {
     cudaEventRecord(H->fork_ev, cs);
     for (int g = 1; g < k; ++g) cudaStreamWaitEvent(H->cap_branch[g - 1], H->fork_ev, 0);
     const std::vector<Plan::Group>& gs = P->groups[k];
+    bool pdl[kMaxGroups] = {};
     for (int stage = 0; stage < kStages; ++stage)
-        for (int g = 0; g < k; ++g) enqueue_group_stage(H, P, gs[g], stage, g == 0 ? cs : H->cap_branch[g - 1]);
+        for (int g = 0; g < k; ++g) enqueue_group_stage(H, P, gs[g], stage, g == 0 ? cs : H->cap_branch[g - 1], pdl[g]);
     for (int g = 1; g < k; ++g) {
         cudaEventRecord(H->join_ev[g - 1], H->cap_branch[g - 1]);
         cudaStreamWaitEvent(cs, H->join_ev[g - 1], 0);
@@ -697,6 +714,20 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     P->cell_tiles = s.cell >= CT_MIN_CELL && s.cell <= CT_MAX_CELL;
     P->aligned_ok = P->cell_tiles && fast_aligned_ok(s.cell);
     P->strip_ok = s.cell <= CS_MAX_CELL;
+    // Sizes of the work items, by the batch's cell-row strips (75 for a VGA level,
+    // 240 for a VGA frame of 8 levels, 1480 for a 1080p one).  The per-warp kernels
+    // hold 2432 warps: fewer items than that leave warps idle while each item's
+    // rows run one after another, so small batches get thirds or halves of a strip
+    // and 8- or 16-row NMS tiles (one VGA frame, whole call: 52 us with full items,
+    // 43 with thirds and 8 rows; three: 64, 57 with halves and 16 rows; one 1080p
+    // frame: 83 either way).
+    int64_t strips = 0;
+    for (const auto& L : P->lay.img)
+        if (L.det) strips += (int64_t)L.tiles_x * L.ncy;
+    const int part = strips < 700 ? (s.cell + 2) / 3 : strips < 1200 ? (s.cell + 1) / 2 : s.cell;
+    P->strip_rows = std::min(s.cell, std::max(part, 8));
+    P->nms_rows = strips < 700 ? 8 : strips < 1200 ? 16 : TILE_H;
+    P->pdl = strips < 12000;
     // The threshold pass flags the cells itself when a band's cells fit its
     // shared array; otherwise the general FAST kernel sets them.
     P->apply_flags = true;
@@ -839,9 +870,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
             G.np_off = (int)P->gp_nms64.size();
             for (int i = 0; i < 2; ++i) G.ftall_off[i] = (int)P->gp_ftall[i].size();
             G.fal_off = (int)P->gp_fal.size();
-            G.cs_off = (int)P->gp_cstrip.size();
             G.csi_off = (int)P->items_cs.size();
             G.dti_off = (int)P->items_dt.size();
+            G.nmi_off = (int)P->items_nm.size();
             for (int j = j0; j < j1; ++j) {
                 const Img& I = P->h_img[P->det_list[j]];
                 const uint32_t ii = (uint32_t)P->det_list[j];
@@ -849,11 +880,17 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                     for (int tx = 0; tx < I.tiles_x; ++tx)
                         P->items_dt.push_back(make_uint2(
                             ii, ((uint32_t)(s.border + ty * TILE_H) << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
+                if (P->nms_rows != TILE_H)
+                    for (int y = s.border; y < I.h - s.border; y += P->nms_rows)
+                        for (int tx = 0; tx < I.tiles_x; ++tx)
+                            P->items_nm.push_back(make_uint2(ii, ((uint32_t)y << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
                 if (P->strip_ok)
                     for (int cy = 0; cy < I.ncy; ++cy)
-                        for (int tx = 0; tx < I.tiles_x; ++tx)
-                            P->items_cs.push_back(make_uint2(
-                                ii, ((uint32_t)(s.border + cy * s.cell) << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
+                        for (int y = s.border + cy * s.cell; y < std::min(s.border + (cy + 1) * s.cell, I.h - s.border);
+                             y += P->strip_rows)
+                            for (int tx = 0; tx < I.tiles_x; ++tx)
+                                P->items_cs.push_back(
+                                    make_uint2(ii, ((uint32_t)y << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
                 P->gp_nms64.push_back(G.nms64_tiles);
                 G.nms64_tiles += I.tiles_x * ((I.h - 2 * s.border + 63) / 64);
                 for (int i = 0; i < 2; ++i) {
@@ -869,9 +906,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                 G.fast_tiles += P->cell_tiles ? I.ftiles_x * ((I.ncy + ct_cell_rows(s.cell) - 1) / ct_cell_rows(s.cell)) : 0;
                 P->gp_rows.push_back(G.n_bands);
                 G.n_bands += I.ncy;
-                P->gp_cstrip.push_back(G.cs_strips);
-                G.cs_strips += P->strip_ok ? I.tiles_x * I.ncy : 0;
             }
+            G.cs_strips = (int)P->items_cs.size() - G.csi_off;
+            G.nm_tiles = (int)P->items_nm.size() - G.nmi_off;
             G.slot_begin = P->h_img[G.img_begin].slot0;
             G.slot_end = f1 < nf ? P->h_img[f1 * nl].slot0 : P->total_slots;
             G.rs_job.assign(nl + 1, 0);
@@ -932,17 +969,17 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     P->tun.resize_tile_h = RS_TILE_HS[1];
     P->tun.resize_tma = 1;
     P->tun.stream_groups = 1;
-    // Untuned plans.  Batches of 4 frames or more start from the autotuner's
-    // choice on 1080p batches: the cell-row strips (form 4, which set the cell
-    // flags) and the per-warp NMS kernel, which applies them (no threshold
-    // pass).  Fewer frames per call are launch-bound; there the cell-tile form
-    // with the block NMS kernel measured faster (0.144 against 0.150 ms for
-    // one 1080p frame per call).
-    const bool big = nf >= 4 && P->strip_ok;
-    P->tun.fast_cell_tiles = big ? 4 : P->cell_tiles ? 1 : 0;
+    // Untuned plans: the cell-row strips (form 4, which set the cell flags) with
+    // an NMS kernel that applies them (no threshold pass).
+    // NMS: the per-warp kernel, which spreads its Harris sums over the warps'
+    // own survivors and wins on small items and on many; between (1200 to 6000
+    // strips: one 1080p frame 80 against 83 us, one 4K frame 208 against 215)
+    // the block kernel, whose Harris phase shares a 64-row tile's survivors.
+    const bool warp_nms = strips < 1200 || strips >= 6000;
+    P->tun.fast_cell_tiles = P->strip_ok ? 4 : P->cell_tiles ? 1 : 0;
     P->tun.fast_tile_h = 32;
     P->tun.fast_blocks_per_sm = plan_fast_bps(P);
-    P->tun.nms_tile_h = big ? 32 : 64;
+    P->tun.nms_tile_h = P->strip_ok && warp_nms ? 32 : 64;
     P->tun.nms_blocks_per_sm = nms_blocks_per_sm(P->tun.nms_tile_h, true);
     for (int i = 0; i < 2; ++i)  // raise the tall kernels' shared-memory limits before any capture
         for (int fl = 0; fl < 2; ++fl) fast_blocks_per_sm(FT_HS[i], fl != 0);
@@ -1010,10 +1047,10 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     }
     P->off_gfal = off;
     off = align_up(off + sizeof(int32_t) * std::max<size_t>(P->gp_fal.size(), 1), 16);
-    P->off_gcs = off;
-    off = align_up(off + sizeof(int32_t) * std::max<size_t>(P->gp_cstrip.size(), 1), 16);
     P->off_ics = off;
     off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_cs.size(), 1), 16);
+    P->off_inm = off;
+    off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_nm.size(), 1), 16);
     P->off_idt = off;
     off = align_up(off + sizeof(uint2) * std::max<size_t>(P->items_dt.size(), 1), 16);
     P->off_ipy = off;
@@ -1069,8 +1106,8 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     put(P->off_gnp, P->gp_nms64.data(), sizeof(int32_t) * P->gp_nms64.size());
     for (int i = 0; i < 2; ++i) put(P->off_gft[i], P->gp_ftall[i].data(), sizeof(int32_t) * P->gp_ftall[i].size());
     put(P->off_gfal, P->gp_fal.data(), sizeof(int32_t) * P->gp_fal.size());
-    put(P->off_gcs, P->gp_cstrip.data(), sizeof(int32_t) * P->gp_cstrip.size());
     put(P->off_ics, P->items_cs.data(), sizeof(uint2) * P->items_cs.size());
+    put(P->off_inm, P->items_nm.data(), sizeof(uint2) * P->items_nm.size());
     put(P->off_idt, P->items_dt.data(), sizeof(uint2) * P->items_dt.size());
     put(P->off_ipy, P->items_py.data(), sizeof(uint2) * P->items_py.size());
     put(P->off_pj, P->h_pj.data(), sizeof(PyrJob) * P->h_pj.size());

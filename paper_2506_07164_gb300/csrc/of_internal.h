@@ -137,13 +137,14 @@ __host__ __device__ __forceinline__ int tile_of(int order, int block, int grid, 
 }  // namespace ofk
 
 // Kernel launchers (implemented in the .cu files).  All take device pointers
-// to the plan's descriptor arrays and launch on `stream`.
+// to the plan's descriptor arrays and launch on `stream`.  pdl: the kernel may
+// start while the one before it on the stream still runs (of_launch.cuh).
 namespace ofk {
 void launch_resize(const Resize* jobs, const int32_t* tile_prefix, int n_jobs, int n_tiles,
                    int tile_h, void* stream);
 // Fused pyramid levels: one block per (frame, tile); items (job, (tile row << 16) | tile column).
 void launch_pyramid(const PyrJob* jobs, const uint2* items, int n_tiles, const CUtensorMap* maps, const Call* call,
-                    int s_bytes, int t_bytes, int x_words, int y_words, void* stream);
+                    int s_bytes, int t_bytes, int x_words, int y_words, void* stream, bool pdl = false);
 int pyramid_smem(int s_bytes, int t_bytes, int x_words, int y_words);
 bool pyramid_raise_smem();
 // General FAST on 128 x tile_h tiles (32, 64, 128 or 256 rows); flags: also
@@ -154,7 +155,7 @@ void launch_fast(const Img* imgs, const int32_t* img_list, const int32_t* tile_p
                  int tile_h = 32);
 void launch_fast_cells(const Img* imgs, const int32_t* img_list, const int32_t* tile_prefix, int n_list,
                        int n_tiles, const CUtensorMap* maps, const Call* call, int t_hi, int t_lo, int border,
-                       int cell, int grid, int order, void* stream);
+                       int cell, int grid, int order, void* stream, bool pdl = false);
 int fast_cells_blocks_per_sm(int cell);
 // Cell-aligned general FAST (120 x 120 tiles of whole cells; cells of 15 or 30 pixels).
 constexpr int FAST_AL_T = 120;
@@ -173,7 +174,8 @@ int fast_warp_blocks_per_sm();
 // of 8..33 pixels): general FAST that also sets the cell flags exactly.
 constexpr int CS_MAX_CELL = 33;
 void launch_fast_cstrip(const Img* imgs, const uint2* items, int n_strips, const CUtensorMap* maps, const Call* call,
-                        int t_hi, int t_lo, int border, int cell, int grid, int order, void* stream);
+                        int t_hi, int t_lo, int border, int cell, int sub, int grid, int order, void* stream,
+                        bool pdl = false);
 int fast_cstrip_blocks_per_sm();
 // Threshold pass: flags 1: sets the cell flags (when the FAST kernel did
 // not), 2: only for images with proposal tiles, 0: never; apply: applies them
@@ -185,7 +187,7 @@ void launch_nms_harris(const Img* imgs, const int32_t* img_list, const int32_t* 
                        int n_list, int n_tiles, const CUtensorMap* img_maps,
                        const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo,
                        int border, int cell, int grid, int order, void* stream,
-                       bool final_scores = false, int tile_h = 32);
+                       bool final_scores = false, int tile_h = 32, bool pdl = false);
 // Resident blocks per SM of the NMS kernel a plan launches for tile_h (32 with
 // final scores: the per-warp kernel).
 int nms_blocks_per_sm(int tile_h, bool final_scores);
@@ -195,13 +197,13 @@ int nms_blocks_per_sm(int tile_h, bool final_scores);
 // Otherwise the maps hold S(p).  Scores outside proposed tiles count as 0.
 void launch_nms_warp(const Img* imgs, const uint2* items, int n_tiles, const CUtensorMap* img_maps,
                      const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo, int border, int cell,
-                     int grid, int order, void* stream, bool apply);
+                     int rows, int grid, int order, void* stream, bool apply, bool pdl = false);
 int nms_warp_blocks_per_sm();
-void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream);
+void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream, bool pdl = false);
 void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream);
 // Slots [slot_begin, slot_end) of images [img_begin, img_begin + n_img) (one frame group).
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,
-                         void* stream, const uint16_t* slot_img = nullptr);
+                         void* stream, const uint16_t* slot_img = nullptr, bool pdl = false);
 // S(p) of image `img` from a dense w x h copy of its map (offset scores):
 // the per-cell thresholds and proposal tiles applied, t_lo - 1 added back.
 void launch_inspect_score_final(const Img* imgs, int img, uint8_t* d, int w, int h, int t_hi, int t_lo, int border,

@@ -1,0 +1,49 @@
+// Launches that overlap the end of the kernel before them.
+//
+// One call is a chain of short kernels (pyramid, FAST, NMS, top-N,
+// orientation), each starting from descriptors that the host wrote before the
+// chain.  Launched with `pdl` (programmatic stream serialization), a kernel may
+// start while its predecessor still runs: it reads descriptors, sets up its
+// barriers and then waits (pdl_wait) for the predecessor's grid to complete
+// and its writes to be visible.  Every kernel of a chain waits in every thread
+// before it ends, so a kernel's completion implies its predecessors'.
+// pdl_trigger lets the next kernel of the chain start; it is called first
+// thing, so that kernel's blocks take their places as soon as the SMs have
+// room.  Without `pdl` both are no-ops.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace ofk {
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// cluster: blocks per cluster (1: none).
+template <typename... P, typename... A>
+inline void launch_chain(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t st, bool pdl, int cluster,
+                         A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (pdl) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    cudaLaunchKernelEx(&cfg, kernel, P(std::forward<A>(args))...);
+}
+
+}  // namespace ofk
