@@ -6,10 +6,9 @@
 // bright or all dark.  The largest such t is
 //   s(p) = max( max_j min_{k<9} I_{j+k} - I_p ,  I_p - min_j max_{k<9} I_{j+k} )
 // (the I_p terms leave the min/max), so corner(t) <=> s(p) >= t for t >= 1.
-// The arc terms use the three-input packed min/max of sm_90+ (DPX):
-// minima of 3 contiguous ring pixels, then of 9 = three 3-runs 3 apart, then
-// the maximum over the 16 starts -- 40 instructions per side for 2 pixels,
-// no branches.  The map stores the offset score s(p) - (t_lo - 1) where
+// The arc terms use the three-input packed min/max of sm_90+ (DPX), windows
+// sharing their common pixels -- 32 instructions per side for 2 pixels, no
+// branches (arc_side).  The map stores the offset score s(p) - (t_lo - 1) where
 // s(p) >= t_lo (the lowest threshold in use), else 0: an order-preserving
 // shift that costs nothing (both terms of the final maximum carry a bias of
 // 512 - (t_lo - 1) per lane and its floor is 512, so each lane's low byte is
@@ -63,8 +62,13 @@ __device__ __forceinline__ uint32_t pair_at(const uint32_t (&h)[6]) {
 
 // One side of the score for the two pixels in the lanes of q[]: MIN = true
 // gives the largest arc minimum max_j min_{k<9} q[j+k], MIN = false the
-// smallest arc maximum.  Minima of 3 contiguous ring pixels, then of three
-// 3-runs 3 apart (9 pixels), then the extremum over the 16 starts.
+// smallest arc maximum.  The windows starting at j and j + 1 share 8 pixels:
+//   max(min q[j..j+8], min q[j+1..j+9]) = min(min q[j+1..j+8], max(q[j], q[j+9])),
+// so 8 windows of 8 at odd starts remain, each 4 consecutive of the 8 pairs
+// p_i = (q[2i+1], q[2i+2]).  Neighbouring windows share 3 pairs, so 4 minima of
+// three pairs serve all 8: 8 pairs + 4 triples + 8 ends + 8 windows + 4 for the
+// extremum = 32 operations (40 with minima of 3, then 9 contiguous pixels at
+// all 16 starts; the kernel is bound by these: see k_fast_cstrip).
 template <bool MIN>
 __device__ __forceinline__ uint32_t arc_side(const uint32_t (&q)[16]) {
     auto f = [](uint32_t a, uint32_t b, uint32_t c) {
@@ -75,15 +79,20 @@ __device__ __forceinline__ uint32_t arc_side(const uint32_t (&q)[16]) {
         if constexpr (MIN) return __vimax3_u16x2(a, b, c);
         else return __vimin3_u16x2(a, b, c);
     };
-    uint32_t m3[16];
+    uint32_t p[8], e[8], r[8];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) m3[i] = f(q[i], q[(i + 1) & 15], q[(i + 2) & 15]);
-    uint32_t m9[16];
+    for (int i = 0; i < 8; ++i) {
+        p[i] = f(q[2 * i + 1], q[(2 * i + 2) & 15], q[2 * i + 1]);
+        e[i] = g(q[2 * i], q[(2 * i + 9) & 15], q[2 * i]);
+    }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) m9[i] = f(m3[i], m3[(i + 3) & 15], m3[(i + 6) & 15]);
-    const uint32_t a0 = g(m9[0], m9[1], m9[2]), a1 = g(m9[3], m9[4], m9[5]), a2 = g(m9[6], m9[7], m9[8]);
-    const uint32_t a3 = g(m9[9], m9[10], m9[11]), a4 = g(m9[12], m9[13], m9[14]);
-    return g(g(a0, a1, a2), a3, g(a4, m9[15], m9[15]));
+    for (int i = 0; i < 4; ++i) {
+        // Windows of the pairs 2i .. 2i+3 and 2i+1 .. 2i+4.
+        const uint32_t t = f(p[2 * i + 1], p[(2 * i + 2) & 7], p[(2 * i + 3) & 7]);
+        r[2 * i] = f(t, p[2 * i], e[2 * i]);
+        r[2 * i + 1] = f(t, p[(2 * i + 4) & 7], e[2 * i + 1]);
+    }
+    return g(g(r[0], r[1], r[2]), g(r[3], r[4], r[5]), g(r[6], r[7], r[7]));
 }
 
 constexpr uint32_t PAIR_BIAS = 0x02000200u;  // 512 per lane: every biased difference stays positive

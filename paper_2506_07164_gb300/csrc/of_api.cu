@@ -972,10 +972,10 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     // Untuned plans: the cell-row strips (form 4, which set the cell flags) with
     // an NMS kernel that applies them (no threshold pass).
     // NMS: the per-warp kernel, which spreads its Harris sums over the warps'
-    // own survivors and wins on small items and on many; between (1200 to 6000
+    // own survivors and wins on small items and on many; between (1200 to 8000
     // strips: one 1080p frame 80 against 83 us, one 4K frame 208 against 215)
     // the block kernel, whose Harris phase shares a 64-row tile's survivors.
-    const bool warp_nms = strips < 1200 || strips >= 6000;
+    const bool warp_nms = strips < 1200 || strips >= 8000;
     P->tun.fast_cell_tiles = P->strip_ok ? 4 : P->cell_tiles ? 1 : 0;
     P->tun.fast_tile_h = 32;
     P->tun.fast_blocks_per_sm = plan_fast_bps(P);
