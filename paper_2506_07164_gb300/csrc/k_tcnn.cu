@@ -7,9 +7,8 @@
 // ReLU): 1 -> 8 channels (32 x 32), 8 -> 16 (16 x 16), 16 -> 16 (8 x 8);
 // global average pool; linear 16 -> 1 logit.  Weights are stored and used as
 // bf16 (rounded from fp32 master copies that Adam updates); every product is
-// accumulated in fp32.  One block per tile; activations stay in shared
-// memory.  Training uses a plain forward that saves activations to global
-// memory for the backward pass; inference runs on the tensor cores.
+// accumulated in fp32.  One block per tile; activations stay in shared memory;
+// inference and training run on the tensor cores.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -32,25 +31,17 @@ constexpr int C1 = 8, C2 = 16, C3 = 16;
 // Flat parameter layout.
 constexpr int W1 = 0, B1 = W1 + C1 * 9, W2 = B1 + C1, B2 = W2 + C2 * C1 * 9, W3 = B2 + C2,
               B3 = W3 + C3 * C2 * 9, WF = B3 + C3, BF = WF + C3, NP = BF + 1;
-constexpr int A1 = C1 * S1 * S1, A2 = C2 * S2 * S2, A3 = C3 * S3 * S3;  // activation sizes
-constexpr int SAVE = A1 + A2 + A3 + C3 + 1;  // per tile: a1, a2, a3, gap, logit
-constexpr int THREADS = 256;
-constexpr int SMEM_FWD = (S0 * S0 + A1 + A2 + A3 + NP + 32) * 4;
-
 static_assert(NP == 3585, "parameter count");
+constexpr int LOSS_AT = (NP + 1) / 2 * 2;  // 8-byte aligned word after the gradient
 
 }  // namespace tn
 
 struct of_tcnn {
     float* master = nullptr;  // fp32 master weights [NP]
     __nv_bfloat16* w = nullptr;  // bf16 compute weights [NP]
-    float* grad = nullptr;    // fp32 gradients [NP]
+    float* grad = nullptr;    // fp32 gradients [NP], then (LOSS_AT) the loss as a double
     float* m = nullptr;       // Adam moments
     float* v = nullptr;
-    float* save = nullptr;    // saved activations [cap * SAVE]
-    float* dz = nullptr;      // dLoss/dlogit [cap]
-    float* loss = nullptr;    // [1]
-    int cap = 0;
     int64_t step = 0;
     int device = 0;
 };
@@ -68,88 +59,6 @@ struct PatchSrc {
     const ofk::Img* imgs;   // in place: image descriptors
     const uint2* items;     // in place: the detect tiles
 };
-
-__device__ void load_patch(const uint8_t* __restrict__ p, float* in) {
-    for (int i = threadIdx.x; i < S0 * S0; i += blockDim.x) in[i] = ((float)p[i] - 128.f) * (1.f / 64.f);
-}
-
-// out[o][y][x] = relu(b[o] + sum_c sum_k w[o][c][k] in[c][2y+ky-1][2x+kx-1])
-__device__ void conv_s2(const float* __restrict__ in, int C, int Sin, const float* __restrict__ w,
-                        const float* __restrict__ b, int O, float* __restrict__ out) {
-    const int Sout = Sin / 2;
-    for (int i = threadIdx.x; i < O * Sout * Sout; i += blockDim.x) {
-        const int o = i / (Sout * Sout), y = (i / Sout) % Sout, x = i % Sout;
-        float acc = b[o];
-        for (int c = 0; c < C; ++c) {
-            const float* wc = w + (o * C + c) * 9;
-            const float* ic = in + c * Sin * Sin;
-#pragma unroll
-            for (int ky = 0; ky < 3; ++ky) {
-                const int iy = 2 * y + ky - 1;
-                if (iy < 0 || iy >= Sin) continue;
-#pragma unroll
-                for (int kx = 0; kx < 3; ++kx) {
-                    const int ix = 2 * x + kx - 1;
-                    if (ix < 0 || ix >= Sin) continue;
-                    acc = fmaf(wc[ky * 3 + kx], ic[iy * Sin + ix], acc);
-                }
-            }
-        }
-        out[i] = relu(acc);
-    }
-}
-
-// Forward pass of tiles [0, n); logits to `logits` (may be null); when `save`
-// is set, activations to save[t * SAVE ...].
-__global__ void __launch_bounds__(THREADS)
-k_forward(const uint8_t* __restrict__ tiles, int n, const __nv_bfloat16* __restrict__ wq, float* __restrict__ logits,
-          float* __restrict__ save) {
-    extern __shared__ float sm[];
-    float* in = sm;
-    float* a1 = in + S0 * S0;
-    float* a2 = a1 + A1;
-    float* a3 = a2 + A2;
-    float* w = a3 + A3;
-    float* red = w + NP;
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) w[i] = __bfloat162float(wq[i]);
-    __syncthreads();
-    for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        load_patch(tiles + (size_t)t * S0 * S0, in);
-        __syncthreads();
-        conv_s2(in, 1, S0, w + W1, w + B1, C1, a1);
-        __syncthreads();
-        conv_s2(a1, C1, S1, w + W2, w + B2, C2, a2);
-        __syncthreads();
-        conv_s2(a2, C2, S2, w + W3, w + B3, C3, a3);
-        __syncthreads();
-        // Global average pool (one warp per 2 channels) and the linear head.
-        if (threadIdx.x < 32 * 8) {
-            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            for (int c = warp; c < C3; c += 8) {
-                float s = a3[c * 64 + lane] + a3[c * 64 + 32 + lane];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-                if (lane == 0) red[c] = s * (1.f / 64.f);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float z = w[BF];
-            for (int c = 0; c < C3; ++c) z = fmaf(w[WF + c], red[c], z);
-            red[16] = z;
-            if (logits) logits[t] = z;
-        }
-        __syncthreads();
-        if (save) {
-            float* sv = save + (size_t)t * SAVE;
-            for (int i = threadIdx.x; i < A1; i += blockDim.x) sv[i] = a1[i];
-            for (int i = threadIdx.x; i < A2; i += blockDim.x) sv[A1 + i] = a2[i];
-            for (int i = threadIdx.x; i < A3; i += blockDim.x) sv[A1 + A2 + i] = a3[i];
-            if (threadIdx.x <= C3) sv[A1 + A2 + A3 + threadIdx.x] = red[threadIdx.x];
-        }
-        __syncthreads();
-    }
-}
 
 // A 64 x 64 patch is 256 16-byte chunks (4 per row).  Chunk q of tile t; pixels
 // outside the image are 0.  Level images and their pitches are multiples of
@@ -269,20 +178,29 @@ __device__ __forceinline__ void mma8(float (&d)[4], const uint32_t (&a)[2], uint
         : "r"(a[0]), "r"(a[1]), "r"(b), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
 }
 
-// The three bf16 parts of two non-negative activations (channels 2t, 2t + 1),
-// packed: truncations, so that finite values never round up to infinity; an
-// infinity is its own leading part.
+// The three bf16 parts of two values (channels 2t, 2t + 1), packed:
+// truncations, so that finite values never round up to infinity; an infinity
+// is its own leading part.
 __device__ __forceinline__ void split3(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
     auto rest = [](float v) {
         const float r = v - __uint_as_float(__float_as_uint(v) & 0xFFFF0000u);
         return r;
     };
-    const bool xi = x > 3.402823466e38f, yi = y > 3.402823466e38f;
+    const bool xi = fabsf(x) > 3.402823466e38f, yi = fabsf(y) > 3.402823466e38f;
     const float rx = xi ? 0.f : rest(x), ry = yi ? 0.f : rest(y);
     const float sx = rest(rx), sy = rest(ry);
     h = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x7632);
     m = __byte_perm(__float_as_uint(rx), __float_as_uint(ry), 0x7632);
     l = __byte_perm(__float_as_uint(sx), __float_as_uint(sy), 0x7632);
+}
+
+// split3 into the planes of the three parts, `plane` bytes apart.
+__device__ __forceinline__ void store3(uint8_t* d, int plane, float x, float y) {
+    uint32_t h, m, l;
+    split3(x, y, h, m, l);
+    *reinterpret_cast<uint32_t*>(d) = h;
+    *reinterpret_cast<uint32_t*>(d + plane) = m;
+    *reinterpret_cast<uint32_t*>(d + 2 * plane) = l;
 }
 
 // Two consecutive input channels (or taps) of a weight matrix as one fragment word.
@@ -400,16 +318,9 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
             }
             float d[4];
             mma16(d, a, b1, zero);
-            uint32_t hh, mm, ll;
             uint8_t* o = p1 + ((y + 1) * T1_ROW + g + 8 * h) * 16 + 4 * t4;
-            split3(relu(d[0] + bb1[0]), relu(d[1] + bb1[1]), hh, mm, ll);
-            *reinterpret_cast<uint32_t*>(o + T1_O * 16) = hh;  // even columns: odd padded columns
-            *reinterpret_cast<uint32_t*>(o + T1_O * 16 + T1_PLANE) = mm;
-            *reinterpret_cast<uint32_t*>(o + T1_O * 16 + 2 * T1_PLANE) = ll;
-            split3(relu(d[2] + bb1[0]), relu(d[3] + bb1[1]), hh, mm, ll);
-            *reinterpret_cast<uint32_t*>(o + 16) = hh;
-            *reinterpret_cast<uint32_t*>(o + 16 + T1_PLANE) = mm;
-            *reinterpret_cast<uint32_t*>(o + 16 + 2 * T1_PLANE) = ll;
+            store3(o + T1_O * 16, T1_PLANE, relu(d[0] + bb1[0]), relu(d[1] + bb1[1]));  // even columns: odd padded ones
+            store3(o + 16, T1_PLANE, relu(d[2] + bb1[0]), relu(d[3] + bb1[1]));
         }
         __syncthreads();
         if (warp == 0 && last >= 0) finish(last, par ^ 1);
@@ -457,15 +368,9 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    uint32_t hh, mm, ll;
-                    split3(relu(acc[j][2 * i] + low[j][2 * i] + bb2[2 * j]),
-                           relu(acc[j][2 * i + 1] + low[j][2 * i + 1] + bb2[2 * j + 1]), hh, mm, ll);
-                    uint8_t* d = o + 64 * i + j * T2_PLANE;
-                    *reinterpret_cast<uint32_t*>(d) = hh;
-                    *reinterpret_cast<uint32_t*>(d + 2 * T2_PLANE) = mm;
-                    *reinterpret_cast<uint32_t*>(d + 4 * T2_PLANE) = ll;
-                }
+                for (int i = 0; i < 2; ++i)
+                    store3(o + 64 * i + j * T2_PLANE, 2 * T2_PLANE, relu(acc[j][2 * i] + low[j][2 * i] + bb2[2 * j]),
+                           relu(acc[j][2 * i + 1] + low[j][2 * i + 1] + bb2[2 * j + 1]));
             }
         }
         __syncthreads();
@@ -510,118 +415,507 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
     }
 }
 
-// Weighted BCE with logits: loss = mean_i w_i (softplus(z_i) - y_i z_i),
-// w_i = pos_weight for y_i = 1; dz_i = w_i (sigmoid(z_i) - y_i) / n.
-__global__ void k_bce(const float* __restrict__ save, const float* __restrict__ y, int n, float pos_weight,
-                      float* __restrict__ dz, float* __restrict__ loss) {
-    float acc = 0.f;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float z = save[(size_t)i * SAVE + A1 + A2 + A3 + C3];
-        const float wt = y[i] > 0.5f ? pos_weight : 1.f;
-        const float sp = z > 0.f ? z + log1pf(expf(-z)) : log1pf(expf(z));
-        acc += wt * (sp - y[i] * z);
-        const float sg = 1.f / (1.f + expf(-z));
-        dz[i] = wt * (sg - y[i]) / (float)n;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc / (float)n);
+// ---------------------------------------------------------------------------
+// One training step's loss and gradient in one kernel.
+//
+// A patch's part of the gradient needs nothing from other patches: its logit
+// gives dLoss/dlogit.  So a block takes a patch through forward, loss and
+// backward with everything in shared memory (the activations used to go out to
+// and back from global memory, 53 KB per patch, between three kernels), and the
+// weight gradients of its patches stay in registers until the end.
+//
+// Every product runs on the tensor cores like the forward's: activations and
+// their gradients as three exact bf16 parts, weights as they are.  Products of
+// two split numbers keep the six part products down to 2^-16 (the rest is below
+// an fp32 rounding); leading parts' sums leave the tensor cores every 16 terms.
+// The gradient entering layer 3 is one number per channel times the ReLU mask,
+//   d3[o][p] = s_o mask[o][p],  s_o = dlogit w_f[o] / 64,
+// so the mask (exact in bf16) is the operand: dW3 = s_o (mask a2), and d2 is
+// (dlogit / 64) times the mask's transposed convolution with w_f[o] w3, a
+// product of two bf16 numbers, hence exact in two.  Transposed stride-2
+// convolutions split by the parity of the pixel: each of the four classes is a
+// small matrix product of 1, 2, 2 or 4 taps over neighbouring pixels.
+//
+// 16 warps, one block per SM.  Phases of a patch, a barrier after each:
+//   1 layer 1 (and the previous patch's dW1)   2 layer 2   3 layer 3, mask, the
+//   next patch's pixels   4 loss, dW3, d2      5 dW2, d1.
+// dW2 lives as one 16 x 72 accumulator per warp (its pixel rows), dW3 as one or
+// two 16 x 8 tiles per warp, dW1 as one 9 x 8 tile per warp (its pixel rows).
+// Bound by the latency of the phases (issue 46 %, shared memory 54 %, tensor
+// pipe 30 %).  2048 patches: 2000 us as three fp32 kernels (1674 of them the
+// backward's scalar loops), 127 us here.  Against 64 bits, 24 batches: gradient
+// 1.7e-7 of its norm off (median; 2.3e-7 before), loss 1.9e-8 (3.3e-8).
+constexpr int TR_THREADS = 512, TR_WARPS = TR_THREADS / 32;
+constexpr int M3_ROW = 9, M3_PLANE = 9 * M3_ROW * 16;      // layer-3 mask: 8 x 8 pixels, a zero row and column; one channel half
+constexpr int D2_ROW = 17, D2_PLANE = 17 * D2_ROW * 16;    // d2: 16 x 16 pixels, a zero row and column; one part and half
+constexpr int D1_PLANE = 32 * 32 * 16;                     // d1: 32 rows of 16 even, then 16 odd columns; one part
+constexpr int FR = 128;                                    // bytes of one fragment register of a warp
+constexpr int TR_IN = 0, TR_P1 = TR_IN + 2 * TI_BYTES, TR_P2 = TR_P1 + 3 * T1_PLANE, TR_M3 = TR_P2 + 6 * T2_PLANE,
+              TR_D2 = TR_M3 + 2 * M3_PLANE, TR_D1 = TR_D2 + 6 * D2_PLANE, TR_F2 = TR_D1 + 3 * D1_PLANE,
+              TR_F3 = TR_F2 + 18 * FR, TR_FQ = TR_F3 + 36 * FR, TR_FT = TR_FQ + 72 * FR, TR_RED = TR_FT + 18 * FR,
+              TR_SMEM = TR_RED + 2 * 4 * C3 * 4 + 64;
+static_assert(TR_SMEM <= 227 * 1024, "shared memory of one block");
+static_assert(TR_M3 % 16 == 0 && TR_D2 % 16 == 0 && TR_D1 % 16 == 0 && TR_F2 % 16 == 0, "16-byte rows for ldmatrix");
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], uint32_t a) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];"
+                 : "=r"(r[0]), "=r"(r[1])
+                 : "r"(a)
+                 : "memory");
 }
 
-// Backward of one strided conv layer given dout (already multiplied by the
-// ReLU derivative): accumulates dW, dB into gw, gb and writes din (without
-// the input's ReLU derivative) when din is not null.
-__device__ void conv_s2_back(const float* __restrict__ in, int C, int Sin, const float* __restrict__ w, int O,
-                             const float* __restrict__ dout, float* __restrict__ gw, float* __restrict__ gb,
-                             float* __restrict__ din) {
-    const int Sout = Sin / 2;
-    // dW[o][c][k] = sum_{y,x} dout[o][y][x] in[c][2y+ky-1][2x+kx-1]
-    for (int i = threadIdx.x; i < O * C * 9; i += blockDim.x) {
-        const int o = i / (C * 9), c = (i / 9) % C, k = i % 9, ky = k / 3, kx = k % 3;
-        float acc = 0.f;
-        for (int y = 0; y < Sout; ++y) {
-            const int iy = 2 * y + ky - 1;
-            if (iy < 0 || iy >= Sin) continue;
-            for (int x = 0; x < Sout; ++x) {
-                const int ix = 2 * x + kx - 1;
-                if (ix < 0 || ix >= Sin) continue;
-                acc = fmaf(dout[(o * Sout + y) * Sout + x], in[(c * Sin + iy) * Sin + ix], acc);
-            }
-        }
-        gw[i] += acc;
-    }
-    for (int o = threadIdx.x; o < O; o += blockDim.x) {
-        float acc = 0.f;
-        for (int j = 0; j < Sout * Sout; ++j) acc += dout[o * Sout * Sout + j];
-        gb[o] += acc;
-    }
-    if (!din) return;
-    // din[c][iy][ix] = sum_{o,ky,kx} dout[o][y][x] w[o][c][ky][kx], iy = 2y+ky-1, ix = 2x+kx-1
-    for (int i = threadIdx.x; i < C * Sin * Sin; i += blockDim.x) {
-        const int c = i / (Sin * Sin), iy = (i / Sin) % Sin, ix = i % Sin;
-        float acc = 0.f;
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
-            const int ty = iy + 1 - ky;
-            if (ty < 0 || (ty & 1) || (ty >> 1) >= Sout) continue;
-#pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {
-                const int tx = ix + 1 - kx;
-                if (tx < 0 || (tx & 1) || (tx >> 1) >= Sout) continue;
-                for (int o = 0; o < O; ++o)
-                    acc = fmaf(dout[(o * Sout + (ty >> 1)) * Sout + (tx >> 1)], w[(o * C + c) * 9 + ky * 3 + kx], acc);
-            }
-        }
-        din[i] = acc;
-    }
-}
+__global__ void __launch_bounds__(TR_THREADS, 1)
+k_train(const uint8_t* __restrict__ tiles, const float* __restrict__ labels, int n, float pos_weight,
+        const __nv_bfloat16* __restrict__ wq, float* __restrict__ grad, double* __restrict__ loss) {
+    extern __shared__ __align__(128) uint8_t tsm[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t4 = lane & 3;
+    uint8_t* const p1 = tsm + TR_P1;
+    uint8_t* const p2 = tsm + TR_P2;
+    uint8_t* const m3 = tsm + TR_M3;
+    uint8_t* const d2 = tsm + TR_D2;
+    uint8_t* const d1 = tsm + TR_D1;
+    float* const red = reinterpret_cast<float*>(tsm + TR_RED);  // [sums, counts][row pair][channel]
+    const uint32_t sb = smem_addr(tsm);
+    for (int i = tid; i < TR_F2 / 16; i += TR_THREADS) reinterpret_cast<uint4*>(tsm)[i] = make_uint4(0u, 0u, 0u, 0u);
 
-// Backward over tiles; per-block gradient sums in shared memory, added to
-// `grad` once per block.
-__global__ void __launch_bounds__(THREADS)
-k_backward(const uint8_t* __restrict__ tiles, int n, const __nv_bfloat16* __restrict__ wq,
-           const float* __restrict__ save, const float* __restrict__ dz, float* __restrict__ grad) {
-    extern __shared__ float sm[];
-    float* in = sm;                 // S0*S0
-    float* d1 = in + S0 * S0;       // A1
-    float* d2 = d1 + A1;            // A2
-    float* d3 = d2 + A2;            // A3
-    float* w = d3 + A3;             // NP
-    float* g = w + NP;              // NP
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) {
-        w[i] = __bfloat162float(wq[i]);
-        g[i] = 0.f;
+    // ---- weight fragments, one word per lane, in shared memory
+    {
+        auto put = [&](int base, int f, uint32_t v) { reinterpret_cast<uint32_t*>(tsm + base + f * FR)[lane] = v; };
+        for (int f = warp; f < 18; f += TR_WARPS) {  // layer 2: (channel half j, step s, register), the ninth tap last
+            const int j = f / 9, k = f % 9, r = W2 + (8 * j + g) * C1 * 9 + 2 * t4 * 9;
+            put(TR_F2, f, k < 8 ? pack_w(wq, r + k, r + 9 + k) : pack_w(wq, r + 8, r + 9 + 8));
+        }
+        for (int f = warp; f < 36; f += TR_WARPS) {  // layer 3: (half j, tap, register)
+            const int j = f / 18, k = f % 18 / 2, h = f & 1;
+            const int r = W3 + (8 * j + g) * C2 * 9 + (8 * h + 2 * t4) * 9;
+            put(TR_F3, f, pack_w(wq, r + k, r + 9 + k));
+        }
+        for (int f = warp; f < 36; f += TR_WARPS) {  // w_f w3 for d2: (half j of c, tap, register), two parts
+            const int j = f / 18, k = f % 18 / 2, o = 8 * (f & 1) + 2 * t4, c = 8 * j + g;
+            uint32_t hi = 0u, lo = 0u;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float q = __bfloat162float(wq[WF + o + e]) * __bfloat162float(wq[W3 + ((o + e) * C2 + c) * 9 + k]);
+                const float h = __uint_as_float(__float_as_uint(q) & 0xFFFF0000u);
+                hi |= (__float_as_uint(h) >> 16) << (16 * e);
+                lo |= (__float_as_uint(q - h) >> 16) << (16 * e);
+            }
+            put(TR_FQ, 2 * f, hi);
+            put(TR_FQ, 2 * f + 1, lo);
+        }
+        for (int f = warp; f < 18; f += TR_WARPS) {  // w2 for d1: (tap, register), depth o, channel c = g
+            const int k = f >> 1, o = 8 * (f & 1) + 2 * t4;
+            put(TR_FT, f, pack_w(wq, W2 + (o * C1 + g) * 9 + k, W2 + ((o + 1) * C1 + g) * 9 + k));
+        }
+    }
+    auto frag = [&](int base, int f) { return reinterpret_cast<const uint32_t*>(tsm + base + f * FR)[lane]; };
+    uint32_t b1[2];
+    {
+        auto w1 = [&](int k) { return k < 12 && (k & 3) ? W1 + g * 9 + (k >> 2) * 3 + (k & 3) - 1 : -1; };
+        b1[0] = pack_w(wq, w1(2 * t4), w1(2 * t4 + 1));
+        b1[1] = pack_w(wq, w1(2 * t4 + 8), w1(2 * t4 + 9));
+    }
+    auto wv = [&](int i) { return __bfloat162float(wq[i]); };
+    const float wf = wv(WF + (lane & 15)), bf = wv(BF);
+    const float wfg[2] = {wv(WF + g), wv(WF + g + 8)};
+    const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+    auto col1 = [](int kx) { return kx == 1 ? T1_O : kx >> 1; };  // E[x], O[x], E[x + 1]
+    auto col2 = [](int kx) { return kx == 1 ? T2_O : kx >> 1; };
+
+    // ---- accumulators over the block's patches
+    float g2[9][4] = {}, g3[2][4] = {}, g1[4] = {}, gb2[2] = {}, gb1[2] = {};
+    float gwf = 0.f, gb3 = 0.f, gbf = 0.f;
+    double lsum = 0.0;  // thread 0
+
+    auto load = [&](int t) {
+        Patch P;
+        P.p = tiles + (size_t)t * S0 * S0;
+        P.x0 = P.y0 = P.w = P.h = P.pitch = 0;
+        return load_chunk(P, tid & 255);
+    };
+    // dW1 of the patch in buffer b: 16 pixels of one row and parity per step, depth = pixels,
+    // rows = taps, columns = channels.
+    auto grad1 = [&](int b) {
+        const uint32_t* const in = reinterpret_cast<const uint32_t*>(tsm + TR_IN + b * TI_BYTES);
+        const int ky = g / 3, kx = g % 3;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int iy = 2 * warp + (i >> 1), par = i & 1;
+            uint32_t bh[2], bm[2], bl[2];
+            const uint32_t ba = sb + TR_D1 + (uint32_t)((iy * 32 + par * 16 + (lane & 15)) * 16);
+            ldsm2t(bh, ba);
+            ldsm2t(bm, ba + D1_PLANE);
+            ldsm2t(bl, ba + 2 * D1_PLANE);
+            // Pixel k of the step is column 2 k + par: input column 4 k + 2 par + kx - 1.
+            auto taps = [&](int ty, int tx, int k0) {  // values for k0 and k0 + 1, packed
+                const uint32_t* r = in + (2 * iy + ty) * TI_ROW + TI_X + par + 2 * k0 - (tx == 0 ? 1 : 0);
+                return __byte_perm(r[0], r[2], tx == 1 ? 0x5410 : 0x7632);
+            };
+            uint32_t a[4] = {taps(ky, kx, 2 * t4), 0u, taps(ky, kx, 2 * t4 + 8), 0u};
+            if (g == 0) {
+                a[1] = taps(2, 2, 2 * t4);
+                a[3] = taps(2, 2, 2 * t4 + 8);
+            }
+            float d[4], low[4];
+            mma16(d, a, bh, zero);
+            mma16(low, a, bl, zero);
+            mma16(low, a, bm, low);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) g1[e] += d[e] + low[e];
+        }
+    };
+
+    int t = blockIdx.x, buf = 0;
+    bool any = false;  // a patch was finished: its dW1 is pending (in buffer buf ^ 1)
+    __syncthreads();
+    if (t < n && tid < 256) stage_bf16(reinterpret_cast<uint32_t*>(tsm + TR_IN), tid, load(t));
+    __syncthreads();
+    for (; t < n; buf ^= 1) {
+        const int tn = t + gridDim.x;
+        uint4 pix = make_uint4(0u, 0u, 0u, 0u);
+        if (tn < n && tid >= 256) pix = load(tn);
+        const float label = __ldg(labels + t);
+        // ---- 1: dW1 of the previous patch; layer 1
+        if (any) grad1(buf ^ 1);
+        {
+            const uint32_t* const in = reinterpret_cast<const uint32_t*>(tsm + TR_IN + buf * TI_BYTES);
+            const float bb[2] = {wv(B1 + 2 * t4), wv(B1 + 2 * t4 + 1)};
+#pragma unroll 2
+            for (int i = warp; i < 64; i += TR_WARPS) {
+                const int y = i >> 1, h = i & 1;
+                const uint32_t* r = in + (2 * y + (t4 >> 1)) * TI_ROW + TI_X - 1 + 2 * g + 16 * h + (t4 & 1);
+                const uint32_t* r2 = in + (2 * y + 2) * TI_ROW + TI_X - 1 + 2 * g + 16 * h + t4;
+                uint32_t a[4] = {r[0], r[1], 0u, 0u};
+                if (t4 < 2) {
+                    a[2] = r2[0];
+                    a[3] = r2[1];
+                }
+                float d[4];
+                mma16(d, a, b1, zero);
+                uint8_t* o = p1 + ((y + 1) * T1_ROW + g + 8 * h) * 16 + 4 * t4;
+                store3(o + T1_O * 16, T1_PLANE, relu(d[0] + bb[0]), relu(d[1] + bb[1]));  // even columns
+                store3(o + 16, T1_PLANE, relu(d[2] + bb[0]), relu(d[3] + bb[1]));
+            }
+        }
+        __syncthreads();
+        // ---- 2: layer 2, one output row per warp
+        {
+            const uint32_t row = sb + TR_P1 + (uint32_t)(2 * warp * T1_ROW * 16);
+            const int x = (lane & 7) + 8 * ((lane >> 3) & 1);
+            float acc[2][4] = {}, low[2][4] = {};
+#pragma unroll
+            for (int s = 0; s < 5; ++s) {
+                const int tap = s < 4 ? 2 * s + (lane >> 4) : 8;
+                const uint32_t a0 = row + (uint32_t)(((tap / 3) * T1_ROW + col1(tap % 3) + x) * 16);
+                if (s < 4) {
+                    uint32_t ah[4], am[4], al[4];
+                    ldsm4(ah, a0);
+                    ldsm4(am, a0 + T1_PLANE);
+                    ldsm4(al, a0 + 2 * T1_PLANE);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const uint32_t b[2] = {frag(TR_F2, 9 * j + 2 * s), frag(TR_F2, 9 * j + 2 * s + 1)};
+                        float d[4];
+                        mma16(d, ah, b, zero);
+                        mma16(low[j], al, b, low[j]);
+                        mma16(low[j], am, b, low[j]);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[j][i] += d[i];
+                    }
+                } else {
+                    uint32_t ah[2], am[2], al[2];
+                    ldsm2(ah, a0);
+                    ldsm2(am, a0 + T1_PLANE);
+                    ldsm2(al, a0 + 2 * T1_PLANE);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const uint32_t b = frag(TR_F2, 9 * j + 8);
+                        float d[4];
+                        mma8(d, ah, b, zero);
+                        mma8(low[j], al, b, low[j]);
+                        mma8(low[j], am, b, low[j]);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[j][i] += d[i];
+                    }
+                }
+            }
+            uint8_t* o = p2 + ((warp + 1) * T2_ROW + ((g & 1) ? (g + 1) >> 1 : T2_O + (g >> 1))) * 16 + 4 * t4;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float bb[2] = {wv(B2 + 8 * j + 2 * t4), wv(B2 + 8 * j + 2 * t4 + 1)};
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    store3(o + 64 * i + j * T2_PLANE, 2 * T2_PLANE, relu(acc[j][2 * i] + low[j][2 * i] + bb[0]),
+                           relu(acc[j][2 * i + 1] + low[j][2 * i + 1] + bb[1]));
+            }
+        }
+        __syncthreads();
+        // ---- 3: layer 3 (warps 0..7: two rows, one channel half), its mask, channel sums and counts
+        if (warp < 8) {
+            const int j = warp & 1, y = 2 * (warp >> 1);
+            const uint32_t a3 =
+                sb + TR_P2 + (uint32_t)((lane >> 4) * T2_PLANE + (2 * (y + ((lane >> 3) & 1)) * T2_ROW + (lane & 7)) * 16);
+            float acc[4] = {}, lm[4] = {}, lw[4] = {};
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const uint32_t a0 = a3 + (uint32_t)(((k / 3) * T2_ROW + col2(k % 3)) * 16);
+                uint32_t ah[4], am[4], al[4];
+                ldsm4(ah, a0);
+                ldsm4(am, a0 + 2 * T2_PLANE);
+                ldsm4(al, a0 + 4 * T2_PLANE);
+                const uint32_t b[2] = {frag(TR_F3, 18 * j + 2 * k), frag(TR_F3, 18 * j + 2 * k + 1)};
+                float d[4];
+                mma16(d, ah, b, zero);
+                mma16(lm, am, b, lm);
+                mma16(lw, al, b, lw);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i] += d[i];
+            }
+            float v[4], s[4];  // channels 2t, 2t + 1 of pixels (y, g), (y + 1, g)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = relu(acc[i] + (lm[i] + lw[i]) + wv(B3 + 8 * j + 2 * t4 + (i & 1)));
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                *reinterpret_cast<uint32_t*>(m3 + j * M3_PLANE + ((y + i) * M3_ROW + g) * 16 + 4 * t4) =
+                    (v[2 * i] > 0.f ? 0x3F80u : 0u) | (v[2 * i + 1] > 0.f ? 0x3F800000u : 0u);
+            s[0] = v[0] + v[2];
+            s[1] = v[1] + v[3];
+            s[2] = (v[0] > 0.f ? 1.f : 0.f) + (v[2] > 0.f ? 1.f : 0.f);
+            s[3] = (v[1] > 0.f ? 1.f : 0.f) + (v[3] > 0.f ? 1.f : 0.f);
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s[i] += __shfl_xor_sync(0xFFFFFFFFu, s[i], o);
+            if (g == 0) {
+                float* r = red + (warp >> 1) * C3 + 8 * j + 2 * t4;
+                r[0] = s[0];
+                r[1] = s[1];
+                r[4 * C3] = s[2];
+                r[4 * C3 + 1] = s[3];
+            }
+        } else if (tn < n) {
+            stage_bf16(reinterpret_cast<uint32_t*>(tsm + TR_IN + (buf ^ 1) * TI_BYTES), tid - 256, pix);
+        }
+        __syncthreads();
+        // ---- 4: logit, loss, dlogit (every warp); dW3; d2
+        float dl;
+        {
+            const float* r = red + (lane & 15);
+            const float gap = ((r[0] + r[C3]) + (r[2 * C3] + r[3 * C3])) * (1.f / 64.f);
+            const float cnt = (r[4 * C3] + r[5 * C3]) + (r[6 * C3] + r[7 * C3]);
+            float z = gap * wf;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+            z += bf;
+            const float wt = label > 0.5f ? pos_weight : 1.f;
+            const float sp = z > 0.f ? z + log1pf(expf(-z)) : log1pf(expf(z));
+            const float sg = 1.f / (1.f + expf(-z));
+            dl = wt * (sg - label) / (float)n;
+            if (tid == 0) lsum += (double)(wt * (sp - label * z));
+            gwf += dl * gap;
+            gb3 += dl * wf * (1.f / 64.f) * cnt;
+            gbf += dl;
+        }
+        // dW3: tile i of (tap, half of c); depth = 16 pixels, two rows at a time.
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = warp + TR_WARPS * q;
+            if (i >= 18) break;
+            const int k = i >> 1, h = i & 1;
+            float acc[4] = {}, low[4] = {};
+#pragma unroll
+            for (int y = 0; y < S3; y += 2) {
+                // The mask transposed: rows = channels o, depth = pixels (y, x), (y + 1, x).
+                uint32_t a[4], bh[2], bm[2], bl[2];
+                ldsm4t(a, sb + TR_M3 +
+                              (uint32_t)(((lane >> 3) & 1) * M3_PLANE + ((y + (lane >> 4)) * M3_ROW + (lane & 7)) * 16));
+                const uint32_t b0 = sb + TR_P2 + (uint32_t)(h * T2_PLANE + ((2 * (y + ((lane >> 3) & 1)) + k / 3) * T2_ROW +
+                                                                            col2(k % 3) + (lane & 7)) * 16);
+                ldsm2t(bh, b0);
+                ldsm2t(bm, b0 + 2 * T2_PLANE);
+                ldsm2t(bl, b0 + 4 * T2_PLANE);
+                float d[4];
+                mma16(d, a, bh, zero);
+                mma16(low, a, bl, low);
+                mma16(low, a, bm, low);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[e] += d[e];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) g3[q][e] += dl * (1.f / 64.f) * wfg[e >> 1] * (acc[e] + low[e]);
+        }
+        // d2: pixels (2u + py, 2v + px), two rows u, half j of the channels; two
+        // classes (py, px) per warp: (0, 0) and (1, 1), or (0, 1) and (1, 0).
+        {
+            const int u = 2 * (warp >> 2), j = (warp >> 1) & 1, c2nd = warp & 1;
+            const uint32_t am = sb + TR_M3 + (uint32_t)((lane >> 4) * M3_PLANE +
+                                                        ((u + ((lane >> 3) & 1)) * M3_ROW + (lane & 7)) * 16);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int py = c, px = c2nd ? 1 - c : c;
+                float acc[4] = {}, low[4] = {};
+                // Rows: even pixels take ky = 1; odd ones ky = 0 from row u + 1 and ky = 2 from row u.
+                for (int ky = py ? 0 : 1; ky < 3; ky += 2)
+                    for (int kx = px ? 0 : 1; kx < 3; kx += 2) {
+                        uint32_t a[4];
+                        ldsm4(a, am + (uint32_t)(((ky == 0 ? 1 : 0) * M3_ROW + (kx == 0 ? 1 : 0)) * 16));
+                        const int f = 2 * (18 * j + 2 * (3 * ky + kx));
+                        const uint32_t bh[2] = {frag(TR_FQ, f), frag(TR_FQ, f + 2)},
+                                       bl[2] = {frag(TR_FQ, f + 1), frag(TR_FQ, f + 3)};
+                        float d[4];
+                        mma16(d, a, bh, zero);
+                        mma16(low, a, bl, low);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[e] += d[e];
+                    }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int iy = 2 * (u + i) + py, ix = 2 * g + px;
+                    // ReLU of layer 2: the leading part is zero where the activation is.
+                    const uint32_t a2 = *reinterpret_cast<const uint32_t*>(
+                        p2 + j * T2_PLANE + ((iy + 1) * T2_ROW + (px ? g + 1 : T2_O + g)) * 16 + 4 * t4);
+                    const float v0 = (a2 & 0xFFFFu) ? dl * (1.f / 64.f) * (acc[2 * i] + low[2 * i]) : 0.f;
+                    const float v1 = (a2 >> 16) ? dl * (1.f / 64.f) * (acc[2 * i + 1] + low[2 * i + 1]) : 0.f;
+                    gb2[0] += v0;
+                    gb2[1] += v1;
+                    store3(d2 + j * D2_PLANE + (iy * D2_ROW + ix) * 16 + 4 * t4, 2 * D2_PLANE, v0, v1);
+                }
+            }
+        }
+        __syncthreads();
+        // ---- 5: dW2 (depth = the 16 pixels of row `warp`), then d1 (row pairs 2u, 2u + 1, u = warp)
+        {
+            uint32_t ah[4], am[4], al[4];
+            const uint32_t a0 = sb + TR_D2 + (uint32_t)(((lane >> 3) & 1) * D2_PLANE +
+                                                        (warp * D2_ROW + (lane & 7) + 8 * (lane >> 4)) * 16);
+            ldsm4t(ah, a0);
+            ldsm4t(am, a0 + 2 * D2_PLANE);
+            ldsm4t(al, a0 + 4 * D2_PLANE);
+            const uint32_t b0 = sb + TR_P1 + (uint32_t)((2 * warp * T1_ROW + (lane & 15)) * 16);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                uint32_t bh[2], bm[2], bl[2];
+                const uint32_t ba = b0 + (uint32_t)(((k / 3) * T1_ROW + col1(k % 3)) * 16);
+                ldsm2t(bh, ba);
+                ldsm2t(bm, ba + T1_PLANE);
+                ldsm2t(bl, ba + 2 * T1_PLANE);
+                float d[4], low[4];
+                mma16(d, ah, bh, zero);
+                mma16(low, al, bh, zero);
+                mma16(low, ah, bl, low);
+                mma16(low, am, bm, low);
+                mma16(low, am, bh, low);
+                mma16(low, ah, bm, low);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) g2[k][e] += d[e] + low[e];
+            }
+        }
+        {
+            float acc[4][4] = {}, low[4][4] = {};  // class 2 py + px
+            const uint32_t a0 = sb + TR_D2 + (uint32_t)((lane >> 4) * D2_PLANE + (warp * D2_ROW + (lane & 15)) * 16);
+#pragma unroll
+            for (int dd = 0; dd < 4; ++dd) {  // d2 pixel (u + dy, v + dx)
+                const int dy = dd >> 1, dx = dd & 1;
+                uint32_t ah[4], am[4], al[4];
+                const uint32_t aa = a0 + (uint32_t)((dy * D2_ROW + dx) * 16);
+                ldsm4(ah, aa);
+                ldsm4(am, aa + 2 * D2_PLANE);
+                ldsm4(al, aa + 4 * D2_PLANE);
+#pragma unroll
+                for (int cl = 0; cl < 4; ++cl) {
+                    const int py = cl >> 1, px = cl & 1;
+                    if ((dy && !py) || (dx && !px)) continue;
+                    const int ky = !py ? 1 : dy ? 0 : 2, kx = !px ? 1 : dx ? 0 : 2;
+                    const uint32_t b[2] = {frag(TR_FT, 2 * (3 * ky + kx)), frag(TR_FT, 2 * (3 * ky + kx) + 1)};
+                    float d[4];
+                    mma16(d, ah, b, zero);
+                    mma16(low[cl], al, b, low[cl]);
+                    mma16(low[cl], am, b, low[cl]);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[cl][e] += d[e];
+                }
+            }
+#pragma unroll
+            for (int cl = 0; cl < 4; ++cl) {
+                const int iy = 2 * warp + (cl >> 1), px = cl & 1;
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int v = g + 8 * i;
+                    const uint32_t a1 = *reinterpret_cast<const uint32_t*>(
+                        p1 + ((iy + 1) * T1_ROW + (px ? v + 1 : T1_O + v)) * 16 + 4 * t4);
+                    const float v0 = (a1 & 0xFFFFu) ? acc[cl][2 * i] + low[cl][2 * i] : 0.f;
+                    const float v1 = (a1 >> 16) ? acc[cl][2 * i + 1] + low[cl][2 * i + 1] : 0.f;
+                    gb1[0] += v0;
+                    gb1[1] += v1;
+                    store3(d1 + (iy * 32 + px * 16 + v) * 16 + 4 * t4, D1_PLANE, v0, v1);
+                }
+            }
+        }
+        any = true;
+        t = tn;
+        __syncthreads();
+    }
+    if (any) grad1(buf ^ 1);
+
+    // ---- the block's sums into the gradient.  dW3's tiles have one owner each; the others are summed over the
+    // warps in shared memory first (the planes are free: every warp is past its last read after the barrier).
+    __syncthreads();
+    if (!any) return;
+    // Per warp: dW2 [16][8][9], dW1 [8][9], db2 [16], db1 [8].
+    constexpr int N2 = C2 * C1 * 9, N1 = C1 * 9, NS = N2 + N1 + C2 + C1;
+    static_assert(TR_WARPS * NS * 4 <= TR_F2 - TR_P1, "the sums fit the planes");
+    float* const sum = reinterpret_cast<float*>(tsm + TR_P1);
+    float* const own = sum + warp * NS;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int o = g + 8 * (e >> 1), c = 2 * t4 + (e & 1);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) own[(o * C1 + c) * 9 + k] = g2[k][e];
+        if (o <= 8) own[N2 + c * 9 + o] = g1[e];  // rows of dW1: taps 0 .. 8
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = warp + TR_WARPS * q;
+            if (i < 18) atomicAdd(grad + W3 + (o * C2 + 8 * (i & 1) + c) * 9 + (i >> 1), g3[q][e]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            gb2[i] += __shfl_xor_sync(0xFFFFFFFFu, gb2[i], o);
+            gb1[i] += __shfl_xor_sync(0xFFFFFFFFu, gb1[i], o);
+        }
+        if (g == 0) {
+            const int j = (warp >> 1) & 1;  // the half of the channels whose d2 this warp made
+            own[N2 + N1 + 8 * j + 2 * t4 + i] = gb2[i];
+            own[N2 + N1 + 8 * (1 - j) + 2 * t4 + i] = 0.f;
+            own[N2 + N1 + C2 + 2 * t4 + i] = gb1[i];
+        }
+    }
+    if (warp == 0) {
+        if (lane < C3) {
+            atomicAdd(grad + WF + lane, gwf);
+            atomicAdd(grad + B3 + lane, gb3);
+        }
+        if (lane == 0) {
+            atomicAdd(grad + BF, gbf);
+            atomicAdd(loss, lsum / (double)n);
+        }
     }
     __syncthreads();
-    for (int t = blockIdx.x; t < n; t += gridDim.x) {
-        const float* sv = save + (size_t)t * SAVE;
-        const float* a1 = sv;
-        const float* a2 = sv + A1;
-        const float* a3 = sv + A1 + A2;
-        const float* gap = sv + A1 + A2 + A3;
-        const float dl = dz[t];
-        const uint8_t* p = tiles + (size_t)t * S0 * S0;
-        for (int i = threadIdx.x; i < S0 * S0; i += blockDim.x) in[i] = ((float)p[i] - 128.f) * (1.f / 64.f);
-        for (int c = threadIdx.x; c < C3; c += blockDim.x) g[WF + c] += dl * gap[c];
-        if (threadIdx.x == 0) g[BF] += dl;
-        // d3 = dgap / 64 * relu'(a3)
-        for (int i = threadIdx.x; i < A3; i += blockDim.x) {
-            const int c = i / 64;
-            d3[i] = a3[i] > 0.f ? dl * w[WF + c] * (1.f / 64.f) : 0.f;
-        }
-        __syncthreads();
-        conv_s2_back(a2, C2, S2, w + W3, C3, d3, g + W3, g + B3, d2);
-        __syncthreads();
-        for (int i = threadIdx.x; i < A2; i += blockDim.x) d2[i] = a2[i] > 0.f ? d2[i] : 0.f;
-        __syncthreads();
-        conv_s2_back(a1, C1, S1, w + W2, C2, d2, g + W2, g + B2, d1);
-        __syncthreads();
-        for (int i = threadIdx.x; i < A1; i += blockDim.x) d1[i] = a1[i] > 0.f ? d1[i] : 0.f;
-        __syncthreads();
-        conv_s2_back(in, 1, S0, w + W1, C1, d1, g + W1, g + B1, nullptr);
-        __syncthreads();
+    for (int i = tid; i < NS; i += TR_THREADS) {
+        float v = 0.f;
+        for (int w = 0; w < TR_WARPS; ++w) v += sum[w * NS + i];
+        const int at = i < N2 ? W2 + i : i < N2 + N1 ? W1 + i - N2 : i < N2 + N1 + C2 ? B2 + i - N2 - N1 : B1 + i - N2 - N1 - C2;
+        atomicAdd(grad + at, v);
     }
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) atomicAdd(&grad[i], g[i]);
 }
 
 __global__ void k_adam(float* __restrict__ master, __nv_bfloat16* __restrict__ wq, const float* __restrict__ g,
@@ -664,36 +958,18 @@ int fail(int code, const std::string& m) {
     return code;
 }
 
-int ensure_cap(of_tcnn* N, int n) {
-    if (n <= N->cap) return OF_OK;
-    if (N->save) cudaFree(N->save);
-    if (N->dz) cudaFree(N->dz);
-    N->save = nullptr;
-    N->dz = nullptr;
-    if (cudaMalloc(&N->save, sizeof(float) * SAVE * (size_t)n) != cudaSuccess ||
-        cudaMalloc(&N->dz, sizeof(float) * (size_t)n) != cudaSuccess) {
-        N->cap = 0;
-        return fail(OF_ERR_CUDA, "tile-net workspace allocation failed");
-    }
-    N->cap = n;
-    return OF_OK;
-}
-
-int grid_for(int n) {
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-    return n < 2 * sms ? n : 2 * sms;
+int sm_count() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
 }
 
 // Blocks of the inference kernel: every SM's three, at most one per tile.
 int fwd_grid(int n) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return n < FWD_BLOCKS * sms ? n : FWD_BLOCKS * sms;
+    const int m = FWD_BLOCKS * sm_count();
+    return n < m ? n : m;
 }
-
-constexpr int SMEM_BWD = (S0 * S0 + A1 + A2 + A3 + 2 * NP) * 4;
 
 // Proposal mask of one listed image per block (see of_detect_learned).
 __global__ void k_propose(const ofk::Img* __restrict__ imgs, const int32_t* __restrict__ list,
@@ -796,8 +1072,7 @@ extern "C" {
 of_tcnn* of_tcnn_create(uint64_t seed) {
     static bool attr = false;
     if (!attr) {
-        cudaFuncSetAttribute(tn::k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::SMEM_FWD);
-        cudaFuncSetAttribute(tn::k_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::SMEM_BWD);
+        cudaFuncSetAttribute(tn::k_train, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::TR_SMEM);
         cudaFuncSetAttribute(tn::k_forward_fast, cudaFuncAttributeMaxDynamicSharedMemorySize, tn::FWD_SMEM);
         attr = true;
     }
@@ -805,8 +1080,8 @@ of_tcnn* of_tcnn_create(uint64_t seed) {
     cudaGetDevice(&N->device);
     const size_t b = sizeof(float) * tn::NP;
     if (cudaMalloc(&N->master, b) != cudaSuccess || cudaMalloc(&N->w, sizeof(__nv_bfloat16) * tn::NP) != cudaSuccess ||
-        cudaMalloc(&N->grad, b) != cudaSuccess || cudaMalloc(&N->m, b) != cudaSuccess ||
-        cudaMalloc(&N->v, b) != cudaSuccess || cudaMalloc(&N->loss, sizeof(float)) != cudaSuccess) {
+        cudaMalloc(&N->grad, sizeof(float) * (tn::LOSS_AT + 2)) != cudaSuccess || cudaMalloc(&N->m, b) != cudaSuccess ||
+        cudaMalloc(&N->v, b) != cudaSuccess) {
         tn::fail(OF_ERR_CUDA, "tile-net allocation failed");
         of_tcnn_destroy(N);
         return nullptr;
@@ -835,8 +1110,7 @@ of_tcnn* of_tcnn_create(uint64_t seed) {
 
 void of_tcnn_destroy(of_tcnn* N) {
     if (!N) return;
-    for (void* q : {(void*)N->master, (void*)N->w, (void*)N->grad, (void*)N->m, (void*)N->v, (void*)N->save,
-                    (void*)N->dz, (void*)N->loss})
+    for (void* q : {(void*)N->master, (void*)N->w, (void*)N->grad, (void*)N->m, (void*)N->v})
         if (q) cudaFree(q);
     delete N;
 }
@@ -886,19 +1160,18 @@ int of_tcnn_forward(of_tcnn* N, const uint8_t* tiles, int n, float* logits, void
 int of_tcnn_loss_grad(of_tcnn* N, const uint8_t* tiles, const float* labels, int n, float pos_weight,
                       float* loss_out, void* stream) {
     if (!N || !tiles || !labels || n < 1 || !(pos_weight > 0.f)) return tn::fail(OF_ERR_ARG, "bad arguments");
-    int rc = tn::ensure_cap(N, n);
-    if (rc != OF_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaMemsetAsync(N->grad, 0, sizeof(float) * tn::NP, st);
-    cudaMemsetAsync(N->loss, 0, sizeof(float), st);
-    tn::k_forward<<<tn::grid_for(n), tn::THREADS, tn::SMEM_FWD, st>>>(tiles, n, N->w, nullptr, N->save);
-    tn::k_bce<<<(n + 255) / 256, 256, 0, st>>>(N->save, labels, n, pos_weight, N->dz, N->loss);
-    tn::k_backward<<<tn::grid_for(n), tn::THREADS, tn::SMEM_BWD, st>>>(tiles, n, N->w, N->save, N->dz, N->grad);
+    double* const loss = reinterpret_cast<double*>(N->grad + tn::LOSS_AT);
+    cudaMemsetAsync(N->grad, 0, sizeof(float) * (tn::LOSS_AT + 2), st);
+    const int sms = tn::sm_count();
+    tn::k_train<<<n < sms ? n : sms, tn::TR_THREADS, tn::TR_SMEM, st>>>(tiles, labels, n, pos_weight, N->w, N->grad, loss);
     if (cudaGetLastError() != cudaSuccess) return tn::fail(OF_ERR_CUDA, "tile-net training launch failed");
     if (loss_out) {
-        if (cudaMemcpyAsync(loss_out, N->loss, sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        double sum = 0.0;
+        if (cudaMemcpyAsync(&sum, loss, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
             return tn::fail(OF_ERR_CUDA, "tile-net loss readback failed");
+        *loss_out = (float)sum;
     }
     return OF_OK;
 }

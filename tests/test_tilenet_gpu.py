@@ -65,6 +65,28 @@ def test_forward_at_grid_edges(n):
     net.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 151, 152, 153, 305])
+def test_gradient_at_grid_edges(n):
+    """Loss and every layer's gradient, one patch per block or fewer and more; the same bounds as the
+    existing gradient test (fp32 against float64; a ReLU input within rounding of 0 may flip)."""
+    net = learned.TileNet(n)
+    tiles = _tiles(n, 6)
+    rng = np.random.default_rng(n)
+    labels = (rng.random(n) < 0.4).astype(np.float32)
+    buf = torch.zeros(tiles.size + 1, dtype=torch.uint8, device="cuda")  # unaligned patches
+    buf[1:] = torch.from_numpy(tiles).cuda().reshape(-1)
+    lab = torch.from_numpy(labels).cuda()
+    for dev in (torch.from_numpy(tiles).cuda(), buf[1:]):
+        loss = ofg.of_tcnn_loss_grad(net.net, dev, lab, n, pos_weight=3.0)
+        g = ofg.of_tcnn_get_params(net.net, 2).astype(np.float64)
+        lo, go = ora.loss_grad(tiles, labels, ofg.of_tcnn_get_params(net.net, 1).astype(np.float64), pos_weight=3.0)
+        assert loss == pytest.approx(lo, rel=1e-5)
+        assert np.linalg.norm(g - go) / np.linalg.norm(go) < 1e-4
+        for a, b in ((0, 72), (72, 80), (80, 1232), (1232, 1248), (1248, 3552), (3552, 3568), (3568, 3584), (3584, 3585)):
+            assert np.linalg.norm(g[a:b] - go[a:b]) <= 1e-3 * np.linalg.norm(go[a:b]) + 1e-12, (a, b)
+    net.close()
+
+
 def test_infinite_activations():
     """Activations that overflow stay infinities (not NaN) through the split into parts."""
     net = learned.TileNet(0)
