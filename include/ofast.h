@@ -143,6 +143,13 @@ void of_destroy(of_handle* h);
 int of_detect(of_handle* h, const uint8_t* img, int w, int h_px, int pitch, int levels,
               float scale, int fast_t, float harris_k, int n_features, of_keypoint* out_kpts);
 
+/* of_detect whose records also arrive in host memory: out_kpts [device] as
+ * of_detect, host_kpts [host] room for n_features records (the count's many are
+ * written).  One synchronisation for count and records.  Returns as of_detect. */
+int of_detect_host(of_handle* h, const uint8_t* img, int w, int h_px, int pitch, int levels,
+                   float scale, int fast_t, float harris_k, int n_features, of_keypoint* out_kpts,
+                   of_keypoint* host_kpts);
+
 /* Detect keypoints in n_frames frames of any sizes in one batched launch
  * sequence (replayed from a cached CUDA graph for a repeated batch shape).
  *   frames [host]         n_frames descriptors, 1 <= n_frames <= max_batch

@@ -21,7 +21,7 @@ import numpy as np
 
 from .build import LIB, build  # noqa: F401
 
-__all__ = ["of_create", "of_destroy", "of_detect", "of_detect_batch", "of_inspect", "of_plan_levels",
+__all__ = ["of_create", "of_destroy", "of_detect", "of_detect_host", "of_detect_batch", "of_inspect", "of_plan_levels",
            "of_time_stages", "OF_N_STAGES", "STAGE_NAMES", "of_detect_level_noalloc", "of_probe_read", "of_sync",
            "of_test_timeout", "OF_ERR_TIMEOUT", "of_autotune", "of_variant_detect", "OfVarPoint",
            "VAR_POINT_DTYPE", "of_set_tuning", "OfTuning", "of_batch_bytes",
@@ -146,6 +146,8 @@ def load(path: str | None = None):
     L.of_detect.argtypes = [C.c_void_p, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_float,
                             C.c_int, C.c_float, C.c_int, C.c_void_p]
     L.of_detect.restype = C.c_int
+    L.of_detect_host.argtypes = [*L.of_detect.argtypes, C.c_void_p]
+    L.of_detect_host.restype = C.c_int
     L.of_detect_batch.argtypes = [C.c_void_p, C.POINTER(OfFrame), C.c_int, C.c_int, C.c_float, C.c_int,
                                   C.c_float, C.c_int, C.c_void_p, C.c_void_p]
     L.of_detect_batch.restype = C.c_int
@@ -266,6 +268,14 @@ def of_detect(h: int, img, w: int, h_px: int, pitch: int, levels: int, scale: fl
               harris_k: float, n_features: int, out_kpts) -> int:
     return _check(load().of_detect(h, _ptr(img), w, h_px, pitch, levels, scale, fast_t, harris_k,
                                    n_features, _ptr(out_kpts)))
+
+
+def of_detect_host(h: int, img, w: int, h_px: int, pitch: int, levels: int, scale: float, fast_t: int,
+                   harris_k: float, n_features: int, out_kpts, host_kpts: np.ndarray) -> int:
+    """of_detect whose records also arrive in ``host_kpts`` (n_features records of KEYPOINT_DTYPE)."""
+    assert host_kpts.dtype == KEYPOINT_DTYPE and host_kpts.size >= n_features and host_kpts.flags.c_contiguous
+    return _check(load().of_detect_host(h, _ptr(img), w, h_px, pitch, levels, scale, fast_t, harris_k,
+                                        n_features, _ptr(out_kpts), host_kpts.ctypes.data))
 
 
 def of_detect_batch(h: int, frames, levels: int, scale: float, fast_t: int, harris_k: float,
@@ -559,9 +569,10 @@ class Detector:
     def detect(self, img, levels=8, scale=1.2, fast_t=20, harris_k=0.04, n_features=1000) -> np.ndarray:
         """One frame (2-D uint8 CUDA tensor, rows may be strided) -> numpy keypoints."""
         assert img.dtype == self.torch.uint8 and img.is_cuda and img.dim() == 2 and img.stride(1) == 1
-        n = of_detect(self.h, img, img.shape[1], img.shape[0], img.stride(0), levels, scale, fast_t,
-                      harris_k, n_features, self.out)
-        return keypoints_to_numpy(self.out[: n * 64])
+        h_px, w = img.shape
+        kp = np.empty(max(n_features, 0), KEYPOINT_DTYPE)
+        n = of_detect_host(self.h, img, w, h_px, img.stride(0), levels, scale, fast_t, harris_k, n_features, self.out, kp)
+        return kp if n == len(kp) else kp[:n].copy()
 
     def detect_batch(self, imgs, levels=8, scale=1.2, fast_t=20, harris_k=0.04, n_features=1000):
         """Queue a batch (list of 2-D uint8 CUDA tensors); returns (records tensor, counts tensor)."""

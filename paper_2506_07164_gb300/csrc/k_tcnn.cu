@@ -26,7 +26,7 @@ void set_last_error(const std::string& msg);
 
 namespace tn {
 
-constexpr int S0 = 64, S1 = 32, S2 = 16, S3 = 8;  // spatial sizes
+constexpr int S0 = 64, S2 = 16, S3 = 8;  // spatial sizes (64, 32, 16, 8)
 constexpr int C1 = 8, C2 = 16, C3 = 16;
 // Flat parameter layout.
 constexpr int W1 = 0, B1 = W1 + C1 * 9, W2 = B1 + C1, B2 = W2 + C2 * C1 * 9, W3 = B2 + C2,

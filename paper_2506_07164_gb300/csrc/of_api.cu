@@ -356,7 +356,8 @@ struct of_handle {
     size_t arena_bytes = 0;
     int32_t* d_counts = nullptr;  // [0] of_detect's count, [4] device status word
     int n_sms = 0;
-    int32_t* h_count = nullptr;   // pinned
+    int32_t* h_count = nullptr;   // pinned: [0] of_detect's count (written by the device), [4..] read-backs
+    of_keypoint* h_rec = nullptr;  // pinned: of_detect_host's records
     std::vector<Plan*> plans;
     Plan* last = nullptr;
     uint64_t clock = 0;
@@ -1471,6 +1472,37 @@ int run_batch(of_handle* H, const of_frame* frames, int n_frames, int levels, fl
     return OF_OK;
 }
 
+// One frame, waited for.  The orientation kernel writes the count to pinned
+// host memory, so the wait needs no copy of it; a wait that expired on the
+// device shows up as a negative count (the status word itself is read, and
+// cleared, only then).  host: the records too, by one copy before the wait.
+int detect_one(of_handle* H, const uint8_t* img, int w, int h_px, int pitch, int levels, float scale, int fast_t,
+               float harris_k, int n_features, of_keypoint* out, of_keypoint* host) {
+    if (!H) return fail(OF_ERR_ARG, "null handle");
+    of_frame F{img, w, h_px, pitch};
+    // No features: no slot publishes a count, run_batch clears it on the device.
+    int32_t* const counts = n_features > 0 ? H->h_count : H->d_counts;
+    const int rc = run_batch(H, &F, 1, levels, scale, fast_t, harris_k, n_features, out, counts);
+    if (rc != OF_OK) return rc;
+    DeviceGuard dg(H->device);
+    if (n_features <= 0)
+        OF_CK(cudaMemcpyAsync(H->h_count, H->d_counts, sizeof(int32_t), cudaMemcpyDeviceToHost, H->stream));
+    else if (host)
+        OF_CK(cudaMemcpyAsync(H->h_rec, out, sizeof(of_keypoint) * n_features, cudaMemcpyDeviceToHost, H->stream));
+    OF_CK(cudaStreamSynchronize(H->stream));
+    const int n = *static_cast<volatile int32_t*>(H->h_count);
+    if (n < 0 || n_features <= 0) {
+        int32_t status = 0;
+        OF_CK(cudaMemcpy(&status, H->d_counts + 4, sizeof(status), cudaMemcpyDeviceToHost));
+        if (status != 0) {
+            OF_CK(cudaMemset(H->d_counts + 4, 0, sizeof(int32_t)));
+            return fail(OF_ERR_TIMEOUT, "a device-side wait expired");
+        }
+    }
+    if (host && n > 0) std::memcpy(host, H->h_rec, sizeof(of_keypoint) * n);
+    return n;
+}
+
 }  // namespace
 
 namespace ofk {
@@ -1562,6 +1594,7 @@ of_handle* of_create(const of_params* pin) {
     e = cudaMemset(H->d_counts, 0, sizeof(int32_t) * 8);
     if (e != cudaSuccess) return bail(e, "cudaMemset(counts)");
     e = cudaMallocHost(&H->h_count, sizeof(int32_t) * 8);
+    if (e == cudaSuccess) e = cudaMallocHost(&H->h_rec, sizeof(of_keypoint) * std::max(p.max_features, 1));
     if (e != cudaSuccess) return bail(e, "cudaMallocHost");
     e = cudaDeviceGetAttribute(&H->n_sms, cudaDevAttrMultiProcessorCount, H->device);
     if (e != cudaSuccess) return bail(e, "cudaDeviceGetAttribute");
@@ -1583,6 +1616,7 @@ void of_destroy(of_handle* H) {
     if (H->arena) cudaFree(H->arena);
     if (H->d_counts) cudaFree(H->d_counts);
     if (H->h_count) cudaFreeHost(H->h_count);
+    if (H->h_rec) cudaFreeHost(H->h_rec);
     if (H->cap_stream) cudaStreamDestroy(H->cap_stream);
     for (int g = 0; g < kMaxGroups - 1; ++g) {
         if (H->cap_branch[g]) cudaStreamDestroy(H->cap_branch[g]);
@@ -1785,20 +1819,14 @@ int of_time_stages(of_handle* H, void* const* events) {
 
 int of_detect(of_handle* H, const uint8_t* img, int w, int h_px, int pitch, int levels,
               float scale, int fast_t, float harris_k, int n_features, of_keypoint* out_kpts) {
-    if (!H) return fail(OF_ERR_ARG, "null handle");
-    of_frame F{img, w, h_px, pitch};
-    const int rc = run_batch(H, &F, 1, levels, scale, fast_t, harris_k, n_features, out_kpts,
-                             H->d_counts);
-    if (rc != OF_OK) return rc;
-    DeviceGuard dg(H->device);
-    OF_CK(cudaMemcpyAsync(H->h_count, H->d_counts, 8 * sizeof(int32_t), cudaMemcpyDeviceToHost,
-                          H->stream));
-    OF_CK(cudaStreamSynchronize(H->stream));
-    if (H->h_count[4] != 0) {
-        OF_CK(cudaMemset(H->d_counts + 4, 0, sizeof(int32_t)));
-        return fail(OF_ERR_TIMEOUT, "a device-side wait expired");
-    }
-    return H->h_count[0];
+    return detect_one(H, img, w, h_px, pitch, levels, scale, fast_t, harris_k, n_features, out_kpts, nullptr);
+}
+
+int of_detect_host(of_handle* H, const uint8_t* img, int w, int h_px, int pitch, int levels,
+                   float scale, int fast_t, float harris_k, int n_features, of_keypoint* out_kpts,
+                   of_keypoint* host_kpts) {
+    if (n_features > 0 && !host_kpts) return fail(OF_ERR_ARG, "null output pointer");
+    return detect_one(H, img, w, h_px, pitch, levels, scale, fast_t, harris_k, n_features, out_kpts, host_kpts);
 }
 
 int of_sync(of_handle* H) {
