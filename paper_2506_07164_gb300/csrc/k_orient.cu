@@ -1,9 +1,12 @@
 // Orientation by intensity centroid (Fig. 1 "Centroid") and the output
 // records.  One warp per output slot (frame, level, rank):
-//   - Harris sums A, B, C of the kept keypoint (Eqs. 2-4), lanes over the 49
-//     window positions, warp reduction;
-//   - moments m10 = sum u I, m01 = sum v I over the disc u^2 + v^2 <= r^2,
-//     lane = column u, loop over rows v, warp reduction;
+//   - the keypoint's patch (31 x 31 for radius 15) goes to shared memory as
+//     aligned words, 9 loads per lane in flight at once;
+//   - lane = column u: moments m10 = sum u I, m01 = sum v I over the disc
+//     u^2 + v^2 <= r^2 from the column's sums, warp reduction;
+//   - Harris sums A, B, C of the kept keypoint (Eqs. 2-4): lanes hold columns,
+//     so the vertical Sobel passes are a lane's own rows and the horizontal
+//     ones two shuffles per row, warp reduction;
 //   - angle = atan2f(m01, m10) (both moments are exact int32, |m| < 2^24, so
 //     their float conversion is exact);
 //   - response = key / kden * (1 / (4*7*255))^4, as key (float) times the
@@ -11,6 +14,13 @@
 //   - level-0 coordinates from the plan's tables (x * scale^level rounded once).
 // Records are level-major in rank order: the slot of a kept keypoint is the
 // number of keypoints kept by the frame's earlier levels plus its rank.
+//
+// Bound by the latency of a warp's chain of loads (descriptors, position,
+// pixels), so each link is one round: the counts of the earlier levels by one
+// lane each, everything that depends on the position together.  128 1080p frames
+// (128 k keypoints): 145 us with byte loads in rounds of 8, two rounds of Sobel
+// loads and the counts and the score one after another, 108 us now, bound by
+// instruction issue (70 %).
 #include <cuda_runtime.h>
 
 #include "of_internal.h"
@@ -18,9 +28,13 @@
 
 namespace ofk {
 
+constexpr int OP_WORDS = 9;                   // aligned words that hold any 31 bytes
+constexpr int OP_SIZE = 31 * OP_WORDS;        // words of a patch
+
 __global__ void __launch_bounds__(ORIENT_WARPS * 32)
 k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin, int slot_end,
          const Call* __restrict__ call, const uint16_t* __restrict__ slot_img) {
+    __shared__ uint32_t patch[ORIENT_WARPS][OP_SIZE];
     const int slot = slot_begin + blockIdx.x * ORIENT_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     pdl_trigger();
@@ -40,97 +54,116 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
     }
     const Img& I = imgs[lo];
     const int rank = slot - I.slot0;
-    const int levels = call->levels;
-    const Img* F = imgs + I.frame * levels;
-    // Descriptor fields, read before the wait.
-    const uint8_t* img = I.img;
-    const int pitch = I.pitch, quota = I.quota, level = I.level;
+    const int levels = call->levels, n_features = call->n_features;
+    // Descriptor fields, read before the wait; lane l < levels: level l's counters.
+    const uint8_t* const img = I.img;
+    const uint8_t* const score = I.score;
+    const float* const fx = I.fx;
+    const float* const fy = I.fy;
+    const int pitch = I.pitch, spitch = I.spitch, quota = I.quota, level = I.level, frame = I.frame;
     const int32_t* const ctr = I.ctr;
+    const int32_t* const lctr = lane < levels ? imgs[frame * levels + lane].ctr : nullptr;
     const uint32_t* const kyx = I.kyx;
-    const bool first = slot == I.frame * call->n_features;
+    const uint64_t* const kkey = I.kkey;
+    const int R = call->radius, H = max(R, 4);  // H: rows and columns around the keypoint that are read
     pdl_wait();  // the kept keypoints
-
+    if (rank >= quota && slot != frame * n_features) return;
+    const int kept_l = lctr ? lctr[1] : 0;
+    const int kept = ctr[1];
+    const bool on = rank < quota;
+    const uint32_t yx = on ? kyx[rank] : 0u;  // issued beside the counts; unused beyond them
+    const uint64_t okey = on ? kkey[rank] : 0ull;
     // The frame's first slot publishes its keypoint count.
-    if (first) {
-        if (lane == 0) {
-            int total = 0;
-            for (int l = 0; l < levels; ++l) total += F[l].ctr[1];
-            // A detect-stage wait that expired leaves partial results: report it instead.
-            call->counts[I.frame] = *call->status ? OF_ERR_TIMEOUT : total;
-        }
+    if (slot == frame * n_features) {
+        const int total = __reduce_add_sync(0xFFFFFFFFu, kept_l);
+        // A detect-stage wait that expired leaves partial results: report it instead.
+        if (lane == 0) call->counts[frame] = *call->status ? OF_ERR_TIMEOUT : total;
     }
-    if (rank >= quota) return;
-    const uint32_t yx = kyx[rank];  // issued beside the count; unused beyond it
-    if (rank >= ctr[1]) return;
-    int base = 0;
-    for (int l = 0; l < level; ++l) base += F[l].ctr[1];
+    if (rank >= quota || rank >= kept) return;
+    const int base = __reduce_add_sync(0xFFFFFFFFu, lane < level ? kept_l : 0);
+
     const int x = (int)(yx & 0xFFFFu), y = (int)(yx >> 16);
-
-    // Harris sums over the 7 x 7 window.
-    int a = 0, b = 0, c = 0;
+    // The patch, columns x - H .. x + H of rows y - H .. y + H, as aligned words
+    // (images and pitches are multiples of 16 bytes; H <= border keeps it inside).
+    uint32_t* const P = patch[threadIdx.x >> 5];
+    const int sh = (x - H) & 3, nw = (sh + 2 * H + 4) >> 2, rows = 2 * H + 1;
+    {
+        const uint8_t* const q = img + (size_t)(y - H) * pitch + (x - H - sh);
+        uint32_t v[OP_WORDS];
 #pragma unroll
-    for (int rep = 0; rep < 2; ++rep) {
-        const int p = lane + 32 * rep;
-        if (p < 49) {
-            const int u = p % 7 - 3, v = p / 7 - 3;
-            const uint8_t* q = img + (size_t)(y + v) * pitch + (x + u);
-            const int l0 = __ldg(q - pitch - 1), c0 = __ldg(q - pitch), r0 = __ldg(q - pitch + 1);
-            const int l1 = __ldg(q - 1), r1 = __ldg(q + 1);
-            const int l2 = __ldg(q + pitch - 1), c2 = __ldg(q + pitch), r2 = __ldg(q + pitch + 1);
-            const int gx = (r0 - l0) + 2 * (r1 - l1) + (r2 - l2);
-            const int gy = (l2 - l0) + 2 * (c2 - c0) + (r2 - r0);
-            a += gx * gx;
-            b += gy * gy;
-            c += gx * gy;
+        for (int k = 0; k < OP_WORDS; ++k) {
+            const int i = lane + 32 * k, r = i / OP_WORDS, c = i - r * OP_WORDS;
+            v[k] = r < rows && c < nw ? __ldg(reinterpret_cast<const uint32_t*>(q + (size_t)r * pitch) + c) : 0u;
         }
+#pragma unroll
+        for (int k = 0; k < OP_WORDS; ++k)
+            if (lane + 32 * k < OP_SIZE) P[lane + 32 * k] = v[k];
     }
-    a = __reduce_add_sync(0xFFFFFFFFu, a);
-    b = __reduce_add_sync(0xFFFFFFFFu, b);
-    c = __reduce_add_sync(0xFFFFFFFFu, c);
+    const int sc = lane == 0 ? (int)score[(size_t)y * spitch + x] : 0;
+    // No tables: a level-0 image (scale^0 = 1; the allocation-free entry point).
+    const float kx = fx ? fx[x] : (float)x, ky = fx ? fy[y] : (float)y;
+    __syncwarp();
 
-    // Centroid moments.
-    const int R = call->radius;
+    // Lane = column u = lane - 15 (lanes beyond H repeat a column of the patch).
     const int u = lane - 15;
+    const uint8_t* const col = reinterpret_cast<const uint8_t*>(P) + sh + H + min(max(u, -H), H);
+    constexpr int RB = 4 * OP_WORDS;  // bytes per patch row
     int m10 = 0, m01 = 0;
-    if (u >= -R && u <= R) {
-        // Rows in groups of 8 so that each lane has 8 loads in flight.
-        const uint8_t* col = img + (size_t)y * pitch + (x + u);
-        for (int v0 = -R; v0 <= R; v0 += 8) {
-            int iv[8];
+    {
+        // Rows of the disc in this column: |v| <= hv (none beyond the radius).
+        const int hv = u >= -R && u <= R ? (int)sqrtf((float)(R * R - u * u)) : -1;
+        const uint8_t* const mid = col + H * RB;
+        int s0 = hv >= 0 ? mid[0] : 0;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int v = v0 + k;
-                iv[k] = (v <= R && u * u + v * v <= R * R) ? __ldg(col + (ptrdiff_t)v * pitch) : 0;
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                m10 += u * iv[k];
-                m01 += (v0 + k) * iv[k];
-            }
+        for (int v = 1; v <= 15; ++v) {
+            const int up = v <= hv ? mid[-v * RB] : 0, dn = v <= hv ? mid[v * RB] : 0;
+            s0 += up + dn;
+            m01 += v * (dn - up);
         }
+        m10 = u * s0;
     }
     m10 = __reduce_add_sync(0xFFFFFFFFu, m10);
     m01 = __reduce_add_sync(0xFFFFFFFFu, m01);
 
+    // Harris sums over the 7 x 7 window: per row the lane's vertical smoothing
+    // s = p(-1) + 2 p + p(+1) and difference d = p(+1) - p(-1), packed, meet the
+    // neighbouring columns': gx = s(u+1) - s(u-1), gy = d(u-1) + 2 d(u) + d(u+1).
+    int a = 0, b = 0, c = 0;
+    {
+        int pm = col[(H - 4) * RB], pc = col[(H - 3) * RB];
+#pragma unroll
+        for (int v = -3; v <= 3; ++v) {
+            const int pn = col[(H + v + 1) * RB];
+            const int sv = pm + 2 * pc + pn, dv = pn - pm;
+            const uint32_t w = ((uint32_t)sv << 16) | (uint32_t)(dv + 512);
+            const uint32_t wl = __shfl_up_sync(0xFFFFFFFFu, w, 1), wr = __shfl_down_sync(0xFFFFFFFFu, w, 1);
+            const int gx = (int)(wr >> 16) - (int)(wl >> 16);
+            const int gy = (int)(wl & 0xFFFFu) + (int)(wr & 0xFFFFu) + 2 * dv - 1024;
+            a += gx * gx;
+            b += gy * gy;
+            c += gx * gy;
+            pm = pc;
+            pc = pn;
+        }
+    }
+    const bool in = u >= -3 && u <= 3;
+    a = __reduce_add_sync(0xFFFFFFFFu, in ? a : 0);
+    b = __reduce_add_sync(0xFFFFFFFFu, in ? b : 0);
+    c = __reduce_add_sync(0xFFFFFFFFu, in ? c : 0);
+
     if (lane == 0) {
-        const uint64_t okey = I.kkey[rank];
         const int64_t key = (int64_t)(okey ^ 0x8000000000000000ull);
         // response = key / kden * (1/(4*7*255))^4 in float: key as hi * 2^32 + lo
         // (two 32-bit conversions), times the host-rounded scale -- no float64 here
         // (the FP64 pipe was the orientation kernel's busiest unit).
         const float keyf = fmaf((float)(int32_t)(key >> 32), 4294967296.0f, (float)(uint32_t)key);
         of_keypoint k;
-        if (I.fx) {
-            k.x = I.fx[x];
-            k.y = I.fy[y];
-        } else {  // no tables: a level-0 image (scale^0 = 1; the allocation-free entry point)
-            k.x = (float)x;
-            k.y = (float)y;
-        }
+        k.x = kx;
+        k.y = ky;
         k.x_l = x;
         k.y_l = y;
-        k.level = I.level;
-        k.fast_score = I.score[(size_t)y * I.spitch + x] + (call->t_lo - 1);  // the map holds s - (t_lo - 1)
+        k.level = level;
+        k.fast_score = sc + (call->t_lo - 1);  // the map holds s - (t_lo - 1)
         k.response = keyf * call->resp_scale;
         k.angle = (m10 == 0 && m01 == 0) ? 0.0f : atan2f((float)m01, (float)m10);
         k.A = a;
@@ -140,11 +173,16 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
         k.m01 = m01;
         k.reserved = 0;
         k.key = key;
-        of_keypoint* dst = call->out + (size_t)I.frame * call->n_features + base + rank;
+        const size_t at = (size_t)frame * n_features + base + rank;
         const uint4* src = reinterpret_cast<const uint4*>(&k);
-        uint4* d4 = reinterpret_cast<uint4*>(dst);
+        uint4* d4 = reinterpret_cast<uint4*>(call->out + at);
 #pragma unroll
         for (int i = 0; i < 4; ++i) d4[i] = src[i];
+        if (call->host_out) {  // of_detect_host: the record into pinned host memory too
+            uint4* h4 = reinterpret_cast<uint4*>(call->host_out + at);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) h4[i] = src[i];
+        }
     }
 }
 

@@ -357,7 +357,7 @@ struct of_handle {
     int32_t* d_counts = nullptr;  // [0] of_detect's count, [4] device status word
     int n_sms = 0;
     int32_t* h_count = nullptr;   // pinned: [0] of_detect's count (written by the device), [4..] read-backs
-    of_keypoint* h_rec = nullptr;  // pinned: of_detect_host's records
+    of_keypoint* h_rec = nullptr;  // pinned: of_detect_host's records (written by the device)
     std::vector<Plan*> plans;
     Plan* last = nullptr;
     uint64_t clock = 0;
@@ -1189,10 +1189,10 @@ int ensure_learned(Plan* P) {
 
 // Point the plan at this call's frames and output, re-uploading the
 // descriptor header when anything changed.
-int bind_plan(of_handle* H, Plan* P, const of_frame* frames, of_keypoint* out, int32_t* counts) {
+int bind_plan(of_handle* H, Plan* P, const of_frame* frames, of_keypoint* out, int32_t* counts, of_keypoint* host) {
     const int nl = P->s.levels;
     const int nf = (int)P->frames.size();
-    bool changed = !P->bound || P->bound_out != out || P->bound_counts != counts;
+    bool changed = !P->bound || P->bound_out != out || P->bound_counts != counts || P->h_call.host_out != host;
     if (!changed)
         for (int f = 0; f < nf; ++f)
             if (!P->frames[f].copy && P->bound_src[f] != frames[f].img) changed = true;
@@ -1221,6 +1221,7 @@ int bind_plan(of_handle* H, Plan* P, const of_frame* frames, of_keypoint* out, i
     }
     P->h_call.out = out;
     P->h_call.counts = counts;
+    P->h_call.host_out = host;
     P->bound_out = out;
     P->bound_counts = counts;
     P->bound = true;
@@ -1245,7 +1246,7 @@ Plan* find_plan(of_handle* H, const std::vector<FrameKey>& frames, const Setting
 // the call's pointers.  Launches nothing.
 int prepare_batch(of_handle* H, const of_frame* frames, int n_frames, int levels, float scale,
                   int fast_t, float harris_k, int n_features, of_keypoint* out, int32_t* counts,
-                  Plan** outP) {
+                  Plan** outP, of_keypoint* host = nullptr) {
     if (!H) return fail(OF_ERR_ARG, "null handle");
     if (!frames || n_frames < 1) return fail(OF_ERR_ARG, "no frames");
     if (n_frames > H->p.max_batch)
@@ -1299,7 +1300,7 @@ int prepare_batch(of_handle* H, const of_frame* frames, int n_frames, int levels
         OF_CK(cudaMemcpy2DAsync(const_cast<uint8_t*>(I.img), I.pitch, frames[i].img, frames[i].pitch,
                                 frames[i].w, frames[i].h, cudaMemcpyDeviceToDevice, H->stream));
     }
-    const int rc = bind_plan(H, P, frames, out, counts);
+    const int rc = bind_plan(H, P, frames, out, counts, host);
     if (rc != OF_OK) return rc;
     *outP = P;
     return OF_OK;
@@ -1444,12 +1445,13 @@ int autotune_plan(of_handle* H, Plan* P, int reps) {
 }
 
 int run_batch(of_handle* H, const of_frame* frames, int n_frames, int levels, float scale,
-              int fast_t, float harris_k, int n_features, of_keypoint* out, int32_t* counts) {
+              int fast_t, float harris_k, int n_features, of_keypoint* out, int32_t* counts,
+              of_keypoint* host = nullptr) {
     if (!H) return fail(OF_ERR_ARG, "null handle");
     DeviceGuard dg(H->device);
     Plan* P = nullptr;
     int rc = prepare_batch(H, frames, n_frames, levels, scale, fast_t, harris_k, n_features, out,
-                           counts, &P);
+                           counts, &P, host);
     if (rc != OF_OK) return rc;
     rc = set_pmask(H, P, false);
     if (rc != OF_OK) return rc;
@@ -1472,23 +1474,21 @@ int run_batch(of_handle* H, const of_frame* frames, int n_frames, int levels, fl
     return OF_OK;
 }
 
-// One frame, waited for.  The orientation kernel writes the count to pinned
-// host memory, so the wait needs no copy of it; a wait that expired on the
-// device shows up as a negative count (the status word itself is read, and
-// cleared, only then).  host: the records too, by one copy before the wait.
+// One frame, waited for.  The orientation kernel writes the count (and for
+// `host` the records) to pinned host memory, so the wait needs no copies; a
+// wait that expired on the device shows up as a negative count (the status word
+// itself is read, and cleared, only then).
 int detect_one(of_handle* H, const uint8_t* img, int w, int h_px, int pitch, int levels, float scale, int fast_t,
                float harris_k, int n_features, of_keypoint* out, of_keypoint* host) {
     if (!H) return fail(OF_ERR_ARG, "null handle");
     of_frame F{img, w, h_px, pitch};
     // No features: no slot publishes a count, run_batch clears it on the device.
     int32_t* const counts = n_features > 0 ? H->h_count : H->d_counts;
-    const int rc = run_batch(H, &F, 1, levels, scale, fast_t, harris_k, n_features, out, counts);
+    const int rc = run_batch(H, &F, 1, levels, scale, fast_t, harris_k, n_features, out, counts, host ? H->h_rec : nullptr);
     if (rc != OF_OK) return rc;
     DeviceGuard dg(H->device);
     if (n_features <= 0)
         OF_CK(cudaMemcpyAsync(H->h_count, H->d_counts, sizeof(int32_t), cudaMemcpyDeviceToHost, H->stream));
-    else if (host)
-        OF_CK(cudaMemcpyAsync(H->h_rec, out, sizeof(of_keypoint) * n_features, cudaMemcpyDeviceToHost, H->stream));
     OF_CK(cudaStreamSynchronize(H->stream));
     const int n = *static_cast<volatile int32_t*>(H->h_count);
     if (n < 0 || n_features <= 0) {

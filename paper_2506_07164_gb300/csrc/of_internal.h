@@ -115,6 +115,7 @@ constexpr int PY_MAX_SMEM = 160 * 1024;
 // Per-call constants.
 struct Call {
     of_keypoint* out;     // n_frames * n_features records
+    of_keypoint* host_out;  // pinned host copy of the records, or null
     int32_t* counts;      // n_frames
     int32_t* status;      // device status word (OF_DEV_* bits), cleared before each call
     int64_t knum, kden;   // Harris k = knum / kden
