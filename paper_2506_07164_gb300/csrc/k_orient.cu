@@ -12,7 +12,11 @@
 //   - response = key / kden * (1 / (4*7*255))^4, as key (float) times the
 //     host-rounded float (1/(4*7*255))^4 / kden (relative error below 3e-7);
 //   - level-0 coordinates from the plan's tables (x * scale^level rounded once).
-// Records are level-major in rank order: the slot of a kept keypoint is the
+//   - rank: the list's own order, or (GROUPED) of a list grouped by key code,
+//     better codes first, the start of the code's run plus the better ones of the
+//     run (key descending, then y, then x ascending); the 32 entries around the
+//     keypoint usually hold the run, and are read beside its patch.
+// Records are level-major in rank order: the place of a kept keypoint is the
 // number of keypoints kept by the frame's earlier levels plus its rank.
 //
 // Bound by the latency of a warp's chain of loads (descriptors, position,
@@ -25,12 +29,14 @@
 
 #include "of_internal.h"
 #include "of_launch.cuh"
+#include "of_rank.cuh"
 
 namespace ofk {
 
 constexpr int OP_WORDS = 9;                   // aligned words that hold any 31 bytes
 constexpr int OP_SIZE = 31 * OP_WORDS;        // words of a patch
 
+template <bool GROUPED>
 __global__ void __launch_bounds__(ORIENT_WARPS * 32)
 k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin, int slot_end,
          const Call* __restrict__ call, const uint16_t* __restrict__ slot_img) {
@@ -53,7 +59,7 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
         }
     }
     const Img& I = imgs[lo];
-    const int rank = slot - I.slot0;
+    const int idx = slot - I.slot0;  // the keypoint in the image's list
     const int levels = call->levels, n_features = call->n_features;
     // Descriptor fields, read before the wait; lane l < levels: level l's counters.
     const uint8_t* const img = I.img;
@@ -67,26 +73,32 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
     const uint64_t* const kkey = I.kkey;
     const int R = call->radius, H = max(R, 4);  // H: rows and columns around the keypoint that are read
     pdl_wait();  // the kept keypoints
-    if (rank >= quota && slot != frame * n_features) return;
+    if (idx >= quota && slot != frame * n_features) return;
     const int kept_l = lctr ? lctr[1] : 0;
     const int kept = ctr[1];
-    const bool on = rank < quota;
-    const uint32_t yx = on ? kyx[rank] : 0u;  // issued beside the counts; unused beyond them
-    const uint64_t okey = on ? kkey[rank] : 0ull;
+    // The keypoint's entry (GROUPED: the 32 around it, itself in lane 16), issued beside
+    // the counts; unused beyond them.
+    const int wj = GROUPED ? idx - 16 + lane : idx;
+    const bool in_list = wj >= 0 && wj < quota;
+    const uint32_t wyx = in_list ? kyx[wj] : 0u;
+    const uint64_t wkey = in_list ? kkey[wj] : 0ull;
     // The frame's first slot publishes its keypoint count.
     if (slot == frame * n_features) {
         const int total = __reduce_add_sync(0xFFFFFFFFu, kept_l);
         // A detect-stage wait that expired leaves partial results: report it instead.
         if (lane == 0) call->counts[frame] = *call->status ? OF_ERR_TIMEOUT : total;
     }
-    if (rank >= quota || rank >= kept) return;
+    if (idx >= quota || idx >= kept) return;
     const int base = __reduce_add_sync(0xFFFFFFFFu, lane < level ? kept_l : 0);
 
+    const uint32_t yx = GROUPED ? __shfl_sync(0xFFFFFFFFu, wyx, 16) : wyx;
+    const uint64_t okey = GROUPED ? __shfl_sync(0xFFFFFFFFu, wkey, 16) : wkey;
     const int x = (int)(yx & 0xFFFFu), y = (int)(yx >> 16);
     // The patch, columns x - H .. x + H of rows y - H .. y + H, as aligned words
     // (images and pitches are multiples of 16 bytes; H <= border keeps it inside).
     uint32_t* const P = patch[threadIdx.x >> 5];
     const int sh = (x - H) & 3, nw = (sh + 2 * H + 4) >> 2, rows = 2 * H + 1;
+    int rank = idx;
     {
         const uint8_t* const q = img + (size_t)(y - H) * pitch + (x - H - sh);
         uint32_t v[OP_WORDS];
@@ -94,6 +106,45 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
         for (int k = 0; k < OP_WORDS; ++k) {
             const int i = lane + 32 * k, r = i / OP_WORDS, c = i - r * OP_WORDS;
             v[k] = r < rows && c < nw ? __ldg(reinterpret_cast<const uint32_t*>(q + (size_t)r * pitch) + c) : 0u;
+        }
+        if (GROUPED) {
+            // The run of this code in a window of 32 entries, and the better ones of it.
+            const uint32_t mine = key_code(okey);
+            auto count = [&](bool in, uint64_t k, uint32_t yx_k, uint32_t& run) {
+                const bool same = in && key_code(k) == mine;
+                run = __ballot_sync(0xFFFFFFFFu, same);
+                return __popc(__ballot_sync(0xFFFFFFFFu, same && rank_less(okey, ~yx, k, ~yx_k)));
+            };
+            uint32_t run;
+            int better = count(wj >= 0 && wj < kept, wkey, wyx, run);
+            const bool more = (run >> 31) != 0u;
+            int start = idx - 16 + __ffs((int)run) - 1;
+            // The run beyond the window: four more windows at a time to one side.
+            auto extend = [&](int w, int dir) {
+                uint64_t k[4];
+                uint32_t p[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int i = w + dir * 32 * j + lane;
+                    k[j] = i >= 0 && i < kept ? kkey[i] : 0ull;
+                    p[j] = i >= 0 && i < kept ? kyx[i] : 0u;
+                }
+                bool on = true;  // the run reaches the next window
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (on) {
+                        const int at = w + dir * 32 * j;
+                        better += count(at + lane >= 0 && at + lane < kept, k[j], p[j], run);
+                        if (dir < 0 && run) start = at + __ffs((int)run) - 1;
+                        on = dir < 0 ? (run & 1u) != 0u : (run >> 31) != 0u;
+                    }
+                return on;
+            };
+            if (run & 1u)
+                for (int w = idx - 48; w > -32 && extend(w, -1); w -= 128) {}
+            if (more)
+                for (int w = idx + 16; w < kept && extend(w, 1); w += 128) {}
+            rank = start + better;
         }
 #pragma unroll
         for (int k = 0; k < OP_WORDS; ++k)
@@ -190,7 +241,7 @@ void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_beg
                          void* stream, const uint16_t* slot_img, bool pdl) {
     if (slot_end <= slot_begin || n_img <= 0) return;
     const int blocks = (slot_end - slot_begin + ORIENT_WARPS - 1) / ORIENT_WARPS;
-    launch_chain(k_orient, blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream, pdl, 1, imgs, img_begin, n_img, slot_begin,
+    launch_chain(select_grouped(n_img) ? k_orient<true> : k_orient<false>, blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream, pdl, 1, imgs, img_begin, n_img, slot_begin,
                  slot_end, call, slot_img);
 }
 

@@ -1,6 +1,7 @@
 // Top-N per level: keep the n_l best NMS survivors of each (frame, level)
-// image in rank order -- Harris key descending, then y ascending, then x
-// ascending (Harris "screens" the FAST points, Sec. 1 and Sec. 3.2).
+// image -- Harris key descending, then y ascending, then x ascending (Harris
+// "screens" the FAST points, Sec. 1 and Sec. 3.2) -- as a list that is either
+// in rank order or grouped by key code, better codes first (select_grouped).
 //
 // Each candidate has a unique 96-bit rank word
 //   R = (key ^ 2^63) << 32 | ~((y << 16) | x),
@@ -8,40 +9,51 @@
 // found in one of two ways:
 //   - coarse pass: a 4096-bin histogram of a code of the key that is
 //     monotone in the key (sign, bit length and the next 5 bits of |key|)
-//     locates the bin b holding the n_l-th largest key; every candidate with
-//     code >= b is gathered (when they fit in shared memory) and sorted,
-//     and the first n_l are kept;
+//     locates the bin b holding the n_l-th largest key.  Sorted list: every
+//     candidate with code >= b is gathered (when they fit in shared memory)
+//     and sorted, and the first n_l are kept.  Grouped list: candidates with
+//     code > b go straight to the places that the counts of the better bins
+//     give them; those of bin b (at most SEL_BND) go through the same step
+//     once more, by the next 9 bits of |key|, and the few of that boundary
+//     are ranked by counting;
 //   - otherwise an MSB-first radix select over 8-bit digits of R (one
 //     shared-memory histogram per pass) fixes, digit by digit, the prefix of
 //     the n_l-th largest R, stopping as soon as every candidate that shares
 //     the fixed prefix is needed, and those candidates are gathered.
-// The gathered candidates are bitonic-sorted by R, descending; strides below
-// 64 run in a warp's registers (shuffles), the rest through shared memory.
+// Sorted lists are bitonic-sorted by R, descending; strides below 64 run in a
+// warp's registers (shuffles), the rest through shared memory.
 //
 // The scans are latency-bound: a 1080p level 0 holds ~43 k candidates, a 4K
 // one ~170 k, and one block scanning them twice set the whole stage's length
-// (41 us for one 1080p frame, 131 us at 4K; now 22 and 41 us, of which ~8 us
+// (41 us for one 1080p frame, 131 us at 4K; now 16 and 27 us, of which ~8 us
 // are the measurement's own launch and events).  So a cluster of C blocks
 // shares an image: every block histograms and gathers its part of the
 // candidates, block r sums bins [4096 r / C, ...) of all C histograms through
-// distributed shared memory, and the gathered entries go to the first block,
-// which sorts.  Every scan keeps SEL_UNROLL 16-byte loads (two keys) in flight
-// per thread; the positions of the gathered candidates only are read.  Images
-// with at most SEL_SOLO candidates are left to the first block.
+// distributed shared memory, and the gathered entries go to the first block.
+// Every scan keeps SEL_UNROLL 16-byte loads (two keys) in flight per thread;
+// the positions of the gathered candidates only are read.  Images with few
+// candidates are left to the first block.  The sort is one block's chain of
+// barriers (of 1000 keypoints: 5 of 21 us with one 1080p frame, of 8192: 35 of
+// 49), while the orientation kernel has a warp for each keypoint: it finds the
+// ranks of grouped lists.
 #include <cuda_runtime.h>
 
 #include <mutex>
 
 #include "of_internal.h"
 #include "of_launch.cuh"
+#include "of_rank.cuh"
 
 namespace ofk {
 
 constexpr int SEL_UNROLL = 4;   // candidates loaded per thread before use
 constexpr int SEL_BINS = 4096;  // coarse-pass histogram bins
 constexpr int SEL_SOLO = 4096;  // candidates one block scans alone (one round of its loads)
+constexpr int SEL_SOLO_G = 8192;  // ... of a grouped list (no sort beside it)
 constexpr int SEL_MIN_SORT = 64;  // entries of the smallest sort (one warp's registers)
 constexpr int SEL_MAX_DYN = 192 * 1024;
+constexpr int SEL_BND = 2048;   // grouped lists: candidates of the boundary bin the first block takes
+constexpr int SEL_GROUPED = 32;  // images of a launch up to which the lists stay grouped
 
 struct SelState {
     uint64_t pre_hi, msk_hi;
@@ -50,22 +62,14 @@ struct SelState {
     int coarse, code_b, n_take;
 };
 
-__device__ __forceinline__ bool rank_less(uint64_t ah, uint32_t al, uint64_t bh, uint32_t bl) {
-    return ah < bh || (ah == bh && al < bl);
-}
-
-// f(x) for 0 <= x < 2^63: 0 for x = 0, else 32 * bitlength(x) + the 5 bits
-// after the leading one -- non-decreasing in x, at most 2047.
-__device__ __forceinline__ uint32_t mag_code(uint64_t x) {
-    if (x == 0ull) return 0u;
+// The 9 bits of the magnitude after the code's, for keys of one code:
+// non-decreasing in key.
+__device__ __forceinline__ uint32_t fine_code(uint64_t u) {
+    const bool pos = (u >> 63) != 0;
+    const uint64_t x = pos ? u & 0x7FFFFFFFFFFFFFFFull : u ^ 0x7FFFFFFFFFFFFFFFull;
     const int L = 64 - __clzll((long long)x);
-    return 32u * (uint32_t)L + (uint32_t)((x << (64 - L)) >> 58 & 31ull);
-}
-
-// Code of the order-preserving key u = key ^ 2^63, non-decreasing in key:
-// keys >= 0 map to 2048 + f(key), keys < 0 to 2047 - f(-key - 1).
-__device__ __forceinline__ uint32_t key_code(uint64_t u) {
-    return (u >> 63) ? 2048u + mag_code(u & 0x7FFFFFFFFFFFFFFFull) : 2047u - mag_code(u ^ 0x7FFFFFFFFFFFFFFFull);
+    const uint32_t f = L > 6 ? (uint32_t)((x << (70 - L)) >> 55) : 0u;
+    return pos ? f : 511u - f;
 }
 
 // ---- cluster primitives (shared::cluster addresses of the other blocks' shared memory)
@@ -170,7 +174,7 @@ __device__ __forceinline__ void bitonic_sort(uint64_t* skey, uint32_t* syx, int 
     }
 }
 
-template <int C>
+template <int C, bool GROUPED>
 __global__ void __launch_bounds__(SELECT_THREADS)
 k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_cap) {
     extern __shared__ __align__(16) uint8_t dyn[];
@@ -179,6 +183,9 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
     __shared__ uint32_t slice_sum[C];  // candidates in each block's slice of the bins
     __shared__ SelState st;
     __shared__ int s_cnt;
+    __shared__ uint64_t bkey[GROUPED ? SEL_BND : 1];  // the boundary bin's candidates (first block)
+    __shared__ uint32_t byx[GROUPED ? SEL_BND : 1];
+    __shared__ int s_bnd, s_left, s_fine;  // their number, that of the fine boundary bin, its code
 
     const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;  // block's place in its image's cluster
     const Img& I = imgs[blockIdx.x / C];
@@ -194,7 +201,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         return;
     }
     // Blocks that share the scan: all of the cluster, or only the first.
-    const bool shared = C > 1 && n > q && n > SEL_SOLO;
+    const bool shared = C > 1 && (GROUPED || n > q) && n > (GROUPED ? SEL_SOLO_G : SEL_SOLO);
     if (rank != 0 && !shared) return;
     const int parts = shared ? C : 1;
     const int m = min(n, q);
@@ -208,16 +215,17 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         st.msk_lo = 0;
         st.need = q;
         st.done = (n <= q);
-        st.coarse = 0;
-        st.code_b = 0;
+        st.coarse = GROUPED && n <= q;  // a grouped list of everything: no boundary bin
+        st.code_b = GROUPED && n <= q ? -1 : 0;
         st.n_take = m;
         s_cnt = 0;
+        s_bnd = 0;
     }
     __syncthreads();
 
     // This block's candidate pairs: first, step (in pairs of keys).
     const int i_first = rank * SELECT_THREADS + tid, i_step = parts * SELECT_THREADS;
-    if (n > q) {
+    if (GROUPED || n > q) {
         // Coarse pass: histogram of the key code, two keys per 16-byte load
         // (the candidate arrays start on 256-byte boundaries).
         const ulonglong2* ck2 = reinterpret_cast<const ulonglong2*>(I.ckey);
@@ -282,23 +290,35 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
             cluster_sync_all();
             for (int c = rank + 1; c < C; ++c) above += (int)slice_sum[c];
         }
-        if (above < q && above + own >= q) {  // exactly one thread: the n_l-th best key is in its bins
+        if (GROUPED) {
+            // Each bin's count becomes, in the first block, the place of its first candidate.
+            int place = above;
+#pragma unroll
+            for (int j = PER1 - 1; j >= 0; --j)
+                if (j < per) {
+                    if (shared) st_rank(map_rank(&hist[b0 + j], 0), (uint32_t)place);
+                    else hist[b0 + j] = (uint32_t)place;
+                    place += bins[j];
+                }
+        }
+        if (n > q && above < q && above + own >= q) {  // exactly one thread: the n_l-th best key is in its bins
             int cum = above;
 #pragma unroll
             for (int j = PER1 - 1; j >= 0; --j) {
                 if (j < per) {
                     const int h = bins[j];
                     if (cum < q && cum + h >= q) {
-                        const int coarse = cum + h <= sort_cap;
+                        const int coarse = GROUPED ? h <= SEL_BND : cum + h <= sort_cap;
+                        const int take = GROUPED ? cum : cum + h;
                         for (int c = 0; c < parts; ++c) {
                             const int to = shared ? c : rank;
                             if (to == rank) {
                                 st.code_b = b0 + j;
-                                st.n_take = cum + h;
+                                st.n_take = take;
                                 st.coarse = coarse;
                             } else {
                                 st_rank(map_rank(&st.code_b, to), (uint32_t)(b0 + j));
-                                st_rank(map_rank(&st.n_take, to), (uint32_t)(cum + h));
+                                st_rank(map_rank(&st.n_take, to), (uint32_t)take);
                                 st_rank(map_rank(&st.coarse, to), (uint32_t)coarse);
                             }
                         }
@@ -309,6 +329,110 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         }
         if (shared) cluster_sync_all();
         else __syncthreads();
+    }
+
+    auto keep = [&](int pos, uint64_t key, uint32_t yx) {
+        I.kkey[pos] = key;
+        I.kyx[pos] = yx;
+    };
+    if (GROUPED && st.coarse) {  // the same in all blocks
+        // Gather: the better bins to their places, the boundary bin to the first block.
+        const int code_b = st.code_b;
+        const ulonglong2* ck2 = reinterpret_cast<const ulonglong2*>(I.ckey);
+        const int n2 = (n + 1) >> 1;
+        // A place of the first block's counter.
+        auto take = [&](void* counter) {
+            return shared ? atomic_add_rank(map_rank(counter, 0), 1) : atomicAdd(static_cast<int*>(counter), 1);
+        };
+        for (int i0 = i_first; i0 < n2; i0 += SEL_UNROLL * i_step) {
+            ulonglong2 v[SEL_UNROLL];
+#pragma unroll
+            for (int k = 0; k < SEL_UNROLL; ++k) {
+                const int i = i0 + k * i_step;
+                if (2 * i + 1 < n) v[k] = __ldg(ck2 + i);
+                else v[k] = make_ulonglong2(2 * i < n ? __ldg(I.ckey + 2 * i) : 0ull, 0ull);
+            }
+#pragma unroll
+            for (int k = 0; k < SEL_UNROLL; ++k) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int i = 2 * (i0 + k * i_step) + h;
+                    if (i >= n) continue;
+                    const uint64_t key = h ? v[k].y : v[k].x;
+                    const int code = (int)key_code(key);
+                    if (code < code_b) continue;
+                    const uint32_t yx = __ldg(I.cyx + i);
+                    if (code > code_b) {
+                        const int pos = take(&hist[code]);
+                        if (pos < q) keep(pos, key, yx);
+                    } else {
+                        const int pos = take(&s_bnd);  // at most SEL_BND of them
+                        if (pos < SEL_BND) {
+                            if (shared) {
+                                st_rank64(map_rank(&bkey[pos], 0), key);
+                                st_rank(map_rank(&byx[pos], 0), yx);
+                            } else {
+                                bkey[pos] = key;
+                                byx[pos] = yx;
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        if (shared) cluster_sync_all();
+        else __syncthreads();
+        if (rank != 0) return;
+        // The boundary bin: its best fill the rest, found by the fine codes.
+        static_assert(SELECT_THREADS == 512, "one fine code per thread");
+        const int nb = min(s_bnd, SEL_BND), above = st.n_take, need = q - above;
+        if (nb == 0) {
+            if (tid == 0) I.ctr[1] = above;
+            return;
+        }
+        hist[tid] = 0u;
+        if (tid == 0) {
+            s_left = 0;
+            s_cnt = above;
+        }
+        __syncthreads();
+        for (int i = tid; i < nb; i += SELECT_THREADS) atomicAdd(&hist[fine_code(bkey[i])], 1u);
+        __syncthreads();
+        const int own = (int)hist[tid];
+        int v = own;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int t = __shfl_down_sync(0xFFFFFFFFu, v, off);
+            if (lane + off < 32) v += t;
+        }
+        if (lane == 0) wsum[warp] = (uint32_t)v;
+        __syncthreads();
+        int better = v - own;
+        for (int w = warp + 1; w < SELECT_THREADS / 32; ++w) better += (int)wsum[w];
+        if (better < need && better + own >= need) s_fine = tid | better << 9;  // exactly one thread
+        __syncthreads();
+        const int fine = s_fine & 511, sure = s_fine >> 9;  // candidates above the fine boundary bin
+        uint16_t* const left = reinterpret_cast<uint16_t*>(hist);  // its candidates' places in the list
+        for (int i = tid; i < nb; i += SELECT_THREADS) {
+            const int c = (int)fine_code(bkey[i]);
+            if (c > fine) {
+                const int pos = atomicAdd(&s_cnt, 1);
+                keep(pos, bkey[i], byx[i]);
+            } else if (c == fine) {
+                left[atomicAdd(&s_left, 1)] = (uint16_t)i;
+            }
+        }
+        __syncthreads();
+        const int nl = s_left;
+        for (int i = tid; i < nl; i += SELECT_THREADS) {
+            const uint64_t key = bkey[left[i]];
+            const uint32_t yx = byx[left[i]];
+            int place = above + sure;
+            for (int j = 0; j < nl; ++j) place += rank_less(key, ~yx, bkey[left[j]], ~byx[left[j]]);
+            if (place < q) keep(place, key, yx);
+        }
+        if (tid == 0) I.ctr[1] = q;
+        return;
     }
 
     // The radix select (and the gather without a coarse bin) is the first block's alone.
@@ -359,6 +483,45 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
             }
             __syncthreads();
         }
+    }
+
+    if (GROUPED) {
+        // Keep the better bins whole, and of bin b every candidate whose masked rank
+        // word is >= the fixed prefix.  The places of the digits' histogram were lost:
+        // count the bins again.
+        const uint64_t pre_hi = st.pre_hi, msk_hi = st.msk_hi;
+        const uint32_t pre_lo = st.pre_lo, msk_lo = st.msk_lo;
+        const int code_b = st.code_b;
+        for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) hist[i] = 0u;
+        if (tid == 0) s_cnt = st.n_take;
+        __syncthreads();
+        for (int i = tid; i < n; i += SELECT_THREADS) {
+            const int c = (int)key_code(__ldg(I.ckey + i));
+            if (c > code_b) atomicAdd(&hist[c], 1u);
+        }
+        __syncthreads();
+        if (tid == 0) {  // a rare path: one thread turns the counts into places
+            uint32_t place = 0u;
+            for (int i = SEL_BINS - 1; i > code_b; --i) {
+                const uint32_t h = hist[i];
+                hist[i] = place;
+                place += h;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < n; i += SELECT_THREADS) {
+            const uint64_t hi = __ldg(I.ckey + i);
+            const uint32_t yx = __ldg(I.cyx + i);
+            const int c = (int)key_code(hi);
+            const uint64_t mh = hi & msk_hi;
+            if (c < code_b || (c == code_b && !(mh > pre_hi || (mh == pre_hi && (~yx & msk_lo) >= pre_lo)))) continue;
+            const int pos = c > code_b ? (int)atomicAdd(&hist[c], 1u) : atomicAdd(&s_cnt, 1);
+            if (pos < q) {
+                keep(pos, hi, yx);
+            }
+        }
+        if (tid == 0) I.ctr[1] = q;
+        return;
     }
 
     // Gather: code >= b (coarse; each block its part of the candidates), else
@@ -470,27 +633,37 @@ int select_smem_bytes(int max_quota) {
     return select_sort_cap(max_quota) * (int)(sizeof(uint64_t) + sizeof(uint32_t));
 }
 
-template <int C>
+// Ranking in the orientation kernel costs its warps a sixth more, which a launch
+// of many keypoints pays and one of few images does not see.  Select + orientation
+// stages, sorted / grouped lists, 8-level 1080p frames with 1000 keypoints each:
+// 1 frame (8 images) 24.7 / 24.1 us, 2 28.7 / 24.7, 4 (32 images) 33.7 / 31.0,
+// 8 (64) 40.6 / 39.3, 16 (128) 49.3 / 58.2; with 8192: 61.6 / 30.8, 67.6 / 45.0,
+// 82.7 / 71.2, 116 / 119, 186 / 217.
+bool select_grouped(int n_img) { return n_img <= SEL_GROUPED; }
+
+template <int C, bool GROUPED>
 static void launch_select_t(const Img* imgs, int n_img, const Call* call, int mq, cudaStream_t st, bool pdl) {
-    launch_chain(k_select<C>, n_img * C, SELECT_THREADS, select_smem_bytes(mq), st, pdl, C, imgs, call,
-                 select_sort_cap(mq));
+    launch_chain(k_select<C, GROUPED>, n_img * C, SELECT_THREADS, GROUPED ? 0 : select_smem_bytes(mq), st, pdl, C, imgs, call,
+                 GROUPED ? 0 : select_sort_cap(mq));
 }
 
 // Blocks per image, by the images of the launch.  A cluster shortens the scan
 // of the largest image, which sets the launch's length, until its blocks no
 // longer fit the chip beside each other (four 512-thread blocks on each of
 // 152 SMs): 8 while every image has SMs of its own, 4 up to 128 images, 2 up
-// to 304.  Measured stage times (1080p, 8 levels; 1 / 2 / 4 / 8 blocks): 8
-// images 41 / 33 / 27 / 22 us, 32 images 43 / 35 / 26 / 28, 128 images 49 / 39
-// / 35 / 41, 304 images 64 / 57 / 64 / 84, 1024 images 97 / 119 / 149 / 218.
+// to 304.  Measured stage times of sorted lists (1080p, 8 levels; 1 / 2 / 4 / 8
+// blocks): 8 images 41 / 33 / 27 / 22 us, 32 images 43 / 35 / 26 / 28, 128
+// images 49 / 39 / 35 / 41, 304 images 64 / 57 / 64 / 84, 1024 images 97 / 119
+// / 149 / 218.
 void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream, bool pdl) {
     if (n_img <= 0) return;
     const int mq = max_quota > 0 ? max_quota : 1;
     const cudaStream_t st = (cudaStream_t)stream;
-    if (n_img <= 16) launch_select_t<8>(imgs, n_img, call, mq, st, pdl);
-    else if (n_img <= 128) launch_select_t<4>(imgs, n_img, call, mq, st, pdl);
-    else if (n_img <= 304) launch_select_t<2>(imgs, n_img, call, mq, st, pdl);
-    else launch_select_t<1>(imgs, n_img, call, mq, st, pdl);
+    if (n_img <= 16) launch_select_t<8, true>(imgs, n_img, call, mq, st, pdl);
+    else if (select_grouped(n_img)) launch_select_t<4, true>(imgs, n_img, call, mq, st, pdl);
+    else if (n_img <= 128) launch_select_t<4, false>(imgs, n_img, call, mq, st, pdl);
+    else if (n_img <= 304) launch_select_t<2, false>(imgs, n_img, call, mq, st, pdl);
+    else launch_select_t<1, false>(imgs, n_img, call, mq, st, pdl);
 }
 
 // The limit is a per-device attribute of the kernel shared by every handle,
@@ -503,11 +676,10 @@ void set_select_smem_limit(int bytes) {
     if (cudaGetDevice(&dev) != cudaSuccess) return;
     std::lock_guard<std::mutex> lock(mu);
     if (dev >= 0 && dev < 64 && bytes <= limit[dev]) return;
-    const bool ok =
-        cudaFuncSetAttribute(k_select<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
-        cudaFuncSetAttribute(k_select<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
-        cudaFuncSetAttribute(k_select<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess &&
-        cudaFuncSetAttribute(k_select<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const bool ok = cudaFuncSetAttribute(k_select<1, false>, attr, bytes) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_select<2, false>, attr, bytes) == cudaSuccess &&
+                    cudaFuncSetAttribute(k_select<4, false>, attr, bytes) == cudaSuccess;
     if (ok && dev >= 0 && dev < 64) limit[dev] = bytes;
 }
 

@@ -60,7 +60,7 @@ struct Img {
     uint32_t* cell;      // per-cell "has a strong pixel" flags, ncx * ncy
     uint64_t* ckey;      // candidates: order-preserving key (signed key ^ 2^63)
     uint32_t* cyx;       // candidates: (y << 16) | x
-    uint64_t* kkey;      // kept (ranked) keys
+    uint64_t* kkey;      // kept keys: ranked, or grouped by code (select_grouped)
     uint32_t* kyx;       // kept positions
     int32_t* ctr;        // [0] candidate count, [1] kept count, [2] overflow flag
     int32_t w, h, pitch, spitch;
@@ -200,6 +200,9 @@ void launch_nms_warp(const Img* imgs, const uint2* items, int n_tiles, const CUt
                      const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo, int border, int cell,
                      int rows, int grid, int order, void* stream, bool apply, bool pdl = false);
 int nms_warp_blocks_per_sm();
+// Whether the top-N kernel leaves the kept lists of a launch of n_img images grouped by
+// key code for the orientation kernel to rank (else it sorts them).
+bool select_grouped(int n_img);
 void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream, bool pdl = false);
 void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream);
 // Slots [slot_begin, slot_end) of images [img_begin, img_begin + n_img) (one frame group).

@@ -58,3 +58,23 @@ def test_radix_path_in_a_cluster():
         for f in FIELDS:
             np.testing.assert_array_equal(got[f], ora[f], err_msg=f)
         det.close()
+
+
+# Grouped lists (up to 32 images; shared scans of 8 and of 4 blocks) and sorted ones, with
+# the ties of a tiled image: runs of one key code beyond the 32 entries read around a
+# keypoint, and beyond the 128 read next.
+@pytest.mark.parametrize("frames", [1, 17, 33])
+@pytest.mark.parametrize("n", [1, 31, 1000, 4097, 8192])
+def test_grouped_and_sorted_lists(frames, n):
+    tile = synth.scene(64, 64, 9, n_rect=6, n_checker=1, noise_sigma=8.0)
+    img = np.tile(tile, (12, 16))
+    dev = torch.from_numpy(img).cuda()
+    det = ofg.Detector(img.shape[1], img.shape[0], max_levels=1, max_features=n, max_batch=frames)
+    det.detect_batch([dev] * frames, levels=1, fast_t=3, n_features=n)
+    torch.cuda.synchronize()
+    ora = oracle.detect(img, levels=1, fast_t=3, n_features=n)
+    for got in det.batch_results(frames, n):
+        assert len(got) == len(ora) == n
+        for f in FIELDS:
+            np.testing.assert_array_equal(got[f], ora[f], err_msg=f)
+    det.close()
