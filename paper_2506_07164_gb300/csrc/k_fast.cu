@@ -258,6 +258,7 @@ k_fast(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
 
     const int tid = threadIdx.x;
     const bool cells = FLAGS && t_hi != t_lo;
+    pdl_trigger();
     if (tid == 0) {
         mbar_init(&mbar[0], 1);
         mbar_init(&mbar[1], 1);

@@ -245,8 +245,8 @@ void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_beg
                  slot_end, call, slot_img);
 }
 
-void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream) {
-    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, stream, nullptr, false);
+void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream, bool pdl) {
+    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, stream, nullptr, pdl);
 }
 
 // ---------------------------------------------------------------- inspect
