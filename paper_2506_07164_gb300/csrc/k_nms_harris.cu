@@ -428,14 +428,23 @@ k_nms_harris(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
 // APPLY: the maps hold s(p) - (t_lo - 1) where s(p) >= t_lo (FAST's output)
 // and the cell flags are set.  Each staged score word becomes S(p) in
 // registers as it is read (bytes below t_hi cleared in flagged cells), so
-// the maps need no threshold pass.  A lane thresholds its own word and the
-// halo word of the warp's edge (lane 0: columns X0-4..X0-1, lane 31:
-// X0+128..X0+131); the 3x3 test's outer neighbours come from lanes +-1.
-// A chunk of NW_CHUNK output rows reads 8 new staged rows, which lie in at
-// most two cell rows for cells of 8 or more rows.  Otherwise the maps hold
-// S(p).  Bytes outside the detect region, and outside the proposed tiles of
-// an image that has them, are zeroed in the staged score box first (in the
-// words of lanes whose word is not wholly inside).
+// the maps need no threshold pass.  A lane thresholds its own word; the one
+// pixel beyond each end of a row is prepared once per tile, a row per lane,
+// and the 3x3 test's outer neighbours come from lanes +-1.  The cell row's
+// flags are loaded when the rows enter it: the 8 new staged rows of a chunk of
+// NW_CHUNK output rows lie in at most two cell rows for cells of 8 or more.
+// Otherwise the maps hold S(p).  Bytes outside the detect region, and outside
+// the proposed tiles of an image that has them, are zeroed in the staged score
+// box first (in the words of lanes whose word is not wholly inside).
+//
+// Bound by instruction issue (~5200 per tile at first, 83 % of the slots): half
+// as many warps again, with one buffer for both boxes, changed nothing (1154
+// against 1132 us for 128 1080p frames), fewer instructions per row did: halo
+// words no longer read and thresholded by every lane 1132 -> 1064 us; halo
+// pixels stored as the test takes them, bits collected by shifting 1034; the
+// survivors' places by one shared atomic per lane instead of a warp scan 1017;
+// flags carried over the chunks 1002.  Harris sums in packed floats (half the
+// multiply-adds, twice the registers): no gain.
 
 constexpr int NW_QCAP = TILE_W * TILE_H / 4;             // strict maxima are never adjacent
 constexpr int NW_SBUF = (S_BOX + 127) / 128 * 128;       // 5504
@@ -494,6 +503,7 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
     extern __shared__ __align__(128) uint8_t nw_raw[];
     uint8_t* const dyn = nw_raw + ((128u - (smem_u32(nw_raw) & 127u)) & 127u);
     __shared__ __align__(8) uint64_t mbar[NW_WARPS][2];  // [0] score box, [1] image box
+    __shared__ int nq[NW_WARPS];                         // queued survivors
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint8_t* const sS = dyn + w * NW_BYTES;
     uint8_t* const sI = sS + NW_SBUF;
@@ -503,6 +513,7 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
         mbar_init(&mbar[w][0], 1);
         mbar_init(&mbar[w][1], 1);
         fence_barrier_init();
+        nq[w] = 0;
     }
     __syncwarp();
     const int nw = gridDim.x * NW_WARPS, gw = w * gridDim.x + blockIdx.x;
@@ -566,7 +577,7 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
             const int xh = lane == 0 ? X0 - 4 : X0 + TILE_W;  // the halo word (used by lanes 0 and 31)
             const int nrows = min(rows, ry1 - Y0);
             const uint8_t* const srow = sS + HALO_X + 4 * lane;
-            const int hoff = xh - xc;
+            const uint8_t* const hrow = sS + HALO_X - 4;
             // Zero the staged bytes outside the detect region, and outside the
             // proposed tiles of an image that has them, in the words the 3x3 test
             // reads (staged rows 0 .. nrows + 1; a lane's word, and the halo word of
@@ -599,20 +610,34 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
                 if (lane == 0 || lane == 31) sanitize(xh, xh - X0);
                 __syncwarp();
             }
-            WordCells wc_c{0u, 0u, 0}, wc_h{0u, 0u, 0};
             const uint32_t* cellp = I.cell;
-            const int ncx = I.ncx;
-            if (APPLY) {
-                wc_c = word_cells(xc, range_mask4(xc, rx0, rx1), rx0, rx0, cell, cell_magic);
-                wc_h = word_cells(xh, range_mask4(xh, rx0, rx1), rx0, rx0, cell, cell_magic);
-            }
-            // Flag masks of staged row iy (APPLY): cell row of iy (rows outside the region hold zeros).
-            auto flags_of = [&](int iy, uint32_t& fc, uint32_t& fh) {
+            const int ncx = I.ncx, ncy = I.ncy;
+            // Flag mask of a word's bytes in staged row iy (APPLY; rows outside the region hold zeros).
+            auto flags_of = [&](const WordCells& wc, int iy) {
                 const int cy = (int)__umulhi((uint32_t)max(iy - ry0, 0), cell_magic);
-                const uint32_t* crow = cellp + (size_t)min(cy, I.ncy - 1) * ncx;
-                fc = word_flags(wc_c, crow);
-                fh = word_flags(wc_h, crow);
+                return word_flags(wc, cellp + (size_t)min(cy, ncy - 1) * ncx);
             };
+            WordCells wc{0u, 0u, 0};
+            if (APPLY) wc = word_cells(xc, range_mask4(xc, rx0, rx1), rx0, rx0, cell, cell_magic);
+            // S of the tile's halo pixels, a row per lane: column X0 - 1 in the upper
+            // half and X0 + 128 in the lower half of the word at X0 - 4.
+            {
+                WordCells wl{0u, 0u, 0}, wr{0u, 0u, 0};
+                if (APPLY) {
+                    wl = word_cells(X0 - 4, range_mask4(X0 - 4, rx0, rx1), rx0, rx0, cell, cell_magic);
+                    wr = word_cells(X0 + TILE_W, range_mask4(X0 + TILE_W, rx0, rx1), rx0, rx0, cell, cell_magic);
+                }
+                for (int k = lane; k < nrows + 2; k += 32) {
+                    uint32_t* p = reinterpret_cast<uint32_t*>(sS + k * SROW + HALO_X - 4);
+                    uint32_t vl = p[0], vr = p[TILE_W / 4 + 1];
+                    if (APPLY && (vl | vr)) {
+                        vl = threshold_word<SMALL_T>(vl, flags_of(wl, Y0 - 1 + k), th);
+                        vr = threshold_word<SMALL_T>(vr, flags_of(wr, Y0 - 1 + k), th);
+                    }
+                    p[0] = (vl >> 24) << 16 | (vr & 0xFFu);
+                }
+                __syncwarp();
+            }
             // Staged row k (image row Y0 - 1 + k) reduced to what the 3x3 test takes
             // from it for the pixel pairs (x, x+2) and (x+1, x+3) in 16-bit lanes: the
             // centres, the maxima of the left and right neighbours (the centre row's
@@ -620,22 +645,19 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
             struct Row3 {
                 uint32_t ctr[2], side[2], all[2];
             };
-            auto load_row = [&](int k, uint32_t fc, uint32_t fh) {
+            auto load_row = [&](int k, uint32_t fc) {
                 const uint8_t* row = srow + k * SROW;
                 uint32_t vc = *reinterpret_cast<const uint32_t*>(row);
-                uint32_t vh = *reinterpret_cast<const uint32_t*>(row + hoff);
-                if (APPLY) {
-                    vc = threshold_word<SMALL_T>(vc, fc, th);
-                    vh = threshold_word<SMALL_T>(vh, fh, th);
-                }
-                uint32_t vm = __shfl_up_sync(0xFFFFFFFFu, vc, 1);
-                uint32_t vq = __shfl_down_sync(0xFFFFFFFFu, vc, 1);
-                if (lane == 0) vm = vh;
-                if (lane == 31) vq = vh;
-                const uint32_t h0 = __byte_perm(vm, vc, 0x0503) & 0x00FF00FFu;  // (x-1, x+1)
-                const uint32_t h1 = __byte_perm(vc, 0u, 0x4240);                 // (x, x+2)
-                const uint32_t h2 = __byte_perm(vc, 0u, 0x4341);                 // (x+1, x+3)
-                const uint32_t h3 = __byte_perm(vc, vq, 0x0402) & 0x00FF00FFu;  // (x+2, x+4)
+                const uint32_t vh = *reinterpret_cast<const uint32_t*>(hrow + k * SROW);
+                if (APPLY) vc = threshold_word<SMALL_T>(vc, fc, th);
+                const uint32_t h1 = __byte_perm(vc, 0u, 0x4240);    // (x, x+2)
+                const uint32_t h2 = __byte_perm(vc, 0u, 0x4341);    // (x+1, x+3)
+                uint32_t hl = __shfl_up_sync(0xFFFFFFFFu, h2, 1);   // (x-3, x-1)
+                uint32_t hr = __shfl_down_sync(0xFFFFFFFFu, h1, 1);  // (x+4, x+6)
+                if (lane == 0) hl = vh;
+                if (lane == 31) hr = vh;
+                const uint32_t h0 = __byte_perm(hl, h2, 0x5432);  // (x-1, x+1)
+                const uint32_t h3 = __byte_perm(h1, hr, 0x5432);  // (x+2, x+4)
                 Row3 o;
                 o.ctr[0] = h1;
                 o.ctr[1] = h2;
@@ -646,49 +668,43 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
                 return o;
             };
             Row3 ra, rb;  // staged rows of the output row's upper neighbours and of the row itself
-            {
-                uint32_t fc = 0u, fh = 0u;
-                if (APPLY) flags_of(Y0 - 1, fc, fh);
-                ra = load_row(0, fc, fh);
-                if (APPLY) flags_of(Y0, fc, fh);
-                rb = load_row(1, fc, fh);
-            }
+            // The flag mask of the cell row reached, and the first row of the next one.
+            uint32_t fa = 0u;
+            int yb = 0;
+            auto enter = [&](int iy) {
+                fa = flags_of(wc, iy);
+                yb = ry0 + ((int)__umulhi((uint32_t)max(iy - ry0, 0), cell_magic) + 1) * cell;
+            };
+            if (APPLY) enter(Y0 - 1);
+            ra = load_row(0, fa);
+            if (APPLY && Y0 >= yb) enter(Y0);
+            rb = load_row(1, fa);
 #pragma unroll 1
             for (int r0 = 0; r0 < nrows; r0 += NW_CHUNK) {
-                // Staged rows r0+2 .. r0+9: cell rows A and (from row yb on) B.
-                uint32_t fa_c = 0u, fa_h = 0u, fb_c = 0u, fb_h = 0u;
-                int yb = 0;
-                if (APPLY) {
-                    const int iy0 = Y0 + 1 + r0;
-                    flags_of(iy0, fa_c, fa_h);
-                    const int cya = (int)__umulhi((uint32_t)max(iy0 - ry0, 0), cell_magic);
-                    yb = ry0 + (cya + 1) * cell;
-                    if (yb <= iy0 + NW_CHUNK - 1) flags_of(yb, fb_c, fb_h);
-                }
+                // Staged rows r0+2 .. r0+9 (image rows from Y0+1+r0): the current cell row
+                // and, from row yb on, the next one.
+                const bool two = APPLY && yb < Y0 + 1 + r0 + NW_CHUNK;
+                const uint32_t fb = two ? flags_of(wc, yb) : 0u;
                 // Survivor bits: byte j (pair j >> 1, lane half j & 1) bit r (chunk row r).
                 uint32_t smask = 0u;
 #pragma unroll
                 for (int r = 0; r < NW_CHUNK; ++r) {
-                    if (r0 + r >= nrows) break;
-                    const bool b_row = APPLY && Y0 + 1 + r0 + r >= yb;
-                    const Row3 rc = load_row(r0 + r + 2, b_row ? fb_c : fa_c, b_row ? fb_h : fa_h);
+                    const Row3 rc = load_row(r0 + r + 2, APPLY && Y0 + 1 + r0 + r >= yb ? fb : fa);
                     // Lane bit 15 set when the centre > its 8 neighbours (values <= 255).
                     const uint32_t k0 = rb.ctr[0] + 0x7FFF7FFFu - __vimax3_u16x2(ra.all[0], rb.side[0], rc.all[0]);
                     const uint32_t k1 = rb.ctr[1] + 0x7FFF7FFFu - __vimax3_u16x2(ra.all[1], rb.side[1], rc.all[1]);
-                    smask |= (__byte_perm(k0, k1, 0x7531) & 0x80808080u) >> (7 - r);
+                    smask = (smask >> 1) | (__byte_perm(k0, k1, 0x7531) & 0x80808080u);
                     ra = rb;
                     rb = rc;
                 }
-                // Append the chunk's survivors: a warp scan of the per-lane counts.
-                const int mine = __popc(smask);
-                int incl = mine;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                    if (lane >= o) incl += v;
+                if (two) {
+                    fa = fb;
+                    yb += cell;
                 }
-                int slot = n + incl - mine;
-                n += __shfl_sync(0xFFFFFFFFu, incl, 31);
+                // Rows beyond the tile's (of a chunk that it ends in) hold no survivors.
+                if (nrows - r0 < NW_CHUNK) smask &= ((1u << (nrows - r0)) - 1u) * 0x01010101u;
+                // Append the chunk's survivors (in any order: the top-N stage ranks them).
+                int slot = smask ? atomicAdd(&nq[w], __popc(smask)) : 0;
                 while (smask) {
                     const int bit = __ffs((int)smask) - 1;
                     smask &= smask - 1u;
@@ -700,6 +716,9 @@ k_nms_warp(const Img* __restrict__ imgs, const uint2* __restrict__ items, int n_
         // The score buffer is free: fetch the next tile's score box.
         fence_proxy_async_smem();
         __syncwarp();
+        n = nq[w];
+        __syncwarp();
+        if (lane == 0) nq[w] = 0;
         if (lane == 0 && tn < n_tiles) issue_s(nxt);
         ok = mbar_wait(&mbar[w][1], par);
         if (__any_sync(0xFFFFFFFFu, !ok)) {
