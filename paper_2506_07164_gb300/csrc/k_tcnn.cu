@@ -135,10 +135,15 @@ __device__ __forceinline__ uint4 load_chunk(const Patch& P, int q) {
 //
 // A block of 8 warps takes one tile at a time, two blocks per SM; a layer's
 // planes have buffers of their own, so a tile needs two barriers, and the next
-// tile's pixels are staged while layer 2 runs.  Bound by shared memory (65 % of
-// its wavefront rate; tensor pipe 36 %, issue 50 %).  16,384 patches: 755 us as
-// fp32 FMAs over shared-memory operands, 397 us register-blocked with packed
-// fp32 FMAs (the smem reads of the weights then bound it), 240 us here.
+// tile's pixels are staged while layer 2 runs.  Layer 3 is four products' rows
+// of work: four warps do it, both channel halves from one read of the
+// activations, while the other four start on the next tile's layer 1.  Bound by
+// shared memory (~2300 wavefronts per tile, 64 % of its rate).  16,384 patches:
+// 755 us as fp32 FMAs over shared-memory operands, 397 us register-blocked with
+// packed fp32 FMAs (the smem reads of the weights then bound it), 240 us on the
+// tensor cores with a channel half of layer 3 per warp (each reading all
+// activations, 2600 wavefronts), 219 us here (219.6, 220.1 and 221.2 us with 4,
+// 5 and 7 instead of 6 layer-1 products per warp that also does layer 3).
 constexpr int FWD_THREADS = 256, FWD_BLOCKS = 2;
 constexpr int TI_ROW = 48, TI_X = 4;                       // input rows: words per row (pixel pairs), word of pixel 0
 constexpr int TI_BYTES = 65 * TI_ROW * 4;                  // row 0: zeros
@@ -147,7 +152,9 @@ constexpr int T1_PLANE = 33 * T1_ROW * 16;                 // one part: 33 rows 
 constexpr int T2_ROW = 21, T2_O = 13;                      // layer-2 rows: 9 even columns, (gap), 8 odd ones
 constexpr int T2_PLANE = 17 * T2_ROW * 16;                 // one part and channel half: 17 rows
 constexpr int FWD_RED = 2 * 4 * C3;                        // per tile parity and row pair: channel sums
-constexpr int FWD_SMEM = TI_BYTES + 3 * T1_PLANE + 6 * T2_PLANE + FWD_RED * 4;
+constexpr int FWD_B3 = 18 * 32;                            // layer-3 weight fragments: a word pair per lane, tap and channel half
+constexpr int FWD_SMEM = TI_BYTES + 3 * T1_PLANE + 6 * T2_PLANE + FWD_RED * 4 + FWD_B3 * 8;
+constexpr int FWD_L1A = 6;                                 // layer-1 products of each of the four warps that also do layer 3
 static_assert(TI_BYTES % 16 == 0 && T1_PLANE % 16 == 0 && T2_PLANE % 16 == 0, "16-byte rows for ldmatrix");
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -232,6 +239,7 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
     uint8_t* const p1 = fsm + TI_BYTES;
     uint8_t* const p2 = p1 + 3 * T1_PLANE;
     float* const red = reinterpret_cast<float*>(p2 + 6 * T2_PLANE);
+    uint2* const b3 = reinterpret_cast<uint2*>(red + FWD_RED);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t4 = lane & 3;
     // Zero the planes once: the pad words are never written afterwards.
@@ -240,8 +248,8 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
 
     // Weight fragments.  Layer 1: depth 4 ky + j, j = 0 a zero weight (the pixel
     // two to the left), j = kx + 1; layer 2: two taps of 8 channels per step, the
-    // ninth alone; layer 3 (this warp's channel half): a tap of 16 channels per step.
-    uint32_t b1[2], b2[2][4][2], b2e[2], b3[9][2];
+    // ninth alone; layer 3: a tap of 16 channels per step, in shared memory.
+    uint32_t b1[2], b2[2][4][2], b2e[2];
     {
         auto w1 = [&](int k) {  // depth k of layer 1, channel g; -1: zero weight
             return k < 12 && (k & 3) ? W1 + g * 9 + (k >> 2) * 3 + (k & 3) - 1 : -1;
@@ -258,17 +266,15 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
             }
             b2e[j] = pack_w(wq, r + 8, r + 9 + 8);
         }
-        const int r = W3 + (8 * (warp & 1) + g) * C2 * 9 + 2 * t4 * 9;
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            b3[k][0] = pack_w(wq, r + k, r + 9 + k);
-            b3[k][1] = pack_w(wq, r + 8 * 9 + k, r + 9 * 9 + k);
+        for (int i = warp; i < 18; i += FWD_THREADS / 32) {
+            const int k = i >> 1, r = W3 + (8 * (i & 1) + g) * C2 * 9 + 2 * t4 * 9;
+            b3[i * 32 + lane] = make_uint2(pack_w(wq, r + k, r + 9 + k), pack_w(wq, r + 8 * 9 + k, r + 9 * 9 + k));
         }
     }
     auto bias = [&](int i) { return __bfloat162float(wq[i]); };
     const float bb1[2] = {bias(B1 + 2 * t4), bias(B1 + 2 * t4 + 1)};
     const float bb2[4] = {bias(B2 + 2 * t4), bias(B2 + 2 * t4 + 1), bias(B2 + 8 + 2 * t4), bias(B2 + 9 + 2 * t4)};
-    const float bb3[2] = {bias(B3 + 8 * (warp & 1) + 2 * t4), bias(B3 + 8 * (warp & 1) + 2 * t4 + 1)};
+    const float bb3[4] = {bias(B3 + 2 * t4), bias(B3 + 2 * t4 + 1), bias(B3 + 8 + 2 * t4), bias(B3 + 9 + 2 * t4)};
     const float wf = bias(WF + (lane & 15)), bf = bias(BF);
     const float zero[4] = {0.f, 0.f, 0.f, 0.f};
 
@@ -285,9 +291,9 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
         off2e = (uint32_t)((2 * T1_ROW + 1 + x) * 16);
     }
     const uint32_t s1 = smem_addr(p1), s2 = smem_addr(p2);
-    // Layer 3: output row 2 (warp / 2) + (bit 3 of the lane), column lane & 7, channel half = bit 4.
+    // Layer 3, warps 0 to 3: output row 2 warp + (bit 3 of the lane), column lane & 7, channel half = bit 4.
     const uint32_t a3base =
-        s2 + (uint32_t)((lane >> 4) * T2_PLANE + (2 * (2 * (warp >> 1) + ((lane >> 3) & 1)) * T2_ROW + (lane & 7)) * 16);
+        s2 + (uint32_t)((lane >> 4) * T2_PLANE + (2 * (2 * warp + ((lane >> 3) & 1)) * T2_ROW + (lane & 7)) * 16);
 
     auto finish = [&](int t, int par) {  // warp 0: the head of a finished tile
         const float* r = red + par * 4 * C3 + (lane & 15);
@@ -306,8 +312,10 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
         uint4 pix = make_uint4(0u, 0u, 0u, 0u);
         if (tn < n) pix = load_chunk(find_patch(src, tn), tid);
         // Layer 1: 64 products of 16 pixels (a row's half: even columns 2 g + 16 h, odd ones).
+        // Warps 4 to 7, without a part of layer 3, start earlier and take more of them.
+        const int l1_0 = warp < 4 ? warp : 4 * FWD_L1A + warp - 4, l1_1 = warp < 4 ? 4 * FWD_L1A : 64;
 #pragma unroll 2
-        for (int i = warp; i < 64; i += 8) {
+        for (int i = l1_0; i < l1_1; i += 4) {
             const int y = i >> 1, h = i & 1;
             const uint32_t* r = in + (2 * y + (t4 >> 1)) * TI_ROW + TI_X - 1 + 2 * g + 16 * h + (t4 & 1);
             const uint32_t* r2 = in + (2 * y + 2) * TI_ROW + TI_X - 1 + 2 * g + 16 * h + t4;
@@ -374,9 +382,9 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
             }
         }
         __syncthreads();
-        // Layer 3: two output rows of 8 pixels, 8 channels per warp; their sums for the mean.
-        {
-            float acc[4] = {}, lm[4] = {}, lw[4] = {};
+        // Layer 3: two output rows of 8 pixels per warp; their sums for the mean.
+        if (warp < 4) {
+            float acc[2][4] = {}, lm[2][4] = {}, lw[2][4] = {};
 #pragma unroll
             for (int k = 0; k < 9; ++k) {
                 const uint32_t a0 = a3base + (uint32_t)(((k / 3) * T2_ROW + (k % 3 == 1 ? T2_O : (k % 3) >> 1)) * 16);
@@ -384,24 +392,33 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
                 ldsm4(ah, a0);
                 ldsm4(am, a0 + 2 * T2_PLANE);
                 ldsm4(al, a0 + 4 * T2_PLANE);
-                float d[4];
-                mma16(d, ah, b3[k], zero);
-                mma16(lm, am, b3[k], lm);
-                mma16(lw, al, b3[k], lw);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[i] += d[i];
-            }
-            float v0 = relu(acc[0] + (lm[0] + lw[0]) + bb3[0]) + relu(acc[2] + (lm[2] + lw[2]) + bb3[0]);
-            float v1 = relu(acc[1] + (lm[1] + lw[1]) + bb3[1]) + relu(acc[3] + (lm[3] + lw[3]) + bb3[1]);
+                for (int j = 0; j < 2; ++j) {
+                    const uint2 w3 = b3[(2 * k + j) * 32 + lane];
+                    const uint32_t b[2] = {w3.x, w3.y};
+                    float d[4];
+                    mma16(d, ah, b, zero);
+                    mma16(lm[j], am, b, lm[j]);
+                    mma16(lw[j], al, b, lw[j]);
 #pragma unroll
-            for (int o = 4; o < 32; o <<= 1) {
-                v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o);
-                v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, o);
+                    for (int i = 0; i < 4; ++i) acc[j][i] += d[i];
+                }
             }
-            if (g == 0) {
-                float* r = red + (par * 4 + (warp >> 1)) * C3 + 8 * (warp & 1) + 2 * t4;
-                r[0] = v0;
-                r[1] = v1;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float c0 = bb3[2 * j], c1 = bb3[2 * j + 1];
+                float v0 = relu(acc[j][0] + (lm[j][0] + lw[j][0]) + c0) + relu(acc[j][2] + (lm[j][2] + lw[j][2]) + c0);
+                float v1 = relu(acc[j][1] + (lm[j][1] + lw[j][1]) + c1) + relu(acc[j][3] + (lm[j][3] + lw[j][3]) + c1);
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    v0 += __shfl_xor_sync(0xFFFFFFFFu, v0, o);
+                    v1 += __shfl_xor_sync(0xFFFFFFFFu, v1, o);
+                }
+                if (g == 0) {
+                    float* r = red + (par * 4 + warp) * C3 + 8 * j + 2 * t4;
+                    r[0] = v0;
+                    r[1] = v1;
+                }
             }
         }
         last = t;
