@@ -437,11 +437,11 @@ k_nms_harris(const Img* __restrict__ imgs, const int32_t* __restrict__ list,
 // the proposed tiles of an image that has them, are zeroed in the staged score
 // box first (in the words of lanes whose word is not wholly inside).
 //
-// Bound by instruction issue (~5200 per tile at first, 83 % of the slots): half
-// as many warps again, with one buffer for both boxes, changed nothing (1154
-// against 1132 us for 128 1080p frames), fewer instructions per row did: halo
-// words no longer read and thresholded by every lane 1132 -> 1064 us; halo
-// pixels stored as the test takes them, bits collected by shifting 1034; the
+// Bound by its instructions (issue 63 % active, the half-rate pipes busier: ALU
+// in the 3x3 test, multiply in the Harris sums): half as many warps again, with
+// one buffer for both boxes, changed nothing (1154 against 1132 us for 128 1080p
+// frames), fewer instructions did (~4300 -> ~3700 per tile): halo words no longer
+// read and thresholded by every lane 1132 -> 1064 us; halo pixels stored as the test takes them, bits collected by shifting 1034; the
 // survivors' places by one shared atomic per lane instead of a warp scan 1017;
 // flags carried over the chunks 1002.  Harris sums in packed floats (half the
 // multiply-adds, twice the registers): no gain.

@@ -138,11 +138,11 @@ __device__ __forceinline__ uint4 load_chunk(const Patch& P, int q) {
 // tile's pixels are staged while layer 2 runs.  Layer 3 is four products' rows
 // of work: four warps do it, both channel halves from one read of the
 // activations, while the other four start on the next tile's layer 1.  Bound by
-// shared memory (~2300 wavefronts per tile, 64 % of its rate).  16,384 patches:
+// shared memory (~2430 wavefronts per tile, 61 % of its rate).  16,384 patches:
 // 755 us as fp32 FMAs over shared-memory operands, 397 us register-blocked with
 // packed fp32 FMAs (the smem reads of the weights then bound it), 240 us on the
 // tensor cores with a channel half of layer 3 per warp (each reading all
-// activations, 2600 wavefronts), 219 us here (219.6, 220.1 and 221.2 us with 4,
+// activations), 219 us here (219.6, 220.1 and 221.2 us with 4,
 // 5 and 7 instead of 6 layer-1 products per warp that also does layer 3).
 constexpr int FWD_THREADS = 256, FWD_BLOCKS = 2;
 constexpr int TI_ROW = 48, TI_X = 4;                       // input rows: words per row (pixel pairs), word of pixel 0

@@ -716,7 +716,7 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     P->aligned_ok = P->cell_tiles && fast_aligned_ok(s.cell);
     P->strip_ok = s.cell <= CS_MAX_CELL;
     // Sizes of the work items, by the batch's cell-row strips (75 for a VGA level,
-    // 240 for a VGA frame of 8 levels, 1480 for a 1080p one).  The per-warp kernels
+    // 240 for a VGA frame of 8 levels, 1640 for a 1080p one).  The per-warp kernels
     // hold 2432 warps: fewer items than that leave warps idle while each item's
     // rows run one after another, so small batches get thirds or halves of a strip
     // and 8- or 16-row NMS tiles (one VGA frame, whole call: 52 us with full items,
@@ -974,8 +974,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     // an NMS kernel that applies them (no threshold pass).
     // NMS: the per-warp kernel, which spreads its Harris sums over the warps'
     // own survivors and wins on small items and on many; between (1200 to 8000
-    // strips: one 1080p frame 80 against 83 us, one 4K frame 208 against 215)
-    // the block kernel, whose Harris phase shares a 64-row tile's survivors.
+    // strips: one 1080p frame 69.9 against 71.2 us, two 97.8 against 100.5, four
+    // 157.6 against 158.0) the block kernel, whose Harris phase shares a 64-row
+    // tile's survivors.
     const bool warp_nms = strips < 1200 || strips >= 8000;
     P->tun.fast_cell_tiles = P->strip_ok ? 4 : P->cell_tiles ? 1 : 0;
     P->tun.fast_tile_h = 32;
