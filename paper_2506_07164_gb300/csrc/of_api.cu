@@ -479,7 +479,7 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
             break;
         }
         case 3:
-            launch_select(P->d_img() + G.img_begin, G.n_img, P->d_call(), P->max_quota, st, pdl);
+            launch_select(P->d_img() + G.img_begin, G.n_img, nl, P->d_call(), P->max_quota, st, pdl);
             pdl = P->pdl;
             break;
         case 4:

@@ -203,7 +203,8 @@ int nms_warp_blocks_per_sm();
 // Whether the top-N kernel leaves the kept lists of a launch of n_img images grouped by
 // key code for the orientation kernel to rank (else it sorts them).
 bool select_grouped(int n_img);
-void launch_select(const Img* imgs, int n_img, const Call* call, int max_quota, void* stream, bool pdl = false);
+// n_img images: frames of `levels` levels each.
+void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, void* stream, bool pdl = false);
 void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream, bool pdl = false);
 // Slots [slot_begin, slot_end) of images [img_begin, img_begin + n_img) (one frame group).
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,

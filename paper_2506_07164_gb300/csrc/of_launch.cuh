@@ -22,10 +22,10 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 
 // cluster: blocks per cluster (1: none).
 template <typename... P, typename... A>
-inline void launch_chain(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t st, bool pdl, int cluster,
+inline void launch_chain(void (*kernel)(P...), dim3 grid, int block, int smem, cudaStream_t st, bool pdl, int cluster,
                          A&&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
