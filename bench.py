@@ -317,7 +317,7 @@ FAST_OPS_PER_PX = 40.5
 # levels, divided by the frames.  Valid while the kernels' code
 # (kernels_sha1) and the per-stage launch choices below are the ones captured;
 # otherwise the line reports null.
-STAGE_TRAFFIC = {"code_sha1": "dad5762bdb94d11651991dfb36ec94ea5cf530e8", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18818564, "fast": 30958692, "nms_harris": 39775687, "select": 2634710, "orient": 2620347}, "dram_bytes_per_frame": {"pyramid": 5583392, "fast": 12761732, "nms_harris": 16266900, "select": 1028100, "orient": 547828}}
+STAGE_TRAFFIC = {"code_sha1": "e973cb94047aa7e4513cf5545ee78383cb9099c1", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18769712, "fast": 31129756, "nms_harris": 39991494, "select": 2689641, "orient": 2609459}, "dram_bytes_per_frame": {"pyramid": 5579720, "fast": 12765512, "nms_harris": 16315564, "select": 1040096, "orient": 547832}}
 
 
 def code_sha1(path):
