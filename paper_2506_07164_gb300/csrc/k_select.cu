@@ -15,7 +15,9 @@
 //     code > b go straight to the places that the counts of the better bins
 //     give them; those of bin b (at most SEL_BND) go through the same step
 //     once more, by the next 9 bits of |key|, and the few of that boundary
-//     are ranked by counting;
+//     are ranked by counting (more than SEL_BND in bin b: the cluster first
+//     splits the bin by the next 12 bits; some 4K frames, whole call 324 us
+//     when the first block's radix select took them, 205 now);
 //   - otherwise an MSB-first radix select over 8-bit digits of R (one
 //     shared-memory histogram per pass) fixes, digit by digit, the prefix of
 //     the n_l-th largest R, stopping as soon as every candidate that shares
@@ -60,16 +62,17 @@ struct SelState {
     uint32_t pre_lo, msk_lo;
     int need, done;
     int coarse, code_b, n_take;
+    int mid_b, sure;  // grouped: boundary of the split bin (-1: not split), candidates above it
 };
 
-// The 9 bits of the magnitude after the code's, for keys of one code:
-// non-decreasing in key.
-__device__ __forceinline__ uint32_t fine_code(uint64_t u) {
+// N bits of the magnitude after the leading one and the next SKIP bits, for keys
+// that agree in those: non-decreasing in key.  The code's bits end at SKIP = 5.
+template <int SKIP, int N>
+__device__ __forceinline__ uint32_t fine_bits(uint64_t u) {
     const bool pos = (u >> 63) != 0;
     const uint64_t x = pos ? u & 0x7FFFFFFFFFFFFFFFull : u ^ 0x7FFFFFFFFFFFFFFFull;
-    const int L = 64 - __clzll((long long)x);
-    const uint32_t f = L > 6 ? (uint32_t)((x << (70 - L)) >> 55) : 0u;
-    return pos ? f : 511u - f;
+    const uint32_t f = x ? (uint32_t)((x << __clzll((long long)x) << (1 + SKIP)) >> (64 - N)) : 0u;
+    return pos ? f : (1u << N) - 1u - f;
 }
 
 // ---- cluster primitives (shared::cluster addresses of the other blocks' shared memory)
@@ -219,6 +222,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         st.coarse = GROUPED && n <= q;  // a grouped list of everything: no boundary bin
         st.code_b = GROUPED && n <= q ? -1 : 0;
         st.n_take = m;
+        st.mid_b = -1;
+        st.sure = 0;
         s_cnt = 0;
         s_bnd = 0;
     }
@@ -332,20 +337,110 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         else __syncthreads();
     }
 
+    if (GROUPED && __builtin_expect(!st.coarse, 0)) {  // the same in all blocks
+        // The boundary bin holds too many for the first block: the cluster splits it by
+        // the next 12 bits of the keys, counted where its candidates go later.
+        uint32_t* const h2 = reinterpret_cast<uint32_t*>(bkey);
+        static_assert(SEL_BND * sizeof(uint64_t) >= SEL_BINS * sizeof(uint32_t), "room for the counts");
+        const uint32_t code_b = (uint32_t)st.code_b;
+        for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) h2[i] = 0u;
+        __syncthreads();
+        for (int i0 = i_first; i0 < n; i0 += 2 * SEL_UNROLL * i_step) {
+            uint64_t v[2 * SEL_UNROLL];
+#pragma unroll
+            for (int k = 0; k < 2 * SEL_UNROLL; ++k) v[k] = i0 + k * i_step < n ? __ldg(I.ckey + i0 + k * i_step) : 0ull;
+#pragma unroll
+            for (int k = 0; k < 2 * SEL_UNROLL; ++k)
+                if (i0 + k * i_step < n && key_code(v[k]) == code_b) atomicAdd(&h2[fine_bits<5, 12>(v[k])], 1u);
+        }
+        if (shared) cluster_sync_all();
+        else __syncthreads();
+        if (rank == 0) {
+            constexpr int PER1 = SEL_BINS / SELECT_THREADS;
+            const int need = q - st.n_take;
+            int bins[PER1], own = 0;
+#pragma unroll
+            for (int j = 0; j < PER1; ++j) {
+                uint32_t h = 0u;
+                for (int c = 0; c < parts; ++c) h += shared ? ld_rank(map_rank(&h2[PER1 * tid + j], c)) : h2[PER1 * tid + j];
+                bins[j] = (int)h;
+                own += (int)h;
+            }
+            int v = own;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int t = __shfl_down_sync(0xFFFFFFFFu, v, off);
+                if (lane + off < 32) v += t;
+            }
+            if (lane == 0) wsum[warp] = (uint32_t)v;
+            __syncthreads();
+            int above = v - own;
+            for (int w = warp + 1; w < SELECT_THREADS / 32; ++w) above += (int)wsum[w];
+            if (above < need && above + own >= need) {  // exactly one thread
+                int cum = above;
+#pragma unroll
+                for (int j = PER1 - 1; j >= 0; --j) {
+                    if (cum < need && cum + bins[j] >= need && bins[j] <= SEL_BND) {
+                        s_cnt = st.n_take;  // where the split bin's sure ones go
+                        st.sure = cum;
+                        for (int c = 0; c < parts; ++c) {
+                            if (c == 0) {
+                                st.mid_b = PER1 * tid + j;
+                                st.coarse = 1;
+                            } else {
+                                st_rank(map_rank(&st.mid_b, c), (uint32_t)(PER1 * tid + j));
+                                st_rank(map_rank(&st.coarse, c), 1u);
+                            }
+                        }
+                    }
+                    cum += bins[j];
+                }
+            }
+        }
+        if (shared) cluster_sync_all();
+        else __syncthreads();
+    }
     auto keep = [&](int pos, uint64_t key, uint32_t yx) {
         I.kkey[pos] = key;
         I.kyx[pos] = yx;
     };
     if (GROUPED && st.coarse) {  // the same in all blocks
         // Gather: the better bins to their places, the boundary bin to the first block.
-        const int code_b = st.code_b;
+        const int code_b = st.code_b, mid_b = st.mid_b;
         const ulonglong2* ck2 = reinterpret_cast<const ulonglong2*>(I.ckey);
         const int n2 = (n + 1) >> 1;
         // A place of the first block's counter.
         auto take = [&](void* counter) {
             return shared ? atomic_add_rank(map_rank(counter, 0), 1) : atomicAdd(static_cast<int*>(counter), 1);
         };
-        for (int i0 = i_first; i0 < n2; i0 += SEL_UNROLL * i_step) {
+        auto bound = [&](uint64_t key, uint32_t yx) {
+            const int pos = take(&s_bnd);  // at most SEL_BND of them
+            if (pos < SEL_BND) {
+                if (shared) {
+                    st_rank64(map_rank(&bkey[pos], 0), key);
+                    st_rank(map_rank(&byx[pos], 0), yx);
+                } else {
+                    bkey[pos] = key;
+                    byx[pos] = yx;
+                }
+            }
+        };
+        if (__builtin_expect(mid_b >= 0, 0)) {
+            for (int i = i_first; i < n; i += i_step) {
+                const uint64_t key = __ldg(I.ckey + i);
+                const int code = (int)key_code(key);
+                const int mid = code == code_b ? (int)fine_bits<5, 12>(key) : -1;
+                if (code < code_b || (code == code_b && mid < mid_b)) continue;
+                const uint32_t yx = __ldg(I.cyx + i);
+                if (code == code_b && mid == mid_b) {
+                    bound(key, yx);
+                } else {
+                    const int pos = code > code_b ? take(&hist[code]) : take(&s_cnt);
+                    if (pos < q) keep(pos, key, yx);
+                }
+            }
+        }
+        for (int i0 = mid_b < 0 ? i_first : n2; i0 < n2; i0 += SEL_UNROLL * i_step) {
             ulonglong2 v[SEL_UNROLL];
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {
@@ -367,16 +462,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
                         const int pos = take(&hist[code]);
                         if (pos < q) keep(pos, key, yx);
                     } else {
-                        const int pos = take(&s_bnd);  // at most SEL_BND of them
-                        if (pos < SEL_BND) {
-                            if (shared) {
-                                st_rank64(map_rank(&bkey[pos], 0), key);
-                                st_rank(map_rank(&byx[pos], 0), yx);
-                            } else {
-                                bkey[pos] = key;
-                                byx[pos] = yx;
-                            }
-                        }
+                        bound(key, yx);
                     }
                 }
             }
@@ -386,7 +472,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         if (rank != 0) return;
         // The boundary bin: its best fill the rest, found by the fine codes.
         static_assert(SELECT_THREADS == 512, "one fine code per thread");
-        const int nb = min(s_bnd, SEL_BND), above = st.n_take, need = q - above;
+        const int nb = min(s_bnd, SEL_BND), above = st.n_take + st.sure, need = q - above;
         if (nb == 0) {
             if (tid == 0) I.ctr[1] = above;
             return;
@@ -397,6 +483,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
             s_cnt = above;
         }
         __syncthreads();
+        auto fine_code = [&](uint64_t key) { return mid_b < 0 ? fine_bits<5, 9>(key) : fine_bits<17, 9>(key); };
         for (int i = tid; i < nb; i += SELECT_THREADS) atomicAdd(&hist[fine_code(bkey[i])], 1u);
         __syncthreads();
         const int own = (int)hist[tid];

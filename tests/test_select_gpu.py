@@ -78,3 +78,23 @@ def test_grouped_and_sorted_lists(frames, n):
         for f in FIELDS:
             np.testing.assert_array_equal(got[f], ora[f], err_msg=f)
     det.close()
+
+
+# Thousands of keys that differ in their last bits only: the boundary bin holds more
+# than the first block takes, so the cluster splits it by further bits of the keys.
+@pytest.mark.parametrize("frames,n", [(1, 1), (1, 2000), (1, 8192), (17, 500)])
+def test_a_full_boundary_bin_is_split(frames, n):
+    rng = np.random.default_rng(7)
+    tile = np.full((16, 16), 60, np.uint8)
+    tile[4:11, 4:11] = 200
+    img = (np.tile(tile, (60, 80)).astype(np.int16) + rng.integers(-1, 2, (960, 1280))).astype(np.uint8)
+    dev = torch.from_numpy(img).cuda()
+    det = ofg.Detector(img.shape[1], img.shape[0], max_levels=1, max_features=n, max_batch=frames)
+    det.detect_batch([dev] * frames, levels=1, fast_t=20, n_features=n)
+    torch.cuda.synchronize()
+    ora = oracle.detect(img, levels=1, fast_t=20, n_features=n)
+    for got in det.batch_results(frames, n):
+        assert len(got) == len(ora) == n
+        for f in FIELDS:
+            np.testing.assert_array_equal(got[f], ora[f], err_msg=f)
+    det.close()
