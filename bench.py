@@ -317,7 +317,7 @@ FAST_OPS_PER_PX = 40.5
 # levels, divided by the frames.  Valid while the kernels' code
 # (kernels_sha1) and the per-stage launch choices below are the ones captured;
 # otherwise the line reports null.
-STAGE_TRAFFIC = {"code_sha1": "e973cb94047aa7e4513cf5545ee78383cb9099c1", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18769712, "fast": 31129756, "nms_harris": 39991494, "select": 2689641, "orient": 2609459}, "dram_bytes_per_frame": {"pyramid": 5579720, "fast": 12765512, "nms_harris": 16315564, "select": 1040096, "orient": 547832}}
+STAGE_TRAFFIC = {"code_sha1": "49a6a0bec6a6decbf570487fa413ba1f6e81c2eb", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18763954, "fast": 31141120, "nms_harris": 39979009, "select": 2689336, "orient": 2607282}, "dram_bytes_per_frame": {"pyramid": 5580852, "fast": 12769388, "nms_harris": 16291260, "select": 1040760, "orient": 547852}}
 
 
 def code_sha1(path):
