@@ -27,6 +27,7 @@
 // instruction issue (70 %).
 #include <cuda_runtime.h>
 
+#include "of_edge.cuh"
 #include "of_internal.h"
 #include "of_launch.cuh"
 #include "of_rank.cuh"
@@ -67,6 +68,7 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
     const float* const fx = I.fx;
     const float* const fy = I.fy;
     const int pitch = I.pitch, spitch = I.spitch, quota = I.quota, level = I.level, frame = I.frame;
+    const int width = I.w, height = I.h;
     const int32_t* const ctr = I.ctr;
     const int32_t* const lctr = lane < levels ? imgs[frame * levels + lane].ctr : nullptr;
     const uint32_t* const kyx = I.kyx;
@@ -95,9 +97,11 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
     const uint64_t okey = GROUPED ? __shfl_sync(0xFFFFFFFFu, wkey, 16) : wkey;
     const int x = (int)(yx & 0xFFFFu), y = (int)(yx >> 16);
     // The patch, columns x - H .. x + H of rows y - H .. y + H, as aligned words
-    // (images and pitches are multiples of 16 bytes; H <= border keeps it inside).
+    // (images and pitches are multiples of 16 bytes; H <= border keeps its pixels
+    // inside, and a word that would pass the caller's frame is read bytewise).
     uint32_t* const P = patch[threadIdx.x >> 5];
-    const int sh = (x - H) & 3, nw = (sh + 2 * H + 4) >> 2, rows = 2 * H + 1;
+    const PatchWords pw = patch_words(x, y, H, width, height, OP_WORDS);
+    const int sh = pw.sh;
     int rank = idx;
     {
         const uint8_t* const q = img + (size_t)(y - H) * pitch + (x - H - sh);
@@ -105,7 +109,7 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
 #pragma unroll
         for (int k = 0; k < OP_WORDS; ++k) {
             const int i = lane + 32 * k, r = i / OP_WORDS, c = i - r * OP_WORDS;
-            v[k] = r < rows && c < nw ? __ldg(reinterpret_cast<const uint32_t*>(q + (size_t)r * pitch) + c) : 0u;
+            v[k] = i < pw.whole && c < pw.nw ? __ldg(reinterpret_cast<const uint32_t*>(q + (size_t)r * pitch) + c) : 0u;
         }
         if (GROUPED) {
             // The run of this code in a window of 32 entries, and the better ones of it.
@@ -149,6 +153,13 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
 #pragma unroll
         for (int k = 0; k < OP_WORDS; ++k)
             if (lane + 32 * k < OP_SIZE) P[lane + 32 * k] = v[k];
+        if (pw.tail && lane == (pw.whole & 31)) {
+            const int x0 = x - H - sh + 4 * (pw.nw - 1);  // its first column, inside the frame
+            const uint8_t* const last = img + (size_t)(y + H) * pitch + x0;
+            uint32_t t = 0u;
+            for (int i = 0; i < 4 && x0 + i < width; ++i) t |= (uint32_t)last[i] << (8 * i);
+            P[pw.whole] = t;
+        }
     }
     const int sc = lane == 0 ? (int)score[(size_t)y * spitch + x] : 0;
     // No tables: a level-0 image (scale^0 = 1; the allocation-free entry point).
