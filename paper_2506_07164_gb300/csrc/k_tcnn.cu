@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "of_edge.cuh"
 #include "of_internal.h"
 #include "ofast.h"
 
@@ -63,7 +64,8 @@ struct PatchSrc {
 // A 64 x 64 patch is 256 16-byte chunks (4 per row).  Chunk q of tile t; pixels
 // outside the image are 0.  Level images and their pitches are multiples of
 // 16 bytes, and a patch starts at a multiple of 16, so a chunk is one aligned
-// load (whole inside the row's pitch); bytes past the row's w are cleared.
+// load (whole inside the row's pitch; bytewise where it would pass the end of a
+// caller's frame); bytes past the row's w are cleared.
 struct Patch {
     const uint8_t* p;       // dense: the tile; in place: the level image
     int x0, y0, w, h, pitch;  // in place; pitch 0: dense
@@ -98,8 +100,16 @@ __device__ __forceinline__ uint4 load_chunk(const Patch& P, int q) {
     }
     const int x = P.x0 + 16 * (q & 3), y = P.y0 + (q >> 2);
     if (x < 0 || x >= P.w || y < 0 || y >= P.h) return make_uint4(0u, 0u, 0u, 0u);
-    uint4 v = __ldg(reinterpret_cast<const uint4*>(P.p + (size_t)y * P.pitch + x));
-    const int n = P.w - x;  // valid bytes
+    const uint8_t* const p = P.p + (size_t)y * P.pitch + x;
+    const int n = ofk::chunk_bytes(x, P.w);
+    if (!ofk::chunk_whole(n, y, P.h)) {  // at most 15 bytes
+        uint32_t v[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int i = 0; i < 15; ++i)
+            if (i < n) v[i >> 2] |= (uint32_t)__ldg(p + i) << (8 * (i & 3));
+        return make_uint4(v[0], v[1], v[2], v[3]);
+    }
+    uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
     if (n < 16) {
         uint32_t* m = &v.x;
 #pragma unroll

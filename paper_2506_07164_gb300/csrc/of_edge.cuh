@@ -25,4 +25,9 @@ __host__ __device__ __forceinline__ PatchWords patch_words(int x, int y, int H, 
     return p;
 }
 
+// Of the 16 bytes from column x of row y (both inside a w x h image), those
+// inside the row; whether they may be read as one 16-byte load.
+__host__ __device__ __forceinline__ int chunk_bytes(int x, int w) { return w - x < 16 ? w - x : 16; }
+__host__ __device__ __forceinline__ bool chunk_whole(int n, int y, int h) { return n == 16 || y < h - 1; }
+
 }  // namespace ofk

@@ -74,6 +74,34 @@ def test_orientation_patch_words_stay_inside_the_frame(tmp_path):
     assert beyond == wide > 0  # whole words alone would pass the end at these positions
 
 
+CHUNK = r"""
+#include <cstdio>
+#include "of_edge.cuh"
+// Every 16-byte chunk of the patches around the tiles of w x h frames.
+int main() {
+    long bad = 0, missing = 0, wide = 0;
+    for (int w = 39; w <= 90; ++w) {
+        const int h = 41, pitch = (w + 15) / 16 * 16, end = (h - 1) * pitch + w;
+        for (int y = 0; y < h; ++y)
+            for (int x = 0; x < w; x += 16) {
+                const int n = ofk::chunk_bytes(x, w), at = y * pitch + x;
+                const int read = ofk::chunk_whole(n, y, h) ? 16 : n;
+                bad += at + read > end;
+                missing += n != (w - x < 16 ? w - x : 16) || read < n;
+                wide += at + 16 > end;  // as a whole chunk
+            }
+    }
+    std::printf("%ld %ld %ld\n", bad, missing, wide);
+}
+"""
+
+
+def test_network_patch_chunks_stay_inside_the_frame(tmp_path):
+    bad, missing, wide = _host(tmp_path, CHUNK)
+    assert bad == 0 and missing == 0
+    assert wide > 0  # whole chunks alone would pass the end of these frames
+
+
 def _ending_frame(img, torch):
     """The frame at a 16-byte pitch in a buffer that ends with its last pixel."""
     h, w = img.shape
@@ -109,3 +137,29 @@ def test_keypoints_at_the_last_admissible_pixel(border, radius, w):
     for f in ("x_l", "y_l", "level", "fast_score", "A", "B", "C", "m10", "m01", "key"):
         np.testing.assert_array_equal(got[f], ora[f], err_msg=f)
     det.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("w,h", [(331, 217), (97, 70), (145, 89), (335, 102), (336, 103)])
+def test_proposal_patches_at_the_frame_end(w, h):
+    """Logits of the tiles read in place, on frames that end with their buffer, equal those of the same
+    patches extracted."""
+    torch = pytest.importorskip("torch")
+    import synth
+    from paper_2506_07164_gb300 import learned
+
+    net = learned.TileNet(0).load(learned.DEFAULT_WEIGHTS)
+    det = ofg.Detector(w, h, max_levels=2, max_features=200, max_batch=1, fast_t_lo=7)
+    t = _ending_frame(synth.scene(w, h, w), torch)
+    ofg.of_detect_learned(det.h, [(t, w, h, t.stride(0))], 2, 1.2, 20, 0.04, 200, net.net, 0.1, 0.0, 1, det.out,
+                          det.counts)
+    for lvl in range(2):
+        raw, dims = det.inspect(ofg.OF_BUF_LOGIT, 0, lvl)
+        n, _ = ofg.of_extract_tiles(det.h, 0, lvl)
+        if n == 0:
+            continue
+        p = torch.empty((n, 64, 64), dtype=torch.uint8, device="cuda")
+        ofg.of_extract_tiles(det.h, 0, lvl, p, n)
+        np.testing.assert_array_equal(raw.view(np.float32), net.logits(p).cpu().numpy())
+    det.close()
+    net.close()
