@@ -13,7 +13,8 @@
 // (when the FAST kernel did not set the flags) the block first ORs, per lane
 // and 16-byte chunk, a "byte >= t_hi" bit over the band's rows (three
 // instructions per word), maps the set bits to cells in shared memory and
-// stores the band's flags.  Then it writes, for up to 4096 columns at a time,
+// stores the band's flags (rows of more than CA_MAX_CELLS cells: in
+// rounds of that many).  Then it writes, for up to 4096 columns at a time,
 // a byte 0xFF where the column's cell in this band is flagged (all rows of a
 // band share their cells' flags), and its warps stream the band's rows in
 // 16-byte chunks against that mask, four chunks in flight per lane, writing a
@@ -68,62 +69,70 @@ k_cell_apply(const Img* __restrict__ imgs, const int32_t* __restrict__ list, con
         const uint32_t* fl = crow;
         const int y0 = border + cy * cell, y1 = min(y0 + cell, ry1);
         if (FLAGS && cells && (pmask || !pmask_only)) {
-            __syncthreads();  // the previous band's readers are done with bflag and colmask
-            for (int i = tid; i < ncx; i += CA_THREADS) bflag[i] = 0u;
-            __syncthreads();
-            for (int c0 = 0; c0 < n_chunks; c0 += 128) {
-                uint4 acc[4];
+            // CA_MAX_CELLS cells of the band at a time (one round but for rows of more).
+            for (int g0 = 0; g0 < ncx; g0 += CA_MAX_CELLS) {
+                const int ng = min(CA_MAX_CELLS, ncx - g0);
+                const int ch0 = (border + g0 * cell - xb0) >> 4;
+                const int ch1 = min(n_chunks, (border + (g0 + ng) * cell - xb0 + 15) >> 4);
+                __syncthreads();  // the last readers of bflag and colmask are done
+                for (int i = tid; i < ng; i += CA_THREADS) bflag[i] = 0u;
+                __syncthreads();
+                for (int c0 = ch0; c0 < ch1; c0 += 128) {
+                    uint4 acc[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) acc[k] = make_uint4(0u, 0u, 0u, 0u);
-                for (int y = y0 + warp; y < y1; y += CA_THREADS / 32) {
-                    const uint8_t* srow = score + (size_t)y * spitch;
-                    const int py = (y - border) >> 5;
+                    for (int k = 0; k < 4; ++k) acc[k] = make_uint4(0u, 0u, 0u, 0u);
+                    for (int y = y0 + warp; y < y1; y += CA_THREADS / 32) {
+                        const uint8_t* srow = score + (size_t)y * spitch;
+                        const int py = (y - border) >> 5;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int c = c0 + lane + 32 * k;
+                            if (c >= ch1) continue;
+                            const int x = xb0 + 16 * c;
+                            // Scores outside proposed tiles are stale: they do not count.
+                            if (pmask && pmask[(size_t)py * 4 * tiles_x + ((x - tile_x0) >> 5)] == 0) continue;
+                            const uint4 v = *reinterpret_cast<const uint4*>(srow + x);
+                            if (SMALL_T) {
+                                acc[k].x |= ge_bits(v.x, th);
+                                acc[k].y |= ge_bits(v.y, th);
+                                acc[k].z |= ge_bits(v.z, th);
+                                acc[k].w |= ge_bits(v.w, th);
+                            } else {
+                                acc[k].x |= bytes_ge_any(v.x, th);
+                                acc[k].y |= bytes_ge_any(v.y, th);
+                                acc[k].z |= bytes_ge_any(v.z, th);
+                                acc[k].w |= bytes_ge_any(v.w, th);
+                            }
+                        }
+                    }
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int c = c0 + lane + 32 * k;
-                        if (c >= n_chunks) continue;
+                        if (c >= ch1) continue;
                         const int x = xb0 + 16 * c;
-                        // Scores outside proposed tiles are stale: they do not count.
-                        if (pmask && pmask[(size_t)py * 4 * tiles_x + ((x - tile_x0) >> 5)] == 0) continue;
-                        const uint4 v = *reinterpret_cast<const uint4*>(srow + x);
-                        if (SMALL_T) {
-                            acc[k].x |= ge_bits(v.x, th);
-                            acc[k].y |= ge_bits(v.y, th);
-                            acc[k].z |= ge_bits(v.z, th);
-                            acc[k].w |= ge_bits(v.w, th);
-                        } else {
-                            acc[k].x |= bytes_ge_any(v.x, th);
-                            acc[k].y |= bytes_ge_any(v.y, th);
-                            acc[k].z |= bytes_ge_any(v.z, th);
-                            acc[k].w |= bytes_ge_any(v.w, th);
-                        }
-                    }
-                }
+                        const uint32_t wd[4] = {acc[k].x & 0x80808080u, acc[k].y & 0x80808080u,
+                                                acc[k].z & 0x80808080u, acc[k].w & 0x80808080u};
+                        if ((wd[0] | wd[1] | wd[2] | wd[3]) == 0u) continue;
+                        int last = -1;  // last cell flagged by this chunk (adjacent bytes share cells)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int c = c0 + lane + 32 * k;
-                    if (c >= n_chunks) continue;
-                    const int x = xb0 + 16 * c;
-                    const uint32_t wd[4] = {acc[k].x & 0x80808080u, acc[k].y & 0x80808080u,
-                                            acc[k].z & 0x80808080u, acc[k].w & 0x80808080u};
-                    if ((wd[0] | wd[1] | wd[2] | wd[3]) == 0u) continue;
-                    int last = -1;  // last cell flagged by this chunk (adjacent bytes share cells)
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int xx = x + i;
-                        if (((wd[i >> 2] >> (8 * (i & 3) + 7)) & 1u) && xx >= border && xx < rx1) {
-                            const int cx = (int)__umulhi((uint32_t)(xx - border), magic);
-                            if (cx != last) {
-                                atomicOr(&bflag[cx], 1u);
-                                last = cx;
+                        for (int i = 0; i < 16; ++i) {
+                            const int xx = x + i;
+                            if (((wd[i >> 2] >> (8 * (i & 3) + 7)) & 1u) && xx >= border && xx < rx1) {
+                                const int cx = (int)__umulhi((uint32_t)(xx - border), magic);
+                                if (cx != last) {
+                                    // A chunk at a round's edge holds cells of both rounds.
+                                    if ((uint32_t)(cx - g0) < (uint32_t)ng) atomicOr(&bflag[cx - g0], 1u);
+                                    last = cx;
+                                }
                             }
                         }
                     }
                 }
+                __syncthreads();
+                for (int i = tid; i < ng; i += CA_THREADS) crow[g0 + i] = bflag[i];
             }
-            __syncthreads();
-            for (int i = tid; i < ncx; i += CA_THREADS) crow[i] = bflag[i];
-            fl = bflag;
+            if (ncx <= CA_MAX_CELLS) fl = bflag;
+            else __syncthreads();  // the flags are read back from memory below
         }
         if constexpr (APPLY) {  // else flags only: NMS applies them on its staged tiles
             for (int s0 = 0; s0 < n_chunks; s0 += CA_SEG) {

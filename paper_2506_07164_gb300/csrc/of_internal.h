@@ -183,7 +183,7 @@ int fast_cstrip_blocks_per_sm();
 // to the maps (else NMS applies them on its staged tiles).
 void launch_cell_apply(const Img* imgs, const int32_t* img_list, const int32_t* band_prefix, int n_list, int n_bands,
                        int t_hi, int t_lo, int border, int cell, int grid, void* stream, int flags, bool apply = true);
-constexpr int CA_MAX_CELLS = 1024;  // cells per band row the threshold pass can flag itself
+constexpr int CA_MAX_CELLS = 1024;  // cells of a band row that the threshold pass flags in one round
 void launch_nms_harris(const Img* imgs, const int32_t* img_list, const int32_t* tile_prefix,
                        int n_list, int n_tiles, const CUtensorMap* img_maps,
                        const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo,
