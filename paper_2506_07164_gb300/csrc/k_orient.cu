@@ -109,7 +109,7 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
 #pragma unroll
         for (int k = 0; k < OP_WORDS; ++k) {
             const int i = lane + 32 * k, r = i / OP_WORDS, c = i - r * OP_WORDS;
-            v[k] = i < pw.whole && c < pw.nw ? __ldg(reinterpret_cast<const uint32_t*>(q + (size_t)r * pitch) + c) : 0u;
+            v[k] = i < pw.whole && c < pw.nw ? reinterpret_cast<const uint32_t*>(q + (size_t)r * pitch)[c] : 0u;
         }
         if (GROUPED) {
             // The run of this code in a window of 32 entries, and the better ones of it.

@@ -241,7 +241,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {
                 const int i = i0 + k * i_step;
-                v[k] = i < n2 ? __ldg(ck2 + i) : make_ulonglong2(0ull, 0ull);
+                v[k] = i < n2 ? ck2[i] : make_ulonglong2(0ull, 0ull);
             }
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k)
@@ -250,7 +250,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
                     atomicAdd(&hist[key_code(v[k].y)], 1u);
                 }
         }
-        if ((n & 1) && tid == 0 && rank == 0) atomicAdd(&hist[key_code(__ldg(I.ckey + n - 1))], 1u);
+        if ((n & 1) && tid == 0 && rank == 0) atomicAdd(&hist[key_code(I.ckey[n - 1])], 1u);
         if (shared) cluster_sync_all();
         else __syncthreads();
         // Suffix sums: higher bins = better keys.  Shared scan: block r owns
@@ -348,7 +348,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         for (int i0 = i_first; i0 < n; i0 += 2 * SEL_UNROLL * i_step) {
             uint64_t v[2 * SEL_UNROLL];
 #pragma unroll
-            for (int k = 0; k < 2 * SEL_UNROLL; ++k) v[k] = i0 + k * i_step < n ? __ldg(I.ckey + i0 + k * i_step) : 0ull;
+            for (int k = 0; k < 2 * SEL_UNROLL; ++k) v[k] = i0 + k * i_step < n ? I.ckey[i0 + k * i_step] : 0ull;
 #pragma unroll
             for (int k = 0; k < 2 * SEL_UNROLL; ++k)
                 if (i0 + k * i_step < n && key_code(v[k]) == code_b) atomicAdd(&h2[fine_bits<5, 12>(v[k])], 1u);
@@ -427,11 +427,11 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         };
         if (__builtin_expect(mid_b >= 0, 0)) {
             for (int i = i_first; i < n; i += i_step) {
-                const uint64_t key = __ldg(I.ckey + i);
+                const uint64_t key = I.ckey[i];
                 const int code = (int)key_code(key);
                 const int mid = code == code_b ? (int)fine_bits<5, 12>(key) : -1;
                 if (code < code_b || (code == code_b && mid < mid_b)) continue;
-                const uint32_t yx = __ldg(I.cyx + i);
+                const uint32_t yx = I.cyx[i];
                 if (code == code_b && mid == mid_b) {
                     bound(key, yx);
                 } else {
@@ -445,8 +445,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {
                 const int i = i0 + k * i_step;
-                if (2 * i + 1 < n) v[k] = __ldg(ck2 + i);
-                else v[k] = make_ulonglong2(2 * i < n ? __ldg(I.ckey + 2 * i) : 0ull, 0ull);
+                if (2 * i + 1 < n) v[k] = ck2[i];
+                else v[k] = make_ulonglong2(2 * i < n ? I.ckey[2 * i] : 0ull, 0ull);
             }
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {
@@ -457,7 +457,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
                     const uint64_t key = h ? v[k].y : v[k].x;
                     const int code = (int)key_code(key);
                     if (code < code_b) continue;
-                    const uint32_t yx = __ldg(I.cyx + i);
+                    const uint32_t yx = I.cyx[i];
                     if (code > code_b) {
                         const int pos = take(&hist[code]);
                         if (pos < q) keep(pos, key, yx);
@@ -539,8 +539,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
 #pragma unroll
                 for (int k = 0; k < SEL_UNROLL; ++k) {
                     const int i = i0 + k * SELECT_THREADS;
-                    hi[k] = i < n ? __ldg(I.ckey + i) : 0ull;
-                    lo[k] = need_lo && i < n ? ~__ldg(I.cyx + i) : 0u;
+                    hi[k] = i < n ? I.ckey[i] : 0ull;
+                    lo[k] = need_lo && i < n ? ~I.cyx[i] : 0u;
                 }
 #pragma unroll
                 for (int k = 0; k < SEL_UNROLL; ++k) {
@@ -584,7 +584,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         if (tid == 0) s_cnt = st.n_take;
         __syncthreads();
         for (int i = tid; i < n; i += SELECT_THREADS) {
-            const int c = (int)key_code(__ldg(I.ckey + i));
+            const int c = (int)key_code(I.ckey[i]);
             if (c > code_b) atomicAdd(&hist[c], 1u);
         }
         __syncthreads();
@@ -598,8 +598,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         }
         __syncthreads();
         for (int i = tid; i < n; i += SELECT_THREADS) {
-            const uint64_t hi = __ldg(I.ckey + i);
-            const uint32_t yx = __ldg(I.cyx + i);
+            const uint64_t hi = I.ckey[i];
+            const uint32_t yx = I.cyx[i];
             const int c = (int)key_code(hi);
             const uint64_t mh = hi & msk_hi;
             if (c < code_b || (c == code_b && !(mh > pre_hi || (mh == pre_hi && (~yx & msk_lo) >= pre_lo)))) continue;
@@ -626,8 +626,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
             for (int k = 0; k < SEL_UNROLL; ++k) {
                 const int i = i0 + k * i_step;
                 if (i < n2) {
-                    if (2 * i + 1 < n) v[k] = __ldg(ck2 + i);
-                    else v[k] = make_ulonglong2(__ldg(I.ckey + 2 * i), 0ull);
+                    if (2 * i + 1 < n) v[k] = ck2[i];
+                    else v[k] = make_ulonglong2(I.ckey[2 * i], 0ull);
                 } else {
                     v[k] = make_ulonglong2(0ull, 0ull);
                 }
@@ -642,7 +642,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
                         const int pos = atomicAdd(&s_cnt, 1);
                         if (pos < sort_cap) {
                             skey[pos] = key;
-                            syx[pos] = __ldg(I.cyx + 2 * i + h);
+                            syx[pos] = I.cyx[2 * i + h];
                         }
                     }
                 }
@@ -673,8 +673,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {
                 const int i = i0 + k * SELECT_THREADS;
-                hi[k] = i < n ? __ldg(I.ckey + i) : 0ull;
-                yx[k] = i < n ? __ldg(I.cyx + i) : 0u;
+                hi[k] = i < n ? I.ckey[i] : 0ull;
+                yx[k] = i < n ? I.cyx[i] : 0u;
             }
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {

@@ -10,6 +10,10 @@
 // pdl_trigger lets the next kernel of the chain start; it is called first
 // thing, so that kernel's blocks take their places as soon as the SMs have
 // room.  Without `pdl` both are no-ops.
+// What a kernel of the chain writes is read by the later ones with plain loads:
+// they may be resident while it is written, and the non-coherent path (__ldg)
+// is for data that does not change while the reading kernel runs.  That path is
+// left to what the host wrote before the chain (descriptors, item tables).
 #pragma once
 #include <cuda_runtime.h>
 
