@@ -676,7 +676,7 @@ k_fast_cstrip(const Img* __restrict__ imgs, const uint2* __restrict__ items, int
                 if (tn < n_tiles) mbar_wait(&mbar[w][b ^ 1], ((it + 1) >> 1) & 1, OF_WAIT_LIMIT_NS / 8);
             }
             __syncwarp();
-            return;
+            break;  // to the wait at the end
         }
         const TileInfo ti = tinfo[w][b];
         const Img& I = imgs[ti.img];
@@ -755,7 +755,7 @@ k_fast_cstrip(const Img* __restrict__ imgs, const uint2* __restrict__ items, int
         }
         __syncwarp();  // every lane is done with buffer b before lane 0 refills it
     }
-    pdl_wait();
+    pdl_wait();  // also behind a wait that expired: this kernel's end implies its predecessors'
 }
 
 void launch_fast_cstrip(const Img* imgs, const uint2* items, int n_strips, const CUtensorMap* maps, const Call* call,

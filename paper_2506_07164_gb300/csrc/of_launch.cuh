@@ -5,8 +5,10 @@
 // chain.  Launched with `pdl` (programmatic stream serialization), a kernel may
 // start while its predecessor still runs: it reads descriptors, sets up its
 // barriers and then waits (pdl_wait) for the predecessor's grid to complete
-// and its writes to be visible.  Every kernel of a chain waits in every thread
-// before it ends, so a kernel's completion implies its predecessors'.
+// and its writes to be visible.  A kernel launched this way waits in every
+// thread before it ends, on every path (one that gives up on an expired wait
+// among them), so a kernel's completion implies its predecessors'; one that is
+// launched plainly starts behind them and need not wait.
 // pdl_trigger lets the next kernel of the chain start; it is called first
 // thing, so that kernel's blocks take their places as soon as the SMs have
 // room.  Without `pdl` both are no-ops.
