@@ -16,6 +16,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -247,7 +248,6 @@ struct Plan {
     std::vector<PyrJob> h_pj;        // jobs of all runs (one per frame and run)
     std::vector<int> pj_frame, pj_level;  // frame and source level of each job
     std::vector<std::pair<int, int>> pj_tiles;  // tile columns and rows of each job
-    std::vector<int32_t> pblk;       // the jobs' axis tables
     std::vector<uint2> items_py;     // (job in its run, (tile row << 16) | tile column) per group and run
     bool cell_tiles = false;     // the cell size allows the cell-tile FAST kernel
     bool apply_flags = false;    // the threshold pass can set the cell flags (else the general FAST kernel does)
@@ -597,68 +597,71 @@ PyrShape pyr_shape(const std::vector<FrameKey>& frames) {
     return {px < 800000 ? 64 : px < 3000000 ? 96 : 128, 1.9};
 }
 
-// Split the levels 1 .. L-1 of every frame into runs that k_pyramid computes in
-// one launch each: a run takes as many levels as keep the seams within the
-// shape's bound.  Frames of one size share their tables.  No runs (the staged
-// kernel) when some level's source steps or pieces do not fit (scales above 3).
-void plan_pyramid(Plan* P) {
-    const int nl = P->s.levels, nf = (int)P->frames.size();
-    struct Piece {
-        int level, nl, ntx, nty, xoff, yoff;
-        ofh::PyrAxis x, y;
+// The runs of a plan's frame sizes, and where each run's tables go: word offsets
+// of its column and row blocks in a part of `words` words.
+struct PyrPlan {
+    struct Size {
+        std::vector<int32_t> ws, hs;
+        std::vector<const int32_t*> xtab, ytab;
+        std::vector<ofh::PyrPiece> pieces;
+        std::vector<std::pair<size_t, size_t>> at;
     };
-    std::map<std::pair<int, int>, std::vector<Piece>> made;  // per frame size: its runs
+    std::map<std::pair<int, int>, Size> made;
+    size_t words = 0;
+    void write(int32_t* to) const {
+        std::memset(to, 0, sizeof(int32_t) * words);
+        for (const auto& m : made)
+            for (size_t i = 0; i < m.second.pieces.size(); ++i)
+                ofh::pyramid_tables(m.second.pieces[i], m.second.ws, m.second.hs, m.second.xtab, m.second.ytab,
+                                    to + m.second.at[i].first, to + m.second.at[i].second);
+    }
+};
+
+// Split the levels 1 .. L-1 of every frame into runs that k_pyramid computes in
+// one launch each (pyramid_pieces); table(n_src, n_dst): the plan's resize table.
+// Frames of one size share their tables.  No runs (the staged kernel) when some
+// level's source steps or pieces do not fit (scales above 3).
+//
+// This is part of the first call with a shape: 128 frames of as many sizes, first
+// call 32 ms when every try of the search made its resize tables and blocks, 13
+// with the plan's tables, ranges alone in the search and the blocks written once,
+// into the upload (12 before the fused kernel; each later call 1.25 times faster).
+template <typename Table>
+PyrPlan plan_pyramid(Plan* P, Table&& table) {
+    const int nl = P->s.levels, nf = (int)P->frames.size();
+    PyrPlan pp;
     const PyrShape shape = pyr_shape(P->frames);
     size_t n_runs = 0;
     bool ok = nl > 1 && pyramid_raise_smem();
     for (int f = 0; f < nf && ok; ++f) {
         const std::pair<int, int> key(P->frames[f].w, P->frames[f].h);
-        if (made.count(key)) continue;
-        std::vector<Piece>& v = made[key];
-        std::vector<int32_t> ws, hs;
+        if (pp.made.count(key)) continue;
+        PyrPlan::Size& z = pp.made[key];
         for (int l = 0; l < nl && P->h_img[f * nl + l].w > 0; ++l) {
-            ws.push_back(P->h_img[f * nl + l].w);
-            hs.push_back(P->h_img[f * nl + l].h);
+            z.ws.push_back(P->h_img[f * nl + l].w);
+            z.hs.push_back(P->h_img[f * nl + l].h);
+            z.xtab.push_back(l > 0 ? table(z.ws[l - 1], z.ws[l]) : nullptr);
+            z.ytab.push_back(l > 0 ? table(z.hs[l - 1], z.hs[l]) : nullptr);
         }
-        for (int a = 0; a + 1 < (int)ws.size() && ok;) {
-            bool found = false;
-            for (int t = shape.tile; t >= 32 && !found; t = t > 128 ? 128 : t / 2)
-                for (int n = std::min((int)ws.size() - 1 - a, PY_MAX_LEVELS); n >= 1 && !found; --n) {
-                    Piece p;
-                    p.level = a;
-                    p.nl = n;
-                    p.ntx = (ws[a] + t - 1) / t;
-                    p.nty = (hs[a] + t - 1) / t;
-                    p.x = ofh::pyramid_axis(ws.data() + a, n, p.ntx, 256);
-                    std::vector<int32_t> row_words(n + 1);
-                    for (int l = 0; l <= n; ++l) row_words[l] = std::max(p.x.extent[l], 16) / 4;
-                    p.y = ofh::pyramid_axis(hs.data() + a, n, p.nty, 256, row_words.data());
-                    if (!p.x.ok || !p.y.ok) continue;
-                    const double seam = (double)p.x.computed * p.y.computed / ((double)p.x.owned * p.y.owned);
-                    if (n > 1 && seam > shape.max_seam) continue;
-                    p.xoff = (int)P->pblk.size();
-                    P->pblk.insert(P->pblk.end(), p.x.blk.begin(), p.x.blk.end());
-                    p.yoff = (int)P->pblk.size();
-                    P->pblk.insert(P->pblk.end(), p.y.blk.begin(), p.y.blk.end());
-                    v.push_back(p);
-                    a += n;
-                    found = true;
-                }
-            ok = found;
+        ok = ofh::pyramid_pieces(z.ws, z.hs, z.xtab, z.ytab, PY_MAX_LEVELS, shape.tile, shape.max_seam, z.pieces);
+        for (const ofh::PyrPiece& p : z.pieces) {
+            const size_t x = pp.words, y = x + (size_t)p.x.stride * p.x.nt;
+            pp.words = y + (size_t)p.y.stride * p.y.nt;
+            z.at.emplace_back(x, y);
         }
-        n_runs = std::max(n_runs, v.size());
+        n_runs = std::max(n_runs, z.pieces.size());
     }
     for (size_t c = 0; c < n_runs && ok; ++c) {
         Plan::Run R;
         R.job_begin = (int)P->h_pj.size();
         for (int f = 0; f < nf; ++f) {
-            const std::vector<Piece>& v = made[std::make_pair(P->frames[f].w, P->frames[f].h)];
-            if (c >= v.size()) continue;
-            const Piece& p = v[c];
+            const PyrPlan::Size& z = pp.made[std::make_pair(P->frames[f].w, P->frames[f].h)];
+            if (c >= z.pieces.size()) continue;
+            const ofh::PyrPiece& p = z.pieces[c];
             PyrJob J;
             std::memset(&J, 0, sizeof(J));
-            J.xblk = reinterpret_cast<const int32_t*>((intptr_t)p.xoff);  // word offsets until the block has an address
-            J.yblk = reinterpret_cast<const int32_t*>((intptr_t)p.yoff);
+            J.xblk = reinterpret_cast<const int32_t*>((intptr_t)z.at[c].first);  // word offsets until the block has an address
+            J.yblk = reinterpret_cast<const int32_t*>((intptr_t)z.at[c].second);
             J.xstride = p.x.stride;
             J.ystride = p.y.stride;
             J.nl = p.nl;
@@ -692,8 +695,9 @@ void plan_pyramid(Plan* P) {
         P->pj_frame.clear();
         P->pj_level.clear();
         P->pj_tiles.clear();
-        P->pblk.clear();
+        pp = PyrPlan();
     }
+    return pp;
 }
 
 int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings& s,
@@ -837,7 +841,7 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
         }
     }
     P->rs_begin[nl] = (int)P->h_rs.size();
-    plan_pyramid(P);
+    const PyrPlan pyr = plan_pyramid(P, [&](int n_src, int n_dst) { return P->tables.data() + tab_of.at(std::make_pair(n_src, n_dst)); });
     for (int i = 0; i < P->n_img; ++i) {
         const Img& I = P->h_img[i];
         if (I.tiles_x > 0) {
@@ -1060,7 +1064,7 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     P->off_pj = off;
     off = align_up(off + sizeof(PyrJob) * std::max<size_t>(P->h_pj.size(), 1), 16);
     P->off_pblk = off;
-    off = align_up(off + sizeof(int32_t) * std::max<size_t>(P->pblk.size(), 1), 16);
+    off = align_up(off + sizeof(int32_t) * std::max<size_t>(pyr.words, 1), 16);
     // Output slot -> image (slots of image i: [slot0, slot0 + layout quota)).
     P->slot_img.assign(std::max(P->total_slots, 1), 0);
     for (int i = 0; i < P->n_img; ++i) {
@@ -1090,9 +1094,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
         J.xblk = d_pblk + reinterpret_cast<intptr_t>(J.xblk);
         J.yblk = d_pblk + reinterpret_cast<intptr_t>(J.yblk);
     }
-    std::vector<uint8_t> blob(off, 0);
+    const std::unique_ptr<uint8_t[]> blob(new uint8_t[off]);  // written below but for the gaps between its parts
     auto put = [&](size_t at, const void* src, size_t n) {
-        if (n) std::memcpy(blob.data() + at, src, n);
+        if (n) std::memcpy(blob.get() + at, src, n);
     };
     put(P->off_call, &C, sizeof(C));
     put(P->off_img, P->h_img.data(), sizeof(Img) * P->h_img.size());
@@ -1113,9 +1117,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     put(P->off_idt, P->items_dt.data(), sizeof(uint2) * P->items_dt.size());
     put(P->off_ipy, P->items_py.data(), sizeof(uint2) * P->items_py.size());
     put(P->off_pj, P->h_pj.data(), sizeof(PyrJob) * P->h_pj.size());
-    put(P->off_pblk, P->pblk.data(), sizeof(int32_t) * P->pblk.size());
+    pyr.write(reinterpret_cast<int32_t*>(blob.get() + P->off_pblk));
     put(P->off_sli, P->slot_img.data(), sizeof(uint16_t) * P->slot_img.size());
-    e = cudaMemcpy(P->dbuf, blob.data(), off, cudaMemcpyHostToDevice);
+    e = cudaMemcpy(P->dbuf, blob.get(), off, cudaMemcpyHostToDevice);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         e = cudaMallocHost(&P->stage[i], P->header_bytes);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->ev[i], cudaEventDisableTiming);

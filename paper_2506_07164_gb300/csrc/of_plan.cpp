@@ -88,44 +88,32 @@ bool k_fraction(float k, int64_t* num, int64_t* den) {
 // A level's column groups n (at most 64) and ceil(2^16 / n), which divides thread numbers by n: n | m << 8.
 static int32_t pack_groups(int n) { return n > 0 ? n | ((65536 + n - 1) / n << 8) : 0; }
 
-PyrAxis pyramid_axis(const int32_t* sizes, int nl, int nt, int max_extent, const int32_t* row_words) {
-    const bool columns = row_words == nullptr;
+static PyrAxis pyramid_ranges(const int32_t* sizes, const int32_t* const* tab, int nl, int nt, int max_extent, bool columns) {
     PyrAxis A;
     A.nt = nt;
     A.nl = nl;
-    A.ok = true;
-    std::vector<std::vector<int32_t>> tab(nl + 1);
-    for (int l = 1; l <= nl; ++l) {
-        tab[l].resize(sizes[l]);
-        resize_table(sizes[l - 1], sizes[l], tab[l].data());
-        if (columns)
-            for (int d = 1; d < sizes[l]; ++d)
-                if ((tab[l][d] >> 12) - (tab[l][d - 1] >> 12) > 3) A.ok = false;
-    }
     // Tile boundaries: equal shares of every level, columns at multiples of 4.
     auto bound = [&](int l, int i) {
         if (i >= nt) return sizes[l];
         const int b = (int)((int64_t)sizes[l] * i / nt);
         return columns ? b & ~3 : b;
     };
-    struct Range {
-        int c0 = 0, c1 = 0, o0 = 0, o1 = 0;
-    };
-    std::vector<std::vector<Range>> tiles(nt, std::vector<Range>(nl + 1));
+    A.ranges.assign((size_t)nt * (nl + 1), PyrRange());
     A.extent.assign(nl + 1, 0);
     int words = 0;
     for (int i = 0; i < nt; ++i) {
+        PyrRange* const tile = A.ranges.data() + (size_t)i * (nl + 1);
         int n = 4 * (nl + 1);
         for (int l = nl; l >= 0; --l) {
-            Range& R = tiles[i][l];
+            PyrRange& R = tile[l];
             int n0 = 0, n1 = 0;  // needed: the owned range and the sources of the next level's computed range
             if (l > 0) {
                 R.o0 = n0 = bound(l, i);
                 R.o1 = n1 = std::max(bound(l, i + 1), R.o0);
             }
-            if (l < nl && tiles[i][l + 1].c1 > tiles[i][l + 1].c0) {
-                const Range& N = tiles[i][l + 1];
-                const int d1 = std::min(N.c1, (int)sizes[l + 1]) - 1;
+            if (l < nl && tile[l + 1].c1 > tile[l + 1].c0) {
+                const PyrRange& N = tile[l + 1];
+                const int d1 = std::min(N.c1, sizes[l + 1]) - 1;
                 const int s0 = tab[l + 1][N.c0] >> 12, s1 = std::min((tab[l + 1][d1] >> 12) + 1, sizes[l] - 1) + 1;
                 if (n1 > n0) {
                     n0 = std::min(n0, s0);
@@ -149,50 +137,98 @@ PyrAxis pyramid_axis(const int32_t* sizes, int nl, int nt, int max_extent, const
         }
         words = std::max(words, n);
     }
-    if (A.extent[0] > max_extent) A.ok = false;
+    A.ok = A.extent[0] <= max_extent;
     A.stride = (words + 3) / 4 * 4;
-    A.blk.assign((size_t)A.stride * nt, 0);
-    if (!A.ok) return A;
-    for (int i = 0; i < nt; ++i) {
-        int32_t* b = A.blk.data() + (size_t)A.stride * i;
+    return A;
+}
+
+static void pyramid_blocks(const PyrAxis& A, const int32_t* sizes, const int32_t* const* tab, const int32_t* row_words,
+                    int32_t* out) {
+    const bool columns = row_words == nullptr;
+    const int nl = A.nl;
+    for (int i = 0; i < A.nt; ++i) {
+        const PyrRange* const tile = A.ranges.data() + (size_t)i * (nl + 1);
+        int32_t* b = out + (size_t)A.stride * i;
         int32_t* e = b + 4 * (nl + 1);
         for (int l = 0; l <= nl; ++l) {
-            const Range& R = tiles[i][l];
+            const PyrRange& R = tile[l];
             b[4 * l] = R.c0;
             b[4 * l + 1] = !columns ? (R.c1 - R.c0) | row_words[l] << 16 : l > 0 ? pack_groups((R.c1 - R.c0) / 4) : R.c1 - R.c0;
             b[4 * l + 2] = R.o0;
             b[4 * l + 3] = R.o1;
             if (l == 0) continue;
-            const int s0 = tiles[i][l - 1].c0;
+            const int s0 = tile[l - 1].c0;
+            const int32_t* const tl = tab[l];
             if (!columns) {
+                const int rw = row_words[l - 1];
                 for (int d = R.c0; d < R.c1; ++d) {
-                    const int t = tab[l][d];
-                    *e++ = (int32_t)((uint32_t)(((t >> 12) - s0) * row_words[l - 1]) << 16) | 2 * (t & 4095);
+                    const int t = tl[d];
+                    *e++ = (int32_t)((uint32_t)(((t >> 12) - s0) * rw) << 16) | 2 * (t & 4095);
                 }
                 continue;
             }
-            for (int d = R.c0; d < R.c1; d += 4) {
-                int xo[4];
-                uint32_t wgt[4], sel[4];
-                for (int k = 0; k < 4; ++k) {
-                    const int t = tab[l][std::min(d + k, sizes[l] - 1)];
-                    const uint32_t a2 = 2u * (uint32_t)(t & 4095);
-                    xo[k] = (t >> 12) - s0;
-                    wgt[k] = (4096u - a2) | (a2 << 16);
-                }
-                const int wa = xo[0] >> 2, wb = xo[2] >> 2;
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t o = (uint32_t)(xo[k] - 4 * (k < 2 ? wa : wb));
-                    sel[k] = o | ((o + 1u) << 4);
-                }
+            auto weights = [](int t) { return (int32_t)(4096u + 2u * (uint32_t)(t & 4095) * 0xFFFFu); };  // 4096 - 2a | 2a << 16
+            auto pair = [](int o) { return (uint32_t)(o | (o + 1) << 4); };  // selects bytes o, o + 1
+            const int last = sizes[l] - 1;
+            for (int d = R.c0; d < R.c1; d += 4, e += 8) {
+                const int t0 = tl[std::min(d, last)], t1 = tl[std::min(d + 1, last)], t2 = tl[std::min(d + 2, last)],
+                          t3 = tl[std::min(d + 3, last)];
+                const int x0 = (t0 >> 12) - s0, x1 = (t1 >> 12) - s0, x2 = (t2 >> 12) - s0, x3 = (t3 >> 12) - s0;
+                const int wa = x0 >> 2, wb = x2 >> 2;
                 e[0] = wa | (wb << 16);
-                e[1] = (int32_t)(sel[0] | (sel[1] << 8) | (sel[2] << 16) | (sel[3] << 24));
-                for (int k = 0; k < 4; ++k) e[2 + k] = (int32_t)wgt[k];
-                e += 8;
+                e[1] = (int32_t)(pair(x0 - 4 * wa) | pair(x1 - 4 * wa) << 8 | pair(x2 - 4 * wb) << 16 | pair(x3 - 4 * wb) << 24);
+                e[2] = weights(t0);
+                e[3] = weights(t1);
+                e[4] = weights(t2);
+                e[5] = weights(t3);
             }
         }
     }
-    return A;
+}
+
+bool pyramid_pieces(const std::vector<int32_t>& ws, const std::vector<int32_t>& hs, const std::vector<const int32_t*>& xtab,
+                    const std::vector<const int32_t*>& ytab, int max_levels, int tile, double max_seam,
+                    std::vector<PyrPiece>& out) {
+    const int nl = (int)ws.size();
+    // Levels whose source columns step by at most 3 (the kernel picks byte pairs of 4 outputs from two
+    // words): a step is at most the ratio of the widths, rounded up.
+    std::vector<char> steps(nl, 1);
+    for (int l = 1; l < nl; ++l)
+        if (10 * (int64_t)ws[l - 1] > 29 * (int64_t)ws[l])
+            for (int d = 1; d < ws[l] && steps[l]; ++d) steps[l] = (xtab[l][d] >> 12) - (xtab[l][d - 1] >> 12) <= 3;
+    for (int a = 0; a + 1 < nl;) {
+        int most = 0;
+        while (a + 1 + most < nl && most < max_levels && steps[a + 1 + most]) ++most;
+        bool found = false;
+        for (int t = tile; t >= 32 && !found; t = t > 128 ? 128 : t / 2)
+            for (int n = most; n >= 1 && !found; --n) {
+                PyrPiece p;
+                p.level = a;
+                p.nl = n;
+                p.ntx = (ws[a] + t - 1) / t;
+                p.nty = (hs[a] + t - 1) / t;
+                p.x = pyramid_ranges(ws.data() + a, xtab.data() + a, n, p.ntx, 256, true);
+                // (A seam is at least its columns' part.)
+                if (!p.x.ok || (n > 1 && (double)p.x.computed > max_seam * (double)p.x.owned)) continue;
+                p.y = pyramid_ranges(hs.data() + a, ytab.data() + a, n, p.nty, 256, false);
+                if (!p.y.ok) continue;
+                const double seam = (double)p.x.computed * p.y.computed / ((double)p.x.owned * p.y.owned);
+                if (n > 1 && seam > max_seam) continue;
+                out.push_back(std::move(p));
+                a += n;
+                found = true;
+            }
+        if (!found) return false;
+    }
+    return true;
+}
+
+void pyramid_tables(const PyrPiece& p, const std::vector<int32_t>& ws, const std::vector<int32_t>& hs,
+                    const std::vector<const int32_t*>& xtab, const std::vector<const int32_t*>& ytab, int32_t* x, int32_t* y) {
+    std::vector<int32_t> row_words(p.nl + 1);
+    for (int l = 0; l <= p.nl; ++l) row_words[l] = std::max(p.x.extent[l], 16) / 4;
+    pyramid_blocks(p.x, ws.data() + p.level, xtab.data() + p.level, nullptr, x);
+    pyramid_blocks(p.y, hs.data() + p.level, ytab.data() + p.level, row_words.data(), y);
 }
 
 float response_scale(int64_t den) {
