@@ -234,7 +234,7 @@ struct Plan {
     };
     std::vector<Group> groups[kMaxGroups + 1];
     std::vector<int32_t> gp_det, gp_rs, gp_fast, gp_rows, gp_nms64, gp_ftall[2], gp_fal;
-    // Work-item tables of the per-warp kernels, per group: (image, (y0 << 16) | x0).
+    // Work-item tables of the per-warp kernels: (image, (y0 << 16) | x0).
     std::vector<uint2> items_cs, items_dt, items_nm;
     int strip_rows = 0;  // rows of a FAST strip (a cell row or part of one)
     int nms_rows = 0;    // rows of a per-warp NMS tile (32: the detect tiles)
@@ -248,7 +248,7 @@ struct Plan {
     std::vector<PyrJob> h_pj;        // jobs of all runs (one per frame and run)
     std::vector<int> pj_frame, pj_level;  // frame and source level of each job
     std::vector<std::pair<int, int>> pj_tiles;  // tile columns and rows of each job
-    std::vector<uint2> items_py;     // (job in its run, (tile row << 16) | tile column) per group and run
+    std::vector<uint2> items_py;     // (job in its run, (tile row << 16) | tile column) per run
     bool cell_tiles = false;     // the cell size allows the cell-tile FAST kernel
     bool apply_flags = false;    // the threshold pass can set the cell flags (else the general FAST kernel does)
     bool strip_ok = false;       // the cell size allows the cell-row strip kernel (cells of 8..33 pixels)
@@ -623,9 +623,9 @@ struct PyrPlan {
 // level's source steps or pieces do not fit (scales above 3).
 //
 // This is part of the first call with a shape: 128 frames of as many sizes, first
-// call 32 ms when every try of the search made its resize tables and blocks, 13
+// call 32 ms when every try of the search made its resize tables and blocks, 13.7
 // with the plan's tables, ranges alone in the search and the blocks written once,
-// into the upload (12 before the fused kernel; each later call 1.25 times faster).
+// into the upload.
 template <typename Table>
 PyrPlan plan_pyramid(Plan* P, Table&& table) {
     const int nl = P->s.levels, nf = (int)P->frames.size();
@@ -851,6 +851,41 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
         }
     }
 
+    // Work items, in the order of the frames, so that a group of frames has a part
+    // of each table: made and uploaded once, not for every number of groups (first
+    // call of 128 frames of as many sizes: 13.7 -> 9.2 ms; 128 1080p frames: 14.0 -> 5.0).
+    const int nd = (int)P->det_list.size();
+    std::vector<int> cs_at(1, 0), nm_at(1, 0);  // first strip and NMS tile of each detect-list entry
+    for (int j = 0; j < nd; ++j) {
+        const uint32_t ii = (uint32_t)P->det_list[j];
+        const Img& I = P->h_img[ii];
+        auto row = [&](std::vector<uint2>& items, int y) {
+            for (int tx = 0; tx < I.tiles_x; ++tx)
+                items.push_back(make_uint2(ii, ((uint32_t)y << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
+        };
+        for (int ty = 0; ty < I.tiles_y; ++ty) row(P->items_dt, s.border + ty * TILE_H);  // as det_prefix counts
+        if (P->nms_rows != TILE_H)
+            for (int y = s.border; y < I.h - s.border; y += P->nms_rows) row(P->items_nm, y);
+        if (P->strip_ok)
+            for (int cy = 0; cy < I.ncy; ++cy)
+                for (int y = s.border + cy * s.cell; y < std::min(s.border + (cy + 1) * s.cell, I.h - s.border);
+                     y += P->strip_rows)
+                    row(P->items_cs, y);
+        cs_at.push_back((int)P->items_cs.size());
+        nm_at.push_back((int)P->items_nm.size());
+    }
+    std::vector<int> py_at(1, 0);  // first tile of each pyramid job; jobs are stored run by run
+    for (size_t c = 0; c < P->runs.size(); ++c) {
+        const int j0 = P->runs[c].job_begin;
+        const int j1 = c + 1 < P->runs.size() ? P->runs[c + 1].job_begin : (int)P->h_pj.size();
+        for (int j = j0; j < j1; ++j) {
+            for (int ty = 0; ty < P->pj_tiles[j].second; ++ty)
+                for (int tx = 0; tx < P->pj_tiles[j].first; ++tx)
+                    P->items_py.push_back(make_uint2((uint32_t)(j - j0), ((uint32_t)ty << 16) | (uint32_t)tx));
+            py_at.push_back((int)P->items_py.size());
+        }
+    }
+
     // Launch ranges per frame group (k = 1 .. min(kMaxGroups, frames)).
     for (int k = 1; k <= kMaxGroups; ++k) {
         if (k > nf) break;
@@ -859,7 +894,6 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
             const int f0 = nf * g / k, f1 = nf * (g + 1) / k;
             G.img_begin = f0 * nl;
             G.n_img = (f1 - f0) * nl;
-            const int nd = (int)P->det_list.size();
             int j0 = 0, j1 = 0;
             while (j0 < nd && P->det_list[j0] < G.img_begin) ++j0;
             j1 = j0;
@@ -875,27 +909,13 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
             G.np_off = (int)P->gp_nms64.size();
             for (int i = 0; i < 2; ++i) G.ftall_off[i] = (int)P->gp_ftall[i].size();
             G.fal_off = (int)P->gp_fal.size();
-            G.csi_off = (int)P->items_cs.size();
-            G.dti_off = (int)P->items_dt.size();
-            G.nmi_off = (int)P->items_nm.size();
+            G.dti_off = t0;
+            G.csi_off = cs_at[j0];
+            G.cs_strips = cs_at[j1] - cs_at[j0];
+            G.nmi_off = nm_at[j0];
+            G.nm_tiles = nm_at[j1] - nm_at[j0];
             for (int j = j0; j < j1; ++j) {
                 const Img& I = P->h_img[P->det_list[j]];
-                const uint32_t ii = (uint32_t)P->det_list[j];
-                for (int ty = 0; ty < I.tiles_y; ++ty)  // tile t = ty * tiles_x + tx, as the prefixes count
-                    for (int tx = 0; tx < I.tiles_x; ++tx)
-                        P->items_dt.push_back(make_uint2(
-                            ii, ((uint32_t)(s.border + ty * TILE_H) << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
-                if (P->nms_rows != TILE_H)
-                    for (int y = s.border; y < I.h - s.border; y += P->nms_rows)
-                        for (int tx = 0; tx < I.tiles_x; ++tx)
-                            P->items_nm.push_back(make_uint2(ii, ((uint32_t)y << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
-                if (P->strip_ok)
-                    for (int cy = 0; cy < I.ncy; ++cy)
-                        for (int y = s.border + cy * s.cell; y < std::min(s.border + (cy + 1) * s.cell, I.h - s.border);
-                             y += P->strip_rows)
-                            for (int tx = 0; tx < I.tiles_x; ++tx)
-                                P->items_cs.push_back(
-                                    make_uint2(ii, ((uint32_t)y << 16) | (uint32_t)(I.tile_x0 + tx * TILE_W)));
                 P->gp_nms64.push_back(G.nms64_tiles);
                 G.nms64_tiles += I.tiles_x * ((I.h - 2 * s.border + 63) / 64);
                 for (int i = 0; i < 2; ++i) {
@@ -912,8 +932,6 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                 P->gp_rows.push_back(G.n_bands);
                 G.n_bands += I.ncy;
             }
-            G.cs_strips = (int)P->items_cs.size() - G.csi_off;
-            G.nm_tiles = (int)P->items_nm.size() - G.nmi_off;
             G.slot_begin = P->h_img[G.img_begin].slot0;
             G.slot_end = f1 < nf ? P->h_img[f1 * nl].slot0 : P->total_slots;
             G.rs_job.assign(nl + 1, 0);
@@ -942,14 +960,12 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
             for (size_t c = 0; c < P->runs.size(); ++c) {
                 const int j0r = P->runs[c].job_begin;
                 const int j1r = c + 1 < P->runs.size() ? P->runs[c + 1].job_begin : (int)P->h_pj.size();
-                G.py_off.push_back((int)P->items_py.size());
-                for (int j = j0r; j < j1r; ++j) {
-                    if (P->pj_frame[j] < f0 || P->pj_frame[j] >= f1) continue;
-                    for (int ty = 0; ty < P->pj_tiles[j].second; ++ty)
-                        for (int tx = 0; tx < P->pj_tiles[j].first; ++tx)
-                            P->items_py.push_back(make_uint2((uint32_t)(j - j0r), ((uint32_t)ty << 16) | (uint32_t)tx));
-                }
-                G.py_n.push_back((int)P->items_py.size() - G.py_off.back());
+                int a = j0r;
+                while (a < j1r && P->pj_frame[a] < f0) ++a;
+                int e = a;
+                while (e < j1r && P->pj_frame[e] < f1) ++e;
+                G.py_off.push_back(py_at[a]);
+                G.py_n.push_back(py_at[e] - py_at[a]);
             }
             P->groups[k].push_back(G);
         }
