@@ -15,13 +15,17 @@
 //     code > b go straight to the places that the counts of the better bins
 //     give them; those of bin b (at most SEL_BND) go through the same step
 //     once more, by the next 9 bits of |key|, and the few of that boundary
-//     are ranked by counting (more than SEL_BND in bin b: the cluster first
-//     splits the bin by the next 12 bits; some 4K frames, whole call 324 us
-//     when the first block's radix select took them, 205 now);
-//   - otherwise an MSB-first radix select over 8-bit digits of R (one
-//     shared-memory histogram per pass) fixes, digit by digit, the prefix of
-//     the n_l-th largest R, stopping as soon as every candidate that shares
-//     the fixed prefix is needed, and those candidates are gathered.
+//     are ranked by counting.  More than SEL_BND in bin b: the cluster first
+//     narrows the bin by 12 bits of R at a time, from the highest bit in which
+//     its candidates differ (one round for most 4K frames that need it, whole
+//     call 324 us by a radix select of the first block, 205 now; equal keys,
+//     say of a printed grid, go straight to the bits of their positions: a grid
+//     at 1080p, 8192 features, top-N stage 256 us by radix select, 39 now);
+//   - sorted lists whose gathered candidates do not fit: an MSB-first radix
+//     select over 8-bit digits of R (one shared-memory histogram per pass)
+//     fixes, digit by digit, the prefix of the n_l-th largest R, stopping as
+//     soon as every candidate that shares the fixed prefix is needed, and
+//     those candidates are gathered.
 // Sorted lists are bitonic-sorted by R, descending; strides below 64 run in a
 // warp's registers (shuffles), the rest through shared memory.
 //
@@ -55,6 +59,7 @@ constexpr int SEL_SOLO_G = 8192;  // ... of a grouped list (no sort beside it)
 constexpr int SEL_MIN_SORT = 64;  // entries of the smallest sort (one warp's registers)
 constexpr int SEL_MAX_DYN = 192 * 1024;
 constexpr int SEL_BND = 2048;   // grouped lists: candidates of the boundary bin the first block takes
+constexpr int SEL_RANK = 128;   // ... and ranks by counting
 constexpr int SEL_GROUPED = 32;  // images of a launch up to which the lists stay grouped
 
 struct SelState {
@@ -62,17 +67,42 @@ struct SelState {
     uint32_t pre_lo, msk_lo;
     int need, done;
     int coarse, code_b, n_take;
-    int mid_b, sure;  // grouped: boundary of the split bin (-1: not split), candidates above it
+    int split, sure;  // grouped: the bin was narrowed to the prefix, its candidates above that
 };
 
-// N bits of the magnitude after the leading one and the next SKIP bits, for keys
-// that agree in those: non-decreasing in key.  The code's bits end at SKIP = 5.
-template <int SKIP, int N>
+// The 9 bits of the magnitude after those of the code, for keys of one code:
+// non-decreasing in key.
 __device__ __forceinline__ uint32_t fine_bits(uint64_t u) {
     const bool pos = (u >> 63) != 0;
     const uint64_t x = pos ? u & 0x7FFFFFFFFFFFFFFFull : u ^ 0x7FFFFFFFFFFFFFFFull;
-    const uint32_t f = x ? (uint32_t)((x << __clzll((long long)x) << (1 + SKIP)) >> (64 - N)) : 0u;
-    return pos ? f : (1u << N) - 1u - f;
+    const uint32_t f = x ? (uint32_t)((x << __clzll((long long)x) << 6) >> 55) : 0u;
+    return pos ? f : 511u - f;
+}
+
+// The N bits of rank words that start at the highest bit in which some of them
+// differ: `all` and `any` are their AND and OR as three words, highest first.
+template <int N>
+struct RankDigit {
+    int sh;  // the digit is bits sh .. sh + N - 1 of the 96; the words agree above
+    __device__ __forceinline__ RankDigit(const uint32_t* all, const uint32_t* any) {
+        const uint32_t d0 = all[0] ^ any[0], d1 = all[1] ^ any[1], d2 = all[2] ^ any[2];
+        const int p = d0 ? 95 - __clz(d0) : d1 ? 63 - __clz(d1) : 31 - __clz(d2);
+        sh = max(p - N + 1, 0);
+    }
+    __device__ __forceinline__ uint32_t of(uint64_t hi, uint32_t lo) const {
+        return (uint32_t)(sh >= 32 ? hi >> (sh - 32) : hi << (32 - sh) | lo >> sh) & ((1u << N) - 1u);
+    }
+};
+// AND (words 0 .. 2) and OR (3 .. 5) of the warps' rank words into `bits`, preset to ones and zeros.
+__device__ __forceinline__ void merge_bits(uint32_t* bits, const uint32_t (&all)[3], const uint32_t (&any)[3], int lane) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const uint32_t a = __reduce_and_sync(0xFFFFFFFFu, all[j]), o = __reduce_or_sync(0xFFFFFFFFu, any[j]);
+        if (lane == 0) {
+            atomicAnd(&bits[j], a);
+            atomicOr(&bits[3 + j], o);
+        }
+    }
 }
 
 // ---- cluster primitives (shared::cluster addresses of the other blocks' shared memory)
@@ -177,6 +207,222 @@ __device__ __forceinline__ void bitonic_sort(uint64_t* skey, uint32_t* syx, int 
     }
 }
 
+// Sum over the block's threads after this one.
+__device__ __forceinline__ int threads_after(int own, uint32_t* wsum, int tid) {
+    const int lane = tid & 31, warp = tid >> 5;
+    int v = own;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int t = __shfl_down_sync(0xFFFFFFFFu, v, off);
+        if (lane + off < 32) v += t;
+    }
+    if (lane == 0) wsum[warp] = (uint32_t)v;
+    __syncthreads();
+    int above = v - own;
+    for (int w = warp + 1; w < SELECT_THREADS / 32; ++w) above += (int)wsum[w];
+    return above;
+}
+
+// What the narrowing of ties shares: AND and OR of rank words (the block's, the
+// cluster's), a split's boundary digit, the number needed of it and held by it.
+struct TieState {
+    uint32_t bits[6], all[6];
+    int pick[3];
+};
+
+// A grouped list's boundary bin that holds too many for the first block: the
+// cluster narrows it, 12 bits of the rank words at a time from the highest bit in
+// which its candidates differ (equal keys differ in their positions), until few
+// enough share the boundary's prefix.  Counted where they go later.  Kept out of
+// the kernel's own code, which most images run through without it.
+template <int C>
+__device__ __noinline__ void narrow_bin(const uint64_t* ckey, const uint32_t* cyx, int n, int parts, int q, uint64_t* bkey,
+                                        uint32_t* wsum, TieState& T, SelState& st, int* s_cnt) {
+    const int tid = threadIdx.x, lane = tid & 31, rank = (int)(blockIdx.x % C);
+    const bool shared = parts > 1;
+    const int i_first = rank * SELECT_THREADS + tid, i_step = parts * SELECT_THREADS;
+    uint32_t* const h2 = reinterpret_cast<uint32_t*>(bkey);
+    static_assert(SEL_BND * sizeof(uint64_t) >= SEL_BINS * sizeof(uint32_t), "room for the counts");
+    const uint32_t code_b = (uint32_t)st.code_b;
+    const int need0 = q - st.n_take;
+    int need = need0;
+    uint64_t pre_hi = 0ull, msk_hi = 0ull;
+    uint32_t pre_lo = 0u, msk_lo = 0u;
+    auto sync = [&] {
+        if (shared) cluster_sync_all();
+        else __syncthreads();
+    };
+    auto each = [&](auto&& f) {  // this block's candidates of the bin with the prefix
+        for (int i0 = i_first; i0 < n; i0 += SEL_UNROLL * i_step) {
+            uint64_t hi[SEL_UNROLL];
+            uint32_t lo[SEL_UNROLL];
+#pragma unroll
+            for (int k = 0; k < SEL_UNROLL; ++k) {
+                const int i = i0 + k * i_step;
+                hi[k] = i < n ? ckey[i] : 0ull;
+                lo[k] = i < n ? ~cyx[i] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < SEL_UNROLL; ++k)
+                if (i0 + k * i_step < n && key_code(hi[k]) == code_b && (hi[k] & msk_hi) == pre_hi &&
+                    (lo[k] & msk_lo) == pre_lo)
+                    f(hi[k], lo[k]);
+        }
+    };
+    for (int left = SEL_BND + 1, round = 0; left > SEL_BND && round < 8; ++round) {  // 12 of 96 bits a round
+        if (tid < 6) T.bits[tid] = tid < 3 ? 0xFFFFFFFFu : 0u;
+        if (tid < 3) T.pick[tid] = 0;  // ends the loop in all blocks alike
+        for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) h2[i] = 0u;
+        __syncthreads();
+        uint32_t all[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, any[3] = {0u, 0u, 0u};
+        each([&](uint64_t hi, uint32_t lo) {
+            const uint32_t w[3] = {(uint32_t)(hi >> 32), (uint32_t)hi, lo};
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                all[j] &= w[j];
+                any[j] |= w[j];
+            }
+        });
+        merge_bits(T.bits, all, any, lane);
+        sync();
+        if (tid < 6) {
+            uint32_t v = T.bits[tid];
+            for (int c = 0; c < parts && shared; ++c) {
+                const uint32_t o = ld_rank(map_rank(&T.bits[tid], c));
+                v = tid < 3 ? v & o : v | o;
+            }
+            T.all[tid] = v;
+        }
+        __syncthreads();
+        const RankDigit<12> dg(T.all, T.all + 3);
+        each([&](uint64_t hi, uint32_t lo) { atomicAdd(&h2[dg.of(hi, lo)], 1u); });
+        sync();
+        if (rank == 0) {
+            constexpr int PER1 = SEL_BINS / SELECT_THREADS;
+            int bins[PER1], own = 0;
+#pragma unroll
+            for (int j = 0; j < PER1; ++j) {
+                uint32_t h = 0u;
+                for (int c = 0; c < parts; ++c) h += shared ? ld_rank(map_rank(&h2[PER1 * tid + j], c)) : h2[PER1 * tid + j];
+                bins[j] = (int)h;
+                own += (int)h;
+            }
+            const int above = threads_after(own, wsum, tid);
+            if (above < need && above + own >= need) {  // exactly one thread
+                int cum = above;
+#pragma unroll
+                for (int j = PER1 - 1; j >= 0; --j) {
+                    if (cum < need && cum + bins[j] >= need) {
+                        const int pick[3] = {PER1 * tid + j, need - cum, bins[j]};
+                        for (int c = 0; c < parts; ++c)
+                            for (int e = 0; e < 3; ++e) {
+                                if (c == 0) T.pick[e] = pick[e];
+                                else st_rank(map_rank(&T.pick[e], c), (uint32_t)pick[e]);
+                            }
+                    }
+                    cum += bins[j];
+                }
+            }
+        }
+        sync();
+        // The words agree above the digit: the prefix is their common bits and the digit.
+        const uint64_t d = (uint64_t)T.pick[0];
+        need = T.pick[1];
+        left = T.pick[2];
+        const int sh = dg.sh;
+        const uint64_t common = (uint64_t)T.all[0] << 32 | T.all[1];
+        if (sh >= 32) {
+            msk_hi = ~0ull << (sh - 32);
+            pre_hi = (common & ~(0xFFFull << (sh - 32)) & msk_hi) | d << (sh - 32);
+        } else {
+            msk_hi = ~0ull;
+            pre_hi = (common & ~(0xFFFull >> (32 - sh))) | d >> (32 - sh);
+            msk_lo = ~0u << sh;
+            pre_lo = (T.all[2] & ~(0xFFFu << sh) & msk_lo) | (uint32_t)d << sh;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        st.pre_hi = pre_hi;
+        st.msk_hi = msk_hi;
+        st.pre_lo = pre_lo;
+        st.msk_lo = msk_lo;
+        st.sure = need0 - need;
+        st.split = 1;
+        st.coarse = 1;
+        *s_cnt = st.n_take;  // where the bin's sure ones go
+    }
+    sync();
+}
+
+// The first block's boundary candidates `left` (nl of them, the best one's place
+// `base`): while they are more than SEL_RANK they are narrowed by 9 bits of their
+// rank words at a time, the better ones kept; the rest is ranked by counting.
+__device__ __noinline__ void rank_ties(const uint64_t* bkey, const uint32_t* byx, uint32_t* hist, uint16_t* left, int nl,
+                                       int base, int q, uint32_t* wsum, TieState& T, int* s_left, int* s_cnt, int* s_fine,
+                                       uint64_t* kkey, uint32_t* kyx) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint16_t* next = reinterpret_cast<uint16_t*>(hist + 2048);
+    static_assert(2 * SEL_BND <= 4 * 1024, "room for the lists behind the 512 counts");
+    for (int round = 0; nl > SEL_RANK && round < 11; ++round) {
+        if (tid < 6) T.bits[tid] = tid < 3 ? 0xFFFFFFFFu : 0u;
+        hist[tid] = 0u;
+        if (tid == 0) {
+            *s_left = 0;
+            *s_cnt = base;
+        }
+        __syncthreads();
+        uint32_t all[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, any[3] = {0u, 0u, 0u};
+        for (int i = tid; i < nl; i += SELECT_THREADS) {
+            const uint64_t hi = bkey[left[i]];
+            const uint32_t w[3] = {(uint32_t)(hi >> 32), (uint32_t)hi, ~byx[left[i]]};
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                all[j] &= w[j];
+                any[j] |= w[j];
+            }
+        }
+        merge_bits(T.bits, all, any, lane);
+        __syncthreads();
+        const RankDigit<9> dg(T.bits, T.bits + 3);
+        for (int i = tid; i < nl; i += SELECT_THREADS) atomicAdd(&hist[dg.of(bkey[left[i]], ~byx[left[i]])], 1u);
+        __syncthreads();
+        const int own = (int)hist[tid], better = threads_after(own, wsum, tid);
+        if (base + better < q && base + better + own >= q) *s_fine = tid | better << 9;
+        __syncthreads();
+        const int fine = *s_fine & 511;
+        for (int i = tid; i < nl; i += SELECT_THREADS) {
+            const int e = left[i], c = (int)dg.of(bkey[e], ~byx[e]);
+            if (c > fine) {
+                const int pos = atomicAdd(s_cnt, 1);
+                if (pos < q) {
+                    kkey[pos] = bkey[e];
+                    kyx[pos] = byx[e];
+                }
+            } else if (c == fine) {
+                next[atomicAdd(s_left, 1)] = (uint16_t)e;
+            }
+        }
+        __syncthreads();
+        base += *s_fine >> 9;
+        nl = *s_left;
+        uint16_t* const t = left;
+        left = next;
+        next = t;
+        __syncthreads();
+    }
+    for (int i = tid; i < nl; i += SELECT_THREADS) {
+        const uint64_t key = bkey[left[i]];
+        const uint32_t yx = byx[left[i]];
+        int place = base;
+        for (int j = 0; j < nl; ++j) place += rank_less(key, ~yx, bkey[left[j]], ~byx[left[j]]);
+        if (place < q) {
+            kkey[place] = key;
+            kyx[place] = yx;
+        }
+    }
+}
+
 template <int C, bool GROUPED>
 __global__ void __launch_bounds__(SELECT_THREADS)
 k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_cap) {
@@ -189,6 +435,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
     __shared__ uint64_t bkey[GROUPED ? SEL_BND : 1];  // the boundary bin's candidates (first block)
     __shared__ uint32_t byx[GROUPED ? SEL_BND : 1];
     __shared__ int s_bnd, s_left, s_fine;  // their number, that of the fine boundary bin, its code
+    __shared__ TieState tie;
 
     const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;  // block's place in its image's cluster
     // Images are stored frame by frame; a grid of two dimensions takes them level by level.
@@ -222,7 +469,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         st.coarse = GROUPED && n <= q;  // a grouped list of everything: no boundary bin
         st.code_b = GROUPED && n <= q ? -1 : 0;
         st.n_take = m;
-        st.mid_b = -1;
+        st.split = 0;
         st.sure = 0;
         s_cnt = 0;
         s_bnd = 0;
@@ -338,67 +585,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
     }
 
     if (GROUPED && __builtin_expect(!st.coarse, 0)) {  // the same in all blocks
-        // The boundary bin holds too many for the first block: the cluster splits it by
-        // the next 12 bits of the keys, counted where its candidates go later.
-        uint32_t* const h2 = reinterpret_cast<uint32_t*>(bkey);
-        static_assert(SEL_BND * sizeof(uint64_t) >= SEL_BINS * sizeof(uint32_t), "room for the counts");
-        const uint32_t code_b = (uint32_t)st.code_b;
-        for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) h2[i] = 0u;
-        __syncthreads();
-        for (int i0 = i_first; i0 < n; i0 += 2 * SEL_UNROLL * i_step) {
-            uint64_t v[2 * SEL_UNROLL];
-#pragma unroll
-            for (int k = 0; k < 2 * SEL_UNROLL; ++k) v[k] = i0 + k * i_step < n ? I.ckey[i0 + k * i_step] : 0ull;
-#pragma unroll
-            for (int k = 0; k < 2 * SEL_UNROLL; ++k)
-                if (i0 + k * i_step < n && key_code(v[k]) == code_b) atomicAdd(&h2[fine_bits<5, 12>(v[k])], 1u);
-        }
-        if (shared) cluster_sync_all();
-        else __syncthreads();
-        if (rank == 0) {
-            constexpr int PER1 = SEL_BINS / SELECT_THREADS;
-            const int need = q - st.n_take;
-            int bins[PER1], own = 0;
-#pragma unroll
-            for (int j = 0; j < PER1; ++j) {
-                uint32_t h = 0u;
-                for (int c = 0; c < parts; ++c) h += shared ? ld_rank(map_rank(&h2[PER1 * tid + j], c)) : h2[PER1 * tid + j];
-                bins[j] = (int)h;
-                own += (int)h;
-            }
-            int v = own;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int t = __shfl_down_sync(0xFFFFFFFFu, v, off);
-                if (lane + off < 32) v += t;
-            }
-            if (lane == 0) wsum[warp] = (uint32_t)v;
-            __syncthreads();
-            int above = v - own;
-            for (int w = warp + 1; w < SELECT_THREADS / 32; ++w) above += (int)wsum[w];
-            if (above < need && above + own >= need) {  // exactly one thread
-                int cum = above;
-#pragma unroll
-                for (int j = PER1 - 1; j >= 0; --j) {
-                    if (cum < need && cum + bins[j] >= need && bins[j] <= SEL_BND) {
-                        s_cnt = st.n_take;  // where the split bin's sure ones go
-                        st.sure = cum;
-                        for (int c = 0; c < parts; ++c) {
-                            if (c == 0) {
-                                st.mid_b = PER1 * tid + j;
-                                st.coarse = 1;
-                            } else {
-                                st_rank(map_rank(&st.mid_b, c), (uint32_t)(PER1 * tid + j));
-                                st_rank(map_rank(&st.coarse, c), 1u);
-                            }
-                        }
-                    }
-                    cum += bins[j];
-                }
-            }
-        }
-        if (shared) cluster_sync_all();
-        else __syncthreads();
+        narrow_bin<C>(I.ckey, I.cyx, n, parts, q, bkey, wsum, tie, st, &s_cnt);
     }
     auto keep = [&](int pos, uint64_t key, uint32_t yx) {
         I.kkey[pos] = key;
@@ -406,7 +593,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
     };
     if (GROUPED && st.coarse) {  // the same in all blocks
         // Gather: the better bins to their places, the boundary bin to the first block.
-        const int code_b = st.code_b, mid_b = st.mid_b;
+        const int code_b = st.code_b;
+        const bool split = st.split != 0;
         const ulonglong2* ck2 = reinterpret_cast<const ulonglong2*>(I.ckey);
         const int n2 = (n + 1) >> 1;
         // A place of the first block's counter.
@@ -425,22 +613,35 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
                 }
             }
         };
-        if (__builtin_expect(mid_b >= 0, 0)) {
-            for (int i = i_first; i < n; i += i_step) {
-                const uint64_t key = I.ckey[i];
-                const int code = (int)key_code(key);
-                const int mid = code == code_b ? (int)fine_bits<5, 12>(key) : -1;
-                if (code < code_b || (code == code_b && mid < mid_b)) continue;
-                const uint32_t yx = I.cyx[i];
-                if (code == code_b && mid == mid_b) {
-                    bound(key, yx);
-                } else {
-                    const int pos = code > code_b ? take(&hist[code]) : take(&s_cnt);
-                    if (pos < q) keep(pos, key, yx);
+        if (__builtin_expect(split, 0)) {
+            const uint64_t pre_hi = st.pre_hi, msk_hi = st.msk_hi;
+            const uint32_t pre_lo = st.pre_lo, msk_lo = st.msk_lo;
+            for (int i0 = i_first; i0 < n; i0 += SEL_UNROLL * i_step) {
+                uint64_t hi[SEL_UNROLL];
+                uint32_t yx[SEL_UNROLL];
+#pragma unroll
+                for (int k = 0; k < SEL_UNROLL; ++k) {
+                    const int i = i0 + k * i_step;
+                    hi[k] = i < n ? I.ckey[i] : 0ull;
+                    yx[k] = i < n ? I.cyx[i] : 0u;
+                }
+#pragma unroll
+                for (int k = 0; k < SEL_UNROLL; ++k) {
+                    const int code = (int)key_code(hi[k]);
+                    if (i0 + k * i_step >= n || code < code_b) continue;
+                    const uint64_t mh = hi[k] & msk_hi;
+                    const uint32_t ml = ~yx[k] & msk_lo;
+                    if (code == code_b && rank_less(mh, ml, pre_hi, pre_lo)) continue;
+                    if (code == code_b && mh == pre_hi && ml == pre_lo) {
+                        bound(hi[k], yx[k]);
+                    } else {
+                        const int pos = code > code_b ? take(&hist[code]) : take(&s_cnt);
+                        if (pos < q) keep(pos, hi[k], yx[k]);
+                    }
                 }
             }
         }
-        for (int i0 = mid_b < 0 ? i_first : n2; i0 < n2; i0 += SEL_UNROLL * i_step) {
+        for (int i0 = split ? n2 : i_first; i0 < n2; i0 += SEL_UNROLL * i_step) {
             ulonglong2 v[SEL_UNROLL];
 #pragma unroll
             for (int k = 0; k < SEL_UNROLL; ++k) {
@@ -471,57 +672,59 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         else __syncthreads();
         if (rank != 0) return;
         // The boundary bin: its best fill the rest, found by the fine codes.
-        static_assert(SELECT_THREADS == 512, "one fine code per thread");
+        static_assert(SELECT_THREADS == 512, "one fine code, or digit of a rank word, per thread");
         const int nb = min(s_bnd, SEL_BND), above = st.n_take + st.sure, need = q - above;
         if (nb == 0) {
             if (tid == 0) I.ctr[1] = above;
             return;
         }
-        hist[tid] = 0u;
-        if (tid == 0) {
-            s_left = 0;
-            s_cnt = above;
-        }
-        __syncthreads();
-        auto fine_code = [&](uint64_t key) { return mid_b < 0 ? fine_bits<5, 9>(key) : fine_bits<17, 9>(key); };
-        for (int i = tid; i < nb; i += SELECT_THREADS) atomicAdd(&hist[fine_code(bkey[i])], 1u);
-        __syncthreads();
-        const int own = (int)hist[tid];
-        int v = own;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int t = __shfl_down_sync(0xFFFFFFFFu, v, off);
-            if (lane + off < 32) v += t;
-        }
-        if (lane == 0) wsum[warp] = (uint32_t)v;
-        __syncthreads();
-        int better = v - own;
-        for (int w = warp + 1; w < SELECT_THREADS / 32; ++w) better += (int)wsum[w];
-        if (better < need && better + own >= need) s_fine = tid | better << 9;  // exactly one thread
-        __syncthreads();
-        const int fine = s_fine & 511, sure = s_fine >> 9;  // candidates above the fine boundary bin
-        uint16_t* const left = reinterpret_cast<uint16_t*>(hist);  // its candidates' places in the list
-        for (int i = tid; i < nb; i += SELECT_THREADS) {
-            const int c = (int)fine_code(bkey[i]);
-            if (c > fine) {
-                const int pos = atomicAdd(&s_cnt, 1);
-                keep(pos, bkey[i], byx[i]);
-            } else if (c == fine) {
-                left[atomicAdd(&s_left, 1)] = (uint16_t)i;
+        uint16_t* const left = reinterpret_cast<uint16_t*>(hist + 1024);  // boundary candidates
+        int base = above, nl = nb;  // the place of the best of them, their number
+        if (!split) {
+            hist[tid] = 0u;
+            if (tid == 0) {
+                s_left = 0;
+                s_cnt = above;
             }
+            __syncthreads();
+            for (int i = tid; i < nb; i += SELECT_THREADS) atomicAdd(&hist[fine_bits(bkey[i])], 1u);
+            __syncthreads();
+            const int own = (int)hist[tid], better = threads_after(own, wsum, tid);
+            if (better < need && better + own >= need) s_fine = tid | better << 9;  // exactly one thread
+            __syncthreads();
+            const int fine = s_fine & 511;
+            base += s_fine >> 9;  // candidates above the fine boundary bin
+            for (int i = tid; i < nb; i += SELECT_THREADS) {
+                const int c = (int)fine_bits(bkey[i]);
+                if (c > fine) {
+                    const int pos = atomicAdd(&s_cnt, 1);
+                    keep(pos, bkey[i], byx[i]);
+                } else if (c == fine) {
+                    left[atomicAdd(&s_left, 1)] = (uint16_t)i;
+                }
+            }
+            __syncthreads();
+            nl = s_left;
+        } else {
+            for (int i = tid; i < nb; i += SELECT_THREADS) left[i] = (uint16_t)i;
+            __syncthreads();
         }
-        __syncthreads();
-        const int nl = s_left;
+        if (__builtin_expect(nl > SEL_RANK, 0)) {
+            rank_ties(bkey, byx, hist, left, nl, base, q, wsum, tie, &s_left, &s_cnt, &s_fine, I.kkey, I.kyx);
+            nl = 0;
+        }
         for (int i = tid; i < nl; i += SELECT_THREADS) {
             const uint64_t key = bkey[left[i]];
             const uint32_t yx = byx[left[i]];
-            int place = above + sure;
+            int place = base;
             for (int j = 0; j < nl; ++j) place += rank_less(key, ~yx, bkey[left[j]], ~byx[left[j]]);
             if (place < q) keep(place, key, yx);
         }
         if (tid == 0) I.ctr[1] = q;
         return;
     }
+
+    if constexpr (GROUPED) return;  // (done above: its boundary bin is always narrowed)
 
     // The radix select (and the gather without a coarse bin) is the first block's alone.
     if (rank != 0 && !st.coarse) return;
@@ -571,45 +774,6 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
             }
             __syncthreads();
         }
-    }
-
-    if (GROUPED) {
-        // Keep the better bins whole, and of bin b every candidate whose masked rank
-        // word is >= the fixed prefix.  The places of the digits' histogram were lost:
-        // count the bins again.
-        const uint64_t pre_hi = st.pre_hi, msk_hi = st.msk_hi;
-        const uint32_t pre_lo = st.pre_lo, msk_lo = st.msk_lo;
-        const int code_b = st.code_b;
-        for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) hist[i] = 0u;
-        if (tid == 0) s_cnt = st.n_take;
-        __syncthreads();
-        for (int i = tid; i < n; i += SELECT_THREADS) {
-            const int c = (int)key_code(I.ckey[i]);
-            if (c > code_b) atomicAdd(&hist[c], 1u);
-        }
-        __syncthreads();
-        if (tid == 0) {  // a rare path: one thread turns the counts into places
-            uint32_t place = 0u;
-            for (int i = SEL_BINS - 1; i > code_b; --i) {
-                const uint32_t h = hist[i];
-                hist[i] = place;
-                place += h;
-            }
-        }
-        __syncthreads();
-        for (int i = tid; i < n; i += SELECT_THREADS) {
-            const uint64_t hi = I.ckey[i];
-            const uint32_t yx = I.cyx[i];
-            const int c = (int)key_code(hi);
-            const uint64_t mh = hi & msk_hi;
-            if (c < code_b || (c == code_b && !(mh > pre_hi || (mh == pre_hi && (~yx & msk_lo) >= pre_lo)))) continue;
-            const int pos = c > code_b ? (int)atomicAdd(&hist[c], 1u) : atomicAdd(&s_cnt, 1);
-            if (pos < q) {
-                keep(pos, hi, yx);
-            }
-        }
-        if (tid == 0) I.ctr[1] = q;
-        return;
     }
 
     // Gather: code >= b (coarse; each block its part of the candidates), else
