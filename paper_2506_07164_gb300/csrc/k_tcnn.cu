@@ -33,14 +33,16 @@ constexpr int C1 = 8, C2 = 16, C3 = 16;
 constexpr int W1 = 0, B1 = W1 + C1 * 9, W2 = B1 + C1, B2 = W2 + C2 * C1 * 9, W3 = B2 + C2,
               B3 = W3 + C3 * C2 * 9, WF = B3 + C3, BF = WF + C3, NP = BF + 1;
 static_assert(NP == 3585, "parameter count");
-constexpr int LOSS_AT = (NP + 1) / 2 * 2;  // 8-byte aligned word after the gradient
+// Behind the gradient, on 8 bytes: the loss and the last bias' gradient, sums over all patches of numbers of
+// both signs, as doubles (the latter rounded where it is read).
+constexpr int LOSS_AT = (NP + 1) / 2 * 2, GRAD_WORDS = LOSS_AT + 4;
 
 }  // namespace tn
 
 struct of_tcnn {
     float* master = nullptr;  // fp32 master weights [NP]
     __nv_bfloat16* w = nullptr;  // bf16 compute weights [NP]
-    float* grad = nullptr;    // fp32 gradients [NP], then (LOSS_AT) the loss as a double
+    float* grad = nullptr;    // fp32 gradients [NP] (the last bias' apart), then (LOSS_AT) what a step sums in double
     float* m = nullptr;       // Adam moments
     float* v = nullptr;
     int64_t step = 0;
@@ -470,8 +472,11 @@ k_forward_fast(PatchSrc src, int n, const __nv_bfloat16* __restrict__ wq, float*
 // two 16 x 8 tiles per warp, dW1 as one 9 x 8 tile per warp (its pixel rows).
 // Bound by the latency of the phases (issue 46 %, shared memory 54 %, tensor
 // pipe 30 %).  2048 patches: 2000 us as three fp32 kernels (1674 of them the
-// backward's scalar loops), 127 us here.  Against 64 bits, 24 batches: gradient
-// 1.7e-7 of its norm off (median; 2.3e-7 before), loss 1.9e-8 (3.3e-8).
+// backward's scalar loops), 127 us here.  Against 64 bits (medians of 48 batches of
+// the committed network; before, as fp32 kernels): gradient 1.6e-7 of its norm off
+// (2.2e-7), by layer, weights and bias: 1.6e-7, 1.2e-7 (2.7e-7, 1.7e-7); 1.7e-7,
+// 1.4e-7 (2.2e-7, 1.9e-7); 1.6e-7, 1.4e-7 (2.2e-7, 1.9e-7); head 1.4e-7, 2.7e-8
+// (1.6e-7, 1.0e-7; its bias summed in fp32 atomics was 1.2e-7 off).
 constexpr int TR_THREADS = 512, TR_WARPS = TR_THREADS / 32;
 constexpr int M3_ROW = 9, M3_PLANE = 9 * M3_ROW * 16;      // layer-3 mask: 8 x 8 pixels, a zero row and column; one channel half
 constexpr int D2_ROW = 17, D2_PLANE = 17 * D2_ROW * 16;    // d2: 16 x 16 pixels, a zero row and column; one part and half
@@ -932,8 +937,8 @@ k_train(const uint8_t* __restrict__ tiles, const float* __restrict__ labels, int
             atomicAdd(grad + B3 + lane, gb3);
         }
         if (lane == 0) {
-            atomicAdd(grad + BF, gbf);
             atomicAdd(loss, lsum / (double)n);
+            atomicAdd(loss + 1, (double)gbf);
         }
     }
     __syncthreads();
@@ -946,11 +951,11 @@ k_train(const uint8_t* __restrict__ tiles, const float* __restrict__ labels, int
 }
 
 __global__ void k_adam(float* __restrict__ master, __nv_bfloat16* __restrict__ wq, const float* __restrict__ g,
-                       float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2, float eps,
+                       const double* __restrict__ g_last, float* __restrict__ m, float* __restrict__ v, float lr, float b1, float b2, float eps,
                        float wd, float c1, float c2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NP) return;
-    const float gi = g[i];
+    const float gi = i == BF ? (float)*g_last : g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
     m[i] = mi;
@@ -1107,7 +1112,7 @@ of_tcnn* of_tcnn_create(uint64_t seed) {
     cudaGetDevice(&N->device);
     const size_t b = sizeof(float) * tn::NP;
     if (cudaMalloc(&N->master, b) != cudaSuccess || cudaMalloc(&N->w, sizeof(__nv_bfloat16) * tn::NP) != cudaSuccess ||
-        cudaMalloc(&N->grad, sizeof(float) * (tn::LOSS_AT + 2)) != cudaSuccess || cudaMalloc(&N->m, b) != cudaSuccess ||
+        cudaMalloc(&N->grad, sizeof(float) * tn::GRAD_WORDS) != cudaSuccess || cudaMalloc(&N->m, b) != cudaSuccess ||
         cudaMalloc(&N->v, b) != cudaSuccess) {
         tn::fail(OF_ERR_CUDA, "tile-net allocation failed");
         of_tcnn_destroy(N);
@@ -1149,7 +1154,7 @@ int of_tcnn_set_params(of_tcnn* N, const float* host) {
     const size_t b = sizeof(float) * tn::NP;
     if (cudaMemcpy(N->master, host, b, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(N->m, 0, b) != cudaSuccess || cudaMemset(N->v, 0, b) != cudaSuccess ||
-        cudaMemset(N->grad, 0, b) != cudaSuccess)
+        cudaMemset(N->grad, 0, sizeof(float) * tn::GRAD_WORDS) != cudaSuccess)
         return tn::fail(OF_ERR_CUDA, "tile-net upload failed");
     tn::k_round<<<(tn::NP + 255) / 256, 256>>>(N->master, N->w);
     N->step = 0;
@@ -1163,7 +1168,12 @@ int of_tcnn_get_params(of_tcnn* N, int which, float* host) {
     if (which == 0) {
         e = cudaMemcpy(host, N->master, b, cudaMemcpyDeviceToHost);
     } else if (which == 2) {
-        e = cudaMemcpy(host, N->grad, b, cudaMemcpyDeviceToHost);
+        std::vector<float> g(tn::GRAD_WORDS);
+        e = cudaMemcpy(g.data(), N->grad, sizeof(float) * tn::GRAD_WORDS, cudaMemcpyDeviceToHost);
+        double last = 0.0;
+        std::memcpy(&last, g.data() + tn::LOSS_AT + 2, sizeof(last));
+        g[tn::BF] = (float)last;
+        if (e == cudaSuccess) std::memcpy(host, g.data(), b);
     } else {
         float* tmp = nullptr;
         e = cudaMalloc(&tmp, b);
@@ -1189,7 +1199,7 @@ int of_tcnn_loss_grad(of_tcnn* N, const uint8_t* tiles, const float* labels, int
     if (!N || !tiles || !labels || n < 1 || !(pos_weight > 0.f)) return tn::fail(OF_ERR_ARG, "bad arguments");
     cudaStream_t st = (cudaStream_t)stream;
     double* const loss = reinterpret_cast<double*>(N->grad + tn::LOSS_AT);
-    cudaMemsetAsync(N->grad, 0, sizeof(float) * (tn::LOSS_AT + 2), st);
+    cudaMemsetAsync(N->grad, 0, sizeof(float) * tn::GRAD_WORDS, st);
     const int sms = tn::sm_count();
     tn::k_train<<<n < sms ? n : sms, tn::TR_THREADS, tn::TR_SMEM, st>>>(tiles, labels, n, pos_weight, N->w, N->grad, loss);
     if (cudaGetLastError() != cudaSuccess) return tn::fail(OF_ERR_CUDA, "tile-net training launch failed");
@@ -1208,7 +1218,8 @@ int of_tcnn_adam(of_tcnn* N, float lr, float beta1, float beta2, float eps, floa
         return tn::fail(OF_ERR_ARG, "bad Adam arguments");
     N->step += 1;
     const float c1 = 1.f - std::pow(beta1, (float)N->step), c2 = 1.f - std::pow(beta2, (float)N->step);
-    tn::k_adam<<<(tn::NP + 255) / 256, 256, 0, (cudaStream_t)stream>>>(N->master, N->w, N->grad, N->m, N->v, lr,
+    const double* const last = reinterpret_cast<const double*>(N->grad + tn::LOSS_AT) + 1;
+    tn::k_adam<<<(tn::NP + 255) / 256, 256, 0, (cudaStream_t)stream>>>(N->master, N->w, N->grad, last, N->m, N->v, lr,
                                                                         beta1, beta2, eps, weight_decay, c1, c2);
     return cudaGetLastError() == cudaSuccess ? OF_OK : tn::fail(OF_ERR_CUDA, "Adam launch failed");
 }
