@@ -125,14 +125,13 @@ __device__ __forceinline__ uint16_t q_entry(int row, int col) { return (uint16_t
 
 // Step 2 for one thread: strict 3x3 maxima of its 4 columns x RPT rows of the
 // staged score rows sS (staged row 0 = tile row -1), appended to queue with
-// one shared atomic per warp (count in *nq; with nq null the queue is the
-// warp's own and the count is returned).  MASK: the staged scores are the
+// one shared atomic per warp (count in *nq).  MASK: the staged scores are the
 // raw maps, so bytes outside [lox, hix) x [ry0, ry1) are masked here.  Rows
 // below the detect region hold no survivor; a warp entirely below it only
 // takes part in the queue.
 template <bool MASK, int RPT>
-__device__ __forceinline__ int nms_queue(const uint8_t* __restrict__ sS, int X0, int Y0, int lox, int hix, int ry0,
-                                         int ry1, int lane, int ty, uint16_t* __restrict__ queue, int* nq) {
+__device__ __forceinline__ void nms_queue(const uint8_t* __restrict__ sS, int X0, int Y0, int lox, int hix, int ry0,
+                                          int ry1, int lane, int ty, uint16_t* __restrict__ queue, int* nq) {
     const int nrows = min(RPT, ry1 - (Y0 + ty * RPT));
     // Survivor bits (2 * row + pair) * 2 + lane: 4 per row, 64-bit beyond 8 rows.
     using SMask = typename std::conditional<(RPT > 8), unsigned long long, uint32_t>::type;
@@ -194,18 +193,15 @@ __device__ __forceinline__ int nms_queue(const uint8_t* __restrict__ sS, int X0,
         const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
         if (lane >= o) incl += v;
     }
-    // nq null: the queue is the warp's own (entries from 0; the count is returned).
     int wbase = 0;
-    if (nq != nullptr && lane == 31 && incl) wbase = atomicAdd(nq, incl);
+    if (lane == 31 && incl) wbase = atomicAdd(nq, incl);
     int slot = __shfl_sync(0xFFFFFFFFu, wbase, 31) + incl - mine;
-    const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
     while (smask) {
         const int bit = (RPT > 8 ? __ffsll((long long)smask) : __ffs((int)smask)) - 1;
         smask &= smask - 1u;
         // bit = 2 (2 row + pair) + lane: column 4 lane + pair + 2 lane
         queue[slot++] = q_entry(ty * RPT + (bit >> 2), 4 * lane + ((bit >> 1) & 1) + 2 * (bit & 1));
     }
-    return total;
 }
 
 // Step 3-4 for the block: Harris sums and key of every queued survivor of the
