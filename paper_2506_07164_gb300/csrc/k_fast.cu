@@ -611,7 +611,7 @@ int fast_warp_blocks_per_sm() {
 // one entry per item instead of searching the image list, which was a chain
 // of dependent loads the rest of the warp waited on (FAST 2.06 -> 1.99 ms).
 // In small batches an item is a part of a cell row (`sub` rows; its flags OR
-// into the same cells): 1480 strips of a 1080p frame are fewer than the 2432
+// into the same cells): 1640 strips of a 1080p frame are fewer than the 2432
 // resident warps.  Items go to blocks first, then to their warps, so that few
 // items spread over all SMs (8 1080p frames: 151 -> 141 us, a stereo pair of
 // 720p frames 32 -> 28).  Launched beside the pyramid's end, the strips of

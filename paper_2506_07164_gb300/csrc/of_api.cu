@@ -250,7 +250,7 @@ struct Plan {
     std::vector<std::pair<int, int>> pj_tiles;  // tile columns and rows of each job
     std::vector<uint2> items_py;     // (job in its run, (tile row << 16) | tile column) per run
     bool cell_tiles = false;     // the cell size allows the cell-tile FAST kernel
-    bool apply_flags = false;    // the threshold pass can set the cell flags (else the general FAST kernel does)
+    bool apply_flags = false;    // the threshold pass sets the cell flags (else the general FAST kernel does)
     bool strip_ok = false;       // the cell size allows the cell-row strip kernel (cells of 8..33 pixels)
     bool aligned_ok = false;     // ... and the cell-aligned general FAST kernel (cells of 15 or 30 pixels)
     int det_tiles = 0, max_quota = 0, total_slots = 0, n_img = 0;
@@ -306,7 +306,7 @@ struct Plan {
 // final scores themselves.  Otherwise the threshold pass applies the cell
 // flags to the maps; it also sets them, unless the FAST kernel did: the
 // cell-row strips (form 4) always, the general block kernel when the pass
-// cannot flag a band's cells (more than CA_MAX_CELLS cells per row).
+// would flag a band's cells in more than one round (CA_MAX_CELLS).
 bool cell_form(const Plan* P) {
     const int f = P->tun.fast_cell_tiles;
     return P->cell_tiles && (f == 1 || f == 2);
@@ -733,8 +733,8 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     P->strip_rows = std::min(s.cell, std::max(part, 8));
     P->nms_rows = strips < 700 ? 8 : strips < 1200 ? 16 : TILE_H;
     P->pdl = strips < 12000;
-    // The threshold pass flags the cells itself when a band's cells fit its
-    // shared array; otherwise the general FAST kernel sets them.
+    // The threshold pass flags the cells itself when it takes a band's cells in
+    // one round; otherwise the general FAST kernel sets them.
     P->apply_flags = true;
     for (const auto& L : P->lay.img)
         if (L.ncx > CA_MAX_CELLS) P->apply_flags = false;
