@@ -72,8 +72,9 @@ k_cell_apply(const Img* __restrict__ imgs, const int32_t* __restrict__ list, con
             // CA_MAX_CELLS cells of the band at a time (one round but for rows of more).
             for (int g0 = 0; g0 < ncx; g0 += CA_MAX_CELLS) {
                 const int ng = min(CA_MAX_CELLS, ncx - g0);
-                const int ch0 = (border + g0 * cell - xb0) >> 4;
-                const int ch1 = min(n_chunks, (border + (g0 + ng) * cell - xb0 + 15) >> 4);
+                // The round's columns and chunks (a chunk at its edge holds cells of two rounds).
+                const int xa = border + g0 * cell, xe = min(rx1, xa + ng * cell);
+                const int ch0 = (xa - xb0) >> 4, ch1 = (xe - xb0 + 15) >> 4;
                 __syncthreads();  // the last readers of bflag and colmask are done
                 for (int i = tid; i < ng; i += CA_THREADS) bflag[i] = 0u;
                 __syncthreads();
@@ -117,11 +118,10 @@ k_cell_apply(const Img* __restrict__ imgs, const int32_t* __restrict__ list, con
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
                             const int xx = x + i;
-                            if (((wd[i >> 2] >> (8 * (i & 3) + 7)) & 1u) && xx >= border && xx < rx1) {
-                                const int cx = (int)__umulhi((uint32_t)(xx - border), magic);
+                            if (((wd[i >> 2] >> (8 * (i & 3) + 7)) & 1u) && xx >= xa && xx < xe) {
+                                const int cx = (int)__umulhi((uint32_t)(xx - xa), magic);
                                 if (cx != last) {
-                                    // A chunk at a round's edge holds cells of both rounds.
-                                    if ((uint32_t)(cx - g0) < (uint32_t)ng) atomicOr(&bflag[cx - g0], 1u);
+                                    atomicOr(&bflag[cx], 1u);
                                     last = cx;
                                 }
                             }
