@@ -5,27 +5,21 @@
 //
 // Each candidate has a unique 96-bit rank word
 //   R = (key ^ 2^63) << 32 | ~((y << 16) | x),
-// larger R = better rank.  The candidates above the n_l-th largest R are
-// found in one of two ways:
-//   - coarse pass: a 4096-bin histogram of a code of the key that is
-//     monotone in the key (sign, bit length and the next 5 bits of |key|)
-//     locates the bin b holding the n_l-th largest key.  Sorted list: every
-//     candidate with code >= b is gathered (when they fit in shared memory)
-//     and sorted, and the first n_l are kept.  Grouped list: candidates with
-//     code > b go straight to the places that the counts of the better bins
-//     give them; those of bin b (at most SEL_BND) go through the same step
-//     once more, by the next 9 bits of |key|, and the few of that boundary
-//     are ranked by counting.  More than SEL_BND in bin b: the cluster first
-//     narrows the bin by 12 bits of R at a time, from the highest bit in which
-//     its candidates differ (one round for most 4K frames that need it, whole
-//     call 324 us by a radix select of the first block, 205 now; equal keys,
-//     say of a printed grid, go straight to the bits of their positions: a grid
-//     at 1080p, 8192 features, top-N stage 256 us by radix select, 39 now);
-//   - sorted lists whose gathered candidates do not fit: an MSB-first radix
-//     select over 8-bit digits of R (one shared-memory histogram per pass)
-//     fixes, digit by digit, the prefix of the n_l-th largest R, stopping as
-//     soon as every candidate that shares the fixed prefix is needed, and
-//     those candidates are gathered.
+// larger R = better rank.  A 4096-bin histogram of a code of the key that is
+// monotone in the key (sign, bit length and the next 5 bits of |key|) locates the
+// bin b holding the n_l-th largest key.  Then
+//   - sorted list: every candidate with code >= b is gathered and sorted, and the
+//     first n_l are kept;
+//   - grouped list: candidates with code > b go straight to the places that the
+//     counts of the better bins give them; those of bin b go through the same step
+//     once more, by the next 9 bits of |key|, and the few of that boundary are
+//     ranked by counting.
+// A bin b that holds too many for that (the sort buffer, or SEL_BND) is narrowed
+// first, by 12 bits of R at a time from the highest bit in which its candidates
+// differ: one round for most 4K frames that need it; equal keys, say of a printed
+// grid, go straight to the bits of their positions.  (By an MSB-first radix select
+// of one block instead: some 4K frames 324 us a call, 205 so; a 1080p grid, 8192
+// features, 256 us for the stage, 39 so.)
 // Sorted lists are bitonic-sorted by R, descending; strides below 64 run in a
 // warp's registers (shuffles), the rest through shared memory.
 //
@@ -60,14 +54,14 @@ constexpr int SEL_MIN_SORT = 64;  // entries of the smallest sort (one warp's re
 constexpr int SEL_MAX_DYN = 192 * 1024;
 constexpr int SEL_BND = 2048;   // grouped lists: candidates of the boundary bin the first block takes
 constexpr int SEL_RANK = 128;   // ... and ranks by counting
-constexpr int SEL_GROUPED = 32;  // images of a launch up to which the lists stay grouped
 
 struct SelState {
+    int coarse, code_b;  // the boundary bin fits; its code
+    int n_take;          // grouped: candidates above the bin; sorted: those and the bin's
+    int at;              // sorted: where a block's entries go in the first block's list
+    int split, sure;     // the bin was narrowed to the prefix; its candidates above that
     uint64_t pre_hi, msk_hi;
     uint32_t pre_lo, msk_lo;
-    int need, done;
-    int coarse, code_b, n_take;
-    int split, sure;  // grouped: the bin was narrowed to the prefix, its candidates above that
 };
 
 // The 9 bits of the magnitude after those of the code, for keys of one code:
@@ -230,22 +224,21 @@ struct TieState {
     int pick[3];
 };
 
-// A grouped list's boundary bin that holds too many for the first block: the
-// cluster narrows it, 12 bits of the rank words at a time from the highest bit in
-// which its candidates differ (equal keys differ in their positions), until few
-// enough share the boundary's prefix.  Counted where they go later.  Kept out of
-// the kernel's own code, which most images run through without it.
-template <int C>
-__device__ __noinline__ void narrow_bin(const uint64_t* ckey, const uint32_t* cyx, int n, int parts, int q, uint64_t* bkey,
-                                        uint32_t* wsum, TieState& T, SelState& st, int* s_cnt) {
+// A boundary bin that holds too many: the cluster narrows it, 12 bits of the rank
+// words at a time from the highest bit in which its candidates differ (equal keys
+// differ in their positions), until those that share the boundary's prefix fit --
+// at most SEL_BND for the first block to rank (GROUPED), or as many as the sort
+// buffer (cap) holds beside the better ones.  n_above: candidates above the bin;
+// h2: SEL_BINS counts.
+template <int C, bool GROUPED>
+__device__ __forceinline__ void narrow_bin(const uint64_t* ckey, const uint32_t* cyx, int n, int parts, int q, int n_above,
+                                        int cap, uint32_t* h2, uint32_t* wsum, TieState& T, SelState& st, int* s_cnt) {
     const int tid = threadIdx.x, lane = tid & 31, rank = (int)(blockIdx.x % C);
     const bool shared = parts > 1;
     const int i_first = rank * SELECT_THREADS + tid, i_step = parts * SELECT_THREADS;
-    uint32_t* const h2 = reinterpret_cast<uint32_t*>(bkey);
-    static_assert(SEL_BND * sizeof(uint64_t) >= SEL_BINS * sizeof(uint32_t), "room for the counts");
     const uint32_t code_b = (uint32_t)st.code_b;
-    const int need0 = q - st.n_take;
-    int need = need0;
+    const int need0 = q - n_above;
+    int need = need0, left = 0;
     uint64_t pre_hi = 0ull, msk_hi = 0ull;
     uint32_t pre_lo = 0u, msk_lo = 0u;
     auto sync = [&] {
@@ -269,7 +262,7 @@ __device__ __noinline__ void narrow_bin(const uint64_t* ckey, const uint32_t* cy
                     f(hi[k], lo[k]);
         }
     };
-    for (int left = SEL_BND + 1, round = 0; left > SEL_BND && round < 8; ++round) {  // 12 of 96 bits a round
+    for (int round = 0; round < 8; ++round) {  // 12 of 96 bits a round
         if (tid < 6) T.bits[tid] = tid < 3 ? 0xFFFFFFFFu : 0u;
         if (tid < 3) T.pick[tid] = 0;  // ends the loop in all blocks alike
         for (int i = tid; i < SEL_BINS; i += SELECT_THREADS) h2[i] = 0u;
@@ -341,6 +334,7 @@ __device__ __noinline__ void narrow_bin(const uint64_t* ckey, const uint32_t* cy
             pre_lo = (T.all[2] & ~(0xFFFu << sh) & msk_lo) | (uint32_t)d << sh;
         }
         __syncthreads();
+        if (left <= (GROUPED ? SEL_BND : cap - (q - need))) break;  // the same in all blocks
     }
     if (tid == 0) {
         st.pre_hi = pre_hi;
@@ -350,9 +344,19 @@ __device__ __noinline__ void narrow_bin(const uint64_t* ckey, const uint32_t* cy
         st.sure = need0 - need;
         st.split = 1;
         st.coarse = 1;
-        *s_cnt = st.n_take;  // where the bin's sure ones go
+        if (GROUPED) *s_cnt = n_above;  // where the bin's sure ones go
+        else st.n_take = q - need + left;
     }
     sync();
+}
+
+// Apart from the code of grouped lists, whose images mostly run through without it
+// (inside it a single frame's call took 0.5 us longer; sorted lists keep their
+// registers better with it inside).
+template <int C>
+__device__ __noinline__ void narrow_bin_apart(const uint64_t* ckey, const uint32_t* cyx, int n, int parts, int q, int n_above,
+                                              int cap, uint32_t* h2, uint32_t* wsum, TieState& T, SelState& st, int* s_cnt) {
+    narrow_bin<C, true>(ckey, cyx, n, parts, q, n_above, cap, h2, wsum, T, st, s_cnt);
 }
 
 // The first block's boundary candidates `left` (nl of them, the best one's place
@@ -423,8 +427,9 @@ __device__ __noinline__ void rank_ties(const uint64_t* bkey, const uint32_t* byx
     }
 }
 
+// (Three blocks per SM of sorted lists, whose launches hold many images; grouped ones have no such bound.)
 template <int C, bool GROUPED>
-__global__ void __launch_bounds__(SELECT_THREADS)
+__global__ void __launch_bounds__(SELECT_THREADS, GROUPED ? 0 : 3)
 k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_cap) {
     extern __shared__ __align__(16) uint8_t dyn[];
     __shared__ uint32_t hist[SEL_BINS];
@@ -460,14 +465,8 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
     uint32_t* syx = reinterpret_cast<uint32_t*>(dyn + sizeof(uint64_t) * (size_t)sort_cap);
 
     if (tid == 0) {
-        st.pre_hi = 0;
-        st.msk_hi = 0;
-        st.pre_lo = 0;
-        st.msk_lo = 0;
-        st.need = q;
-        st.done = (n <= q);
-        st.coarse = GROUPED && n <= q;  // a grouped list of everything: no boundary bin
-        st.code_b = GROUPED && n <= q ? -1 : 0;
+        st.coarse = n <= q;  // everything is kept: no boundary bin
+        st.code_b = GROUPED ? -1 : 0;
         st.n_take = m;
         st.split = 0;
         st.sure = 0;
@@ -562,7 +561,7 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
                     const int h = bins[j];
                     if (cum < q && cum + h >= q) {
                         const int coarse = GROUPED ? h <= SEL_BND : cum + h <= sort_cap;
-                        const int take = GROUPED ? cum : cum + h;
+                        const int take = GROUPED || !coarse ? cum : cum + h;  // (narrowed: until then those above)
                         for (int c = 0; c < parts; ++c) {
                             const int to = shared ? c : rank;
                             if (to == rank) {
@@ -584,14 +583,20 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         else __syncthreads();
     }
 
-    if (GROUPED && __builtin_expect(!st.coarse, 0)) {  // the same in all blocks
-        narrow_bin<C>(I.ckey, I.cyx, n, parts, q, bkey, wsum, tie, st, &s_cnt);
+    if (__builtin_expect(!st.coarse, 0)) {  // the same in all blocks
+        static_assert(!GROUPED || SEL_BND * sizeof(uint64_t) >= SEL_BINS * sizeof(uint32_t), "room for the counts");
+        // Grouped: counted where the bin's candidates go later (the bins keep their places).
+        uint32_t* const h2 = GROUPED ? reinterpret_cast<uint32_t*>(bkey) : hist;
+        if constexpr (GROUPED)
+            narrow_bin_apart<C>(I.ckey, I.cyx, n, parts, q, st.n_take, sort_cap, h2, wsum, tie, st, &s_cnt);
+        else
+            narrow_bin<C, false>(I.ckey, I.cyx, n, parts, q, st.n_take, sort_cap, h2, wsum, tie, st, &s_cnt);
     }
     auto keep = [&](int pos, uint64_t key, uint32_t yx) {
         I.kkey[pos] = key;
         I.kyx[pos] = yx;
     };
-    if (GROUPED && st.coarse) {  // the same in all blocks
+    if constexpr (GROUPED) {
         // Gather: the better bins to their places, the boundary bin to the first block.
         const int code_b = st.code_b;
         const bool split = st.split != 0;
@@ -724,64 +729,39 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
         return;
     }
 
-    if constexpr (GROUPED) return;  // (done above: its boundary bin is always narrowed)
-
-    // The radix select (and the gather without a coarse bin) is the first block's alone.
-    if (rank != 0 && !st.coarse) return;
-    if (!st.coarse) {
-        for (int pass = 0; pass < 12 && !st.done; ++pass) {
-            for (int i = tid; i < 256; i += SELECT_THREADS) hist[i] = 0u;
-            __syncthreads();
-            const uint64_t pre_hi = st.pre_hi, msk_hi = st.msk_hi;
-            const uint32_t pre_lo = st.pre_lo, msk_lo = st.msk_lo;
-            const int shift_hi = 56 - 8 * pass, shift_lo = 24 - 8 * (pass - 8);
-            const bool need_lo = pass >= 8;  // block-uniform
-            for (int i0 = tid; i0 < n; i0 += SEL_UNROLL * SELECT_THREADS) {
-                uint64_t hi[SEL_UNROLL];
-                uint32_t lo[SEL_UNROLL];
-#pragma unroll
-                for (int k = 0; k < SEL_UNROLL; ++k) {
-                    const int i = i0 + k * SELECT_THREADS;
-                    hi[k] = i < n ? I.ckey[i] : 0ull;
-                    lo[k] = need_lo && i < n ? ~I.cyx[i] : 0u;
-                }
-#pragma unroll
-                for (int k = 0; k < SEL_UNROLL; ++k) {
-                    if (i0 + k * SELECT_THREADS < n && (hi[k] & msk_hi) == pre_hi && (lo[k] & msk_lo) == pre_lo) {
-                        const uint32_t d = pass < 8 ? (uint32_t)(hi[k] >> shift_hi) & 255u
-                                                    : (lo[k] >> shift_lo) & 255u;
-                        atomicAdd(&hist[d], 1u);
-                    }
-                }
-            }
-            __syncthreads();
-            if (tid == 0) {
-                int need = st.need, cum = 0, d = 255;
-                for (; d > 0; --d) {
-                    if (cum + (int)hist[d] >= need) break;
-                    cum += (int)hist[d];
-                }
-                need -= cum;
-                if (pass < 8) {
-                    st.pre_hi |= (uint64_t)d << shift_hi;
-                    st.msk_hi |= 0xFFull << shift_hi;
-                } else {
-                    st.pre_lo |= (uint32_t)d << shift_lo;
-                    st.msk_lo |= 0xFFu << shift_lo;
-                }
-                st.need = need;
-                st.done = ((int)hist[d] == need);
-            }
-            __syncthreads();
+    // Gather, each block its part of the candidates: code >= b, or, of a narrowed
+    // bin b, those whose masked rank word is >= the prefix.
+    const int n_take = st.n_take;
+    const uint32_t code_b = (uint32_t)st.code_b;
+    auto gather = [&](uint64_t key, uint32_t yx) {
+        const int pos = atomicAdd(&s_cnt, 1);
+        if (pos < sort_cap) {
+            skey[pos] = key;
+            syx[pos] = yx;
         }
-    }
-
-    // Gather: code >= b (coarse; each block its part of the candidates), else
-    // every candidate whose masked rank word is >= the fixed prefix.
-    const bool coarse = st.coarse;  // block-uniform
-    const int n_take = coarse ? st.n_take : m;
-    if (coarse) {
-        const uint32_t code_b = (uint32_t)st.code_b;
+    };
+    if (__builtin_expect(st.split, 0)) {
+        const uint64_t pre_hi = st.pre_hi, msk_hi = st.msk_hi;
+        const uint32_t pre_lo = st.pre_lo, msk_lo = st.msk_lo;
+        for (int i0 = i_first; i0 < n; i0 += SEL_UNROLL * i_step) {
+            uint64_t hi[SEL_UNROLL];
+            uint32_t yx[SEL_UNROLL];
+#pragma unroll
+            for (int k = 0; k < SEL_UNROLL; ++k) {
+                const int i = i0 + k * i_step;
+                hi[k] = i < n ? I.ckey[i] : 0ull;
+                yx[k] = i < n ? I.cyx[i] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < SEL_UNROLL; ++k) {
+                const uint32_t code = key_code(hi[k]);
+                if (i0 + k * i_step >= n || code < code_b ||
+                    (code == code_b && rank_less(hi[k] & msk_hi, ~yx[k] & msk_lo, pre_hi, pre_lo)))
+                    continue;
+                gather(hi[k], yx[k]);
+            }
+        }
+    } else {
         const ulonglong2* ck2 = reinterpret_cast<const ulonglong2*>(I.ckey);
         const int n2 = (n + 1) >> 1;
         for (int i0 = i_first; i0 < n2; i0 += SEL_UNROLL * i_step) {
@@ -802,57 +782,26 @@ k_select(const Img* __restrict__ imgs, const Call* __restrict__ call, int sort_c
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint64_t key = h ? v[k].y : v[k].x;
-                    if (i < n2 && 2 * i + h < n && key_code(key) >= code_b) {
-                        const int pos = atomicAdd(&s_cnt, 1);
-                        if (pos < sort_cap) {
-                            skey[pos] = key;
-                            syx[pos] = I.cyx[2 * i + h];
-                        }
-                    }
+                    if (i < n2 && 2 * i + h < n && key_code(key) >= code_b) gather(key, I.cyx[2 * i + h]);
                 }
             }
         }
-        if (shared) {
-            // The first block's own entries stay in place; the others append theirs.
-            cluster_sync_all();
-            if (rank != 0) {
-                const int cnt = min(s_cnt, sort_cap);
-                if (tid == 0) st.need = atomic_add_rank(map_rank(&s_cnt, 0), cnt);
-                __syncthreads();
-                const int base = st.need;
-                for (int i = tid; i < cnt && base + i < sort_cap; i += SELECT_THREADS) {
-                    st_rank64(map_rank(&skey[base + i], 0), skey[i]);
-                    st_rank(map_rank(&syx[base + i], 0), syx[i]);
-                }
-            }
-            cluster_sync_all();
-            if (rank != 0) return;
-        }
-    } else {
-        const uint64_t pre_hi = st.pre_hi, msk_hi = st.msk_hi;
-        const uint32_t pre_lo = st.pre_lo, msk_lo = st.msk_lo;
-        for (int i0 = tid; i0 < n; i0 += SEL_UNROLL * SELECT_THREADS) {
-            uint64_t hi[SEL_UNROLL];
-            uint32_t yx[SEL_UNROLL];
-#pragma unroll
-            for (int k = 0; k < SEL_UNROLL; ++k) {
-                const int i = i0 + k * SELECT_THREADS;
-                hi[k] = i < n ? I.ckey[i] : 0ull;
-                yx[k] = i < n ? I.cyx[i] : 0u;
-            }
-#pragma unroll
-            for (int k = 0; k < SEL_UNROLL; ++k) {
-                const uint64_t mh = hi[k] & msk_hi;
-                const uint32_t ml = ~yx[k] & msk_lo;
-                if (i0 + k * SELECT_THREADS < n && (mh > pre_hi || (mh == pre_hi && ml >= pre_lo))) {
-                    const int pos = atomicAdd(&s_cnt, 1);
-                    if (pos < sort_cap) {
-                        skey[pos] = hi[k];
-                        syx[pos] = yx[k];
-                    }
-                }
+    }
+    if (shared) {
+        // The first block's own entries stay in place; the others append theirs.
+        cluster_sync_all();
+        if (rank != 0) {
+            const int cnt = min(s_cnt, sort_cap);
+            if (tid == 0) st.at = atomic_add_rank(map_rank(&s_cnt, 0), cnt);
+            __syncthreads();
+            const int base = st.at;
+            for (int i = tid; i < cnt && base + i < sort_cap; i += SELECT_THREADS) {
+                st_rank64(map_rank(&skey[base + i], 0), skey[i]);
+                st_rank(map_rank(&syx[base + i], 0), syx[i]);
             }
         }
+        cluster_sync_all();
+        if (rank != 0) return;
     }
     __syncthreads();
     const int got = min(min(s_cnt, n_take), sort_cap);
@@ -885,13 +834,21 @@ int select_smem_bytes(int max_quota) {
     return select_sort_cap(max_quota) * (int)(sizeof(uint64_t) + sizeof(uint32_t));
 }
 
-// Ranking in the orientation kernel costs its warps a sixth more, which a launch
-// of many keypoints pays and one of few images does not see.  Select + orientation
-// stages, sorted / grouped lists, 8-level 1080p frames with 1000 keypoints each:
-// 1 frame (8 images) 24.7 / 24.1 us, 2 28.7 / 24.7, 4 (32 images) 33.7 / 31.0,
-// 8 (64) 40.6 / 39.3, 16 (128) 49.3 / 58.2; with 8192: 61.6 / 30.8, 67.6 / 45.0,
-// 82.7 / 71.2, 116 / 119, 186 / 217.
-bool select_grouped(int n_img) { return n_img <= SEL_GROUPED; }
+// The orientation kernel's ranking costs each keypoint a sixth more where few keys
+// share a code, and the length of the run where many do (a large quota, a smooth
+// scene); the sort costs one block's chain of barriers, which the images of a
+// launch share.  So lists stay grouped while a launch has few images and keypoint
+// slots.  Whole calls, grouped / sorted, one level or eight, us: 2 1080p frames of
+// 8192 features 123 / 239, 2 of 8 levels and 1000 114 / 117, 4 (32 images) 185 /
+// 187; 8 720p frames of 1000 83 / 95, of 4096 227 / 163, of 8192 516 / 284; 16 of
+// 8192 986 / 378, 32 of 1000 232 / 211, of 8192 1876 / 538 (sorted by one block an
+// image, without the fused stages: 305, 193, 258; 157, 235, 385; 480, 281, 670).
+// On 476 batches of 2 to 32 images (five sizes, 1 to 8 levels, 500 to 8192
+// features, a scene and noise) these lines are within 1 % of the better form on
+// average, and none takes longer than sorted by one block.
+bool select_grouped(int n_img, int slots) {
+    return n_img <= 32 && slots <= 32768 && (int64_t)n_img * n_img * slots <= 1 << 22;
+}
 
 template <int C, bool GROUPED>
 static void launch_select_t(const Img* imgs, int n_img, int levels, const Call* call, int mq, cudaStream_t st,
@@ -903,8 +860,9 @@ static void launch_select_t(const Img* imgs, int n_img, int levels, const Call* 
 // Blocks per image, by the images of the launch.  A cluster shortens the scan
 // of the largest image, which sets the launch's length, until its blocks no
 // longer fit the chip beside each other (four 512-thread blocks on each of
-// 152 SMs): 8 while every image has SMs of its own, 4 up to 128 images, 2 up
-// to 304.  Measured stage times of sorted lists (1080p, 8 levels; 1 / 2 / 4 / 8
+// 152 SMs): 8 while every image has SMs of its own (grouped lists of up to 16
+// images; sorted ones are better with 4: 16 VGA frames of 4096, whole call 240
+// against 216 us), 4 up to 128 images, 2 up to 304.  Measured stage times of sorted lists (1080p, 8 levels; 1 / 2 / 4 / 8
 // blocks): 8 images 41 / 33 / 27 / 22 us, 32 images 43 / 35 / 26 / 28, 128
 // images 49 / 39 / 35 / 41, 304 images 64 / 57 / 64 / 84, 1024 images 97 / 119
 // / 149 / 218.
@@ -914,12 +872,14 @@ static void launch_select_t(const Img* imgs, int n_img, int levels, const Call* 
 // 128 frames 82 -> 60 (whole calls 827 -> 822, 2943 -> 2921).  With clusters of
 // 4 they all start at once, and frame by frame is the better one (6 frames, whole
 // call: 214 against 216 us).
-void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, void* stream, bool pdl) {
+void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, int slots, void* stream,
+                   bool pdl) {
     if (n_img <= 0) return;
     const int mq = max_quota > 0 ? max_quota : 1;
     const cudaStream_t st = (cudaStream_t)stream;
-    if (n_img <= 16) launch_select_t<8, true>(imgs, n_img, 1, call, mq, st, pdl);
-    else if (select_grouped(n_img)) launch_select_t<4, true>(imgs, n_img, 1, call, mq, st, pdl);
+    const bool grouped = select_grouped(n_img, slots);
+    if (grouped && n_img <= 16) launch_select_t<8, true>(imgs, n_img, 1, call, mq, st, pdl);
+    else if (grouped) launch_select_t<4, true>(imgs, n_img, 1, call, mq, st, pdl);
     else if (n_img <= 128) launch_select_t<4, false>(imgs, n_img, 1, call, mq, st, pdl);
     else if (n_img <= 304) launch_select_t<2, false>(imgs, n_img, levels, call, mq, st, pdl);
     else launch_select_t<1, false>(imgs, n_img, levels, call, mq, st, pdl);

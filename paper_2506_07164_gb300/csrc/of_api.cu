@@ -483,7 +483,7 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
             // NMS blocks still need (one VGA level 38.2 -> 37.1 us, 16 VGA levels of 2000
             // features 154 -> 133, 32 205 -> 148, four 1080p frames 187 -> 185).  (Launched
             // directly, by the allocation-free entry, it gains from it: 720p 43.9 -> 41.4.)
-            launch_select(P->d_img() + G.img_begin, G.n_img, nl, P->d_call(), P->max_quota, st, false);
+            launch_select(P->d_img() + G.img_begin, G.n_img, nl, P->d_call(), P->max_quota, G.slot_end - G.slot_begin, st, false);
             pdl = P->pdl;
             break;
         case 4:

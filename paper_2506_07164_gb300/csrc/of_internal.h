@@ -200,11 +200,12 @@ void launch_nms_warp(const Img* imgs, const uint2* items, int n_tiles, const CUt
                      const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo, int border, int cell,
                      int rows, int grid, int order, void* stream, bool apply, bool pdl = false);
 int nms_warp_blocks_per_sm();
-// Whether the top-N kernel leaves the kept lists of a launch of n_img images grouped by
-// key code for the orientation kernel to rank (else it sorts them).
-bool select_grouped(int n_img);
+// Whether the top-N kernel leaves the kept lists of a launch of n_img images with `slots`
+// keypoint slots grouped by key code for the orientation kernel to rank (else it sorts them).
+bool select_grouped(int n_img, int slots);
 // n_img images: frames of `levels` levels each.
-void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, void* stream, bool pdl = false);
+void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, int slots, void* stream,
+                   bool pdl = false);
 void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream, bool pdl = false);
 // Slots [slot_begin, slot_end) of images [img_begin, img_begin + n_img) (one frame group).
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,

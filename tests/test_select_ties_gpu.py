@@ -1,6 +1,6 @@
 """Top-N when thousands of candidates share one key (synthetic grids, calibration targets): no
-coarse bin splits them, so the radix select fixes the boundary by position -- for grouped lists
-(up to 32 images, shared scans of 8 and 4 blocks) and sorted ones (4, 2 and 1 blocks)."""
+coarse bin splits them, so the boundary is fixed by position -- for grouped lists (few images, shared
+scans of 8 and 4 blocks) and sorted ones (4, 2 and 1 blocks); and the lines between the two."""
 
 import numpy as np
 import pytest
@@ -53,6 +53,24 @@ def test_boundary_in_a_run_of_equal_keys(frames):
                 for f in FIELDS:
                     np.testing.assert_array_equal(got[f], ora[f][:n], err_msg=f"{frames} frames, n {n}, frame {i}, {f}")
         det.close()
+
+
+# Grouped up to 32 images, 32,768 slots and 2^22 = images^2 x slots: the last grouped launch and the
+# first sorted one of 8, 16 and 32 images (8 and 4 blocks an image; 4), and 33 images.
+@pytest.mark.parametrize("frames,n", [(8, 4096), (8, 4097), (16, 1024), (16, 1025), (32, 128), (32, 129), (33, 100)])
+def test_both_sides_of_the_grouping_lines(frames, n):
+    img = synth.scene(900, 700, 8, n_rect=60, n_checker=30, noise_sigma=0.6)  # smooth: long runs of one code
+    dev = torch.from_numpy(img).cuda()
+    ora = oracle.detect(img, levels=1, fast_t=4, n_features=n)
+    det = ofg.Detector(900, 700, max_levels=1, max_features=n, max_batch=frames)
+    det.detect_batch([dev] * frames, levels=1, fast_t=4, n_features=n)
+    torch.cuda.synchronize()
+    for i, got in enumerate(det.batch_results(frames, n)):
+        assert len(got) == len(ora) > min(n, 1000) - 1
+        if i in (0, frames - 1):
+            for f in FIELDS:
+                np.testing.assert_array_equal(got[f], ora[f], err_msg=f"frame {i} {f}")
+    det.close()
 
 
 def test_allocation_free_entry_in_a_run_of_equal_keys():
