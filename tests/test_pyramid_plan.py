@@ -1,4 +1,4 @@
-"""Host planning of the fused pyramid (csrc/of_plan.cpp), compiled with a small driver.
+"""Host planning of the fused pyramid (csrc/of_plan.cpp), compiled with a small program.
 
 Runs and tables: every pixel of every level is owned by one tile; what a tile computes covers what
 it owns and what its later levels read; weights, byte pairs and row offsets give each output's
@@ -15,7 +15,7 @@ import paper_2506_07164_gb300 as ofg
 
 b = sys.modules[ofg.build.__module__]  # the build module (the package exports its function under the same name)
 
-DRIVER = r"""
+PROGRAM = r"""
 #include <algorithm>
 #include <chrono>
 #include <cstdio>
@@ -145,26 +145,26 @@ int main(int, char** a) {
 
 
 @pytest.fixture(scope="module")
-def driver(tmp_path_factory):
+def planner(tmp_path_factory):
     d = tmp_path_factory.mktemp("plan")
-    (d / "driver.cpp").write_text(DRIVER)
-    exe = str(d / "driver")
-    r = subprocess.run(["g++", *b.CXX_FLAGS, str(d / "driver.cpp"), os.path.join(b.CSRC, "of_plan.cpp"), "-o", exe],
+    (d / "planner.cpp").write_text(PROGRAM)
+    exe = str(d / "planner")
+    r = subprocess.run(["g++", *b.CXX_FLAGS, str(d / "planner.cpp"), os.path.join(b.CSRC, "of_plan.cpp"), "-o", exe],
                        capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     return exe
 
 
 @pytest.mark.parametrize("seed", [1, 2, 3])
-def test_runs_and_tables(driver, seed):
-    r = subprocess.run([driver, "c", str(seed)], capture_output=True, text=True)
+def test_runs_and_tables(planner, seed):
+    r = subprocess.run([planner, "c", str(seed)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
     assert int(r.stdout) > 200
 
 
-def test_planning_costs_no_more_than_a_few_tables(driver):
+def test_planning_costs_no_more_than_a_few_tables(planner):
     """64 frame sizes at 8 levels, in short runs (what large batches take): 7 times the resize tables when
     every try of the search made tables and blocks of its own, about half of them with the search on ranges."""
-    r = subprocess.run([driver, "t"], capture_output=True, text=True)
+    r = subprocess.run([planner, "t"], capture_output=True, text=True)
     assert r.returncode == 0
     assert float(r.stdout) < 4.0, r.stdout
