@@ -737,6 +737,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     const int part = strips < 700 ? (s.cell + 2) / 3 : strips < 1200 ? (s.cell + 1) / 2 : s.cell;
     P->strip_rows = std::min(s.cell, std::max(part, 8));
     P->nms_rows = strips < 700 ? 8 : strips < 1200 ? 16 : TILE_H;
+    // Chained launches: six 1080p frames 223 us a call, 234 without; ten 333 against
+    // 342, but 24 with cell tiles 1136 against 1116 and 128 in seven frame groups 3114
+    // against 3104.
     P->pdl = strips < 12000;
     // The threshold pass flags the cells itself when it takes a band's cells in
     // one round; otherwise the general FAST kernel sets them.
@@ -998,11 +1001,12 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     // Untuned plans: the cell-row strips (form 4, which set the cell flags) with
     // an NMS kernel that applies them (no threshold pass).
     // NMS: the per-warp kernel, which spreads its Harris sums over the warps'
-    // own survivors and wins on small items and on many; between (1200 to 8000
-    // strips: one 1080p frame 69.9 against 71.2 us, two 97.8 against 100.5, four
-    // 157.6 against 158.0) the block kernel, whose Harris phase shares a 64-row
-    // tile's survivors.
-    const bool warp_nms = strips < 1200 || strips >= 8000;
+    // own survivors and wins on small items and on many; between (1200 to 3000
+    // strips) the block kernel, whose Harris phase shares a 64-row tile's survivors.
+    // Whole calls, block / per-warp: two 720p frames (1456 strips) 65.9 / 68.1 us,
+    // one 1080p (1640) 70.7 / 73.5; two 1080p (3280) 105.8 / 103.8, 16 VGA (3872)
+    // 122.2 / 116.6, four 1080p (6560) 173.4 / 168.9, one 4K 178.5 / 177.1.
+    const bool warp_nms = strips < 1200 || strips >= 3000;
     P->tun.fast_cell_tiles = P->strip_ok ? 4 : P->cell_tiles ? 1 : 0;
     P->tun.fast_tile_h = 32;
     P->tun.fast_blocks_per_sm = plan_fast_bps(P);

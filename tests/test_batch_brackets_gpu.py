@@ -1,5 +1,5 @@
 """Default dispatch on both sides of every line that a batch's cell-row strips decide: 700 and 1200
-(parts of strips, 8- and 16-row NMS tiles), 8000 (block or per-warp NMS kernel), 12000 (launches
+(parts of strips, 8- and 16-row NMS tiles), 3000 (block or per-warp NMS kernel), 12000 (launches
 chained programmatically or not).  Each frame's records equal those of a call of its own, whose
 forms are another bracket's, and one frame's the oracle's."""
 
@@ -36,7 +36,7 @@ def _sizes(target):
     return out, left
 
 
-@pytest.mark.parametrize("line", [700, 1200, 8000, 12000])
+@pytest.mark.parametrize("line", [700, 1200, 3000, 12000])
 @pytest.mark.parametrize("below", [True, False])
 def test_both_sides_of_every_line(line, below):
     sizes, left = _sizes(line - 1 if below else line)
