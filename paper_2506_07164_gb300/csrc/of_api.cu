@@ -728,9 +728,9 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
     // 240 for a VGA frame of 8 levels, 1640 for a 1080p one).  The per-warp kernels
     // hold 2432 warps: fewer items than that leave warps idle while each item's
     // rows run one after another, so small batches get thirds or halves of a strip
-    // and 8- or 16-row NMS tiles (one VGA frame, whole call: 52 us with full items,
-    // 43 with thirds and 8 rows; three: 64, 57 with halves and 16 rows; one 1080p
-    // frame: 83 either way).
+    // and 8- or 16-row NMS tiles (one VGA frame, whole call: 43.6 us with full items,
+    // 41.0 with halves and 16 rows, 37.5 with thirds and 8; three: 53.3, 48.1, 51.5;
+    // one 1080p frame: 71.1, 71.8, 73.3).
     int64_t strips = 0;
     for (const auto& L : P->lay.img)
         if (L.det) strips += (int64_t)L.tiles_x * L.ncy;
