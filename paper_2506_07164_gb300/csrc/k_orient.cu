@@ -249,15 +249,15 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
 }
 
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,
-                         void* stream, const uint16_t* slot_img, bool pdl) {
+                         bool grouped, void* stream, const uint16_t* slot_img, bool pdl) {
     if (slot_end <= slot_begin || n_img <= 0) return;
     const int blocks = (slot_end - slot_begin + ORIENT_WARPS - 1) / ORIENT_WARPS;
-    launch_chain(select_grouped(n_img, slot_end - slot_begin) ? k_orient<true> : k_orient<false>, blocks, ORIENT_WARPS * 32,
-                 0, (cudaStream_t)stream, pdl, 1, imgs, img_begin, n_img, slot_begin, slot_end, call, slot_img);
+    launch_chain(grouped ? k_orient<true> : k_orient<false>, blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream, pdl, 1, imgs,
+                 img_begin, n_img, slot_begin, slot_end, call, slot_img);
 }
 
-void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream, bool pdl) {
-    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, stream, nullptr, pdl);
+void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, bool grouped, void* stream, bool pdl) {
+    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, grouped, stream, nullptr, pdl);
 }
 
 // ---------------------------------------------------------------- inspect

@@ -38,6 +38,7 @@
 // ranks of grouped lists.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "of_internal.h"
@@ -835,19 +836,19 @@ int select_smem_bytes(int max_quota) {
 }
 
 // The orientation kernel's ranking costs each keypoint a sixth more where few keys
-// share a code, and the length of the run where many do (a large quota, a smooth
-// scene); the sort costs one block's chain of barriers, which the images of a
-// launch share.  So lists stay grouped while a launch has few images and keypoint
-// slots.  Whole calls, grouped / sorted, one level or eight, us: 2 1080p frames of
-// 8192 features 123 / 239, 2 of 8 levels and 1000 114 / 117, 4 (32 images) 185 /
-// 187; 8 720p frames of 1000 83 / 95, of 4096 227 / 163, of 8192 516 / 284; 16 of
-// 8192 986 / 378, 32 of 1000 232 / 211, of 8192 1876 / 538 (sorted by one block an
-// image, without the fused stages: 305, 193, 258; 157, 235, 385; 480, 281, 670).
-// On 476 batches of 2 to 32 images (five sizes, 1 to 8 levels, 500 to 8192
-// features, a scene and noise) these lines are within 1 % of the better form on
-// average, and none takes longer than sorted by one block.
-bool select_grouped(int n_img, int slots) {
-    return n_img <= 32 && slots <= 32768 && (int64_t)n_img * n_img * slots <= 1 << 22;
+// share a code, and the length of its run where many do (a smooth scene): with n_l
+// keypoints over a fixed number of codes, n_l^2 an image, 0.75 us per million.  The
+// sort is one block's chain of barriers, which the images of a launch share: 6 us
+// for 1000 keypoints, 15 for 2000, 55 for 4096, 150 for 8192, so at least three
+// times the largest image's ranking.  Lists stay grouped while the images' n_l^2 add
+// up to at most four times the largest's (a frame of 8 levels counts 1.9), or to no
+// more than a short sort costs.  Whole calls, grouped / sorted, us: two 1080p levels
+// of 8192 features 123 / 239, two 1080p frames of 8 levels and 8192 137 / 156, and
+// 1000 114 / 117; 8 720p levels of 1000 83 / 95, of 4096 227 / 163, of 8192 516 / 284;
+// 16 of 8192 986 / 378; 32 of 1000 232 / 211, of 8192 1876 / 538 (sorted by one block
+// an image, without the fused stages: 351, 246, 193; 157, 235, 385; 480; 281, 670).
+bool select_grouped(int n_img, int64_t quota_sq, int max_quota) {
+    return n_img <= 32 && quota_sq <= std::max<int64_t>(4ll * max_quota * max_quota, 16000000);
 }
 
 template <int C, bool GROUPED>
@@ -872,12 +873,11 @@ static void launch_select_t(const Img* imgs, int n_img, int levels, const Call* 
 // 128 frames 82 -> 60 (whole calls 827 -> 822, 2943 -> 2921).  With clusters of
 // 4 they all start at once, and frame by frame is the better one (6 frames, whole
 // call: 214 against 216 us).
-void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, int slots, void* stream,
+void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, bool grouped, void* stream,
                    bool pdl) {
     if (n_img <= 0) return;
     const int mq = max_quota > 0 ? max_quota : 1;
     const cudaStream_t st = (cudaStream_t)stream;
-    const bool grouped = select_grouped(n_img, slots);
     if (grouped && n_img <= 16) launch_select_t<8, true>(imgs, n_img, 1, call, mq, st, pdl);
     else if (grouped) launch_select_t<4, true>(imgs, n_img, 1, call, mq, st, pdl);
     else if (n_img <= 128) launch_select_t<4, false>(imgs, n_img, 1, call, mq, st, pdl);

@@ -228,6 +228,7 @@ struct Plan {
         int fal_tiles = 0, fal_off = 0;             // cell-aligned FAST: tiles and prefix offset in gp_fal
         int n_bands = 0, rp_off = 0;                // threshold pass: cell rows and prefix offset in gp_rows
         int slot_begin = 0, slot_end = 0;
+        bool grouped = false;                       // kept lists grouped by key code (select_grouped)
         std::vector<int> rs_job, rs_n;              // per level: first resize job, jobs
         std::vector<int> rsp_off[2], rs_tiles[2];   // per level and resize tile height
         std::vector<int> py_off, py_n;              // per fused run: its tiles in items_py
@@ -484,11 +485,11 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
             // NMS blocks still need (one VGA level 38.2 -> 37.1 us, 16 VGA levels of 2000
             // features 154 -> 133, 32 205 -> 148, four 1080p frames 187 -> 185).  (Launched
             // directly, by the allocation-free entry, it gains from it: 720p 43.9 -> 41.4.)
-            launch_select(P->d_img() + G.img_begin, G.n_img, nl, P->d_call(), P->max_quota, G.slot_end - G.slot_begin, st, false);
+            launch_select(P->d_img() + G.img_begin, G.n_img, nl, P->d_call(), P->max_quota, G.grouped, st, false);
             pdl = P->pdl;
             break;
         case 4:
-            launch_orient_range(P->d_img(), G.img_begin, G.n_img, G.slot_begin, G.slot_end, P->d_call(), st,
+            launch_orient_range(P->d_img(), G.img_begin, G.n_img, G.slot_begin, G.slot_end, P->d_call(), G.grouped, st,
                                 P->n_img <= 65536 ? P->d_sli() : nullptr, pdl);
             break;
     }
@@ -941,6 +942,14 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                 G.n_bands += I.ncy;
             }
             G.slot_begin = P->h_img[G.img_begin].slot0;
+            int64_t quota_sq = 0;
+            int quota = 0;
+            for (int i = G.img_begin; i < G.img_begin + G.n_img; ++i) {
+                const Img& I = P->h_img[i];
+                quota_sq += (int64_t)I.quota * I.quota;
+                quota = std::max(quota, I.quota);
+            }
+            G.grouped = select_grouped(G.n_img, quota_sq, quota);
             G.slot_end = f1 < nf ? P->h_img[f1 * nl].slot0 : P->total_slots;
             G.rs_job.assign(nl + 1, 0);
             G.rs_n.assign(nl + 1, 0);

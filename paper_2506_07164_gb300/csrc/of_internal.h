@@ -200,16 +200,18 @@ void launch_nms_warp(const Img* imgs, const uint2* items, int n_tiles, const CUt
                      const CUtensorMap* score_maps, const Call* call, int t_hi, int t_lo, int border, int cell,
                      int rows, int grid, int order, void* stream, bool apply, bool pdl = false);
 int nms_warp_blocks_per_sm();
-// Whether the top-N kernel leaves the kept lists of a launch of n_img images with `slots`
-// keypoint slots grouped by key code for the orientation kernel to rank (else it sorts them).
-bool select_grouped(int n_img, int slots);
+// Whether the top-N kernel leaves the kept lists of a launch of n_img images grouped by key
+// code for the orientation kernel to rank (else it sorts them); quota_sq: the sum of the
+// images' squared quotas.
+bool select_grouped(int n_img, int64_t quota_sq, int max_quota);
 // n_img images: frames of `levels` levels each.
-void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, int slots, void* stream,
+void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, bool grouped, void* stream,
                    bool pdl = false);
-void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, void* stream, bool pdl = false);
+void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, bool grouped, void* stream,
+                   bool pdl = false);
 // Slots [slot_begin, slot_end) of images [img_begin, img_begin + n_img) (one frame group).
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,
-                         void* stream, const uint16_t* slot_img = nullptr, bool pdl = false);
+                         bool grouped, void* stream, const uint16_t* slot_img = nullptr, bool pdl = false);
 // S(p) of image `img` from a dense w x h copy of its map (offset scores):
 // the per-cell thresholds and proposal tiles applied, t_lo - 1 added back.
 void launch_inspect_score_final(const Img* imgs, int img, uint8_t* d, int w, int h, int t_hi, int t_lo, int border,

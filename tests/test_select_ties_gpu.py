@@ -55,9 +55,11 @@ def test_boundary_in_a_run_of_equal_keys(frames):
         det.close()
 
 
-# Grouped up to 32 images, 32,768 slots and 2^22 = images^2 x slots: the last grouped launch and the
-# first sorted one of 8, 16 and 32 images (8 and 4 blocks an image; 4), and 33 images.
-@pytest.mark.parametrize("frames,n", [(8, 4096), (8, 4097), (16, 1024), (16, 1025), (32, 128), (32, 129), (33, 100)])
+# Grouped up to 32 images whose squared quotas add up to 16 million or four times the largest: the last
+# grouped launch and the first sorted one of 5, 16 and 32 images (8 and 4 blocks an image; 4), four images
+# of any quota, and 33 images.
+@pytest.mark.parametrize("frames,n", [(8, 4096), (8, 4097), (16, 1024), (16, 1025), (32, 128), (32, 129), (33, 100),
+                                      (4, 8192), (5, 1788), (5, 1789), (16, 1000), (16, 1001), (32, 707), (32, 708)])
 def test_both_sides_of_the_grouping_lines(frames, n):
     img = synth.scene(900, 700, 8, n_rect=60, n_checker=30, noise_sigma=0.6)  # smooth: long runs of one code
     dev = torch.from_numpy(img).cuda()
