@@ -878,10 +878,14 @@ void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int
     if (n_img <= 0) return;
     const int mq = max_quota > 0 ? max_quota : 1;
     const cudaStream_t st = (cudaStream_t)stream;
+    // Sorted lists of large quotas: no more blocks than are resident at once, by their shared
+    // memory (whole calls of 40 VGA levels of 4096 features: 352 us with four blocks each, 286
+    // with two; of 96 720p levels of 8192: 1351 and 1167).
+    const int per_sm = std::min(4, (227 * 1024) / (select_smem_bytes(mq) + 18 * 1024)), fit = 152 * std::max(per_sm, 1);
     if (grouped && n_img <= 16) launch_select_t<8, true>(imgs, n_img, 1, call, mq, st, pdl);
     else if (grouped) launch_select_t<4, true>(imgs, n_img, 1, call, mq, st, pdl);
-    else if (n_img <= 128) launch_select_t<4, false>(imgs, n_img, 1, call, mq, st, pdl);
-    else if (n_img <= 304) launch_select_t<2, false>(imgs, n_img, levels, call, mq, st, pdl);
+    else if (n_img <= 128 && 4 * n_img <= fit) launch_select_t<4, false>(imgs, n_img, 1, call, mq, st, pdl);
+    else if (n_img <= 304 && 2 * n_img <= fit) launch_select_t<2, false>(imgs, n_img, levels, call, mq, st, pdl);
     else launch_select_t<1, false>(imgs, n_img, levels, call, mq, st, pdl);
 }
 
