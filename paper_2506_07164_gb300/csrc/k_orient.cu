@@ -37,7 +37,7 @@ namespace ofk {
 constexpr int OP_WORDS = 9;                   // aligned words that hold any 31 bytes
 constexpr int OP_SIZE = 31 * OP_WORDS;        // words of a patch
 
-template <bool GROUPED>
+template <bool GROUPED, bool SPARSE>
 __global__ void __launch_bounds__(ORIENT_WARPS * 32)
 k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin, int slot_end,
          const Call* __restrict__ call, const uint16_t* __restrict__ slot_img) {
@@ -62,14 +62,22 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
     const Img& I = imgs[lo];
     const int idx = slot - I.slot0;  // the keypoint in the image's list
     const int levels = call->levels, n_features = call->n_features;
+    const int quota = I.quota, frame = I.frame;
+    const int32_t* const ctr = I.ctr;
+    if (SPARSE) {
+        // More slots than the images can be expected to fill: those beyond their list go
+        // before the rest is read (96 160 x 120 frames of 8192 features, whole call 151 us
+        // otherwise, 132 so; with full lists the later reads would cost 4 % of this kernel).
+        pdl_wait();
+        if (slot != frame * n_features && (idx >= quota || idx >= ctr[1])) return;
+    }
     // Descriptor fields, read before the wait; lane l < levels: level l's counters.
     const uint8_t* const img = I.img;
     const uint8_t* const score = I.score;
     const float* const fx = I.fx;
     const float* const fy = I.fy;
-    const int pitch = I.pitch, spitch = I.spitch, quota = I.quota, level = I.level, frame = I.frame;
+    const int pitch = I.pitch, spitch = I.spitch, level = I.level;
     const int width = I.w, height = I.h;
-    const int32_t* const ctr = I.ctr;
     const int32_t* const lctr = lane < levels ? imgs[frame * levels + lane].ctr : nullptr;
     const uint32_t* const kyx = I.kyx;
     const uint64_t* const kkey = I.kkey;
@@ -249,15 +257,18 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
 }
 
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,
-                         bool grouped, void* stream, const uint16_t* slot_img, bool pdl) {
+                         bool grouped, bool sparse, void* stream, const uint16_t* slot_img, bool pdl) {
     if (slot_end <= slot_begin || n_img <= 0) return;
     const int blocks = (slot_end - slot_begin + ORIENT_WARPS - 1) / ORIENT_WARPS;
-    launch_chain(grouped ? k_orient<true> : k_orient<false>, blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream, pdl, 1, imgs,
-                 img_begin, n_img, slot_begin, slot_end, call, slot_img);
+    const auto kernel = grouped ? (sparse ? k_orient<true, true> : k_orient<true, false>)
+                                : (sparse ? k_orient<false, true> : k_orient<false, false>);
+    launch_chain(kernel, blocks, ORIENT_WARPS * 32, 0, (cudaStream_t)stream, pdl, 1, imgs, img_begin, n_img, slot_begin,
+                 slot_end, call, slot_img);
 }
 
-void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, bool grouped, void* stream, bool pdl) {
-    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, grouped, stream, nullptr, pdl);
+void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, bool grouped, bool sparse, void* stream,
+                   bool pdl) {
+    launch_orient_range(imgs, 0, n_img, 0, total_slots, call, grouped, sparse, stream, nullptr, pdl);
 }
 
 // ---------------------------------------------------------------- inspect

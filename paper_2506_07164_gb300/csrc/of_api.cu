@@ -229,6 +229,7 @@ struct Plan {
         int n_bands = 0, rp_off = 0;                // threshold pass: cell rows and prefix offset in gp_rows
         int slot_begin = 0, slot_end = 0;
         bool grouped = false;                       // kept lists grouped by key code (select_grouped)
+        bool sparse = false;                        // slots many for the images (orient_sparse)
         std::vector<int> rs_job, rs_n;              // per level: first resize job, jobs
         std::vector<int> rsp_off[2], rs_tiles[2];   // per level and resize tile height
         std::vector<int> py_off, py_n;              // per fused run: its tiles in items_py
@@ -489,7 +490,7 @@ void enqueue_group_stage(of_handle* H, Plan* P, const Plan::Group& G, int stage,
             pdl = P->pdl;
             break;
         case 4:
-            launch_orient_range(P->d_img(), G.img_begin, G.n_img, G.slot_begin, G.slot_end, P->d_call(), G.grouped, st,
+            launch_orient_range(P->d_img(), G.img_begin, G.n_img, G.slot_begin, G.slot_end, P->d_call(), G.grouped, G.sparse, st,
                                 P->n_img <= 65536 ? P->d_sli() : nullptr, pdl);
             break;
     }
@@ -942,15 +943,17 @@ int build_plan(of_handle* H, const std::vector<FrameKey>& frames, const Settings
                 G.n_bands += I.ncy;
             }
             G.slot_begin = P->h_img[G.img_begin].slot0;
-            int64_t quota_sq = 0;
+            int64_t quota_sq = 0, px = 0;
             int quota = 0;
             for (int i = G.img_begin; i < G.img_begin + G.n_img; ++i) {
                 const Img& I = P->h_img[i];
                 quota_sq += (int64_t)I.quota * I.quota;
                 quota = std::max(quota, I.quota);
+                if (I.tiles_x > 0) px += (int64_t)(I.w - 2 * s.border) * (I.h - 2 * s.border);
             }
             G.grouped = select_grouped(G.n_img, quota_sq, quota);
             G.slot_end = f1 < nf ? P->h_img[f1 * nl].slot0 : P->total_slots;
+            G.sparse = orient_sparse(G.slot_end - G.slot_begin, px);
             G.rs_job.assign(nl + 1, 0);
             G.rs_n.assign(nl + 1, 0);
             for (int v = 0; v < 2; ++v) {

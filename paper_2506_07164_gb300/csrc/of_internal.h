@@ -207,11 +207,15 @@ bool select_grouped(int n_img, int64_t quota_sq, int max_quota);
 // n_img images: frames of `levels` levels each.
 void launch_select(const Img* imgs, int n_img, int levels, const Call* call, int max_quota, bool grouped, void* stream,
                    bool pdl = false);
-void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, bool grouped, void* stream,
+// sparse: more than one slot for 8 pixels that detection covers, which images do not fill (4800 pixels
+// of a dense scene have some 300 maxima): k_orient looks at the count before the rest.
+inline bool orient_sparse(int64_t slots, int64_t detect_px) { return 8 * slots > detect_px; }
+void launch_orient(const Img* imgs, int n_img, const Call* call, int total_slots, bool grouped, bool sparse, void* stream,
                    bool pdl = false);
 // Slots [slot_begin, slot_end) of images [img_begin, img_begin + n_img) (one frame group).
 void launch_orient_range(const Img* imgs, int img_begin, int n_img, int slot_begin, int slot_end, const Call* call,
-                         bool grouped, void* stream, const uint16_t* slot_img = nullptr, bool pdl = false);
+                         bool grouped, bool sparse, void* stream, const uint16_t* slot_img = nullptr,
+                         bool pdl = false);
 // S(p) of image `img` from a dense w x h copy of its map (offset scores):
 // the per-cell thresholds and proposal tiles applied, t_lo - 1 added back.
 void launch_inspect_score_final(const Img* imgs, int img, uint8_t* d, int w, int h, int t_hi, int t_lo, int border,

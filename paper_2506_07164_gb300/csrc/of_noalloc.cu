@@ -234,7 +234,7 @@ extern "C" int of_detect_level_noalloc(const uint8_t* img, int w, int h, int pit
     launch_nms_harris(d_img, d_list, d_list + 1, 1, tiles, d_maps, d_maps + 1, d_call, fast_t, t_lo, border, cell,
                       grid_nms, 0, st, false, TILE_H, true);
     launch_select(d_img, 1, 1, d_call, quota, true, st, tiles > 0);
-    launch_orient(d_img, 1, d_call, n_features, true, st, true);
+    launch_orient(d_img, 1, d_call, n_features, true, orient_sparse(n_features, det ? (int64_t)rw * rh : 0), st, true);
     e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(OF_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     return OF_OK;

@@ -62,7 +62,7 @@ void launch_nms_harris(const Img*, const int32_t*, const int32_t*, int, int n_ti
     if (n_tiles > 0) std::printf("nms %d\n", pdl);
 }
 void launch_select(const Img*, int, int, const Call*, int, bool, void*, bool pdl) { std::printf("select %d\n", pdl); }
-void launch_orient(const Img*, int, const Call*, int total_slots, bool, void*, bool pdl) {
+void launch_orient(const Img*, int, const Call*, int total_slots, bool, bool, void*, bool pdl) {
     if (total_slots > 0) std::printf("orient %d\n", pdl);
 }
 }  // namespace ofk

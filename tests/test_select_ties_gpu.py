@@ -75,6 +75,26 @@ def test_both_sides_of_the_grouping_lines(frames, n):
     det.close()
 
 
+# More slots than the frames can fill, from one for 8 pixels of their 80 x 60 up: the orientation
+# kernel looks at the count first.  Grouped lists (1 frame), sorted ones (33), several levels, none.
+@pytest.mark.parametrize("frames,levels,n", [(1, 1, 600), (1, 1, 601), (33, 1, 600), (33, 1, 601), (33, 1, 4096), (2, 3, 4096),
+                                             (40, 3, 4096)])
+@pytest.mark.parametrize("size", [(118, 98), (38, 60)])
+def test_slots_beyond_the_keypoints(frames, levels, n, size):
+    w, h = size
+    img = np.ascontiguousarray(synth.scene(640, 480, 8, n_rect=60, n_checker=30)[100 : 100 + h, 200 : 200 + w])
+    dev = torch.from_numpy(img).cuda()
+    ora = oracle.detect(img, levels=levels, fast_t=4, n_features=n)
+    det = ofg.Detector(w, h, max_levels=levels, max_features=n, max_batch=frames)
+    det.detect_batch([dev] * frames, levels=levels, fast_t=4, n_features=n)
+    torch.cuda.synchronize()
+    for i, got in enumerate(det.batch_results(frames, n)):
+        assert len(got) == len(ora)
+        for f in FIELDS:
+            np.testing.assert_array_equal(got[f], ora[f], err_msg=f"frame {i} {f}")
+    det.close()
+
+
 def test_allocation_free_entry_in_a_run_of_equal_keys():
     img = _grid()
     h, w = img.shape
