@@ -317,7 +317,7 @@ FAST_OPS_PER_PX = 40.5
 # levels, divided by the frames.  Valid while the kernels' code
 # (kernels_sha1) and the per-stage launch choices below are the ones captured;
 # otherwise the line reports null.
-STAGE_TRAFFIC = {"code_sha1": "5dd2d09191308a5b3108080edb32182e00b0622f", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18822407, "fast": 30957815, "nms_harris": 39787938, "select": 2696679, "orient": 2621280}, "dram_bytes_per_frame": {"pyramid": 5594228, "fast": 12762532, "nms_harris": 16263324, "select": 1041100, "orient": 547784}}
+STAGE_TRAFFIC = {"code_sha1": "3be1c7debac274f90385577e4011f00f5d532167", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18866905, "fast": 30960126, "nms_harris": 39819129, "select": 2697469, "orient": 2623437}, "dram_bytes_per_frame": {"pyramid": 5586128, "fast": 12761732, "nms_harris": 16288680, "select": 1038800, "orient": 547832}}
 
 
 def code_sha1(path):
