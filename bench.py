@@ -317,7 +317,7 @@ FAST_OPS_PER_PX = 40.5
 # levels, divided by the frames.  Valid while the kernels' code
 # (kernels_sha1) and the per-stage launch choices below are the ones captured;
 # otherwise the line reports null.
-STAGE_TRAFFIC = {"code_sha1": "3be1c7debac274f90385577e4011f00f5d532167", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18866905, "fast": 30960126, "nms_harris": 39819129, "select": 2697469, "orient": 2623437}, "dram_bytes_per_frame": {"pyramid": 5586128, "fast": 12761732, "nms_harris": 16288680, "select": 1038800, "orient": 547832}}
+STAGE_TRAFFIC = {"code_sha1": "3fa530d3a6a60f381588e8541b378134b76ed377", "frames": 64, "tuning": {"resize_tma": 1, "resize_tile_h": 64, "fast_cell_tiles": 4, "fast_tile_h": 32, "nms_tile_h": 32}, "l2_bytes_per_frame": {"pyramid": 18828605, "fast": 31466758, "nms_harris": 40388239, "select": 2701252, "orient": 2631057}, "dram_bytes_per_frame": {"pyramid": 5580892, "fast": 12775568, "nms_harris": 16323124, "select": 1040636, "orient": 547864}}
 
 
 def code_sha1(path):

@@ -69,7 +69,10 @@ k_orient(const Img* __restrict__ imgs, int img_begin, int n_img, int slot_begin,
         // before the rest is read (96 160 x 120 frames of 8192 features, whole call 151 us
         // otherwise, 132 so; with full lists the later reads would cost 4 % of this kernel).
         pdl_wait();
-        if (slot != frame * n_features && (idx >= quota || idx >= ctr[1])) return;
+        if (slot != frame * n_features && (idx >= quota || idx >= ctr[1])) {
+            pdl_wait();  // long over: every exit stands directly behind a wait
+            return;
+        }
     }
     // Descriptor fields, read before the wait; lane l < levels: level l's counters.
     const uint8_t* const img = I.img;
